@@ -72,12 +72,12 @@ def draw(rng):
     elif what == "split":
         n_rep = rng.choice([1, 1, 2, 2, 3])
         over = rng.random() < 0.15   # auxiliary sets beyond 64, with small orbital sets
-        c = _eval("", "diamond", min(n_rep, 2) if over else n_rep, str(rng.randint(3, 9) if over else rng.randint(4, 16 if n_rep < 3 else 13)),
+        c = _eval("", "diamond", min(n_rep, 2) if over else n_rep, str(rng.randint(3, 9) if over else rng.randint(4, 15 if n_rep < 3 else 13)),
                   str(rng.randint(65, 80) if over else rng.randint(9, 64 if n_rep < 3 else 50)),
                   round(rng.uniform(2.6, 3.7), 2), rng.choice(["bf16x6", "bf16x6", "bf16x3"]),
                   graph=rng.random() < 0.2, strain=rng.choice([0.0, 0.03]))
     elif what == "ragged":
-        c = _eval("", "perovskite", rng.choice([1, 2, 2]), ",".join(str(rng.randint(3, 16)) for _ in range(3)),
+        c = _eval("", "perovskite", rng.choice([1, 2, 2]), ",".join(str(rng.randint(3, 15)) for _ in range(3)),
                   ",".join(str(rng.randint(9, 64)) for _ in range(3)), round(rng.uniform(3.0, 4.2), 2), "bf16x6",
                   deterministic=rng.random() < 0.3)
     else:
