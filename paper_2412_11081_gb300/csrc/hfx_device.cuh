@@ -1,9 +1,10 @@
 // Device helpers shared by the split-precision translation units
-// (hfx_mixed.cu, hfx_t1umma.cu): index lookups, bf16 splitting, warp sums and
+// (hfx_mixed.cu, hfx_t1umma.cu): index lookups, operand splitting, warp sums and
 // the tcgen05 / mbarrier / bulk-copy wrappers (inline PTX).
 #pragma once
 
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -33,35 +34,63 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
-// x = p0 + p1 (+ p2) + r with p_i bf16, each the round-to-nearest of what the
-// earlier pieces leave.
-template <int NP>
+// Split modes (the plan's precision): every operand is two 16-bit pieces
+// x = p0 + p1 + r, p0 the round-to-nearest of x and p1 of what p0 leaves.
+//   kSplitBf16 (HFX_BF16X3): bf16 pieces, 16 significant bits, any FP32 range
+//   kSplitHalf (HFX_BF16X6): fp16 pieces, 22 significant bits.  fp16 has
+//     five exponent bits, so the stores hold x times a power of two
+//     (SplitScale) that keeps every element's magnitude within 2^15: the low
+//     piece is exact to 2^-25 of the stored scale, so elements down to 2^-18
+//     of that bound keep all 22 bits and the rest an absolute error of 2^-40
+//     of it.  Three products of two such pieces carry what six products of
+//     three bf16 pieces did, at half the tensor-core work and two thirds of
+//     the operand bytes.
+constexpr int NP = kPieces;
+
+// A factor of SplitScale: 1 (and no multiplication) with bf16 pieces.
+template <int SP>
+__device__ __forceinline__ float scf(float s) {
+  return SP == kSplitHalf ? s : 1.f;
+}
+
+template <int SP>
 __device__ __forceinline__ void split_f(float x, uint16_t (&p)[NP]) {
-  float r = x;
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(r);
-    p[i] = __bfloat16_as_ushort(h);
-    r -= __bfloat162float(h);
+  if (SP == kSplitHalf) {
+    const __half h = __float2half_rn(x);
+    p[0] = __half_as_ushort(h);
+    p[1] = __half_as_ushort(__float2half_rn(x - __half2float(h)));
+  } else {
+    const __nv_bfloat16 h = __float2bfloat16_rn(x);
+    p[0] = __bfloat16_as_ushort(h);
+    p[1] = __bfloat16_as_ushort(__float2bfloat16_rn(x - __bfloat162float(h)));
   }
 }
 
-// The same split for four consecutive values, packed as 4 bf16 per piece
-// (element 0 in the low half of .x).
-template <int NP>
-__device__ __forceinline__ void split4(const float (&x)[4], uint2 (&p)[NP]) {
-  float r0 = x[0], r1 = x[1], r2 = x[2], r3 = x[3];
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    const __nv_bfloat162 h01 = __floats2bfloat162_rn(r0, r1);
-    const __nv_bfloat162 h23 = __floats2bfloat162_rn(r2, r3);
-    p[i].x = *reinterpret_cast<const uint32_t*>(&h01);
-    p[i].y = *reinterpret_cast<const uint32_t*>(&h23);
-    r0 -= __low2float(h01);
-    r1 -= __high2float(h01);
-    r2 -= __low2float(h23);
-    r3 -= __high2float(h23);
+// The pieces of two values, x0 in the low half of each word.
+template <int SP>
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t (&p)[NP]) {
+  if (SP == kSplitHalf) {
+    const __half2 h = __floats2half2_rn(x0, x1);
+    const float2 f = __half22float2(h);
+    const __half2 l = __floats2half2_rn(x0 - f.x, x1 - f.y);
+    p[0] = *reinterpret_cast<const uint32_t*>(&h);
+    p[1] = *reinterpret_cast<const uint32_t*>(&l);
+  } else {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - __low2float(h), x1 - __high2float(h));
+    p[0] = *reinterpret_cast<const uint32_t*>(&h);
+    p[1] = *reinterpret_cast<const uint32_t*>(&l);
   }
+}
+
+// The same for four consecutive values (element 0 in the low half of .x).
+template <int SP>
+__device__ __forceinline__ void split4(const float (&x)[4], uint2 (&p)[NP]) {
+  uint32_t a[NP], b[NP];
+  split2<SP>(x[0], x[1], a);
+  split2<SP>(x[2], x[3], b);
+#pragma unroll
+  for (int i = 0; i < NP; ++i) p[i] = make_uint2(a[i], b[i]);
 }
 
 __device__ __forceinline__ int ylut_get(const DevPlan& P, int i, int j, int r0, int r1, int r2) {
@@ -79,54 +108,43 @@ __device__ __forceinline__ int dlut_get(const DevPlan& P, int i, int j, int r0, 
 }
 
 // ------------------------------------------------------------- warp-level MMA
-// bf16 m16n8k16 MMAs with FP32 accumulation, the split products over NP
-// pieces and the ldmatrix loads of their fragments.
+// m16n8k16 MMAs on the pieces with FP32 accumulation, the split products and
+// the ldmatrix loads of their fragments.
 __device__ __forceinline__ uint32_t pack2(uint16_t lo, uint16_t hi) { return (uint32_t)lo | ((uint32_t)hi << 16); }
 
+template <int SP>
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-  asm(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+  if (SP == kSplitHalf)
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+  else
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// All piece products (i, j) with i + j < NP, smallest first.
-template <int NP>
+// The piece products (0,1), (1,0), (0,0), smallest first.
+template <int SP>
 __device__ __forceinline__ void mma_split(float (&c)[4], const uint32_t (&a)[NP][4], const uint32_t (&b)[NP][2]) {
-  if (NP == 3) {
-    mma16816(c, a[1], b[1]);
-    mma16816(c, a[0], b[2]);
-    mma16816(c, a[2], b[0]);
-  }
-  if (NP >= 2) {
-    mma16816(c, a[0], b[1]);
-    mma16816(c, a[1], b[0]);
-  }
-  mma16816(c, a[0], b[0]);
+  mma16816<SP>(c, a[0], b[1]);
+  mma16816<SP>(c, a[1], b[0]);
+  mma16816<SP>(c, a[0], b[0]);
 }
 
 // Two independent accumulators with their product chains interleaved, so the
 // dependent MMAs of one tile overlap the other's.
-template <int NP>
+template <int SP>
 __device__ __forceinline__ void mma_split2(float (&c0)[4], const uint32_t (&a0)[NP][4], const uint32_t (&b0)[NP][2],
                                            float (&c1)[4], const uint32_t (&a1)[NP][4], const uint32_t (&b1)[NP][2]) {
-  if (NP == 3) {
-    mma16816(c0, a0[1], b0[1]);
-    mma16816(c1, a1[1], b1[1]);
-    mma16816(c0, a0[0], b0[2]);
-    mma16816(c1, a1[0], b1[2]);
-    mma16816(c0, a0[2], b0[0]);
-    mma16816(c1, a1[2], b1[0]);
-  }
-  if (NP >= 2) {
-    mma16816(c0, a0[0], b0[1]);
-    mma16816(c1, a1[0], b1[1]);
-    mma16816(c0, a0[1], b0[0]);
-    mma16816(c1, a1[1], b1[0]);
-  }
-  mma16816(c0, a0[0], b0[0]);
-  mma16816(c1, a1[0], b1[0]);
+  mma16816<SP>(c0, a0[0], b0[1]);
+  mma16816<SP>(c1, a1[0], b1[1]);
+  mma16816<SP>(c0, a0[1], b0[0]);
+  mma16816<SP>(c1, a1[1], b1[0]);
+  mma16816<SP>(c0, a0[0], b0[0]);
+  mma16816<SP>(c1, a1[0], b1[0]);
 }
 
 __device__ __forceinline__ void ldm_x4(uint32_t (&r)[4], const void* p) {
@@ -169,11 +187,13 @@ __device__ __forceinline__ uint64_t sdesc2(uint32_t saddr, uint32_t lbo, uint32_
   return d;
 }
 
-// Instruction descriptor of kind::f16 with bf16 A and B, FP32 accumulator;
-// b_mn = 1 reads B as MN-major.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int b_mn) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_mn << 16) | ((uint32_t)(N >> 3) << 17) |
-         ((uint32_t)(M >> 4) << 24);
+// Instruction descriptor of kind::f16 with A and B of the split's piece type
+// (fp16 or bf16, both operands alike), FP32 accumulator; b_mn = 1 reads B as
+// MN-major.
+template <int SP>
+__host__ __device__ constexpr uint32_t idesc_split(int M, int N, int b_mn) {
+  return (1u << 4) | (SP == kSplitHalf ? 0u : (1u << 7) | (1u << 10)) | ((uint32_t)b_mn << 16) |
+         ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 // One potentially blocking test: the thread may sleep in hardware up to
@@ -232,7 +252,7 @@ __device__ __forceinline__ void bulk_g2s(uint32_t sdst, const void* gsrc, uint32
                : "memory");
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void umma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
   asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
                "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));

@@ -183,8 +183,13 @@ struct hfx_plan {
   int beta_chunk = 1, alpha_chunk = 1;
   size_t smem_t1 = 0, smem_t2 = 0;
 
-  // split-precision path (np = bf16 pieces per operand; 0 = FP64 path)
+  // split-precision path (np = pieces per operand; 0 = FP64 path)
   int np = 0;
+  int sp = 0;                  // piece type, hfx::kSplitBf16 or kSplitHalf
+  std::vector<double> cmax;    // [S*S] bound of |C| / f(r)
+  double dmax = 0, vmax = 0, vrow = 0;   // bounds of |D|, |V| and sum_beta |V|
+  double ymax = 0;             // bound of |Y| over the skin of the current lists
+  hfx::SplitScale scale;
   uint16_t* Dsp = nullptr;
   long long* dsp_off = nullptr;
   uint16_t* Ysp = nullptr;
@@ -315,6 +320,10 @@ void upload_model(hfx_plan* P, const hfx_system* sys, const hfx_model* m) {
       msz += (long long)P->n_abf[a] * P->n_abf[b];
     }
   std::vector<double> G(gsz), M(msz), Gp, Mnorm(S * S), Gmom(3 * S * S, 0.0);
+  P->cmax.assign(S * S, 0.0);
+  double elen = 0;   // |d.e| <= |e| R_C where f(r) > 0
+  for (int k = 0; k < 3; ++k) elen += m->aniso_dir[k] * m->aniso_dir[k];
+  elen = m->G_aniso ? std::sqrt(elen) : 0.0;
   if (m->G_aniso) Gp.resize(gsz);
   double mmax = 0;
   for (int a = 0; a < S; ++a)
@@ -336,6 +345,16 @@ void upload_model(hfx_plan* P, const hfx_system* sys, const hfx_model* m) {
         gm[0] += gv * gv;
         gm[1] += gv * gq;
         gm[2] += gq * gq;
+        P->cmax[a * S + b] = std::max(P->cmax[a * S + b], std::fabs(gv) + elen * std::fabs(gq));
+      }
+      for (int x = 0; x < P->n_abf[a]; ++x) {   // h(r) <= 1
+        double row = 0;
+        for (int y = 0; y < P->n_abf[b]; ++y) {
+          const double v = std::fabs(M[moff[a * S + b] + (long long)x * P->n_abf[b] + y]);
+          row += v;
+          P->vmax = std::max(P->vmax, v);
+        }
+        P->vrow = std::max(P->vrow, row);
       }
       Mnorm[a * S + b] = std::sqrt(s2);
       mmax = std::max(mmax, Mnorm[a * S + b]);
@@ -411,6 +430,7 @@ void upload_density(hfx_plan* P, const hfx_model* m) {
   }
   const long long nvals = off[nd];
   if (!finite_all(m->d_values, (size_t)nvals)) fail(HFX_ERR_INVALID, "non-finite D values");
+  for (long long k = 0; k < nvals; ++k) P->dmax = std::max(P->dmax, std::fabs(m->d_values[k]));
   for (int c = 0; c < 3; ++c) P->HD[c] = H[c];
   const long long n0 = 2 * H[0] + 1, n1 = 2 * H[1] + 1, n2 = 2 * H[2] + 1;
   const long long lut_n = (long long)N * N * n0 * n1 * n2;
@@ -495,6 +515,7 @@ DevPlan make_devplan(hfx_plan* P, const double* lattice) {
   D.thdV = P->opt.theta_dV;
   D.thD = P->opt.theta_D;
   D.thCS = P->opt.theta_CS;
+  D.sc = P->scale;
   D.terms = P->opt.terms;
   D.h0 = P->chunks.empty() ? 0 : P->chunks.front().first;
   D.h1 = P->chunks.empty() ? P->N : P->chunks.back().second;
@@ -558,6 +579,39 @@ DevPlan make_devplan(hfx_plan* P, const double* lattice) {
   }
   D.cnt = reinterpret_cast<unsigned long long*>(P->d_tot + kTot);
   return D;
+}
+
+// Powers of two of the fp16 stores (hfx::SplitScale) from the bounds of the
+// blocks: |C| <= cmax f, |D| <= dmax, |V| <= vmax, |Y| <= ymax,
+// |U| <= n_ao dmax ymax, |Z| <= vrow ymax.  bf16 pieces hold the values as
+// they are.
+void set_scale(hfx_plan* P) {
+  P->scale = hfx::SplitScale{};
+  if (P->sp != hfx::kSplitHalf) return;
+  int nao = 1;
+  for (int n : P->n_ao) nao = std::max(nao, n);
+  auto ex = [](double bound) {   // bound * 2^ex in (2^14, 2^15]
+    if (!(bound > 0)) return 0;
+    int k = 0;
+    std::frexp(bound, &k);
+    return std::max(-100, std::min(100, 15 - k));
+  };
+  const int eC = ex(*std::max_element(P->cmax.begin(), P->cmax.end())), eD = ex(P->dmax), eV = ex(P->vmax);
+  const int eY = ex(P->ymax), eU = ex(nao * P->dmax * P->ymax), eZ = ex(P->vrow * P->ymax);
+  auto f = [](int e) { return std::ldexp(1.f, std::max(-126, std::min(127, e))); };
+  hfx::SplitScale& s = P->scale;
+  s.c = f(eC);
+  s.v = f(eV);
+  s.d = f(eD);
+  s.y = f(eY - eC - eD);
+  s.yf = f(-eY);
+  s.u = f(eU - eD - eY);
+  s.uf = f(eU);
+  s.z = f(eZ - eV - eY);
+  s.r1 = std::ldexp(1.0, -eC - eU);
+  s.q1 = std::ldexp(1.0, -eV - eU);
+  s.r2 = std::ldexp(1.0, -2 * eY);
+  s.q2 = std::ldexp(1.0, -eZ - eD);
 }
 
 // Pair lists (K0): C pairs within R_C + skin, V pairs within the V radius
@@ -715,6 +769,25 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
   v_ptr[N] = (int)v_j.size();
   y_ptr[N] = (int)y_j.size();
   const int nC = c_ptr[N], nV = v_ptr[N], nY = y_ptr[N];
+  // bound of |Y^{XZ}| = |sum_W C_XW D_WZ| at every geometry these lists cover
+  // (no pair distance moves by more than the skin before they are rebuilt)
+  P->ymax = 0;
+  for (int A = 0; A < N; ++A) {
+    double y = 0;
+    for (int q = c_ptr[A]; q < c_ptr[A + 1]; ++q) {
+      double d2 = 0;
+      for (int k = 0; k < 3; ++k) {
+        const double dv = pos[3 * c_j[q] + k] + c_R[3 * q] * L[k] + c_R[3 * q + 1] * L[3 + k] +
+                          c_R[3 * q + 2] * L[6 + k] - pos[3 * A + k];
+        d2 += dv * dv;
+      }
+      const double r = std::max(0.0, std::sqrt(d2) - skin), t = std::max(0.0, 1.0 - r * r / (P->RC * P->RC));
+      y += t * t * t * std::exp(-0.5 * r * r) * P->cmax[P->species[A] * P->S + P->species[c_j[q]]] *
+           P->n_ao[P->species[c_j[q]]];
+    }
+    P->ymax = std::max(P->ymax, y * P->dmax);
+  }
+  set_scale(P);
   int maxC = 0, maxV = 0;
   for (int A = 0; A < N; ++A) {
     maxC = std::max(maxC, c_ptr[A + 1] - c_ptr[A]);
@@ -822,7 +895,7 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
     std::vector<long long> cw_off(nC + 1, 0);
     for (int p = 0; p < nC; ++p) {
       const int sA = P->species[c_home[p]], sj = P->species[c_j[p]];
-      cw_off[p + 1] = cw_off[p] + hfx::wide_cpieces_size(P->np, P->n_abf[sA], P->n_ao[sA], P->n_ao[sj]);
+      cw_off[p + 1] = cw_off[p] + hfx::wide_cpieces_size(P->n_abf[sA], P->n_ao[sA], P->n_ao[sj]);
     }
     P->cw_off = P->lalloc<long long>(nC + 1);
     P->Cw = P->lalloc<uint16_t>(std::max(1LL, cw_off[nC]));
@@ -941,13 +1014,13 @@ void setup_shapes(hfx_plan* P) {
   if (P->np && maxAO > 16) {
     // n_ao beyond the 16-column tiles of the tensor-memory kernels: the wide kernels
     P->wide = true;
-    P->ws = hfx::wide_shapes(P->np, maxABF, maxAO, limit);
+    P->ws = hfx::wide_shapes(maxABF, maxAO, limit);
     if (!P->ws.ok) fail(HFX_ERR_UNSUPPORTED, "block shapes too large for the split-precision kernels");
     int maxrows = 0;
     for (int a = 0; a < P->S; ++a) maxrows = std::max(maxrows, P->n_abf[a] * P->n_ao[a]);
     P->wide_RB = hfx::wide_ybuild_row_blocks(maxrows);
     P->wide_maxrows = maxrows;
-    ck(hfx::set_wide_smem_limits(P->np), "smem attributes");
+    ck(hfx::set_wide_smem_limits(P->sp), "smem attributes");
     return;
   }
   if (P->np) {
@@ -967,8 +1040,14 @@ void setup_shapes(hfx_plan* P) {
     P->MC = (maxrows + 127) / 128;
     P->zblk = (long long)P->np * P->MC * 128 * 16;   // 128-row tiles of 16 columns, per piece
     P->YRmax = r16(maxABF * maxAO);
-    P->smem_m1 = hfx::term1_mma_smem(P->np, P->MAmax, P->MBmax, P->KSmax, P->YRmax);
-    P->smem_m2 = hfx::term2_mma_smem(P->np, P->MAmax, P->KZmax);
+    // The accepted shapes of HFX_BF16X6 are those whose operands would fit in
+    // three pieces each; its first-product kernel stages Y too where that fits.
+    const size_t lim = P->sp == hfx::kSplitHalf ? limit * 2 / 3 : limit;
+    if (P->sp == hfx::kSplitHalf && hfx::term1_mma_smem(P->MAmax, P->MBmax, P->KSmax, P->YRmax) > limit) P->YRmax = 0;
+    P->smem_m1 = hfx::term1_mma_smem(P->MAmax, P->MBmax, P->KSmax, P->YRmax);
+    P->smem_m2 = hfx::term2_mma_smem(P->MAmax, P->KZmax);
+    const bool m1_fits = P->sp == hfx::kSplitHalf ? hfx::term1_mma_smem(P->MAmax, P->MBmax, P->KSmax, 0) <= lim
+                                                  : P->smem_m1 <= limit;
     // term 1: each warp owns one alpha tile and ceil(NTq / (16 / MT)) Q tiles (at most 16);
     // the second product's GEMM holds two column tiles per F (n_ao <= 16)
     const int MT = P->MAmax / 16, wpm = MT > 0 ? 16 / MT : 0;
@@ -992,7 +1071,8 @@ void setup_shapes(hfx_plan* P) {
       while (fs > 1 && slots(fs) < 2) --fs;
       P->t1u_FS = fs;
       P->t1u_NS = (int)std::min<long long>(slots(fs), hfx::t1u_max_slots());
-      if (P->t1u_NS >= 2) {
+      const size_t base = hfx::t1u_smem(P->sp == hfx::kSplitHalf ? 3 : 2, P->t1u_KP, 2, 1);
+      if (base <= limit && P->t1u_NS >= 2) {
         P->t1u = true;
         P->smem_t1u = hfx::t1u_smem(P->np, P->t1u_KP, P->t1u_NS, P->t1u_FS);
         // kept B per FP32 run of the Q accumulator: 32 for BF16X3, whose
@@ -1000,23 +1080,23 @@ void setup_shapes(hfx_plan* P) {
         // at most on the jittered si64 geometries against 5.4e-6 with 32,
         // and fewer FP64 flushes)
         const char* sg = std::getenv("HFX_T1_SEG");
-        P->t1u_seg = sg ? std::max(1, std::atoi(sg)) : (P->np == 3 ? 128 : 32);
-        ck(hfx::t1u_set_smem(P->np), "smem attributes");
+        P->t1u_seg = sg ? std::max(1, std::atoi(sg)) : (P->sp == hfx::kSplitHalf ? 128 : 32);
+        ck(hfx::t1u_set_smem(P->sp), "smem attributes");
         // the second product's R2 and Z on tcgen05 as well (HFX_T2_KERNEL=mma keeps the warp-level kernel)
         const char* t2k = std::getenv("HFX_T2_KERNEL");
-        P->smem_t2u = hfx::t2u_smem(P->np, maxAO);
-        if (!(t2k && std::string(t2k) == "mma") && P->smem_t2u <= limit) {
+        P->smem_t2u = hfx::t2u_smem(maxAO);
+        if (!(t2k && std::string(t2k) == "mma") && P->smem_t2u <= lim) {
           P->t2u = true;
-          ck(hfx::t2u_set_smem(P->np), "smem attributes");
+          ck(hfx::t2u_set_smem(P->sp), "smem attributes");
         }
       }
     }
     if (!P->t1u) {
       if (t1k && std::string(t1k) == "umma")
         fail(HFX_ERR_UNSUPPORTED, "HFX_T1_KERNEL=umma: shapes outside the tcgen05 first-product kernel");
-      if (P->smem_m1 > limit || qtiles > 16) fail(HFX_ERR_UNSUPPORTED, "block shapes too large for the split-precision kernels");
+      if (!m1_fits || qtiles > 16) fail(HFX_ERR_UNSUPPORTED, "block shapes too large for the split-precision kernels");
     }
-    if (P->smem_m2 > limit || maxAO > 16)
+    if (P->smem_m2 > lim || maxAO > 16)
       fail(HFX_ERR_UNSUPPORTED, "block shapes too large for the split-precision kernels");
     // 128-row tiles per CTA of the tcgen05 Y build and Q2 GEMM (the autotuner
     // may change them; HFX_Y_TILES = 1 or 2, HFX_Q2_TILES = 1, 2 or 3 set the initial choice)
@@ -1024,10 +1104,10 @@ void setup_shapes(hfx_plan* P) {
     const char* qt = std::getenv("HFX_Q2_TILES");
     P->ybtpc = yt && std::atoi(yt) == 1 ? 1 : 2;
     // (BF16X6 starts from the deep pipeline: si1000 second product 172.6 -> 139.6 ms)
-    P->q2tpc = qt && (std::atoi(qt) >= 1 && std::atoi(qt) <= 3) ? std::atoi(qt) : (P->np == 3 ? 3 : 2);
+    P->q2tpc = qt && (std::atoi(qt) >= 1 && std::atoi(qt) <= 3) ? std::atoi(qt) : (P->sp == hfx::kSplitHalf ? 3 : 2);
     const char* qf = std::getenv("HFX_Q2_FLUSH");
-    P->q2_flush = qf ? std::max(1, std::atoi(qf)) : (P->np == 3 ? 128 : 32);   // as t1u_seg
-    ck(hfx::set_mixed_smem_limits(P->np), "smem attributes");
+    P->q2_flush = qf ? std::max(1, std::atoi(qf)) : (P->sp == hfx::kSplitHalf ? 128 : 32);   // as t1u_seg
+    ck(hfx::set_mixed_smem_limits(P->sp), "smem attributes");
   }
 }
 
@@ -1045,7 +1125,7 @@ void split_density(hfx_plan* P) {
     P->Dw = P->mem.alloc<uint16_t>(off[P->n_d]);
     upload(P->dw_off, off, P->stream);
     DevPlan D = make_devplan(P, P->lat_ref.data());
-    ck(hfx::launch_dsplit_w(D, P->np, P->Dw, P->dw_off, P->stream), "D pieces");
+    ck(hfx::launch_dsplit_w(D, P->sp, P->Dw, P->dw_off, P->stream), "D pieces");
     ck(cudaStreamSynchronize(P->stream), "D pieces");
     return;
   }
@@ -1080,13 +1160,13 @@ void split_density(hfx_plan* P) {
   }
   DevPlan D = make_devplan(P, P->lat_ref.data());
   hfx::MixPlan X{P->Dsp, P->dsp_off, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  ck(hfx::launch_dsplit(D, X, P->np, P->stream), "dsplit");
+  ck(hfx::launch_dsplit(D, X, P->sp, P->stream), "dsplit");
   if (P->t1u) {
     P->d_work = P->mem.alloc<int>(1);
     P->Df = P->mem.alloc<float>((size_t)P->n_d * 256);
     hfx::T1UPlan U{};
     U.Df = P->Df;
-    ck(hfx::launch_t1u_stores(D, U, P->np, nullptr, 0, true, P->stream), "D FP32 store");
+    ck(hfx::launch_t1u_stores(D, U, P->sp, nullptr, 0, true, P->stream), "D FP32 store");
   }
   ck(cudaStreamSynchronize(P->stream), "dsplit");
 }
@@ -1306,8 +1386,8 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     ck(hfx::launch_ybuild(D, P->y_list, (int)P->tot[1], s), "ybuild");
   } else if (P->wide) {
     ensure_buf(P, P->Ysp, P->Yspcap, std::max(1LL, P->tot[0]));
-    ck(hfx::launch_cpieces_w(D, P->np, P->Cw, P->cw_off, P->dCf, s), "C pieces");
-    ck(hfx::launch_ybuild_w(D, P->np, P->Ysp, P->Cw, P->cw_off, P->Dw, P->dw_off, P->y_list, P->gX, P->gS, P->gN,
+    ck(hfx::launch_cpieces_w(D, P->sp, P->Cw, P->cw_off, P->dCf, s), "C pieces");
+    ck(hfx::launch_ybuild_w(D, P->sp, P->Ysp, P->Cw, P->cw_off, P->Dw, P->dw_off, P->y_list, P->gX, P->gS, P->gN,
                             (int)P->tot[9], P->wide_RB, s),
        "ybuild");
   } else {
@@ -1326,7 +1406,7 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
       ck(hfx::launch_t1_lists(D, X, 1, s), "t1 fill");
     }
     X.blist = P->blist;
-    ck(hfx::launch_cpieces(D, X, P->np, s), "cpieces");
+    ck(hfx::launch_cpieces(D, X, P->sp, s), "cpieces");
     if (P->t1u) {
       U.KP = P->t1u_KP;
       U.NS = P->t1u_NS;
@@ -1349,7 +1429,7 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     ensure_buf(P, P->ytab, P->ytabcap, std::max(1LL, hfx::ytab_size((int)P->tot[9], P->maxC)));
     X.ytab = P->ytab;
     X.ytab_stride = 8 * P->maxC;
-    ck(hfx::launch_ybuild_mma(D, X, P->np, P->y_list, P->gX, P->gS, P->gN, (int)P->tot[9], P->MC, P->drows, P->d_err, s),
+    ck(hfx::launch_ybuild_mma(D, X, P->sp, P->y_list, P->gX, P->gS, P->gN, (int)P->tot[9], P->MC, P->drows, P->d_err, s),
        "ybuild");
   }
   tm.mark();  // 3
@@ -1370,7 +1450,7 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
       ck(hfx::launch_vblocks(D, P->v_list + v0, (int)ct[CT_VN], s), "vblocks");
       k1a.push_back(tm.mark());
       if (P->wide)
-        ck(hfx::launch_term1_w(D, P->np, P->Ysp, P->Cw, P->cw_off, P->Dw, P->dw_off, P->dCf, P->t1_list + v0,
+        ck(hfx::launch_term1_w(D, P->sp, P->Ysp, P->Cw, P->cw_off, P->Dw, P->dw_off, P->dCf, P->t1_list + v0,
                                (int)ct[CT_T1], P->ws, s),
            "term1");
       else
@@ -1381,7 +1461,7 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
       if (P->wide) {
         ensure_buf(P, P->Zw, P->Zwcap,
                    std::max(1LL, ct[CT_T2]) * P->np * hfx::wide_zplane(P->wide_maxrows, P->ws.KZ));
-        ck(hfx::launch_term2_w(D, P->np, P->Ysp, P->Zw, P->Dw, P->dw_off, P->dCf, P->t2_list + v0, P->t2_idx, (int)ct[CT_T2],
+        ck(hfx::launch_term2_w(D, P->sp, P->Ysp, P->Zw, P->Dw, P->dw_off, P->dCf, P->t2_list + v0, P->t2_idx, (int)ct[CT_T2],
                                a0, a1, P->wide_maxrows, P->maxC, P->ws, s),
            "term2");
       } else
@@ -1403,15 +1483,15 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
         ensure_buf(P, P->Vu, P->Vucap, std::max(1LL, ct[CT_T1]) * U.vu_blk);
         U.Cu = P->Cu;
         U.Vu = P->Vu;
-        ck(hfx::launch_t1u_stores(D, U, P->np, t1items + c0, (int)ct[CT_Q], false, s), "term-1 C store");
-        ck(hfx::launch_vstores(D, X, U, P->np, P->v_list + v0, (int)ct[CT_VN], s), "V stores");
+        ck(hfx::launch_t1u_stores(D, U, P->sp, t1items + c0, (int)ct[CT_Q], false, s), "term-1 C store");
+        ck(hfx::launch_vstores(D, X, U, P->sp, P->v_list + v0, (int)ct[CT_VN], s), "V stores");
         k1a.push_back(tm.mark());
-        ck(hfx::launch_t1_umma(D, X, U, P->np, t1items + c0, (int)ct[CT_Q], P->smem_t1u, P->d_work, P->d_err, s),
+        ck(hfx::launch_t1_umma(D, X, U, P->sp, t1items + c0, (int)ct[CT_Q], P->smem_t1u, P->d_work, P->d_err, s),
            "term1");
       } else {
-        ck(hfx::launch_vpieces(D, X, P->np, P->v_list + v0, (int)ct[CT_VN], s), "vpieces");
+        ck(hfx::launch_vpieces(D, X, P->sp, P->v_list + v0, (int)ct[CT_VN], s), "vpieces");
         k1a.push_back(tm.mark());
-        ck(hfx::launch_term1_mma(D, X, P->np, t1items + c0, (int)ct[CT_Q], P->MAmax, P->MBmax, P->KSmax, P->YRmax,
+        ck(hfx::launch_term1_mma(D, X, P->sp, t1items + c0, (int)ct[CT_Q], P->MAmax, P->MBmax, P->KSmax, P->YRmax,
                                  P->smem_m1, s),
            "term1");
       }
@@ -1430,10 +1510,10 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
       X.stall_q2 = stall && stall[0] == '1' ? 1 : 0;
       k2a.push_back(tm.mark());
       if (P->t2u)
-        ck(hfx::launch_t2_umma(D, X, P->np, P->t2_list + v0, (int)ct[CT_T2], P->zblk, P->smem_t2u, P->d_err, s),
+        ck(hfx::launch_t2_umma(D, X, P->sp, P->t2_list + v0, (int)ct[CT_T2], P->zblk, P->smem_t2u, P->d_err, s),
            "term2 R2 and Z");
-      ck(hfx::launch_term2_mma(D, X, P->np, P->t2_list + v0, P->t2_idx, (int)ct[CT_T2], a0, a1, P->MAmax, P->KZmax,
-                               P->zblk, P->ZROWS, FC, P->MC, hfx::q2_umma_segments(P->maxV, P->np, P->q2tpc), P->q2_flush,
+      ck(hfx::launch_term2_mma(D, X, P->sp, P->t2_list + v0, P->t2_idx, (int)ct[CT_T2], a0, a1, P->MAmax, P->KZmax,
+                               P->zblk, P->ZROWS, FC, P->MC, hfx::q2_umma_segments(P->maxV, P->q2tpc), P->q2_flush,
                                P->drows, P->smem_m2, P->d_err, s, P->t2u),
          "term2");
     }
@@ -1609,7 +1689,8 @@ hfx_status hfx_plan_create(const hfx_system* sys, const hfx_model* model, const 
     P->S = model->n_species;
     P->RC = 2.0 * model->r_c;
     P->omega = model->omega;
-    P->np = opt->precision == HFX_BF16X3 ? 2 : opt->precision == HFX_BF16X6 ? 3 : 0;
+    P->sp = opt->precision == HFX_BF16X3 ? hfx::kSplitBf16 : opt->precision == HFX_BF16X6 ? hfx::kSplitHalf : 0;
+    P->np = P->sp ? hfx::kPieces : 0;
     // passes of the plan's home atoms
     const int want = opt->home_chunk > 0 ? opt->home_chunk : 128;
     const int npass = (h1 - h0 + want - 1) / want;

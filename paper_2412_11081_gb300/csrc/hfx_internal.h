@@ -16,6 +16,23 @@ constexpr int kMaxABF = 128;
 constexpr int kMaxCPerAtom = 256;     // C-pair candidates per home atom (mask width)
 constexpr int kMaskWords = kMaxCPerAtom / 32;
 
+// Piece type of the split-precision operands (hfx_device.cuh).
+enum { kSplitBf16 = 2, kSplitHalf = 3 };
+constexpr int kPieces = 2;            // pieces per operand
+
+// Powers of two between the split path's stores and the values they stand
+// for (all 1 for bf16 pieces).  The stored C, V, D, Y, U and Z are the values
+// times 2^e with e chosen on the host from bounds that hold at every geometry
+// the lists cover, so that no stored element exceeds 2^15.
+struct SplitScale {
+  float c = 1.f, v = 1.f, d = 1.f;   // stored piece = c * C, v * V, d * D
+  float y = 1.f, yf = 1.f;           // C.D accumulator -> stored Y; stored Y -> FP32 Y
+  float u = 1.f, uf = 1.f;           // D.Y accumulator -> stored U; FP32 U -> stored U
+  float z = 1.f;                     // V.Y accumulator -> stored Z
+  double r1 = 1.0, q1 = 1.0;         // C.U and V.U accumulators -> R, Q
+  double r2 = 1.0, q2 = 1.0;         // Y.Y and Z.D accumulators -> R2, Q2
+};
+
 // Everything a kernel needs, passed by value.  All pointers are device
 // pointers.  Pair p of a list is (home atom *_home[p] -> atom *_j[p], image
 // *_R[3p..3p+2]); its vector is d = tau_j + R.L - tau_home.
@@ -41,6 +58,7 @@ struct DevPlan {
   double e[3];
   double RC, omega;
   double thC, thdC, thV, thdV, thD, thCS;
+  SplitScale sc;
   int terms;
   int h0, h1;                  // home atoms A whose items are screened in: [h0, h1)
 
@@ -125,9 +143,9 @@ struct MixPlan {
   int* qcnt;                   // [nC] kept B per (A,F)
   long long* qoff;             // [nC] offsets into blist
   int* blist;                  // V pairs (A,B) per (A,F), in V-pair order
-  float* Yf = nullptr;         // Y^{XZ} in FP32 as [z][alpha][16], offsets y_off / np (tcgen05 term 1 only)
+  float* Yf = nullptr;         // Y^{XZ} in FP32 as [z][alpha][16], offsets y_off / 2 (tcgen05 term 1 only)
   uint16_t* YspT = nullptr;    // Y^{XZ} transposed, bf16 pieces [piece][(alpha,x)][16 z] (z padded), yT_blk per key
-  long long yT_blk = 0;        // uint16 units per key of YspT (np x 128-row tiles x 16)
+  long long yT_blk = 0;        // uint16 units per key of YspT (2 pieces x 128-row tiles x 16)
   const long long* y_idx = nullptr;   // key -> its position in the needed-key list (YspT block)
   int* ytab = nullptr;         // Y build: D block (256-element units) per (key group, C slot t, key i), or -1
   int ytab_stride = 0;         // ints per key group (8 * most C pairs of an atom)
@@ -164,9 +182,9 @@ __host__ __device__ inline int gc_off(int row, int f) {
 
 // Operand stores of the tcgen05 first-product kernel (hfx_t1umma.cu).
 struct T1UPlan {
-  uint16_t* Cu;                // per item (A,F): np bf16 pieces of C as [alpha 64][(f,a) KP], then C, grad C FP32 [4][64][KP]
+  uint16_t* Cu;                // per item (A,F): pieces of C as [alpha 64][(f,a) KP], then C, grad C FP32 [4][64][KP]
   long long cu_blk;            // uint16 units per item
-  uint16_t* Vu;                // per term-1 V pair: np pieces of V [alpha 64][beta 64], then grad V FP32 [3][64][64]
+  uint16_t* Vu;                // per term-1 V pair: pieces of V [alpha 64][beta 64], then grad V FP32 [3][64][64]
   long long vu_blk;            // uint16 units per V pair
   const long long* t1_idx;     // V pair -> its position in the term-1 V list
   float* Yf;                   // see MixPlan::Yf
@@ -214,11 +232,11 @@ size_t lri_fit_smem(int n);
 cudaError_t launch_lri_fit(int batch, int n, int w, const double* A, const double* B, const double* dA,
                            const double* dB, double* X, double* dX, int* err, cudaStream_t s);
 
-// Split-precision kernels (hfx_mixed.cu); np = bf16 pieces per operand (2 or 3).
+// Split-precision kernels (hfx_mixed.cu); sp = kSplitBf16 or kSplitHalf.
 long long mixed_launch_count();
-cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, int np, cudaStream_t s);
-cudaError_t launch_cpieces(const DevPlan& P, const MixPlan& X, int np, cudaStream_t s);
-cudaError_t launch_vpieces(const DevPlan& P, const MixPlan& X, int np, const int* list, int n, cudaStream_t s);
+cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, int sp, cudaStream_t s);
+cudaError_t launch_cpieces(const DevPlan& P, const MixPlan& X, int sp, cudaStream_t s);
+cudaError_t launch_vpieces(const DevPlan& P, const MixPlan& X, int sp, const int* list, int n, cudaStream_t s);
 cudaError_t launch_ygroups(const DevPlan& P, const long long* y_idx, const long long* y_total, int* gcnt,
                            const long long* goff, int* gX, int* gS, int* gN, int phase, cudaStream_t s);
 // The D piece store viewed as a 2-D tensor of 512-byte rows (one row per
@@ -228,37 +246,37 @@ struct DRows {
   CUtensorMap map;             // box: one row of 256 bf16
   int zero_row;
 };
-cudaError_t launch_ybuild_mma(const DevPlan& P, const MixPlan& X, int np, const int* ylist, const int* gX,
+cudaError_t launch_ybuild_mma(const DevPlan& P, const MixPlan& X, int sp, const int* ylist, const int* gX,
                               const int* gS, const int* gN, int ngroups, int MC, const DRows& drows, int* err,
                               cudaStream_t s);
 // ints of the D-block tables (MixPlan::ytab, MixPlan::q2tab)
 long long ytab_size(int ngroups, int maxC);
 long long q2tab_size(int n_slots, int FC);
 cudaError_t launch_t1_lists(const DevPlan& P, const MixPlan& X, int phase, cudaStream_t s);
-size_t term1_mma_smem(int np, int MAmax, int MBmax, int KSmax, int YRmax);
-size_t term2_mma_smem(int np, int MAmax, int KZmax);
-cudaError_t set_mixed_smem_limits(int np);
-cudaError_t launch_term1_mma(const DevPlan& P, const MixPlan& X, int np, const int* qlist, int n, int MAmax,
+size_t term1_mma_smem(int MAmax, int MBmax, int KSmax, int YRmax);
+size_t term2_mma_smem(int MAmax, int KZmax);
+cudaError_t set_mixed_smem_limits(int sp);
+cudaError_t launch_term1_mma(const DevPlan& P, const MixPlan& X, int sp, const int* qlist, int n, int MAmax,
                              int MBmax, int KSmax, int YRmax, size_t smem, cudaStream_t s);
 // Second product of the home atoms [a0, a1): list / slot0 / n are that pass's
 // pair list, its slot of every V pair of those atoms and its length.
-cudaError_t launch_term2_mma(const DevPlan& P, const MixPlan& X, int np, const int* list, const long long* slot0,
+cudaError_t launch_term2_mma(const DevPlan& P, const MixPlan& X, int sp, const int* list, const long long* slot0,
                              int n, int a0, int a1, int MAmax, int KZmax, long long zblk, int zrows, int FC, int MC,
                              int nseg, int flush, const DRows& drows, size_t smem, int* err, cudaStream_t s,
                              bool pairs_done = false);
-int q2_umma_segments(int max_pairs_per_atom, int np, int tpc);
+int q2_umma_segments(int max_pairs_per_atom, int tpc);
 // R2 and Z of the pass's second-product pairs on tcgen05 (hfx_t1umma.cu),
 // shapes n_abf <= 64, n_ao <= 16, with X.ycm and X.Vz set: E, g^V and the Z
 // store that k_q2_umma reads (launch_term2_mma with pairs_done then skips
 // its warp-level R2 / Z kernel).
-size_t t2u_smem(int np, int max_ao);
-cudaError_t t2u_set_smem(int np);
-cudaError_t launch_t2_umma(const DevPlan& P, const MixPlan& X, int np, const int* list, int n, long long zblk,
+size_t t2u_smem(int max_ao);
+cudaError_t t2u_set_smem(int sp);
+cudaError_t launch_t2_umma(const DevPlan& P, const MixPlan& X, int sp, const int* list, int n, long long zblk,
                            size_t smem, int* err, cudaStream_t s);
 
 // tcgen05 first exchange product (hfx_t1umma.cu): shapes n_abf <= 64, n_ao <= 16.
 long long t1u_launch_count();
-size_t t1u_smem(int np, int KP, int NS, int FS);
+size_t t1u_smem(int pieces, int KP, int NS, int FS);
 // Columns of one FP32 plane of C / grad C in the operand store (KP rounded up to 32).
 __host__ __device__ inline int t1u_kp32(int KP) { return (KP + 31) & ~31; }
 // Items of the first product in a chosen order: list[0..*n) (n read on the
@@ -270,14 +288,14 @@ constexpr int kLptBuckets = 4096;
 cudaError_t launch_lpt_order(const int* key, int asc, const int* list, int n_max, const long long* n_dev, int* hist,
                              int* out, cudaStream_t s);
 int t1u_max_slots();
-cudaError_t t1u_set_smem(int np);
+cudaError_t t1u_set_smem(int sp);
 // Needed V pairs: the second product's V store (MixPlan::Vm) and, with U.Vu
 // set, the tcgen05 first product's V store, in one pass per pair.
-cudaError_t launch_vstores(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int np, const int* list, int n,
+cudaError_t launch_vstores(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int sp, const int* list, int n,
                            cudaStream_t s);
-cudaError_t launch_t1u_stores(const DevPlan& P, const T1UPlan& U, int np, const int* qlist, int nq, bool dstore,
+cudaError_t launch_t1u_stores(const DevPlan& P, const T1UPlan& U, int sp, const int* qlist, int nq, bool dstore,
                               cudaStream_t s);
-cudaError_t launch_t1_umma(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int np, const int* qlist, int n,
+cudaError_t launch_t1_umma(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int sp, const int* qlist, int n,
                            size_t smem, int* work, int* err, cudaStream_t s);
 
 // Split-precision kernels for n_ao up to 32 and n_abf up to 128 (hfx_wide.cu):
@@ -293,27 +311,27 @@ struct WideShapes {
   bool ok = false;             // every shape fits the kernels' shared memory and tiles
 };
 long long wide_launch_count();
-WideShapes wide_shapes(int np, int maxABF, int maxAO, size_t limit);
+WideShapes wide_shapes(int maxABF, int maxAO, size_t limit);
 int wide_ybuild_row_blocks(int max_rows);
-cudaError_t set_wide_smem_limits(int np);
+cudaError_t set_wide_smem_limits(int sp);
 // C pieces: per kept C pair, NP planes [alpha][rup8(n_ao(A) n_ao(F))] at Cw + cw_off[q]
-long long wide_cpieces_size(int np, int n_abf, int n_ao_a, int n_ao_f);
-cudaError_t launch_cpieces_w(const DevPlan& P, int np, uint16_t* Cw, const long long* cw_off, float* dCf,
+long long wide_cpieces_size(int n_abf, int n_ao_a, int n_ao_f);
+cudaError_t launch_cpieces_w(const DevPlan& P, int sp, uint16_t* Cw, const long long* cw_off, float* dCf,
                              cudaStream_t s);
-cudaError_t launch_ybuild_w(const DevPlan& P, int np, uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
+cudaError_t launch_ybuild_w(const DevPlan& P, int sp, uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
                             const uint16_t* Dw, const long long* dw_off, const int* ylist, const int* gX,
                             const int* gS, const int* gN, int ngroups, int RB, cudaStream_t s);
-cudaError_t launch_term1_w(const DevPlan& P, int np, const uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
+cudaError_t launch_term1_w(const DevPlan& P, int sp, const uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
                            const uint16_t* Dw, const long long* dw_off, const float* dCf, const int* list, int n,
                            const WideShapes& w, cudaStream_t s);
 // elements per bf16 piece plane of one pair slot of the Z store (rows (alpha, a), row stride KZ)
 long long wide_zplane(int max_rows, int KZ);
 // bf16 pieces of every D block (fixed for the plan): NP planes of
 // rup16(n_ao(I)) x rup16(n_ao(J)) at Dw + dw_off[k] (multiples of 256)
-cudaError_t launch_dsplit_w(const DevPlan& P, int np, uint16_t* Dw, const long long* dw_off, cudaStream_t s);
+cudaError_t launch_dsplit_w(const DevPlan& P, int sp, uint16_t* Dw, const long long* dw_off, cudaStream_t s);
 // Second product of the home atoms [a0, a1): k_term2_w over the pass's pair
 // list (E, g^V and the Z piece store), then k_q2_w (grad C); slot0 as launch_term2_mma.
-cudaError_t launch_term2_w(const DevPlan& P, int np, const uint16_t* Yp, uint16_t* Zw, const uint16_t* Dw,
+cudaError_t launch_term2_w(const DevPlan& P, int sp, const uint16_t* Yp, uint16_t* Zw, const uint16_t* Dw,
                            const long long* dw_off, const float* dCf, const int* list, const long long* slot0, int n,
                            int a0, int a1, int max_rows, int max_c, const WideShapes& w, cudaStream_t s);
 

@@ -1,6 +1,6 @@
 // Split-precision tensor-core kernels of the HFX force/stress hot path.
 //
-// Every FP64 operand x of a contraction is written as NP bf16 pieces
+// Every FP64 operand x of a contraction is written as NP pieces
 // x = p0 + p1 (+ p2) + r (p0 = bf16(x), p1 = bf16(x - p0), ...), and each
 // product keeps the piece pairs (i, j) with i + j < NP: three warp-level
 // MMAs for NP = 2, six for NP = 3 (the BF16x3 / BF16x6 splits of Henry,
@@ -8,8 +8,8 @@
 // short run; the screening, the pair gradients, E, F and sigma stay FP64.
 //
 // Operand stores, written once per evaluation from the FP64 blocks
-// (k_cpieces, k_vpieces): per C pair, NP bf16 planes of C [(alpha,a)][rup16(f)]
-// and grad C in FP32; per needed V pair, NP bf16 planes of V [alpha][rup16(beta)]
+// (k_cpieces, k_vpieces): per C pair, NP planes of C [(alpha,a)][rup16(f)]
+// and grad C in FP32; per needed V pair, NP planes of V [alpha][rup16(beta)]
 // and V, grad V in FP32.  No FP64 arithmetic runs inside the item loops.
 //
 // Same factorisation as the FP64 kernels (Eq. exx_expand by the
@@ -79,8 +79,8 @@ __device__ void block_sum_n(double (&v)[NV], double* red) {
 }
 
 // ------------------------------------------------------------------ D split
-// D block k (n_ao(I) x n_ao(J)) -> NP bf16 planes of rup16(n_ao(I)) x rup16(n_ao(J)), zero padded.
-template <int NP>
+// D block k (n_ao(I) x n_ao(J)) -> NP planes of rup16(n_ao(I)) x rup16(n_ao(J)), zero padded.
+template <int SP>
 __global__ void k_dsplit(DevPlan P, MixPlan X) {
   for (long long k = blockIdx.x; k < P.n_d; k += gridDim.x) {
     const int I = P.Didx[5 * k], J = P.Didx[5 * k + 1];
@@ -91,7 +91,7 @@ __global__ void k_dsplit(DevPlan P, MixPlan X) {
     for (int e = threadIdx.x; e < pa * pb; e += blockDim.x) {
       const int a = e / pb, b = e - a * pb;
       uint16_t pc[NP];
-      split_f<NP>((a < na && b < nb) ? (float)src[a * nb + b] : 0.f, pc);
+      split_f<SP>((a < na && b < nb) ? (float)src[a * nb + b] * scf<SP>(P.sc.d) : 0.f, pc);
 #pragma unroll
       for (int p = 0; p < NP; ++p) out[p * pa * pb + tix(a, b)] = pc[p];
     }
@@ -99,10 +99,10 @@ __global__ void k_dsplit(DevPlan P, MixPlan X) {
 }
 
 // ------------------------------------------------------------------ pieces
-// C pair q: NP bf16 pieces of C[(alpha,a)][f] in 128-row tiles of the
+// C pair q: NP pieces of C[(alpha,a)][f] in 128-row tiles of the
 // tensor cores' core-matrix order ([tile][piece][128 x 16], f padded to 16),
 // then grad C in FP32 ([3][(alpha,a)][f]).
-template <int NP>
+template <int SP>
 __global__ void k_cpieces(DevPlan P, MixPlan X) {
   for (int q = blockIdx.x; q < P.nC; q += gridDim.x) {
     if (!P.c_keep[q]) continue;
@@ -119,7 +119,7 @@ __global__ void k_cpieces(DevPlan P, MixPlan X) {
     for (int e = threadIdx.x; e < nt * 128 * 16; e += blockDim.x) {
       const int r = e >> 4, c = e & 15;
       uint16_t pc[NP];
-      split_f<NP>((r < rows && c < nF) ? model::c_value_f(P, scf, go, r * nF + c, 0) : 0.f, pc);
+      split_f<SP>((r < rows && c < nF) ? model::c_value_f(P, scf, go, r * nF + c, 0) * scf<SP>(P.sc.c) : 0.f, pc);
 #pragma unroll
       for (int p = 0; p < NP; ++p) out[((r >> 7) * NP + p) * 2048 + tix(r & 127, c)] = pc[p];
     }
@@ -133,9 +133,9 @@ __global__ void k_cpieces(DevPlan P, MixPlan X) {
   }
 }
 
-// needed V pair p: NP bf16 planes of V[alpha][rup16(n_abf(B))] then V, grad V (FP32),
+// needed V pair p: NP planes of V[alpha][rup16(n_abf(B))] then V, grad V (FP32),
 // evaluated from the block model (V = M h, grad V = M g) without an FP64 store.
-template <int NP>
+template <int SP>
 __global__ void k_vpieces(DevPlan P, MixPlan X, const int* list, int n_list) {
   for (int k = blockIdx.x; k < n_list; k += gridDim.x) {
     const int p = list[k];
@@ -150,7 +150,7 @@ __global__ void k_vpieces(DevPlan P, MixPlan X, const int* list, int n_list) {
     for (int e = threadIdx.x; e < mA * MB; e += blockDim.x) {
       const int al = e / MB, be = e - al * MB;
       uint16_t pc[NP];
-      split_f<NP>(be < mB ? M[al * mB + be] * hf : 0.f, pc);
+      split_f<SP>(be < mB ? M[al * mB + be] * hf * scf<SP>(P.sc.v) : 0.f, pc);
 #pragma unroll
       for (int pp = 0; pp < NP; ++pp) out[pp * mA * MB + e] = pc[pp];
     }
@@ -212,10 +212,10 @@ constexpr int kYS = 24;     // row stride (elements) of the staged Y rows (16 + 
 //                    prefetched while the previous B's R and Q run)
 // Per-B metadata (block offsets) is resolved in chunks of kMeta B by all
 // threads before the chunk's loop.
-template <int NP>
+template <int SP>
 __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X, const int* qlist, int n_list,
                                                             int MAmax, int MBmax, int KSmax, int YRmax) {
-  constexpr bool kStageY = NP == 2;
+  const bool kStageY = YRmax > 0;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[32 * 4];
   __shared__ double sacc[4];    // E (over the item) and g^V partials of the current triplet
@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
                   bf1[pp][0] = *reinterpret_cast<const uint32_t*>(Db + 128);
                   bf1[pp][1] = *reinterpret_cast<const uint32_t*>(Db + 192);
                 }
-                mma_split2<NP>(acc[nt], af, bf0, acc[nt + 1], af, bf1);
+                mma_split2<SP>(acc[nt], af, bf0, acc[nt + 1], af, bf1);
               }
             }
 #pragma unroll
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
                 if (r < rowsU && a < nA) {
                   const int be = r / nF, ff = r - be * nF;
                   uint16_t pc[NP];
-                  split_f<NP>(acc[nt][c], pc);
+                  split_f<SP>(acc[nt][c] * scf<SP>(P.sc.u), pc);
 #pragma unroll
                   for (int pp = 0; pp < NP; ++pp) Us[(size_t)pp * MB * KS + (size_t)be * KS + a * nF + ff] = pc[pp];
                 }
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
                   ldm_x2(bf1[pp], Us + (size_t)pp * MB * KS + (size_t)((two ? nt1 : nt0) * 8 + (lane & 7)) * KS + k0 +
                                       (((lane >> 3) & 1) << 3));
                 }
-                mma_split2<NP>(acc0, af, bf0, acc1, af, bf1);
+                mma_split2<SP>(acc0, af, bf0, acc1, af, bf1);
               }
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
@@ -455,9 +455,9 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
           const float w = warp_sum_f(evf[c]);
           if (lane == 0) {
             if (P.fxC)   // deterministic plan: straight into the exact cells
-              (c == 0) ? dev::add_E(P, -(double)w) : dev::add_gV(P, 3 * p + c - 1, -(double)w);
+              (c == 0) ? dev::add_E(P, -(double)w * P.sc.r1) : dev::add_gV(P, 3 * p + c - 1, -(double)w * P.sc.r1);
             else
-              atomicAdd(&sacc[c], (double)w);
+              atomicAdd(&sacc[c], (double)w * P.sc.r1);
           }
         }
         // Q += V_AB . U (M = alpha, N = (a,f), K = beta).  Warp -> one alpha tile
@@ -482,8 +482,8 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
                   ldm_x2_trans(bf0[pp], Us + (size_t)pp * MB * KS + (size_t)(k0 + (lane & 15)) * KS + nt0 * 8);
                   ldm_x2_trans(bf1[pp], Us + (size_t)pp * MB * KS + (size_t)(k0 + (lane & 15)) * KS + (two ? nt1 : nt0) * 8);
                 }
-                if (two) mma_split2<NP>(qacc[i], af, bf0, qacc[i + 1], af, bf1);
-                else mma_split<NP>(qacc[i], af, bf0);
+                if (two) mma_split2<SP>(qacc[i], af, bf0, qacc[i + 1], af, bf1);
+                else mma_split<SP>(qacc[i], af, bf0);
               }
             }
           }
@@ -513,9 +513,9 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
               qacc[i][c] = 0.f;
             }
           }
-          g[0] += (double)gf[0];
-          g[1] += (double)gf[1];
-          g[2] += (double)gf[2];
+          g[0] += (double)gf[0] * P.sc.q1;
+          g[1] += (double)gf[1] * P.sc.q1;
+          g[2] += (double)gf[2] * P.sc.q1;
         }
       }
     }
@@ -543,7 +543,7 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
 // R2^T[beta][alpha] = sum_{(a,b)} Yb[beta][(a,b)] Ya[alpha][(a,b)], dotted with V, grad V;
 // Z[alpha][(a,b)] = sum_beta V[alpha][beta] Yb[beta][(a,b)] -> Z store of slot s as
 // NP planes [(alpha,a)][pB].
-template <int NP>
+template <int SP>
 __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan X, const int* list, int n_list,
                                                              int MAmax, int KZmax, long long zblk, int zrows) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
             ldm_x4(af[pp], Yb + (size_t)pp * MB * KZ + (size_t)(mt * 16 + (lane & 15)) * KZ + k0 + ((lane >> 4) << 3));
             ldm_x2(bf[pp], Ya + (size_t)pp * MA * KZ + (size_t)(nt * 8 + (lane & 7)) * KZ + k0 + (((lane >> 3) & 1) << 3));
           }
-          mma_split<NP>(acc, af, bf);
+          mma_split<SP>(acc, af, bf);
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -659,7 +659,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp)
               ldm_x2_trans(bf[pp], Yb + (size_t)pp * MB * KZ + (size_t)(ks * 16 + (lane & 15)) * KZ + nt * 8);
-            mma_split<NP>(acc, ak[ks], bf);
+            mma_split<SP>(acc, ak[ks], bf);
           }
         } else {
           for (int k0 = 0; k0 < MB; k0 += 16) {
@@ -675,7 +675,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp)
               ldm_x2_trans(bf[pp], Yb + (size_t)pp * MB * KZ + (size_t)(k0 + (lane & 15)) * KZ + nt * 8);
-            mma_split<NP>(acc, af, bf);
+            mma_split<SP>(acc, af, bf);
           }
         }
 #pragma unroll
@@ -685,8 +685,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
           if (al < mA) {
             const int a = col >> 4, bb = col & 15;
             uint16_t p0[NP], p1[NP];
-            split_f<NP>(acc[2 * h], p0);
-            split_f<NP>(acc[2 * h + 1], p1);
+            split_f<SP>(acc[2 * h] * scf<SP>(P.sc.z), p0);
+            split_f<SP>(acc[2 * h + 1] * scf<SP>(P.sc.z), p1);
             const int r = al * nA + a;
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp)
@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const float w = warp_sum_f(evf[c]);
-      ev[c] = lane == 0 ? (double)w : 0.0;
+      ev[c] = lane == 0 ? (double)w * P.sc.r2 : 0.0;
     }
     block_sum_n<4>(ev, red);
     if (threadIdx.x == 0) {
@@ -750,7 +750,6 @@ __device__ __forceinline__ void gather4_rows(uint32_t sdst, const CUtensorMap* m
 // Stage the B operand of one K step: D rows of the eight keys i (row md[i] +
 // piece, the zero row where md[i] < 0), piece pp and key half h by lane
 // 1 + 2 pp + h.
-template <int NP>
 __device__ __forceinline__ void stage_d(int lane, uint16_t* stB, const int* md, const CUtensorMap* map, int zrow,
                                         uint32_t mbar) {
   if (lane >= 1 && lane <= 2 * NP) {
@@ -770,22 +769,21 @@ __device__ __forceinline__ void stage_d(int lane, uint16_t* stB, const int* md, 
 
 // TPC row tiles of 128 rows per CTA share each K step's D blocks (the B
 // operand): with TPC = 2 a step moves 3 NP tiles for two tiles' work instead
-// of 2 NP for one, in 3 stages (2 with NP = 3, so that two CTAs still fit an
-// SM), one accumulator per tile (no double buffer; two CTAs per SM overlap
+// of 2 NP for one, in 3 stages (two CTAs fit an SM), one accumulator per tile (no double buffer; two CTAs per SM overlap
 // one's epilogue with the other's MMAs) and 512 pairs of metadata; TPC = 1
 // keeps 4 stages and two accumulators.  DEEP = 1 (with TPC = 2) runs one
-// CTA per SM instead: 5 stages (6 with NP = 2) to cover the copies' latency
+// CTA per SM instead: 6 stages to cover the copies' latency
 // and two accumulators per tile (all 512 tensor-memory columns), so the
 // epilogue of one run overlaps the next run's MMAs within the CTA.
-template <int NP, int TPC, int DEEP = 0>
+template <int TPC, int DEEP = 0>
 struct Q2Shape {
-  static constexpr int kS = DEEP ? (NP == 2 ? 6 : 5) : TPC == 2 ? (NP == 2 ? 3 : 2) : umma::kStages;   // stages
-  static constexpr int kMP = TPC == 2 ? 512 : umma::kMetaPairs;    // pairs per CTA segment
-  static constexpr int kNB = TPC == 2 && !DEEP ? 1 : 2;            // accumulator buffers
-  static constexpr int kCols = kNB * TPC * 128;                    // tensor-memory columns
+  static constexpr int kS = DEEP ? 6 : TPC == 2 ? 3 : umma::kStages;   // stages
+  static constexpr int kMP = TPC == 2 ? 512 : umma::kMetaPairs;        // pairs per CTA segment
+  static constexpr int kNB = TPC == 2 && !DEEP ? 1 : 2;                // accumulator buffers
+  static constexpr int kCols = kNB * TPC * 128;                        // tensor-memory columns
 };
 
-template <int NP, int TPC, int DEEP>
+template <int SP, int TPC, int DEEP>
 __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int* list, const long long* slot0,
                                                  int n_slots, int a0, int a1, int FC8, int MC, int NSEG,
                                                  long long zblk, int flush, const __grid_constant__ DRows drows,
@@ -797,8 +795,8 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
   // the accumulators (each its 32-lane quarter of tensor memory) and dot
   // them with grad C_AF.  No block barrier inside the pipeline.
   using namespace umma;
-  constexpr int KS = Q2Shape<NP, TPC, DEEP>::kS, KMP = Q2Shape<NP, TPC, DEEP>::kMP, NB = Q2Shape<NP, TPC, DEEP>::kNB;
-  constexpr int TCOLS = Q2Shape<NP, TPC, DEEP>::kCols;
+  constexpr int KS = Q2Shape<TPC, DEEP>::kS, KMP = Q2Shape<TPC, DEEP>::kMP, NB = Q2Shape<TPC, DEEP>::kNB;
+  constexpr int TCOLS = Q2Shape<TPC, DEEP>::kCols;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   uint16_t* stA = reinterpret_cast<uint16_t*>(smem_raw);                  // [KS][TPC][NP][kTileElems]
   uint16_t* stB = stA + (size_t)KS * TPC * NP * kTileElems;               // [KS][NP][kTileElems]
@@ -905,12 +903,12 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
         bulk_g2s((uint32_t)__cvta_generic_to_shared(stA + (size_t)s * TPC * NP * kTileElems),
                  X.Zst + (p0 + t) * zblk + (long long)mc * NP * kTileElems, abytes, mfull + 8 * s);
       }
-      stage_d<NP>(lane, stB + (size_t)s * NP * kTileElems, m_dblk + t * 8, &drows.map, drows.zero_row, mfull + 8 * s);
+      stage_d(lane, stB + (size_t)s * NP * kTileElems, m_dblk + t * 8, &drows.map, drows.zero_row, mfull + 8 * s);
     }
   } else if (warp == 1) {
     if (lane == 0) {
       // MMA issuer: D f32, A/B bf16, both K-major, N = 128, M = 128
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+      const uint32_t idesc = idesc_split<SP>(128, 128, 0);
       for (int r = 0; r < nruns && !s_abort; ++r) {
         const int b = r % NB;
         if (r >= NB && !mbar_wait<kMixTryNs>(macce + 8 * b, (uint32_t)((r / NB - 1) & 1))) {
@@ -993,9 +991,9 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
             g1 = fmaf(w[1][f4].x, x0, fmaf(w[1][f4].y, x1, fmaf(w[1][f4].z, x2, fmaf(w[1][f4].w, x3, g1))));
             g2 = fmaf(w[2][f4].x, x0, fmaf(w[2][f4].y, x1, fmaf(w[2][f4].z, x2, fmaf(w[2][f4].w, x3, g2))));
           }
-          gd[i][0] += (double)g0;
-          gd[i][1] += (double)g1;
-          gd[i][2] += (double)g2;
+          gd[i][0] += (double)g0 * P.sc.q2;
+          gd[i][1] += (double)g1 * P.sc.q2;
+          gd[i][2] += (double)g2 * P.sc.q2;
         }
       }
       }
@@ -1034,16 +1032,12 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
 // bf16 pieces and writes the Y store ([alpha][z][16], x padding zeroed).
 // TPC row tiles of 128 rows per CTA share each K step's D blocks (one
 // accumulator of 128 columns per tile).
-// stages of the Y build's ring: 4, or 2 for two six-product tiles (so that
-// two CTAs still fit an SM)
-__host__ __device__ constexpr int yb_stages(int np, int tpc) { return tpc == 2 && np == 3 ? 2 : umma::kStages; }
 
-template <int NP, int TPC>
+template <int SP, int TPC>
 __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const int* ylist, const int* gX,
                                                      const int* gS, const int* gN, int MC,
                                                      const __grid_constant__ DRows drows, int* err) {
   using namespace umma;
-  constexpr int kStages = yb_stages(NP, TPC);
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   uint16_t* stA = reinterpret_cast<uint16_t*>(smem_raw);                     // [kStages][TPC][NP][kTileElems]
   uint16_t* stB = stA + (size_t)kStages * TPC * NP * kTileElems;           // [kStages][NP][kTileElems]
@@ -1130,11 +1124,11 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
         bulk_g2s((uint32_t)__cvta_generic_to_shared(stA + (size_t)s * TPC * NP * kTileElems),
                  X.Cm + X.cm_off[q0 + t] + (long long)mc * NP * kTileElems, abytes, mfull + 8 * s);
       }
-      stage_d<NP>(lane, stB + (size_t)s * NP * kTileElems, m_d + t * 8, &drows.map, drows.zero_row, mfull + 8 * s);
+      stage_d(lane, stB + (size_t)s * NP * kTileElems, m_d + t * 8, &drows.map, drows.zero_row, mfull + 8 * s);
     }
   } else if (warp == 1) {
     if (lane == 0 && nsteps > 0) {
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+      const uint32_t idesc = idesc_split<SP>(128, 128, 0);
       for (int k = 0; k < nsteps; ++k) {
         const int s = k % kStages;
         if (!mbar_wait<kMixTryNs>(mfull + 8 * s, (uint32_t)((k / kStages) & 1))) {
@@ -1198,7 +1192,7 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
         }
         float* er = ep + (q * 32 + lane) * 33;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) er[j] = __uint_as_float(v[j]);
+        for (int j = 0; j < 32; ++j) er[j] = __uint_as_float(v[j]) * scf<SP>(P.sc.y);
       }
       asm volatile("bar.sync 1, 128;\n" ::: "memory");
 #pragma unroll 1
@@ -1236,8 +1230,8 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
             f1[k] = 8 * hf + 4 + k < nX ? eh[(rl + 4 + k) * 33 + zz] : 0.f;
           }
           uint2 p0[NP], p1[NP];
-          split4<NP>(f0, p0);
-          split4<NP>(f1, p1);
+          split4<SP>(f0, p0);
+          split4<SP>(f1, p1);
           uint16_t* yo = Yo + (cm ? cmx(al, zz * 16 + 8 * hf, KZc) : ((long long)al * nZ + zz) * 16 + 8 * hf);
 #pragma unroll
           for (int pp = 0; pp < NP; ++pp)
@@ -1253,10 +1247,10 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
             const int x0 = 4 * (cq ^ (2 * ((al >> 1) & 1)));
             const int rl = al * nX - row0 + x0;
             float4 o;
-            o.x = x0 < nX ? eh[rl * 33 + zz] : 0.f;
-            o.y = x0 + 1 < nX ? eh[(rl + 1) * 33 + zz] : 0.f;
-            o.z = x0 + 2 < nX ? eh[(rl + 2) * 33 + zz] : 0.f;
-            o.w = x0 + 3 < nX ? eh[(rl + 3) * 33 + zz] : 0.f;
+            o.x = x0 < nX ? eh[rl * 33 + zz] * scf<SP>(P.sc.yf) : 0.f;
+            o.y = x0 + 1 < nX ? eh[(rl + 1) * 33 + zz] * scf<SP>(P.sc.yf) : 0.f;
+            o.z = x0 + 2 < nX ? eh[(rl + 2) * 33 + zz] * scf<SP>(P.sc.yf) : 0.f;
+            o.w = x0 + 3 < nX ? eh[(rl + 3) * 33 + zz] * scf<SP>(P.sc.yf) : 0.f;
             *reinterpret_cast<float4*>(Yf + ((long long)zz * mX + al) * 16 + 4 * cq) = o;
           }
         }
@@ -1290,8 +1284,8 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
               f1[k] = 8 * hz + 4 + k < nZ ? eh[rl * 33 + 8 * hz + 4 + k] : 0.f;
             }
             uint2 p0[NP], p1[NP];
-            split4<NP>(f0, p0);
-            split4<NP>(f1, p1);
+            split4<SP>(f0, p0);
+            split4<SP>(f1, p1);
             uint16_t* dst = yt + rl * 16 + 8 * hz;
             if (cm) {
               const int r = row0 + rl, al = r / nX, x = r - al * nX;
@@ -1312,13 +1306,13 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
             const int zz = c / nr, r = r0 + (c - zz * nr), x = r - al * nX;
             const float y = eh[(r - row0) * 33 + zz];
             uint16_t pc[NP];
-            split_f<NP>(y, pc);
+            split_f<SP>(y, pc);
             const long long o = cm ? cmx(al, zz * 16, KZc) : ((long long)al * nZ + zz) * 16;   // + x (x < 16)
             const int sw = 2 * ((al >> 1) & 1);
             float* yr = Yf ? Yf + ((long long)zz * mX + al) * 16 : nullptr;
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp) Yo[pp * plane + o + (cm ? ((x >> 3) << 6) + (x & 7) : x)] = pc[pp];
-            if (yr) yr[(((x >> 2) ^ sw) << 2) + (x & 3)] = y;
+            if (yr) yr[(((x >> 2) ^ sw) << 2) + (x & 3)] = y * scf<SP>(P.sc.yf);
             if (x == nX - 1)
               for (int xp = nX; xp < 16; ++xp) {
 #pragma unroll
@@ -1427,19 +1421,18 @@ __global__ void k_q2tab(DevPlan P, MixPlan X, const int* list, int n_slots, int 
   if ((threadIdx.x & 31) == 0 && fl != 0.0) atomicAdd(&P.acc[ACC_F2], fl);
 }
 
-size_t ybuild_umma_smem(int np, int tpc) {
-  return (size_t)(tpc + 1) * yb_stages(np, tpc) * np * umma::kTileElems * sizeof(uint16_t) +
+size_t ybuild_umma_smem(int tpc) {
+  return (size_t)(tpc + 1) * umma::kStages * NP * umma::kTileElems * sizeof(uint16_t) +
          (size_t)kMaxCPerAtom * 8 * sizeof(int);
 }
 
-size_t q2_umma_smem(int np, int tpc) {
-  if (tpc >= 2) {   // 3: two tiles, the deep pipeline
-    const int ks = tpc == 3 ? (np == 2 ? Q2Shape<2, 2, 1>::kS : Q2Shape<3, 2, 1>::kS)
-                            : (np == 2 ? Q2Shape<2, 2>::kS : Q2Shape<3, 2>::kS);
-    return (size_t)ks * 3 * np * umma::kTileElems * sizeof(uint16_t) + (size_t)Q2Shape<2, 2>::kMP * 8 * sizeof(int);
+size_t q2_umma_smem(int tpc) {   // tpc 3: two tiles, the deep pipeline
+  if (tpc >= 2) {
+    const int ks = tpc == 3 ? Q2Shape<2, 1>::kS : Q2Shape<2>::kS;
+    return (size_t)ks * 3 * NP * umma::kTileElems * sizeof(uint16_t) + (size_t)Q2Shape<2>::kMP * 8 * sizeof(int);
   }
-  return (size_t)2 * Q2Shape<2, 1>::kS * np * umma::kTileElems * sizeof(uint16_t) +
-         (size_t)Q2Shape<2, 1>::kMP * 8 * sizeof(int);
+  return (size_t)2 * Q2Shape<1>::kS * NP * umma::kTileElems * sizeof(uint16_t) +
+         (size_t)Q2Shape<1>::kMP * 8 * sizeof(int);
 }
 
 int grid_for(long long n, int cap) {
@@ -1454,32 +1447,32 @@ long long mixed_launch_count() { return g_mix_launches; }
 long long ytab_size(int ngroups, int maxC) { return (long long)ngroups * 8 * maxC; }
 long long q2tab_size(int n_slots, int FC) { return (long long)n_slots * ((FC * 4 + 7) / 8) * 8; }
 
-int q2_umma_segments(int max_pairs_per_atom, int np, int tpc) {
-  const int kmp = tpc >= 2 ? Q2Shape<2, 2>::kMP : Q2Shape<2, 1>::kMP;
+int q2_umma_segments(int max_pairs_per_atom, int tpc) {
+  const int kmp = tpc >= 2 ? Q2Shape<2>::kMP : Q2Shape<1>::kMP;
   return (max_pairs_per_atom + kmp - 1) / kmp;
 }
 
-cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, int np, cudaStream_t s) {
+cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, int sp, cudaStream_t s) {
   if (P.n_d == 0) return cudaSuccess;
   ++g_mix_launches;
-  if (np == 2) k_dsplit<2><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X);
-  else k_dsplit<3><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X);
+  if (sp == kSplitBf16) k_dsplit<kSplitBf16><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X);
+  else k_dsplit<kSplitHalf><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X);
   return cudaGetLastError();
 }
 
-cudaError_t launch_cpieces(const DevPlan& P, const MixPlan& X, int np, cudaStream_t s) {
+cudaError_t launch_cpieces(const DevPlan& P, const MixPlan& X, int sp, cudaStream_t s) {
   if (P.nC == 0) return cudaSuccess;
   ++g_mix_launches;
-  if (np == 2) k_cpieces<2><<<grid_for(P.nC, 152 * 32), 256, 0, s>>>(P, X);
-  else k_cpieces<3><<<grid_for(P.nC, 152 * 32), 256, 0, s>>>(P, X);
+  if (sp == kSplitBf16) k_cpieces<kSplitBf16><<<grid_for(P.nC, 152 * 32), 256, 0, s>>>(P, X);
+  else k_cpieces<kSplitHalf><<<grid_for(P.nC, 152 * 32), 256, 0, s>>>(P, X);
   return cudaGetLastError();
 }
 
-cudaError_t launch_vpieces(const DevPlan& P, const MixPlan& X, int np, const int* list, int n, cudaStream_t s) {
+cudaError_t launch_vpieces(const DevPlan& P, const MixPlan& X, int sp, const int* list, int n, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   ++g_mix_launches;
-  if (np == 2) k_vpieces<2><<<grid_for(n, 152 * 32), 256, 0, s>>>(P, X, list, n);
-  else k_vpieces<3><<<grid_for(n, 152 * 32), 256, 0, s>>>(P, X, list, n);
+  if (sp == kSplitBf16) k_vpieces<kSplitBf16><<<grid_for(n, 152 * 32), 256, 0, s>>>(P, X, list, n);
+  else k_vpieces<kSplitHalf><<<grid_for(n, 152 * 32), 256, 0, s>>>(P, X, list, n);
   return cudaGetLastError();
 }
 
@@ -1490,7 +1483,7 @@ cudaError_t launch_ygroups(const DevPlan& P, const long long* y_idx, const long 
   return cudaGetLastError();
 }
 
-cudaError_t launch_ybuild_mma(const DevPlan& P, const MixPlan& X, int np, const int* ylist, const int* gX,
+cudaError_t launch_ybuild_mma(const DevPlan& P, const MixPlan& X, int sp, const int* ylist, const int* gX,
                               const int* gS, const int* gN, int ngroups, int MC, const DRows& drows, int* err,
                               cudaStream_t s) {
   if (ngroups == 0) return cudaSuccess;
@@ -1499,11 +1492,11 @@ cudaError_t launch_ybuild_mma(const DevPlan& P, const MixPlan& X, int np, const 
                                                                                           ngroups);
   const int tpc = X.ybtpc == 1 ? 1 : 2;
   const long long grid = (long long)ngroups * ((MC + tpc - 1) / tpc);
-  const size_t sm = ybuild_umma_smem(np, tpc);
-  if (np == 2 && tpc == 2) k_ybuild_umma<2, 2><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
-  else if (np == 2) k_ybuild_umma<2, 1><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
-  else if (tpc == 2) k_ybuild_umma<3, 2><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
-  else k_ybuild_umma<3, 1><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
+  const size_t sm = ybuild_umma_smem(tpc);
+  if (sp == kSplitBf16 && tpc == 2) k_ybuild_umma<kSplitBf16, 2><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
+  else if (sp == kSplitBf16) k_ybuild_umma<kSplitBf16, 1><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
+  else if (tpc == 2) k_ybuild_umma<kSplitHalf, 2><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
+  else k_ybuild_umma<kSplitHalf, 1><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
   return cudaGetLastError();
 }
 
@@ -1513,25 +1506,21 @@ cudaError_t launch_t1_lists(const DevPlan& P, const MixPlan& X, int phase, cudaS
   return cudaGetLastError();
 }
 
-size_t term1_mma_smem(int np, int MAmax, int MBmax, int KSmax, int YRmax) {
-  size_t e = (size_t)np * (MAmax * KSmax + MBmax * KSmax + 2 * MAmax * (MBmax + 8));
-  if (np == 2) e += (size_t)np * YRmax * kYS;
-  return e * sizeof(uint16_t);
+size_t term1_mma_smem(int MAmax, int MBmax, int KSmax, int YRmax) {
+  return (size_t)NP * (MAmax * KSmax + MBmax * KSmax + 2 * MAmax * (MBmax + 8) + YRmax * kYS) * sizeof(uint16_t);
 }
 
-size_t term2_mma_smem(int np, int MAmax, int KZmax) {
-  return (size_t)np * 2 * MAmax * KZmax * sizeof(uint16_t);
-}
+size_t term2_mma_smem(int MAmax, int KZmax) { return (size_t)NP * 2 * MAmax * KZmax * sizeof(uint16_t); }
 
-cudaError_t set_mixed_smem_limits(int np) {
+cudaError_t set_mixed_smem_limits(int sp) {
   const void* f[7] = {
-      np == 2 ? (const void*)k_ybuild_umma<2, 2> : (const void*)k_ybuild_umma<3, 2>,
-      np == 2 ? (const void*)k_ybuild_umma<2, 1> : (const void*)k_ybuild_umma<3, 1>,
-      np == 2 ? (const void*)k_q2_umma<2, 2, 0> : (const void*)k_q2_umma<3, 2, 0>,
-      np == 2 ? (const void*)k_q2_umma<2, 2, 1> : (const void*)k_q2_umma<3, 2, 1>,
-      np == 2 ? (const void*)k_q2_umma<2, 1, 0> : (const void*)k_q2_umma<3, 1, 0>,
-      np == 2 ? (const void*)k_term1_mma<2> : (const void*)k_term1_mma<3>,
-      np == 2 ? (const void*)k_term2_pairs<2> : (const void*)k_term2_pairs<3>};
+      sp == kSplitBf16 ? (const void*)k_ybuild_umma<kSplitBf16, 2> : (const void*)k_ybuild_umma<kSplitHalf, 2>,
+      sp == kSplitBf16 ? (const void*)k_ybuild_umma<kSplitBf16, 1> : (const void*)k_ybuild_umma<kSplitHalf, 1>,
+      sp == kSplitBf16 ? (const void*)k_q2_umma<kSplitBf16, 2, 0> : (const void*)k_q2_umma<kSplitHalf, 2, 0>,
+      sp == kSplitBf16 ? (const void*)k_q2_umma<kSplitBf16, 2, 1> : (const void*)k_q2_umma<kSplitHalf, 2, 1>,
+      sp == kSplitBf16 ? (const void*)k_q2_umma<kSplitBf16, 1, 0> : (const void*)k_q2_umma<kSplitHalf, 1, 0>,
+      sp == kSplitBf16 ? (const void*)k_term1_mma<kSplitBf16> : (const void*)k_term1_mma<kSplitHalf>,
+      sp == kSplitBf16 ? (const void*)k_term2_pairs<kSplitBf16> : (const void*)k_term2_pairs<kSplitHalf>};
   for (const void* k : f) {
     const cudaError_t e = allow_max_dynamic_smem(k);
     if (e != cudaSuccess) return e;
@@ -1539,18 +1528,18 @@ cudaError_t set_mixed_smem_limits(int np) {
   return cudaSuccess;
 }
 
-cudaError_t launch_term1_mma(const DevPlan& P, const MixPlan& X, int np, const int* qlist, int n, int MAmax, int MBmax,
+cudaError_t launch_term1_mma(const DevPlan& P, const MixPlan& X, int sp, const int* qlist, int n, int MAmax, int MBmax,
                              int KSmax, int YRmax, size_t smem, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   ++g_mix_launches;
-  if (np == 2)
-    k_term1_mma<2><<<grid_for(n, 152 * 16), kWarps1 * 32, smem, s>>>(P, X, qlist, n, MAmax, MBmax, KSmax, YRmax);
+  if (sp == kSplitBf16)
+    k_term1_mma<kSplitBf16><<<grid_for(n, 152 * 16), kWarps1 * 32, smem, s>>>(P, X, qlist, n, MAmax, MBmax, KSmax, YRmax);
   else
-    k_term1_mma<3><<<grid_for(n, 152 * 16), kWarps1 * 32, smem, s>>>(P, X, qlist, n, MAmax, MBmax, KSmax, YRmax);
+    k_term1_mma<kSplitHalf><<<grid_for(n, 152 * 16), kWarps1 * 32, smem, s>>>(P, X, qlist, n, MAmax, MBmax, KSmax, YRmax);
   return cudaGetLastError();
 }
 
-cudaError_t launch_term2_mma(const DevPlan& P, const MixPlan& X, int np, const int* list, const long long* slot0,
+cudaError_t launch_term2_mma(const DevPlan& P, const MixPlan& X, int sp, const int* list, const long long* slot0,
                              int n, int a0, int a1, int MAmax, int KZmax, long long zblk, int zrows, int FC, int MC,
                              int nseg, int flush, const DRows& drows, size_t smem, int* err, cudaStream_t s,
                              bool pairs_done) {
@@ -1559,23 +1548,23 @@ cudaError_t launch_term2_mma(const DevPlan& P, const MixPlan& X, int np, const i
   const int FC8 = (FC * 4 + 7) / 8;     // groups of 8 C slots for the tcgen05 kernel
   k_q2tab<<<grid_for(((long long)n * FC8 * 8 + 255) / 256, 152 * 16), 256, 0, s>>>(P, X, list, n, FC8);
   const int tpc = X.q2tpc == 1 ? 1 : 2, deep = X.q2tpc == 3 ? 1 : 0;   // row tiles per CTA; the deep pipeline
-  const size_t sq = q2_umma_smem(np, X.q2tpc == 1 ? 1 : (deep ? 3 : 2));
+  const size_t sq = q2_umma_smem(X.q2tpc == 1 ? 1 : (deep ? 3 : 2));
   const long long grid = (long long)(a1 - a0) * FC8 * ((MC + tpc - 1) / tpc) * nseg;
   auto q2 = [&](auto kern) {
     kern<<<(unsigned)grid, 192, sq, s>>>(P, X, list, slot0, n, a0, a1, FC8, MC, nseg, zblk, flush, drows, err);
   };
-  if (np == 2) {
+  if (sp == kSplitBf16) {
     if (!pairs_done)
-      k_term2_pairs<2><<<grid_for(n, 152 * 32), kWarps * 32, smem, s>>>(P, X, list, n, MAmax, KZmax, zblk, zrows);
-    if (tpc == 1) q2(k_q2_umma<2, 1, 0>);
-    else if (deep) q2(k_q2_umma<2, 2, 1>);
-    else q2(k_q2_umma<2, 2, 0>);
+      k_term2_pairs<kSplitBf16><<<grid_for(n, 152 * 32), kWarps * 32, smem, s>>>(P, X, list, n, MAmax, KZmax, zblk, zrows);
+    if (tpc == 1) q2(k_q2_umma<kSplitBf16, 1, 0>);
+    else if (deep) q2(k_q2_umma<kSplitBf16, 2, 1>);
+    else q2(k_q2_umma<kSplitBf16, 2, 0>);
   } else {
     if (!pairs_done)
-      k_term2_pairs<3><<<grid_for(n, 152 * 32), kWarps * 32, smem, s>>>(P, X, list, n, MAmax, KZmax, zblk, zrows);
-    if (tpc == 1) q2(k_q2_umma<3, 1, 0>);
-    else if (deep) q2(k_q2_umma<3, 2, 1>);
-    else q2(k_q2_umma<3, 2, 0>);
+      k_term2_pairs<kSplitHalf><<<grid_for(n, 152 * 32), kWarps * 32, smem, s>>>(P, X, list, n, MAmax, KZmax, zblk, zrows);
+    if (tpc == 1) q2(k_q2_umma<kSplitHalf, 1, 0>);
+    else if (deep) q2(k_q2_umma<kSplitHalf, 2, 1>);
+    else q2(k_q2_umma<kSplitHalf, 2, 0>);
   }
   return cudaGetLastError();
 }

@@ -75,7 +75,7 @@ __device__ __forceinline__ void ep_at(int w, int& alpha, int& col) {
   col = 32 * j + 16 * (l >> 4) + 4 * t + k;
 }
 
-// Item kk (C pair q = list[kk]): NP bf16 pieces of C_AF as [alpha (64)][(f,a) (KP)]
+// Item kk (C pair q = list[kk]): NP pieces of C_AF as [alpha (64)][(f,a) (KP)]
 // in core-matrix order (8-row groups of KP/8 core matrices), then C and
 // grad C in FP32 as four planes of 64 x KP32 (KP rounded up to 32) in
 // epilogue load order (ep_at).  Zero padded.  Each plane of the C pair
@@ -83,7 +83,7 @@ __device__ __forceinline__ void ep_at(int w, int& alpha, int& col) {
 // FP32; the outputs are written in storage order, four elements per thread.
 constexpr int kCStoreSmem = 64 * 16 * 16 * 4;   // one plane of n_abf <= 64, n_ao <= 16
 
-template <int NP>
+template <int SP>
 __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
   extern __shared__ float cs[];
   const int KP = U.KP, KP32 = t1u_kp32(KP), PL = 64 * KP32;
@@ -113,9 +113,10 @@ __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
           const int t = 4 * t4;
           const int g8 = t / (KP * 8), rem = t - g8 * KP * 8;
           const int al = g8 * 8 + ((rem >> 3) & 7), col = (rem >> 6) * 8 + (rem & 7);
-          const float x[4] = {val(al, col), val(al, col + 1), val(al, col + 2), val(al, col + 3)};
+          const float x[4] = {val(al, col) * scf<SP>(P.sc.c), val(al, col + 1) * scf<SP>(P.sc.c), val(al, col + 2) * scf<SP>(P.sc.c),
+                              val(al, col + 3) * scf<SP>(P.sc.c)};
           uint2 pc[NP];
-          split4<NP>(x, pc);
+          split4<SP>(x, pc);
 #pragma unroll
           for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(out + (long long)pp * 64 * KP + t) = pc[pp];
         }
@@ -133,7 +134,7 @@ __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
 // Every needed V pair p = list[k], in one pass: V and grad V evaluated once
 // from the block model into shared memory (FP32), then
 //   the warp-level second product's store X.Vm at vm_off[p] (unless X.Vz is
-//   set): NP bf16 planes [alpha][rup16(n_abf(B))] and V, grad V in FP32
+//   set): NP planes [alpha][rup16(n_abf(B))] and V, grad V in FP32
 //   [4][n_abf(A) n_abf(B)];
 //   for the pairs of the first product (any bit of v_mask), the tcgen05
 //   store U.Vu at t1_idx[p]: NP pieces [alpha 64][beta 64] in core-matrix
@@ -143,7 +144,7 @@ __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
 // Outputs are written in storage order, four elements per thread.
 constexpr int kVStoreSmem = 4 * 64 * 64 * 4;
 
-template <int NP>
+template <int SP>
 __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int n) {
   extern __shared__ float vsm[];   // [4][mA * mB]: V, grad V
   for (int k = blockIdx.x; k < n; k += gridDim.x) {
@@ -171,9 +172,9 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
         const int e = 4 * e4, al = e / MB, be = e - al * MB;
         float x[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] = be + j < mB ? vsm[al * mB + be + j] : 0.f;
+        for (int j = 0; j < 4; ++j) x[j] = be + j < mB ? vsm[al * mB + be + j] * scf<SP>(P.sc.v) : 0.f;
         uint2 pc[NP];
-        split4<NP>(x, pc);
+        split4<SP>(x, pc);
 #pragma unroll
         for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(out + (long long)pp * mA * MB + e) = pc[pp];
       }
@@ -197,9 +198,9 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
         const int al = ((t >> 9) << 3) + ((t >> 3) & 7), be = (((t >> 6) & 7) << 3) + (t & 7);
         float x[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] = (al < mA && be + j < mB) ? vsm[al * mB + be + j] : 0.f;
+        for (int j = 0; j < 4; ++j) x[j] = (al < mA && be + j < mB) ? vsm[al * mB + be + j] * scf<SP>(P.sc.v) : 0.f;
         uint2 pc[NP];
-        split4<NP>(x, pc);
+        split4<SP>(x, pc);
 #pragma unroll
         for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(vu + pp * 4096 + t) = pc[pp];
       }
@@ -288,7 +289,7 @@ __global__ void k_lpt_scatter(const int* key, int asc, const int* list, const lo
 }
 
 // ------------------------------------------------------------------- kernel
-template <int NP>
+template <int SP>
 __global__ void __launch_bounds__(kThreads, 1)
     k_t1_umma(DevPlan P, MixPlan X, T1UPlan U, const int* qlist, int n_list, int* work, int* err) {
   const int KP = U.KP, KP32 = t1u_kp32(KP), NF = KP >> 4, FH = (NF + 1) >> 1, NS = U.NS, SEG = U.seg, FS = U.FS;
@@ -511,26 +512,22 @@ __global__ void __launch_bounds__(kThreads, 1)
     // step) into one of two accumulators of kRCols columns.  A U piece
     // plane is 64 rows, i.e. eight 8-row groups, after the previous one, so
     // pieces 0 and 1 together are one N = 128 operand: block 0 (columns
-    // 0-63) collects the products with U_0 (and U_2), block 1 those with U_1,
-    // and R = block 0 + block 1.  BF16X6: C0 [U0;U1], C0 U2, C1 [U0;U1]
-    // (C1 U1 comes with it), C2 U0; BF16X3: C0 [U0;U1], C1 U0.  Descriptors
+    // 0-63) collects the products with U_0, block 1 those with U_1, and
+    // R = block 0 + block 1: C0 [U0;U1], C1 U0.  Descriptors
     // are formed once; a k step adds 16 (256 bytes).
-    constexpr int NR = NP == 3 ? 4 : 2;   // MMAs per k step
-    const uint32_t idR128 = idesc_bf16(64, 128, 0), idR64 = idesc_bf16(64, 64, 0);
+    constexpr int NR = 2;   // MMAs per k step
+    const uint32_t idR128 = idesc_split<SP>(64, 128, 0), idR64 = idesc_split<SP>(64, 64, 0);
     const uint32_t rowg = 16u * KP;   // bytes between 8-row groups of C and U
     const uint64_t dC = sdesc2(sa(Cs), 128, rowg), dUR = sdesc2(sa(Us), 128, rowg);
     uint64_t pa[NR], pb[NR];
     uint32_t pid[NR];
     {
-      const int ca[4] = {0, 0, 1, 2}, ub[4] = {0, 2, 0, 0}, wide[4] = {1, 0, 1, 0};   // BF16X6
-      const int ca2[2] = {0, 1}, ub2[2] = {0, 0}, wide2[2] = {1, 0};                  // BF16X3
-#pragma unroll
-      for (int k = 0; k < NR; ++k) {
-        const int c = NP == 3 ? ca[k] : ca2[k], u = NP == 3 ? ub[k] : ub2[k], w = NP == 3 ? wide[k] : wide2[k];
-        pa[k] = dC + ((uint64_t)(c * CPB) >> 4);
-        pb[k] = dUR + ((uint64_t)(u * CPB) >> 4);
-        pid[k] = w ? idR128 : idR64;
-      }
+      pa[0] = dC;   // C0 [U0;U1]
+      pb[0] = dUR;
+      pid[0] = idR128;
+      pa[1] = dC + ((uint64_t)CPB >> 4);   // C1 U0
+      pb[1] = dUR;
+      pid[1] = idR64;
     }
     uint32_t rb = 0, it = 0, ik = 0;
     bool ok = true;
@@ -556,7 +553,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int f = f0; f < f1; ++f) {
               const uint64_t o = 16u * (uint32_t)f;
 #pragma unroll
-              for (int k = 0; k < NR; ++k) umma_bf16(dR, pa[k] + o, pb[k] + o, pid[k], (f > 0 || k > 0) ? 1u : 0u);
+              for (int k = 0; k < NR; ++k) umma_f16(dR, pa[k] + o, pb[k] + o, pid[k], (f > 0 || k > 0) ? 1u : 0u);
             }
             umma_commit(ue + 8 * c);
             if (c == 1) umma_commit(rf + 8 * rbuf);
@@ -573,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Q[:, chunk] += V_AB . U_B[:, chunk] (M = 64 alpha, N = the chunk's
     // (f,a) columns, K = beta in four k steps; U read MN-major).
     const int N0 = 16 * FH, N1 = 16 * (NF - FH);
-    const uint32_t idQ0 = idesc_bf16(64, N0, 1), idQ1 = N1 > 0 ? idesc_bf16(64, N1, 1) : 0u;
+    const uint32_t idQ0 = idesc_split<SP>(64, N0, 1), idQ1 = N1 > 0 ? idesc_split<SP>(64, N1, 1) : 0u;
     const uint32_t rowg = 16u * KP;
     const uint64_t dV = sdesc2(sa(Vs), 128, 1024), dUQ = sdesc2(sa(Us), rowg, 128);
     uint64_t pa[NPROD], pb[NPROD];
@@ -613,7 +610,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               for (int kb = 0; kb < 4; ++kb)
 #pragma unroll
                 for (int k = 0; k < NPROD; ++k)
-                  umma_bf16(tq, pa[k] + kbA * kb, pb[k] + oB + kbB * kb, idQ, (first && kb == 0 && k == 0) ? 0u : 1u);
+                  umma_f16(tq, pa[k] + kbA * kb, pb[k] + oB + kbB * kb, idQ, (first && kb == 0 && k == 0) ? 0u : 1u);
             }
             umma_commit(ue + 8 * c);
           }
@@ -731,7 +728,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (lane == 0 && ok)
 #pragma unroll
             for (int c = 0; c < 3; ++c)
-              if (gv[c] != 0.f) dev::add_gV(P, 3 * p + c, -(double)gv[c]);
+              if (gv[c] != 0.f) dev::add_gV(P, 3 * p + c, -(double)gv[c] * P.sc.r1);
           if (ew == 0 && lane == 0) fl += 2.0 * mB * nA * nB * nF + 4.0 * mA * mB * nA * nF;
           ++rb;
           // ---- end of a run: Q -> E, g^C
@@ -785,10 +782,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int c = 0; c < 3; ++c) g_it[c] = warp_sum_d(g_it[c]);
       if (lane == 0 && ok) {
-        if (e_it != 0.0) dev::add_E(P, -e_it);
+        if (e_it != 0.0) dev::add_E(P, -e_it * P.sc.q1);
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-          if (g_it[c] != 0.0) dev::add_gC(P, 3 * q + c, -2.0 * g_it[c]);
+          if (g_it[c] != 0.0) dev::add_gC(P, 3 * q + c, -2.0 * g_it[c] * P.sc.q1);
       }
     }
     if (!ok) *abort_flag = 1;
@@ -849,42 +846,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               const int sl = (int)(ys % NS);
               ok = wait_all(yf + 8 * sl, (ys / NS) & 1);
               if (!ok) break;
-              if (NP == 3) {
-                // BF16X6 (tighter on registers): one row per pass, each lane
-                // reads the row's four 16-byte chunks (chunk c stored at c ^ ysw)
-                for (int f = fa; f < fb; ++f) {
-                  float y[16];
-#pragma unroll
-                  for (int c4 = 0; c4 < 4; ++c4) {
-                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (beta < mB)
-                      a = *reinterpret_cast<const float4*>(Ys + sl * SLOT + ((f - fa) * mB + beta) * 16 + 4 * (c4 ^ ysw));
-                    y[4 * c4] = a.x;
-                    y[4 * c4 + 1] = a.y;
-                    y[4 * c4 + 2] = a.z;
-                    y[4 * c4 + 3] = a.w;
-                  }
-                  float uf4[4] = {0.f, 0.f, 0.f, 0.f};
-                  if (beta < mB)
-#pragma unroll
-                    for (int b = 0; b < 16; ++b)
-#pragma unroll
-                      for (int j = 0; j < 2; ++j) {
-                        uf4[2 * j] = fmaf(y[b], dd[j][b].x, uf4[2 * j]);
-                        uf4[2 * j + 1] = fmaf(y[b], dd[j][b].y, uf4[2 * j + 1]);
-                      }
-                  if (f + 1 >= fb) {   // the slot's rows have been read and used
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(ye + 8 * sl);
-                  }
-                  uint2 pk[NP];
-                  split4<NP>(uf4, pk);
-#pragma unroll
-                  for (int pp = 0; pp < NP; ++pp)
-                    *reinterpret_cast<uint2*>(urow + (size_t)pp * 64 * KP + (2 * f + (qa >> 1)) * 64) = pk[pp];
-                }
-              } else {
-                // BF16X3: the run's rows rho = (f - fa) mB + beta (the slot's
+              {
+                // the run's rows rho = (f - fa) mB + beta (the slot's
                 // own order) are shared by all U warps, two per lane and pass
                 // (rho = 16 g + r8 and 16 g + 8 + r8 for row groups g = uw,
                 // uw + kNU, ...), so every warp gets the same share whatever
@@ -934,16 +897,16 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                   uint2 pk[NP];
                   if (v0) {
-                    float uf4[4] = {u0[0].x, u0[0].y, u0[1].x, u0[1].y};
-                    split4<NP>(uf4, pk);
+                    float uf4[4] = {u0[0].x * scf<SP>(P.sc.uf), u0[0].y * scf<SP>(P.sc.uf), u0[1].x * scf<SP>(P.sc.uf), u0[1].y * scf<SP>(P.sc.uf)};
+                    split4<SP>(uf4, pk);
                     uint16_t* ur = Us + (be[0] >> 3) * KP * 8 + (be[0] & 7) * 8 + (qa & 1) * 4 +
                                    (2 * (fa + fr[0]) + (qa >> 1)) * 64;
   #pragma unroll
                     for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(ur + (size_t)pp * 64 * KP) = pk[pp];
                   }
                   if (v1) {
-                    float ug4[4] = {u1[0].x, u1[0].y, u1[1].x, u1[1].y};
-                    split4<NP>(ug4, pk);
+                    float ug4[4] = {u1[0].x * scf<SP>(P.sc.uf), u1[0].y * scf<SP>(P.sc.uf), u1[1].x * scf<SP>(P.sc.uf), u1[1].y * scf<SP>(P.sc.uf)};
+                    split4<SP>(ug4, pk);
                     uint16_t* ur = Us + (be[1] >> 3) * KP * 8 + (be[1] & 7) * 8 + (qa & 1) * 4 +
                                    (2 * (fa + fr[1]) + (qa >> 1)) * 64;
   #pragma unroll
@@ -955,9 +918,9 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
               ++ys;
             }
-            // rows beta >= n_abf(B) (BF16X3 computes only the rows it reads)
-            // and rows f >= nF of the chunk are zero
-            if (NP == 2 && beta >= mB)
+            // rows beta >= n_abf(B) (only the rows read are computed) and rows
+            // f >= nF of the chunk are zero
+            if (beta >= mB)
               for (int f = f0; f < e; ++f)
 #pragma unroll
                 for (int pp = 0; pp < NP; ++pp)
@@ -1002,7 +965,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 constexpr int kT2Threads = 192;
 constexpr int kT2RCol = 256;   // tensor-memory column of the first R2 accumulator (Z at column 0)
 
-template <int NP>
+template <int SP>
 __global__ void __launch_bounds__(kT2Threads, 1)
     k_t2_umma(DevPlan P, MixPlan X, const int* list, int n_list, int KKmax, long long zblk, int* err) {
   constexpr int NPROD = NP * (NP + 1) / 2;
@@ -1081,7 +1044,7 @@ __global__ void __launch_bounds__(kT2Threads, 1)
   } else if (warp == 1) {
     // ----------------------------------------------------------- MMA issuer
     if (lane == 0) {
-      const uint32_t idR = idesc_bf16(64, 64, 0);
+      const uint32_t idR = idesc_split<SP>(64, 64, 0);
       uint32_t i = 0;
       bool ok = true;
       for (int kk = blockIdx.x; kk < n_list && ok; kk += gridDim.x, ++i) {
@@ -1095,7 +1058,7 @@ __global__ void __launch_bounds__(kT2Threads, 1)
         const uint32_t rowg = 16u * (uint32_t)KK;      // bytes between 8-row groups
         const uint64_t dA = sdesc2(sa(Ya), 128, rowg), dBK = sdesc2(sa(Yb), 128, rowg);
         const uint64_t dV = sdesc2(sa(Vs), 128, 1024), dBM = sdesc2(sa(Yb), rowg, 128);
-        const uint32_t idZ = idesc_bf16(64, KK, 1);
+        const uint32_t idZ = idesc_split<SP>(64, KK, 1);
         const int rbuf = i & 1;
         ok = mbar_wait(mAf, i & 1) && mbar_wait(mBf, i & 1) && (i < 2 || mbar_wait(re + 8 * rbuf, ((i >> 1) - 1) & 1));
         if (!ok) break;
@@ -1109,7 +1072,7 @@ __global__ void __launch_bounds__(kT2Threads, 1)
           for (int sum = NP - 1; sum >= 0; --sum)
 #pragma unroll
             for (int ia = 0; ia <= sum; ++ia, ++k)
-              umma_bf16(tR, dA + ((uint64_t)(ia * PB) >> 4) + o, dBK + ((uint64_t)((sum - ia) * PB) >> 4) + o, idR,
+              umma_f16(tR, dA + ((uint64_t)(ia * PB) >> 4) + o, dBK + ((uint64_t)((sum - ia) * PB) >> 4) + o, idR,
                         (a > 0 || k > 0) ? 1u : 0u);
         }
         umma_commit(mAe);
@@ -1124,7 +1087,7 @@ __global__ void __launch_bounds__(kT2Threads, 1)
           for (int sum = NP - 1; sum >= 0; --sum)
 #pragma unroll
             for (int ia = 0; ia <= sum; ++ia, ++k)
-              umma_bf16(T, dV + ((uint64_t)(ia * 8192) >> 4) + 16u * kb,
+              umma_f16(T, dV + ((uint64_t)(ia * 8192) >> 4) + 16u * kb,
                         dBM + ((uint64_t)((sum - ia) * PB) >> 4) + ((uint64_t)(2 * rowg * kb) >> 4), idZ,
                         (kb > 0 || k > 0) ? 1u : 0u);
         }
@@ -1205,10 +1168,10 @@ __global__ void __launch_bounds__(kT2Threads, 1)
 #pragma unroll
       for (int c = 0; c < 4; ++c) ev[c] = warp_sum_f(ev[c]);
       if (lane == 0 && ok) {
-        if (ev[0] != 0.f) dev::add_E(P, -(double)ev[0]);
+        if (ev[0] != 0.f) dev::add_E(P, -(double)ev[0] * P.sc.r2);
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-          if (ev[c + 1] != 0.f) dev::add_gV(P, 3 * p + c, -(double)ev[c + 1]);
+          if (ev[c + 1] != 0.f) dev::add_gV(P, 3 * p + c, -(double)ev[c + 1] * P.sc.r2);
       }
       // ---- Z -> the Z store: NP planes of 128-row tiles of rows (alpha, a),
       // 16 columns b each, in the core-matrix order of tix; a thread writes
@@ -1232,11 +1195,15 @@ __global__ void __launch_bounds__(kT2Threads, 1)
             uint16_t* d = Zo + (long long)(r >> 7) * NP * 2048 + (((r & 127) >> 3) << 7) + ((r & 7) << 3);
 #pragma unroll
             for (int hb = 0; hb < 2; ++hb) {
-              const float x0[4] = {x[8 * hb], x[8 * hb + 1], x[8 * hb + 2], x[8 * hb + 3]};
-              const float x1[4] = {x[8 * hb + 4], x[8 * hb + 5], x[8 * hb + 6], x[8 * hb + 7]};
+              float x0[4], x1[4];
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                x0[k] = x[8 * hb + k] * scf<SP>(P.sc.z);
+                x1[k] = x[8 * hb + 4 + k] * scf<SP>(P.sc.z);
+              }
               uint2 p0[NP], p1[NP];
-              split4<NP>(x0, p0);
-              split4<NP>(x1, p1);
+              split4<SP>(x0, p0);
+              split4<SP>(x1, p1);
 #pragma unroll
               for (int pp = 0; pp < NP; ++pp)
                 *reinterpret_cast<uint4*>(d + pp * 2048 + 64 * hb) = make_uint4(p0[pp].x, p0[pp].y, p1[pp].x, p1[pp].y);
@@ -1274,28 +1241,28 @@ int num_sms() {
 
 long long t1u_launch_count() { return g_t1u_launches; }
 
-size_t t1u_smem(int np, int KP, int NS, int FS) {
-  return (size_t)np * 64 * KP * 2 * 2 + (size_t)np * 8192 + 2 * 256 * 4 + (size_t)NS * FS * 1024 * 4;
+size_t t1u_smem(int pieces, int KP, int NS, int FS) {
+  return (size_t)pieces * 64 * KP * 2 * 2 + (size_t)pieces * 8192 + 2 * 256 * 4 + (size_t)NS * FS * 1024 * 4;
 }
 
 int t1u_max_slots() { return kMaxNS; }
 
-cudaError_t t1u_set_smem(int np) {
-  return allow_max_dynamic_smem(np == 2 ? (const void*)k_t1_umma<2> : (const void*)k_t1_umma<3>);
+cudaError_t t1u_set_smem(int sp) {
+  return allow_max_dynamic_smem(sp == kSplitBf16 ? (const void*)k_t1_umma<kSplitBf16> : (const void*)k_t1_umma<kSplitHalf>);
 }
 
-cudaError_t launch_t1u_stores(const DevPlan& P, const T1UPlan& U, int np, const int* qlist, int nq, bool dstore,
+cudaError_t launch_t1u_stores(const DevPlan& P, const T1UPlan& U, int sp, const int* qlist, int nq, bool dstore,
                               cudaStream_t s) {
   if (nq > 0) {
     ++g_t1u_launches;
     static std::once_flag attr;
     std::call_once(attr, [] {
-      cudaFuncSetAttribute(k_t1u_cstore<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCStoreSmem);
-      cudaFuncSetAttribute(k_t1u_cstore<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCStoreSmem);
+      cudaFuncSetAttribute(k_t1u_cstore<kSplitBf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCStoreSmem);
+      cudaFuncSetAttribute(k_t1u_cstore<kSplitHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCStoreSmem);
     });
     const int g = nq < 152 * 3 ? nq : 152 * 3;
-    if (np == 2) k_t1u_cstore<2><<<g, 256, kCStoreSmem, s>>>(P, U, qlist, nq);
-    else k_t1u_cstore<3><<<g, 256, kCStoreSmem, s>>>(P, U, qlist, nq);
+    if (sp == kSplitBf16) k_t1u_cstore<kSplitBf16><<<g, 256, kCStoreSmem, s>>>(P, U, qlist, nq);
+    else k_t1u_cstore<kSplitHalf><<<g, 256, kCStoreSmem, s>>>(P, U, qlist, nq);
   }
   if (dstore && P.n_d > 0) {
     ++g_t1u_launches;
@@ -1318,47 +1285,47 @@ cudaError_t launch_lpt_order(const int* key, int asc, const int* list, int n_max
   return cudaGetLastError();
 }
 
-cudaError_t launch_vstores(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int np, const int* list, int n,
+cudaError_t launch_vstores(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int sp, const int* list, int n,
                            cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   ++g_t1u_launches;
   static std::once_flag attr;
   std::call_once(attr, [] {
-    cudaFuncSetAttribute(k_vstores<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kVStoreSmem);
-    cudaFuncSetAttribute(k_vstores<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kVStoreSmem);
+    cudaFuncSetAttribute(k_vstores<kSplitBf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kVStoreSmem);
+    cudaFuncSetAttribute(k_vstores<kSplitHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, kVStoreSmem);
   });
   const int g = n < 152 * 3 ? n : 152 * 3;
-  if (np == 2) k_vstores<2><<<g, 256, kVStoreSmem, s>>>(P, X, U, list, n);
-  else k_vstores<3><<<g, 256, kVStoreSmem, s>>>(P, X, U, list, n);
+  if (sp == kSplitBf16) k_vstores<kSplitBf16><<<g, 256, kVStoreSmem, s>>>(P, X, U, list, n);
+  else k_vstores<kSplitHalf><<<g, 256, kVStoreSmem, s>>>(P, X, U, list, n);
   return cudaGetLastError();
 }
 
-size_t t2u_smem(int np, int max_ao) { return (size_t)np * (2 * 64 * 16 * (size_t)max_ao * 2 + 8192); }
+size_t t2u_smem(int max_ao) { return (size_t)NP * (2 * 64 * 16 * (size_t)max_ao * 2 + 8192); }
 
-cudaError_t t2u_set_smem(int np) {
-  return allow_max_dynamic_smem(np == 2 ? (const void*)k_t2_umma<2> : (const void*)k_t2_umma<3>);
+cudaError_t t2u_set_smem(int sp) {
+  return allow_max_dynamic_smem(sp == kSplitBf16 ? (const void*)k_t2_umma<kSplitBf16> : (const void*)k_t2_umma<kSplitHalf>);
 }
 
-cudaError_t launch_t2_umma(const DevPlan& P, const MixPlan& X, int np, const int* list, int n, long long zblk,
+cudaError_t launch_t2_umma(const DevPlan& P, const MixPlan& X, int sp, const int* list, int n, long long zblk,
                            size_t smem, int* err, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   ++g_t1u_launches;
   const int grid = n < num_sms() ? n : num_sms();
-  const int KKmax = (int)(smem / np - 8192) / (2 * 64 * 2);   // 16 x the largest n_ao
-  if (np == 2) k_t2_umma<2><<<grid, kT2Threads, smem, s>>>(P, X, list, n, KKmax, zblk, err);
-  else k_t2_umma<3><<<grid, kT2Threads, smem, s>>>(P, X, list, n, KKmax, zblk, err);
+  const int KKmax = (int)(smem / NP - 8192) / (2 * 64 * 2);   // 16 x the largest n_ao
+  if (sp == kSplitBf16) k_t2_umma<kSplitBf16><<<grid, kT2Threads, smem, s>>>(P, X, list, n, KKmax, zblk, err);
+  else k_t2_umma<kSplitHalf><<<grid, kT2Threads, smem, s>>>(P, X, list, n, KKmax, zblk, err);
   return cudaGetLastError();
 }
 
-cudaError_t launch_t1_umma(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int np, const int* qlist, int n,
+cudaError_t launch_t1_umma(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int sp, const int* qlist, int n,
                            size_t smem, int* work, int* err, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   ++g_t1u_launches;
   const int grid = n < num_sms() ? n : num_sms();
   cudaError_t e = cudaMemsetAsync(work, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
-  if (np == 2) k_t1_umma<2><<<grid, kThreads, smem, s>>>(P, X, U, qlist, n, work, err);
-  else k_t1_umma<3><<<grid, kThreads, smem, s>>>(P, X, U, qlist, n, work, err);
+  if (sp == kSplitBf16) k_t1_umma<kSplitBf16><<<grid, kThreads, smem, s>>>(P, X, U, qlist, n, work, err);
+  else k_t1_umma<kSplitHalf><<<grid, kThreads, smem, s>>>(P, X, U, qlist, n, work, err);
   return cudaGetLastError();
 }
 

@@ -59,20 +59,20 @@ template <int N>
 __device__ __forceinline__ void cpa_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // piece pp of (x0, x1) packed as one 32-bit word, x0 in the low half
-template <int NP>
+template <int SP>
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t (&w)[NP]) {
   uint16_t p0[NP], p1[NP];
-  split_f<NP>(x0, p0);
-  split_f<NP>(x1, p1);
+  split_f<SP>(x0, p0);
+  split_f<SP>(x1, p1);
 #pragma unroll
   for (int pp = 0; pp < NP; ++pp) w[pp] = pack2(p0[pp], p1[pp]);
 }
 
 // element e of a [rows][S] bf16 plane set (NP planes of `plane` elements): the NP pieces of x
-template <int NP>
+template <int SP>
 __device__ __forceinline__ void put_pieces(uint16_t* base, long long plane, int e, float x) {
   uint16_t pc[NP];
-  split_f<NP>(x, pc);
+  split_f<SP>(x, pc);
 #pragma unroll
   for (int pp = 0; pp < NP; ++pp) base[pp * plane + e] = pc[pp];
 }
@@ -112,7 +112,7 @@ struct RTiles {
 
 // acc += A . B^T over K in [0, K): A rows (M) at As (stride SA), B rows (N) at Bs
 // (stride SB), both K-contiguous, for tile pair (mt, nt0, nt0 + 1).
-template <int NP>
+template <int SP>
 __device__ __forceinline__ void gemm_pair_kk(float (&acc)[2][4], const uint16_t* As, long long pa, int SA,
                                              const uint16_t* Bs, long long pb, int SB, int mt, int nt0, bool two, int K) {
   const int lane = threadIdx.x & 31;
@@ -125,13 +125,13 @@ __device__ __forceinline__ void gemm_pair_kk(float (&acc)[2][4], const uint16_t*
       ldm_x2(b0[pp], Bs + pp * pb + (long long)(nt0 * 8 + (lane & 7)) * SB + k0 + (((lane >> 3) & 1) << 3));
       ldm_x2(b1[pp], Bs + pp * pb + (long long)(nt1 * 8 + (lane & 7)) * SB + k0 + (((lane >> 3) & 1) << 3));
     }
-    mma_split2<NP>(acc[0], af, b0, acc[1], af, b1);
+    mma_split2<SP>(acc[0], af, b0, acc[1], af, b1);
   }
 }
 
 // acc += A . B over K in [0, K): A rows (M) K-contiguous at As (stride SA), B
 // rows (K) N-contiguous at Bs (stride SB), for tile pair (mt, nt0, nt0 + 1).
-template <int NP>
+template <int SP>
 __device__ __forceinline__ void gemm_pair_kn(float (&acc)[2][4], const uint16_t* As, long long pa, int SA,
                                              const uint16_t* Bs, long long pb, int SB, int mt, int nt0, bool two, int K) {
   const int lane = threadIdx.x & 31;
@@ -144,14 +144,14 @@ __device__ __forceinline__ void gemm_pair_kn(float (&acc)[2][4], const uint16_t*
       ldm_x2_trans(b0[pp], Bs + pp * pb + (long long)(k0 + (lane & 15)) * SB + nt0 * 8);
       ldm_x2_trans(b1[pp], Bs + pp * pb + (long long)(k0 + (lane & 15)) * SB + nt1 * 8);
     }
-    mma_split2<NP>(acc[0], af, b0, acc[1], af, b1);
+    mma_split2<SP>(acc[0], af, b0, acc[1], af, b1);
   }
 }
 
 // ------------------------------------------------------------------ D pieces
-// D block k (fixed for the plan) -> NP bf16 planes of rup16(n_ao(I)) x
+// D block k (fixed for the plan) -> NP planes of rup16(n_ao(I)) x
 // rup16(n_ao(J)), row-major, zero padded, at Dw + dw_off[k].
-template <int NP>
+template <int SP>
 __global__ void k_dsplit_w(DevPlan P, uint16_t* Dw, const long long* dw_off) {
   for (long long k = blockIdx.x; k < P.n_d; k += gridDim.x) {
     const int I = P.Didx[5 * k], J = P.Didx[5 * k + 1];
@@ -161,7 +161,7 @@ __global__ void k_dsplit_w(DevPlan P, uint16_t* Dw, const long long* dw_off) {
     uint16_t* out = Dw + dw_off[k];
     for (int e = threadIdx.x; e < pa * pb; e += blockDim.x) {
       const int a = e / pb, b = e - a * pb;
-      put_pieces<NP>(out, (long long)pa * pb, e, (a < na && b < nb) ? (float)src[a * nb + b] : 0.f);
+      put_pieces<SP>(out, (long long)pa * pb, e, (a < na && b < nb) ? (float)src[a * nb + b] * scf<SP>(P.sc.d) : 0.f);
     }
   }
 }
@@ -177,7 +177,7 @@ __host__ __device__ inline int cw_cols(int nA, int nF) { return (nA * nF + 7) & 
 // ... and grad C in FP32 (dCf, the layout of P.dCst), which the first
 // product's Q epilogue reads in MMA-fragment order: half the bytes of the
 // FP64 blocks, and the same values (the epilogue rounds to FP32 anyway).
-template <int NP>
+template <int SP>
 __global__ void k_cpieces_w(DevPlan P, uint16_t* Cw, const long long* cw_off, float* dCf) {
   for (int q = blockIdx.x; q < P.nC; q += gridDim.x) {
     if (!P.c_keep[q]) continue;
@@ -188,12 +188,12 @@ __global__ void k_cpieces_w(DevPlan P, uint16_t* Cw, const long long* cw_off, fl
     uint16_t* out = Cw + cw_off[q];
     for (int e = threadIdx.x; e < mA * CW; e += blockDim.x) {
       const int al = e / CW, c = e - al * CW;
-      put_pieces<NP>(out, (long long)mA * CW, e, c < naf ? (float)src[(long long)al * naf + c] : 0.f);
+      put_pieces<SP>(out, (long long)mA * CW, e, c < naf ? (float)src[(long long)al * naf + c] * scf<SP>(P.sc.c) : 0.f);
     }
     uint16_t* cy = out + (long long)NP * mA * CW;
     for (int e = threadIdx.x; e < mA * nA * KW; e += blockDim.x) {
       const int r = e / KW, c = e - r * KW;
-      put_pieces<NP>(cy, (long long)mA * nA * KW, e, c < nF ? (float)src[(long long)r * nF + c] : 0.f);
+      put_pieces<SP>(cy, (long long)mA * nA * KW, e, c < nF ? (float)src[(long long)r * nF + c] * scf<SP>(P.sc.c) : 0.f);
     }
     const double* dsrc = P.dCst + 3 * P.c_off[q];
     float* dst = dCf + 3 * P.c_off[q];
@@ -211,9 +211,9 @@ __global__ void k_cpieces_w(DevPlan P, uint16_t* Cw, const long long* cw_off, fl
 constexpr int kYRows = 64;
 constexpr int kYSA = 24;
 constexpr int kYSB = 8 * 32 + 8;
-size_t ybuild_w_smem(int np) { return (size_t)2 * np * (kYRows * kYSA + 16 * kYSB) * sizeof(uint16_t); }
+size_t ybuild_w_smem() { return (size_t)2 * NP * (kYRows * kYSA + 16 * kYSB) * sizeof(uint16_t); }
 
-template <int NP>
+template <int SP>
 __global__ void __launch_bounds__(kWThreads) k_ybuild_w(DevPlan P, uint16_t* __restrict__ Yp,
                                                         const uint16_t* __restrict__ Cw, const long long* cw_off,
                                                         const uint16_t* __restrict__ Dw, const long long* dw_off,
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kWThreads) k_ybuild_w(DevPlan P, uint16_t* __r
         uint32_t bf[NP][2];
 #pragma unroll
         for (int pp = 0; pp < NP; ++pp) ldm_x2_trans(bf[pp], Bs + pp * pB + (lane & 15) * kYSB + i * 32 + nt * 8);
-        mma_split<NP>(acc[ii][nt], af, bf);
+        mma_split<SP>(acc[ii][nt], af, bf);
       }
     }
     __syncthreads();   // buffer k & 1 is free for step k + 2
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kWThreads) k_ybuild_w(DevPlan P, uint16_t* __r
         if (row < rows && z < nZ) {
           const int al = row / nX, x = row - al * nX;
           const long long o = ((long long)al * nZ + z) * KX;
-          put_pieces<NP>(Y, plane, (int)(o + x), acc[ii][nt][c]);
+          put_pieces<SP>(Y, plane, (int)(o + x), acc[ii][nt][c] * scf<SP>(P.sc.y));
           if (x == nX - 1)
             for (int xp = nX; xp < KX; ++xp)
 #pragma unroll
@@ -384,11 +384,11 @@ struct T1W {
   int MA, MB, KC, da;
 };
 
-__host__ __device__ inline size_t term1w_smem(int np, int MA, int MB, int KC) {
-  return (size_t)np * 2 * ((size_t)MA * (MB + 8) + 48 * 40 + (size_t)MA * (KC + 8) + (size_t)MB * (KC + 8));
+__host__ __device__ inline size_t term1w_smem(int MA, int MB, int KC) {
+  return (size_t)NP * 2 * ((size_t)MA * (MB + 8) + 48 * 40 + (size_t)MA * (KC + 8) + (size_t)MB * (KC + 8));
 }
 
-template <int NP>
+template <int SP>
 __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16_t* __restrict__ Yp,
                                                        const uint16_t* __restrict__ Cw, const long long* cw_off,
                                                        const uint16_t* __restrict__ Dw, const long long* dw_off,
@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
     }
     for (int e = threadIdx.x; e < MA * SV; e += blockDim.x) {
       const int al = e / SV, be = e - al * SV;
-      put_pieces<NP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] : 0.f);
+      put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * scf<SP>(P.sc.v) : 0.f);
     }
     for (int e = threadIdx.x; e < 48 * SD; e += blockDim.x) {
       const int a = e / SD, bb = e - a * SD;
@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
           }
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c) ev[c] += (double)evf[c];
+      for (int c = 0; c < 4; ++c) ev[c] += (double)evf[c] * P.sc.r1;
     };
     const int q0 = P.c_ptr[A];
     double fl = 0.0;
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
                   bf[pp][0] = in ? *reinterpret_cast<const uint32_t*>(yr) : 0u;
                   bf[pp][1] = in ? *reinterpret_cast<const uint32_t*>(yr + 8) : 0u;
                 }
-                mma_split<NP>(acc, af[ks], bf);
+                mma_split<SP>(acc, af[ks], bf);
               }
               // acc[0], acc[1]: row a0 + gid, columns (beta, f) = nt * 8 + 2 tig, + 1
               if (gid < dA) {
@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
                   const int r = nt * 8 + 2 * tig + c;
                   if (r < rowsU) {
                     const int be = r / nF, ff = r - be * nF;
-                    put_pieces<NP>(Us, pU, be * SK + gid * nF + ff, acc[c]);
+                    put_pieces<SP>(Us, pU, be * SK + gid * nF + ff, acc[c] * scf<SP>(P.sc.u));
                   }
                 }
               }
@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
             const int pr = warp + kPW * i;
             if (pr >= rt.count()) break;
             const int mt = pr / rt.NTP, nt0 = 2 * (pr - mt * rt.NTP);
-            gemm_pair_kk<NP>(racc[i], Cs, pC, SK, Us, pU, SK, mt, nt0, nt0 + 1 < rt.NT, KCc);
+            gemm_pair_kk<SP>(racc[i], Cs, pC, SK, Us, pU, SK, mt, nt0, nt0 + 1 < rt.NT, KCc);
           }
           // Q = V_AB . U (M = alpha, N = columns, K = beta), dotted with grad C_AF
           {
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
             for (int pr = warp; pr < npairs; pr += kPW) {
               const int mt = pr / NPQ, nt0 = 2 * (pr - mt * NPQ);
               float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-              gemm_pair_kn<NP>(acc, Vs, pV, SV, Us, pU, SK, mt, nt0, nt0 + 1 < NTQ, MBp);
+              gemm_pair_kn<SP>(acc, Vs, pV, SV, Us, pU, SK, mt, nt0, nt0 + 1 < NTQ, MBp);
 #pragma unroll
               for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -617,8 +617,9 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
         for (int c = 0; c < 3; ++c) {
           const float w = warp_sum_f(gq[c]);
           if (lane == 0) {
-            if (P.fxC) dev::add_gC(P, 3 * q + c, -2.0 * (double)w);   // deterministic plan: straight into the exact cell
-            else atomicAdd(&s_g[c], (double)w);
+            const double wd = (double)w * P.sc.q1;
+            if (P.fxC) dev::add_gC(P, 3 * q + c, -2.0 * wd);   // deterministic plan: straight into the exact cell
+            else atomicAdd(&s_g[c], wd);
           }
         }
         fl += 2.0 * mB * nA * nB * nF + 4.0 * mA * mB * nA * nF;
@@ -656,11 +657,11 @@ struct T2W {
   long long zplane;    // elements per piece plane of a slot (most rows x KZ)
 };
 
-__host__ __device__ inline size_t term2w_smem(int np, int MA, int MB, int KC) {
-  return (size_t)np * 2 * ((size_t)MA * (MB + 8) + (size_t)MA * (KC + 8) + (size_t)MB * (KC + 8));
+__host__ __device__ inline size_t term2w_smem(int MA, int MB, int KC) {
+  return (size_t)NP * 2 * ((size_t)MA * (MB + 8) + (size_t)MA * (KC + 8) + (size_t)MB * (KC + 8));
 }
 
-template <int NP>
+template <int SP>
 __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16_t* __restrict__ Yp,
                                                        uint16_t* __restrict__ Zw, const int* list, int n_list, T2W S) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -699,7 +700,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
     }
     for (int e = threadIdx.x; e < MA * SV; e += blockDim.x) {
       const int al = e / SV, be = e - al * SV;
-      put_pieces<NP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] : 0.f);
+      put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * scf<SP>(P.sc.v) : 0.f);
     }
     // Y^{BA} rows beyond n_abf(B) stay zero (K of Z)
     for (int e = threadIdx.x; e < (MB - mB) * SK; e += blockDim.x)
@@ -760,7 +761,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
         const int pr = warp + kPW * i;
         if (pr >= rt.count()) break;
         const int mt = pr / rt.NTP, nt0 = 2 * (pr - mt * rt.NTP);
-        gemm_pair_kk<NP>(racc[i], Ya, pA, SK, Yb, pB, SK, mt, nt0, nt0 + 1 < rt.NT, KCc);
+        gemm_pair_kk<SP>(racc[i], Ya, pA, SK, Yb, pB, SK, mt, nt0, nt0 + 1 < rt.NT, KCc);
       }
       // Z = V_AB . Y^{BA} (M = alpha, N = (a, b), K = beta) -> Z store rows (alpha, a)
       {
@@ -769,7 +770,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
         for (int pr = warp; pr < npairs; pr += kPW) {
           const int mt = pr / NPZ, nt0 = 2 * (pr - mt * NPZ);
           float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-          gemm_pair_kn<NP>(acc, Vs, pV, SV, Yb, pB, SK, mt, nt0, nt0 + 1 < NTZ, MBp);
+          gemm_pair_kn<SP>(acc, Vs, pV, SV, Yb, pB, SK, mt, nt0, nt0 + 1 < NTZ, MBp);
 #pragma unroll
           for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -778,7 +779,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
               const int n = (nt0 + h) * 8 + 2 * tig + (c & 1);
               if (al < mA && n < dcols && nt0 + h < NTZ) {
                 const int bb = n / dA, a = n - bb * dA;
-                put_pieces<NP>(Z, S.zplane, (int)(((long long)al * nA + a0 + a) * S.KZ + bb), acc[h][c]);
+                put_pieces<SP>(Z, S.zplane, (int)(((long long)al * nA + a0 + a) * S.KZ + bb), acc[h][c] * scf<SP>(P.sc.z));
               }
             }
         }
@@ -810,7 +811,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
           }
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c) ev[c] = (double)evf[c];
+      for (int c = 0; c < 4; ++c) ev[c] = (double)evf[c] * P.sc.r2;
     }
     block_sum_w<4, kPW>(ev, red);
     if (threadIdx.x == 0) {
@@ -839,11 +840,11 @@ constexpr int kQ2Slots = 8;
 constexpr int kQ2Seg = 256;   // pairs per segment of D-block metadata
 constexpr int kQ2Run = 64;    // pairs per FP32 run
 
-__host__ __device__ inline size_t q2w_smem(int np, int KZ) {
-  return (size_t)2 * np * 2 * (size_t)(kQ2Rows + kQ2Slots * 32) * (KZ + 8);
+__host__ __device__ inline size_t q2w_smem(int KZ) {
+  return (size_t)2 * NP * 2 * (size_t)(kQ2Rows + kQ2Slots * 32) * (KZ + 8);
 }
 
-template <int NP>
+template <int SP>
 __global__ void __launch_bounds__(kQ2Threads, 1) k_q2_w(DevPlan P, const uint16_t* __restrict__ Zw, long long zplane,
                                                         int KZ, const uint16_t* __restrict__ Dw,
                                                         const long long* __restrict__ dw_off, const int* list,
@@ -926,7 +927,7 @@ __global__ void __launch_bounds__(kQ2Threads, 1) k_q2_w(DevPlan P, const uint16_
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const float w = warp_sum_f(g[c]);
-        if (lane == 0) s_ev[warp][i][c] += (double)w;
+        if (lane == 0) s_ev[warp][i][c] += (double)w * P.sc.q2;
       }
     }
   };
@@ -1016,7 +1017,7 @@ __global__ void __launch_bounds__(kQ2Threads, 1) k_q2_w(DevPlan P, const uint16_
             for (int pp = 0; pp < NP; ++pp)
               ldm_x2(bf[pp], Bs + pp * pB + ((4 * sh + i) * 32 + nt * 8 + (lane & 7)) * SZ + ks +
                                  (((lane >> 3) & 1) << 3));
-            mma_split<NP>(acc[i][nt], af, bf);
+            mma_split<SP>(acc[i][nt], af, bf);
           }
         }
       }
@@ -1053,125 +1054,125 @@ long long wide_launch_count() { return g_wide_launches.load(); }
 
 int wide_ybuild_row_blocks(int max_rows) { return (max_rows + kYRows - 1) / kYRows; }
 
-WideShapes wide_shapes(int np, int maxABF, int maxAO, size_t limit) {
+WideShapes wide_shapes(int maxABF, int maxAO, size_t limit) {
   WideShapes w{};
   w.MA = w.MB = (maxABF + 15) / 16 * 16;
   w.KZ = (maxAO + 15) / 16 * 16;
   for (int da : {8, 4, 2, 1}) {
     const int KC = (da * maxAO + 15) / 16 * 16;
-    if (term1w_smem(np, w.MA, w.MB, KC) <= limit) {
+    if (term1w_smem(w.MA, w.MB, KC) <= limit) {
       w.t1_da = da;
       w.t1_KC = KC;
-      w.smem_t1 = term1w_smem(np, w.MA, w.MB, KC);
+      w.smem_t1 = term1w_smem(w.MA, w.MB, KC);
       break;
     }
   }
   for (int da : {8, 4, 2, 1}) {
     const int KC = (da * maxAO + 15) / 16 * 16;
-    if (term2w_smem(np, w.MA, w.MB, KC) <= limit) {
+    if (term2w_smem(w.MA, w.MB, KC) <= limit) {
       w.t2_da = da;
       w.t2_KC = KC;
-      w.smem_t2 = term2w_smem(np, w.MA, w.MB, KC);
+      w.smem_t2 = term2w_smem(w.MA, w.MB, KC);
       break;
     }
   }
-  w.smem_q2 = q2w_smem(np, w.KZ);
+  w.smem_q2 = q2w_smem(w.KZ);
   // R tiles: (MA / 16) x (MB / 16) pairs over the warps, kPRP each
   w.ok = w.t1_da > 0 && w.t2_da > 0 && w.smem_q2 <= limit && (w.MA / 16) * (w.MB / 16) <= kPW * kPRP &&
          maxAO <= 32;
   return w;
 }
 
-cudaError_t set_wide_smem_limits(int np) {
+cudaError_t set_wide_smem_limits(int sp) {
   cudaError_t e = cudaSuccess;
   auto one = [&](const void* f) {
     const cudaError_t r = allow_max_dynamic_smem(f);
     if (r != cudaSuccess) e = r;
   };
-  if (np == 2) {
-    one((const void*)k_ybuild_w<2>);
-    one((const void*)k_term1_w<2>);
-    one((const void*)k_term2_w<2>);
-    one((const void*)k_q2_w<2>);
+  if (sp == kSplitBf16) {
+    one((const void*)k_ybuild_w<kSplitBf16>);
+    one((const void*)k_term1_w<kSplitBf16>);
+    one((const void*)k_term2_w<kSplitBf16>);
+    one((const void*)k_q2_w<kSplitBf16>);
   } else {
-    one((const void*)k_ybuild_w<3>);
-    one((const void*)k_term1_w<3>);
-    one((const void*)k_term2_w<3>);
-    one((const void*)k_q2_w<3>);
+    one((const void*)k_ybuild_w<kSplitHalf>);
+    one((const void*)k_term1_w<kSplitHalf>);
+    one((const void*)k_term2_w<kSplitHalf>);
+    one((const void*)k_q2_w<kSplitHalf>);
   }
   return e;
 }
 
-cudaError_t launch_cpieces_w(const DevPlan& P, int np, uint16_t* Cw, const long long* cw_off, float* dCf,
+cudaError_t launch_cpieces_w(const DevPlan& P, int sp, uint16_t* Cw, const long long* cw_off, float* dCf,
                              cudaStream_t s) {
   if (P.nC <= 0) return cudaSuccess;
   const int grid = grid_cap(P.nC, 1 << 16);
-  if (np == 2) k_cpieces_w<2><<<grid, 256, 0, s>>>(P, Cw, cw_off, dCf);
-  else k_cpieces_w<3><<<grid, 256, 0, s>>>(P, Cw, cw_off, dCf);
+  if (sp == kSplitBf16) k_cpieces_w<kSplitBf16><<<grid, 256, 0, s>>>(P, Cw, cw_off, dCf);
+  else k_cpieces_w<kSplitHalf><<<grid, 256, 0, s>>>(P, Cw, cw_off, dCf);
   ++g_wide_launches;
   return cudaGetLastError();
 }
 
-long long wide_cpieces_size(int np, int n_abf, int n_ao_a, int n_ao_f) {
-  return (long long)np * n_abf * (cw_cols(n_ao_a, n_ao_f) + n_ao_a * ((n_ao_f + 15) / 16 * 16));
+long long wide_cpieces_size(int n_abf, int n_ao_a, int n_ao_f) {
+  return (long long)NP * n_abf * (cw_cols(n_ao_a, n_ao_f) + n_ao_a * ((n_ao_f + 15) / 16 * 16));
 }
 
-cudaError_t launch_ybuild_w(const DevPlan& P, int np, uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
+cudaError_t launch_ybuild_w(const DevPlan& P, int sp, uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
                             const uint16_t* Dw, const long long* dw_off, const int* ylist, const int* gX,
                             const int* gS, const int* gN, int ngroups, int RB, cudaStream_t s) {
   if (ngroups <= 0) return cudaSuccess;
   const long long grid = (long long)ngroups * RB;
-  const size_t smem = ybuild_w_smem(np);
-  if (np == 2)
-    k_ybuild_w<2><<<(unsigned)grid, kWThreads, smem, s>>>(P, Yp, Cw, cw_off, Dw, dw_off, ylist, gX, gS, gN, RB);
+  const size_t smem = ybuild_w_smem();
+  if (sp == kSplitBf16)
+    k_ybuild_w<kSplitBf16><<<(unsigned)grid, kWThreads, smem, s>>>(P, Yp, Cw, cw_off, Dw, dw_off, ylist, gX, gS, gN, RB);
   else
-    k_ybuild_w<3><<<(unsigned)grid, kWThreads, smem, s>>>(P, Yp, Cw, cw_off, Dw, dw_off, ylist, gX, gS, gN, RB);
+    k_ybuild_w<kSplitHalf><<<(unsigned)grid, kWThreads, smem, s>>>(P, Yp, Cw, cw_off, Dw, dw_off, ylist, gX, gS, gN, RB);
   ++g_wide_launches;
   return cudaGetLastError();
 }
 
-cudaError_t launch_term1_w(const DevPlan& P, int np, const uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
+cudaError_t launch_term1_w(const DevPlan& P, int sp, const uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
                            const uint16_t* Dw, const long long* dw_off, const float* dCf, const int* list, int n,
                            const WideShapes& w, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const T1W S{w.MA, w.MB, w.t1_KC, w.t1_da};
   const int grid = grid_cap(n, 1 << 20);
-  if (np == 2) k_term1_w<2><<<grid, kPW * 32, w.smem_t1, s>>>(P, Yp, Cw, cw_off, Dw, dw_off, dCf, list, n, S);
-  else k_term1_w<3><<<grid, kPW * 32, w.smem_t1, s>>>(P, Yp, Cw, cw_off, Dw, dw_off, dCf, list, n, S);
+  if (sp == kSplitBf16) k_term1_w<kSplitBf16><<<grid, kPW * 32, w.smem_t1, s>>>(P, Yp, Cw, cw_off, Dw, dw_off, dCf, list, n, S);
+  else k_term1_w<kSplitHalf><<<grid, kPW * 32, w.smem_t1, s>>>(P, Yp, Cw, cw_off, Dw, dw_off, dCf, list, n, S);
   ++g_wide_launches;
   return cudaGetLastError();
 }
 
 long long wide_zplane(int max_rows, int KZ) { return (long long)max_rows * KZ; }
 
-cudaError_t launch_dsplit_w(const DevPlan& P, int np, uint16_t* Dw, const long long* dw_off, cudaStream_t s) {
+cudaError_t launch_dsplit_w(const DevPlan& P, int sp, uint16_t* Dw, const long long* dw_off, cudaStream_t s) {
   if (P.n_d <= 0) return cudaSuccess;
   const int grid = grid_cap(P.n_d, 1 << 16);
-  if (np == 2) k_dsplit_w<2><<<grid, 256, 0, s>>>(P, Dw, dw_off);
-  else k_dsplit_w<3><<<grid, 256, 0, s>>>(P, Dw, dw_off);
+  if (sp == kSplitBf16) k_dsplit_w<kSplitBf16><<<grid, 256, 0, s>>>(P, Dw, dw_off);
+  else k_dsplit_w<kSplitHalf><<<grid, 256, 0, s>>>(P, Dw, dw_off);
   ++g_wide_launches;
   return cudaGetLastError();
 }
 
-cudaError_t launch_term2_w(const DevPlan& P, int np, const uint16_t* Yp, uint16_t* Zw, const uint16_t* Dw,
+cudaError_t launch_term2_w(const DevPlan& P, int sp, const uint16_t* Yp, uint16_t* Zw, const uint16_t* Dw,
                            const long long* dw_off, const float* dCf, const int* list, const long long* slot0, int n,
                            int a0, int a1, int max_rows, int max_c, const WideShapes& w, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const T2W S{w.MA, w.MB, w.t2_KC, w.t2_da, w.KZ, wide_zplane(max_rows, w.KZ)};
   const int grid = grid_cap(n, 1 << 20);
-  if (np == 2) k_term2_w<2><<<grid, kPW * 32, w.smem_t2, s>>>(P, Yp, Zw, list, n, S);
-  else k_term2_w<3><<<grid, kPW * 32, w.smem_t2, s>>>(P, Yp, Zw, list, n, S);
+  if (sp == kSplitBf16) k_term2_w<kSplitBf16><<<grid, kPW * 32, w.smem_t2, s>>>(P, Yp, Zw, list, n, S);
+  else k_term2_w<kSplitHalf><<<grid, kPW * 32, w.smem_t2, s>>>(P, Yp, Zw, list, n, S);
   ++g_wide_launches;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int RBQ = (max_rows + kQ2Rows - 1) / kQ2Rows, SG = (max_c + kQ2Slots - 1) / kQ2Slots;
   const long long qgrid = (long long)(a1 - a0) * RBQ * SG;
   if (qgrid <= 0) return cudaSuccess;
-  if (np == 2)
-    k_q2_w<2><<<(unsigned)qgrid, kQ2Threads, w.smem_q2, s>>>(P, Zw, S.zplane, w.KZ, Dw, dw_off, list, slot0, n, a0, a1,
+  if (sp == kSplitBf16)
+    k_q2_w<kSplitBf16><<<(unsigned)qgrid, kQ2Threads, w.smem_q2, s>>>(P, Zw, S.zplane, w.KZ, Dw, dw_off, list, slot0, n, a0, a1,
                                                              RBQ, SG, dCf);
   else
-    k_q2_w<3><<<(unsigned)qgrid, kQ2Threads, w.smem_q2, s>>>(P, Zw, S.zplane, w.KZ, Dw, dw_off, list, slot0, n, a0, a1,
+    k_q2_w<kSplitHalf><<<(unsigned)qgrid, kQ2Threads, w.smem_q2, s>>>(P, Zw, S.zplane, w.KZ, Dw, dw_off, list, slot0, n, a0, a1,
                                                              RBQ, SG, dCf);
   ++g_wide_launches;
   return cudaGetLastError();
