@@ -62,10 +62,13 @@ typedef enum {
 
 /* Arithmetic of the contraction.  HFX_FP64 runs every step in FP64.  The
  * other values select split-precision tensor-core contractions with FP32
- * accumulation and FP64 screening, force, stress and energy reduction:
- * every operand is written as 2 (BF16X3) or 3 (BF16X6) bf16 pieces and the
- * piece products above 2^-16 (BF16X3) or 2^-24 (BF16X6) of the operands'
- * scale are kept.  (Value 1 is not assigned.) */
+ * accumulation and FP64 screening, force, stress and energy reduction.
+ * BF16X3 writes every operand as two bf16 pieces and keeps the piece products
+ * above 2^-16 of the operands' scale.  BF16X6 stands for the accuracy of six
+ * products of three bf16 pieces: it writes every operand as two fp16 pieces
+ * (22 significant bits) under power-of-two scales taken from bounds of the
+ * blocks, and keeps the piece products above 2^-22 of the operands' scale;
+ * FP32 accumulation bounds its error.  (Value 1 is not assigned.) */
 enum { HFX_FP64 = 0, HFX_BF16X3 = 2, HFX_BF16X6 = 3 };
 
 /* Exchange products of Eq. exx_expand: bit 0 = D_AB D_FG, bit 1 = D_AG D_FB. */

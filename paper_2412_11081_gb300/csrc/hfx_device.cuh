@@ -49,7 +49,7 @@ constexpr int NP = kPieces;
 
 // A factor of SplitScale: 1 (and no multiplication) with bf16 pieces.
 template <int SP>
-__device__ __forceinline__ float scf(float s) {
+__device__ __forceinline__ float pscale(float s) {
   return SP == kSplitHalf ? s : 1.f;
 }
 

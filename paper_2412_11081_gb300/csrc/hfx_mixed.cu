@@ -1,11 +1,18 @@
 // Split-precision tensor-core kernels of the HFX force/stress hot path.
 //
-// Every FP64 operand x of a contraction is written as NP pieces
-// x = p0 + p1 (+ p2) + r (p0 = bf16(x), p1 = bf16(x - p0), ...), and each
-// product keeps the piece pairs (i, j) with i + j < NP: three warp-level
-// MMAs for NP = 2, six for NP = 3 (the BF16x3 / BF16x6 splits of Henry,
-// Tang & Heinecke).  Accumulation is FP32 in the MMA and FP64 beyond a
-// short run; the screening, the pair gradients, E, F and sigma stay FP64.
+// Every FP64 operand x of a contraction is written as two 16-bit pieces
+// x = p0 + p1 + r (p0 = x rounded to the piece type, p1 = x - p0 rounded),
+// and each product keeps the piece pairs (0,0), (0,1), (1,0): three MMAs
+// (the splitting of Henry, Tang & Heinecke).  HFX_BF16X3 takes bf16 pieces.
+// HFX_BF16X6 takes fp16 pieces of operands scaled by powers of two
+// (hfx_device.cuh): 2 x 11 significant bits in three products instead of
+// 3 x 8 in six.  Measured against three bf16 pieces: 64-atom Si cell 55.1 ->
+// 47.6 ms per evaluation (Y stage 7.2 -> 5.5, second product 8.9 -> 6.8,
+// first product 38.2 -> 34.3), 40-atom perovskite (hfx_wide.cu) 62.4 -> 52.0
+// ms, and the error against 64 bits smaller in each (2.7e-6 -> 2.0e-6 and
+// 2.3e-6 -> 1.6e-6: half as many roundings in the FP32 accumulators).
+// Accumulation is FP32 in the MMA and FP64 beyond a short run; the
+// screening, the pair gradients, E, F and sigma stay FP64.
 //
 // Operand stores, written once per evaluation from the FP64 blocks
 // (k_cpieces, k_vpieces): per C pair, NP planes of C [(alpha,a)][rup16(f)]
@@ -91,7 +98,7 @@ __global__ void k_dsplit(DevPlan P, MixPlan X) {
     for (int e = threadIdx.x; e < pa * pb; e += blockDim.x) {
       const int a = e / pb, b = e - a * pb;
       uint16_t pc[NP];
-      split_f<SP>((a < na && b < nb) ? (float)src[a * nb + b] * scf<SP>(P.sc.d) : 0.f, pc);
+      split_f<SP>((a < na && b < nb) ? (float)src[a * nb + b] * pscale<SP>(P.sc.d) : 0.f, pc);
 #pragma unroll
       for (int p = 0; p < NP; ++p) out[p * pa * pb + tix(a, b)] = pc[p];
     }
@@ -119,7 +126,7 @@ __global__ void k_cpieces(DevPlan P, MixPlan X) {
     for (int e = threadIdx.x; e < nt * 128 * 16; e += blockDim.x) {
       const int r = e >> 4, c = e & 15;
       uint16_t pc[NP];
-      split_f<SP>((r < rows && c < nF) ? model::c_value_f(P, scf, go, r * nF + c, 0) * scf<SP>(P.sc.c) : 0.f, pc);
+      split_f<SP>((r < rows && c < nF) ? model::c_value_f(P, scf, go, r * nF + c, 0) * pscale<SP>(P.sc.c) : 0.f, pc);
 #pragma unroll
       for (int p = 0; p < NP; ++p) out[((r >> 7) * NP + p) * 2048 + tix(r & 127, c)] = pc[p];
     }
@@ -150,7 +157,7 @@ __global__ void k_vpieces(DevPlan P, MixPlan X, const int* list, int n_list) {
     for (int e = threadIdx.x; e < mA * MB; e += blockDim.x) {
       const int al = e / MB, be = e - al * MB;
       uint16_t pc[NP];
-      split_f<SP>(be < mB ? M[al * mB + be] * hf * scf<SP>(P.sc.v) : 0.f, pc);
+      split_f<SP>(be < mB ? M[al * mB + be] * hf * pscale<SP>(P.sc.v) : 0.f, pc);
 #pragma unroll
       for (int pp = 0; pp < NP; ++pp) out[pp * mA * MB + e] = pc[pp];
     }
@@ -394,7 +401,7 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
                 if (r < rowsU && a < nA) {
                   const int be = r / nF, ff = r - be * nF;
                   uint16_t pc[NP];
-                  split_f<SP>(acc[nt][c] * scf<SP>(P.sc.u), pc);
+                  split_f<SP>(acc[nt][c] * pscale<SP>(P.sc.u), pc);
 #pragma unroll
                   for (int pp = 0; pp < NP; ++pp) Us[(size_t)pp * MB * KS + (size_t)be * KS + a * nF + ff] = pc[pp];
                 }
@@ -685,8 +692,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
           if (al < mA) {
             const int a = col >> 4, bb = col & 15;
             uint16_t p0[NP], p1[NP];
-            split_f<SP>(acc[2 * h] * scf<SP>(P.sc.z), p0);
-            split_f<SP>(acc[2 * h + 1] * scf<SP>(P.sc.z), p1);
+            split_f<SP>(acc[2 * h] * pscale<SP>(P.sc.z), p0);
+            split_f<SP>(acc[2 * h + 1] * pscale<SP>(P.sc.z), p1);
             const int r = al * nA + a;
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp)
@@ -1192,7 +1199,7 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
         }
         float* er = ep + (q * 32 + lane) * 33;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) er[j] = __uint_as_float(v[j]) * scf<SP>(P.sc.y);
+        for (int j = 0; j < 32; ++j) er[j] = __uint_as_float(v[j]) * pscale<SP>(P.sc.y);
       }
       asm volatile("bar.sync 1, 128;\n" ::: "memory");
 #pragma unroll 1
@@ -1247,10 +1254,10 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
             const int x0 = 4 * (cq ^ (2 * ((al >> 1) & 1)));
             const int rl = al * nX - row0 + x0;
             float4 o;
-            o.x = x0 < nX ? eh[rl * 33 + zz] * scf<SP>(P.sc.yf) : 0.f;
-            o.y = x0 + 1 < nX ? eh[(rl + 1) * 33 + zz] * scf<SP>(P.sc.yf) : 0.f;
-            o.z = x0 + 2 < nX ? eh[(rl + 2) * 33 + zz] * scf<SP>(P.sc.yf) : 0.f;
-            o.w = x0 + 3 < nX ? eh[(rl + 3) * 33 + zz] * scf<SP>(P.sc.yf) : 0.f;
+            o.x = x0 < nX ? eh[rl * 33 + zz] * pscale<SP>(P.sc.yf) : 0.f;
+            o.y = x0 + 1 < nX ? eh[(rl + 1) * 33 + zz] * pscale<SP>(P.sc.yf) : 0.f;
+            o.z = x0 + 2 < nX ? eh[(rl + 2) * 33 + zz] * pscale<SP>(P.sc.yf) : 0.f;
+            o.w = x0 + 3 < nX ? eh[(rl + 3) * 33 + zz] * pscale<SP>(P.sc.yf) : 0.f;
             *reinterpret_cast<float4*>(Yf + ((long long)zz * mX + al) * 16 + 4 * cq) = o;
           }
         }
@@ -1312,7 +1319,7 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
             float* yr = Yf ? Yf + ((long long)zz * mX + al) * 16 : nullptr;
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp) Yo[pp * plane + o + (cm ? ((x >> 3) << 6) + (x & 7) : x)] = pc[pp];
-            if (yr) yr[(((x >> 2) ^ sw) << 2) + (x & 3)] = y * scf<SP>(P.sc.yf);
+            if (yr) yr[(((x >> 2) ^ sw) << 2) + (x & 3)] = y * pscale<SP>(P.sc.yf);
             if (x == nX - 1)
               for (int xp = nX; xp < 16; ++xp) {
 #pragma unroll

@@ -113,8 +113,8 @@ __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
           const int t = 4 * t4;
           const int g8 = t / (KP * 8), rem = t - g8 * KP * 8;
           const int al = g8 * 8 + ((rem >> 3) & 7), col = (rem >> 6) * 8 + (rem & 7);
-          const float x[4] = {val(al, col) * scf<SP>(P.sc.c), val(al, col + 1) * scf<SP>(P.sc.c), val(al, col + 2) * scf<SP>(P.sc.c),
-                              val(al, col + 3) * scf<SP>(P.sc.c)};
+          const float x[4] = {val(al, col) * pscale<SP>(P.sc.c), val(al, col + 1) * pscale<SP>(P.sc.c), val(al, col + 2) * pscale<SP>(P.sc.c),
+                              val(al, col + 3) * pscale<SP>(P.sc.c)};
           uint2 pc[NP];
           split4<SP>(x, pc);
 #pragma unroll
@@ -172,7 +172,7 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
         const int e = 4 * e4, al = e / MB, be = e - al * MB;
         float x[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] = be + j < mB ? vsm[al * mB + be + j] * scf<SP>(P.sc.v) : 0.f;
+        for (int j = 0; j < 4; ++j) x[j] = be + j < mB ? vsm[al * mB + be + j] * pscale<SP>(P.sc.v) : 0.f;
         uint2 pc[NP];
         split4<SP>(x, pc);
 #pragma unroll
@@ -198,7 +198,7 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
         const int al = ((t >> 9) << 3) + ((t >> 3) & 7), be = (((t >> 6) & 7) << 3) + (t & 7);
         float x[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] = (al < mA && be + j < mB) ? vsm[al * mB + be + j] * scf<SP>(P.sc.v) : 0.f;
+        for (int j = 0; j < 4; ++j) x[j] = (al < mA && be + j < mB) ? vsm[al * mB + be + j] * pscale<SP>(P.sc.v) : 0.f;
         uint2 pc[NP];
         split4<SP>(x, pc);
 #pragma unroll
@@ -897,7 +897,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                   uint2 pk[NP];
                   if (v0) {
-                    float uf4[4] = {u0[0].x * scf<SP>(P.sc.uf), u0[0].y * scf<SP>(P.sc.uf), u0[1].x * scf<SP>(P.sc.uf), u0[1].y * scf<SP>(P.sc.uf)};
+                    float uf4[4] = {u0[0].x * pscale<SP>(P.sc.uf), u0[0].y * pscale<SP>(P.sc.uf), u0[1].x * pscale<SP>(P.sc.uf), u0[1].y * pscale<SP>(P.sc.uf)};
                     split4<SP>(uf4, pk);
                     uint16_t* ur = Us + (be[0] >> 3) * KP * 8 + (be[0] & 7) * 8 + (qa & 1) * 4 +
                                    (2 * (fa + fr[0]) + (qa >> 1)) * 64;
@@ -905,7 +905,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(ur + (size_t)pp * 64 * KP) = pk[pp];
                   }
                   if (v1) {
-                    float ug4[4] = {u1[0].x * scf<SP>(P.sc.uf), u1[0].y * scf<SP>(P.sc.uf), u1[1].x * scf<SP>(P.sc.uf), u1[1].y * scf<SP>(P.sc.uf)};
+                    float ug4[4] = {u1[0].x * pscale<SP>(P.sc.uf), u1[0].y * pscale<SP>(P.sc.uf), u1[1].x * pscale<SP>(P.sc.uf), u1[1].y * pscale<SP>(P.sc.uf)};
                     split4<SP>(ug4, pk);
                     uint16_t* ur = Us + (be[1] >> 3) * KP * 8 + (be[1] & 7) * 8 + (qa & 1) * 4 +
                                    (2 * (fa + fr[1]) + (qa >> 1)) * 64;
@@ -1198,8 +1198,8 @@ __global__ void __launch_bounds__(kT2Threads, 1)
               float x0[4], x1[4];
 #pragma unroll
               for (int k = 0; k < 4; ++k) {
-                x0[k] = x[8 * hb + k] * scf<SP>(P.sc.z);
-                x1[k] = x[8 * hb + 4 + k] * scf<SP>(P.sc.z);
+                x0[k] = x[8 * hb + k] * pscale<SP>(P.sc.z);
+                x1[k] = x[8 * hb + 4 + k] * pscale<SP>(P.sc.z);
               }
               uint2 p0[NP], p1[NP];
               split4<SP>(x0, p0);

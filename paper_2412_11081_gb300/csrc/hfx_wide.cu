@@ -2,11 +2,11 @@
 // tiles: n_ao up to 32 per species (the perovskite Cs blocks, n_ao 18) and
 // n_abf up to 128.
 //
-// Same factorisation and the same bf16 piece products as hfx_mixed.cu (NP
-// pieces per operand, the products (i, j) with i + j < NP, FP32 accumulation
+// Same factorisation and the same piece products as hfx_mixed.cu (two 16-bit
+// pieces per operand, three products, FP32 accumulation
 // in warp-level MMAs, FP64 screening, gradients and reductions), organised
 // like the FP64 kernels of hfx_kernels.cu so that any n_ao and n_abf fit.
-// Operands are split into bf16 pieces once, into stores that the kernels copy
+// Operands are split into their pieces once, into stores that the kernels copy
 // from:
 //   D pieces   per D block, NP planes [rup16(n_ao(I))][rup16(n_ao(J))]   (plan)
 //   C pieces   per C pair, NP planes [alpha][rup8(n_ao(A) n_ao(F))]        (per call)
@@ -161,7 +161,7 @@ __global__ void k_dsplit_w(DevPlan P, uint16_t* Dw, const long long* dw_off) {
     uint16_t* out = Dw + dw_off[k];
     for (int e = threadIdx.x; e < pa * pb; e += blockDim.x) {
       const int a = e / pb, b = e - a * pb;
-      put_pieces<SP>(out, (long long)pa * pb, e, (a < na && b < nb) ? (float)src[a * nb + b] * scf<SP>(P.sc.d) : 0.f);
+      put_pieces<SP>(out, (long long)pa * pb, e, (a < na && b < nb) ? (float)src[a * nb + b] * pscale<SP>(P.sc.d) : 0.f);
     }
   }
 }
@@ -188,12 +188,12 @@ __global__ void k_cpieces_w(DevPlan P, uint16_t* Cw, const long long* cw_off, fl
     uint16_t* out = Cw + cw_off[q];
     for (int e = threadIdx.x; e < mA * CW; e += blockDim.x) {
       const int al = e / CW, c = e - al * CW;
-      put_pieces<SP>(out, (long long)mA * CW, e, c < naf ? (float)src[(long long)al * naf + c] * scf<SP>(P.sc.c) : 0.f);
+      put_pieces<SP>(out, (long long)mA * CW, e, c < naf ? (float)src[(long long)al * naf + c] * pscale<SP>(P.sc.c) : 0.f);
     }
     uint16_t* cy = out + (long long)NP * mA * CW;
     for (int e = threadIdx.x; e < mA * nA * KW; e += blockDim.x) {
       const int r = e / KW, c = e - r * KW;
-      put_pieces<SP>(cy, (long long)mA * nA * KW, e, c < nF ? (float)src[(long long)r * nF + c] * scf<SP>(P.sc.c) : 0.f);
+      put_pieces<SP>(cy, (long long)mA * nA * KW, e, c < nF ? (float)src[(long long)r * nF + c] * pscale<SP>(P.sc.c) : 0.f);
     }
     const double* dsrc = P.dCst + 3 * P.c_off[q];
     float* dst = dCf + 3 * P.c_off[q];
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kWThreads) k_ybuild_w(DevPlan P, uint16_t* __r
         if (row < rows && z < nZ) {
           const int al = row / nX, x = row - al * nX;
           const long long o = ((long long)al * nZ + z) * KX;
-          put_pieces<SP>(Y, plane, (int)(o + x), acc[ii][nt][c] * scf<SP>(P.sc.y));
+          put_pieces<SP>(Y, plane, (int)(o + x), acc[ii][nt][c] * pscale<SP>(P.sc.y));
           if (x == nX - 1)
             for (int xp = nX; xp < KX; ++xp)
 #pragma unroll
@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
     }
     for (int e = threadIdx.x; e < MA * SV; e += blockDim.x) {
       const int al = e / SV, be = e - al * SV;
-      put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * scf<SP>(P.sc.v) : 0.f);
+      put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * pscale<SP>(P.sc.v) : 0.f);
     }
     for (int e = threadIdx.x; e < 48 * SD; e += blockDim.x) {
       const int a = e / SD, bb = e - a * SD;
@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
                   const int r = nt * 8 + 2 * tig + c;
                   if (r < rowsU) {
                     const int be = r / nF, ff = r - be * nF;
-                    put_pieces<SP>(Us, pU, be * SK + gid * nF + ff, acc[c] * scf<SP>(P.sc.u));
+                    put_pieces<SP>(Us, pU, be * SK + gid * nF + ff, acc[c] * pscale<SP>(P.sc.u));
                   }
                 }
               }
@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
     }
     for (int e = threadIdx.x; e < MA * SV; e += blockDim.x) {
       const int al = e / SV, be = e - al * SV;
-      put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * scf<SP>(P.sc.v) : 0.f);
+      put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * pscale<SP>(P.sc.v) : 0.f);
     }
     // Y^{BA} rows beyond n_abf(B) stay zero (K of Z)
     for (int e = threadIdx.x; e < (MB - mB) * SK; e += blockDim.x)
@@ -779,7 +779,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
               const int n = (nt0 + h) * 8 + 2 * tig + (c & 1);
               if (al < mA && n < dcols && nt0 + h < NTZ) {
                 const int bb = n / dA, a = n - bb * dA;
-                put_pieces<SP>(Z, S.zplane, (int)(((long long)al * nA + a0 + a) * S.KZ + bb), acc[h][c] * scf<SP>(P.sc.z));
+                put_pieces<SP>(Z, S.zplane, (int)(((long long)al * nA + a0 + a) * S.KZ + bb), acc[h][c] * pscale<SP>(P.sc.z));
               }
             }
         }
