@@ -226,16 +226,15 @@ struct hfx_plan {
   size_t smem_m1 = 0, smem_m2 = 0;
   // tcgen05 first product (n_abf <= 64, n_ao <= 16): operand stores and shape
   bool t1u = false;
-  int t1u_KP = 0, t1u_NS = 0, t1u_FS = 1, t1u_seg = 32;
-  size_t t1u_limit = 0;        // dynamic shared memory the Y ring may fill up to
+  int t1u_KP = 0, t1u_G = 0, t1u_UB = 2, t1u_NS = 0, t1u_seg = 32;
   size_t smem_t1u = 0;
   uint16_t* Cu = nullptr;
   long long Cucap = 0;
   uint16_t* Vu = nullptr;
   long long Vucap = 0;
-  float* Yf = nullptr;
-  long long Yfcap = 0;
-  float* Df = nullptr;
+  uint16_t* Yh = nullptr;      // fp16 Y and D pieces, where Ysp and Dsp hold another form
+  long long Yhcap = 0;
+  uint16_t* Dh = nullptr;
   int* d_work = nullptr;       // item counter of the tcgen05 first-product kernel
   // tcgen05 R2 / Z of the second product (same shapes): core-matrix Y stores, V store per pair slot
   bool t2u = false;
@@ -587,7 +586,7 @@ DevPlan make_devplan(hfx_plan* P, const double* lattice) {
 // they are.
 void set_scale(hfx_plan* P) {
   P->scale = hfx::SplitScale{};
-  if (P->sp != hfx::kSplitHalf) return;
+  if (!P->sp) return;
   int nao = 1;
   for (int n : P->n_ao) nao = std::max(nao, n);
   auto ex = [](double bound) {   // bound * 2^ex in (2^14, 2^15]
@@ -597,16 +596,21 @@ void set_scale(hfx_plan* P) {
     return std::max(-100, std::min(100, 15 - k));
   };
   const int eC = ex(*std::max_element(P->cmax.begin(), P->cmax.end())), eD = ex(P->dmax), eV = ex(P->vmax);
-  const int eY = ex(P->ymax), eU = ex(nao * P->dmax * P->ymax), eZ = ex(P->vrow * P->ymax);
+  // (U with a bit to spare: rows past n_abf(B) hold other blocks' Y, bounded by 2^15 as stored)
+  const int eY = ex(P->ymax), eU = ex(2 * nao * P->dmax * P->ymax), eZ = ex(P->vrow * P->ymax);
   auto f = [](int e) { return std::ldexp(1.f, std::max(-126, std::min(127, e))); };
   hfx::SplitScale& s = P->scale;
+  s.dh = f(eD);
+  if (P->sp != hfx::kSplitHalf) {   // bf16 pieces hold the values as they are
+    s.yh = f(eY);
+    s.u1 = f(-eD - eY);
+    return;
+  }
   s.c = f(eC);
   s.v = f(eV);
   s.d = f(eD);
   s.y = f(eY - eC - eD);
-  s.yf = f(-eY);
-  s.u = f(eU - eD - eY);
-  s.uf = f(eU);
+  s.u = s.u1 = f(eU - eD - eY);
   s.z = f(eZ - eV - eY);
   s.r1 = std::ldexp(1.0, -eC - eU);
   s.q1 = std::ldexp(1.0, -eV - eU);
@@ -824,9 +828,9 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
     v_size[p] = 4ll * P->n_abf[P->species[v_home[p]]] * P->n_abf[P->species[v_j[p]]];
   for (int y = 0; y < nY; ++y) {
     const int sX = P->species[y_home[y]], sz = P->species[y_j[y]];
-    if (P->t2u)  // bf16 pieces of 64 rows alpha x (z, x) columns in core-matrix order
-      y_size[y] = (long long)P->np * 64 * 16 * P->n_ao[sz];
-    else if (P->np)  // bf16 pieces of [alpha][z][rup16(n_ao(X))]
+    if (P->t2u)  // pieces of rup8(n_abf(X)) rows alpha x (z, x) columns in core-matrix order
+      y_size[y] = (long long)P->np * ((P->n_abf[sX] + 7) / 8 * 8) * 16 * P->n_ao[sz];
+    else if (P->np)  // pieces of [alpha][z][rup16(n_ao(X))]
       y_size[y] = (long long)P->np * P->n_abf[sX] * P->n_ao[sz] * ((P->n_ao[sX] + 15) / 16 * 16);
     else
       y_size[y] = (long long)P->n_abf[sX] * P->n_ao[sX] * P->n_ao[sz];
@@ -987,12 +991,6 @@ double list_drift(const hfx_plan* P, const double* L, const double* pos) {
   return 2.0 * disp + P->list_Rabs * dl;
 }
 
-// Y slots of fs rows that fit next to the first product's fixed shared memory.
-long long t1u_slots(const hfx_plan* P, int fs) {
-  const size_t base = hfx::t1u_smem(P->np, P->t1u_KP, 0, 1);
-  return base < P->t1u_limit ? (long long)((P->t1u_limit - base) / ((size_t)fs * 4096)) : 0LL;
-}
-
 void setup_shapes(hfx_plan* P) {
   int dev_smem = 0;
   ck(cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, P->dev), "attr");
@@ -1059,22 +1057,20 @@ void setup_shapes(hfx_plan* P) {
     P->t1u = false;
     if (want_umma && maxABF <= 64 && maxAO <= 16) {
       P->t1u_KP = 16 * maxAO;
-      // Y ring: slots of FS rows f.  Half a U chunk per slot (one wait and one
-      // release per run of rows) when three such slots fit, else runs of two
-      // rows (measured best for BF16X6 on si64), else single rows
-      // (HFX_T1_FS overrides the run length).
-      P->t1u_limit = limit;
-      const int fh = (P->t1u_KP / 16 + 1) / 2;
-      auto slots = [&](int fs) { return t1u_slots(P, fs); };
-      const char* fse = std::getenv("HFX_T1_FS");
-      int fs = fse ? std::max(1, std::min(fh, std::atoi(fse))) : (slots(fh) >= 3 ? fh : (slots(2) >= 3 ? 2 : 1));
-      while (fs > 1 && slots(fs) < 2) --fs;
-      P->t1u_FS = fs;
-      P->t1u_NS = (int)std::min<long long>(slots(fs), hfx::t1u_max_slots());
-      const size_t base = hfx::t1u_smem(P->sp == hfx::kSplitHalf ? 3 : 2, P->t1u_KP, 2, 1);
-      if (base <= limit && P->t1u_NS >= 2) {
+      P->t1u_G = (maxABF + 7) / 8;
+      // two buffers of U where three slots of the Y ring still fit beside them
+      // (n_ao 13: n_abf up to 56), else one
+      auto slots = [&](int ub) {
+        const size_t base = hfx::t1u_smem(P->t1u_KP, P->t1u_G, ub, 0);
+        return base < limit ? (int)std::min<size_t>((limit - base) / 16384, hfx::t1u_max_slots()) : 0;
+      };
+      P->t1u_UB = slots(2) >= 3 ? 2 : 1;
+      P->t1u_NS = slots(P->t1u_UB);
+      // HFX_BF16X6 takes the shapes whose operands would fit in three pieces each
+      const size_t np = P->sp == hfx::kSplitHalf ? 3 : 2;
+      if (np * (64 * P->t1u_KP * 4 + 8192) + 2048 + 8192 <= limit && P->t1u_NS >= 3) {
         P->t1u = true;
-        P->smem_t1u = hfx::t1u_smem(P->np, P->t1u_KP, P->t1u_NS, P->t1u_FS);
+        P->smem_t1u = hfx::t1u_smem(P->t1u_KP, P->t1u_G, P->t1u_UB, P->t1u_NS);
         // kept B per FP32 run of the Q accumulator: 32 for BF16X3, whose
         // stress error is closest to the 1e-5 bound; 128 for BF16X6 (6.5e-6
         // at most on the jittered si64 geometries against 5.4e-6 with 32,
@@ -1160,13 +1156,13 @@ void split_density(hfx_plan* P) {
   }
   DevPlan D = make_devplan(P, P->lat_ref.data());
   hfx::MixPlan X{P->Dsp, P->dsp_off, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  ck(hfx::launch_dsplit(D, X, P->sp, P->stream), "dsplit");
+  ck(hfx::launch_dsplit(D, X, P->Dsp, P->scale.d, P->sp, P->stream), "dsplit");
   if (P->t1u) {
     P->d_work = P->mem.alloc<int>(1);
-    P->Df = P->mem.alloc<float>((size_t)P->n_d * 256);
-    hfx::T1UPlan U{};
-    U.Df = P->Df;
-    ck(hfx::launch_t1u_stores(D, U, P->sp, nullptr, 0, true, P->stream), "D FP32 store");
+    if (P->sp != hfx::kSplitHalf) {
+      P->Dh = P->mem.alloc<uint16_t>((size_t)P->n_d * 512);
+      ck(hfx::launch_dsplit(D, X, P->Dh, P->scale.dh, hfx::kSplitHalf, P->stream), "dsplit");
+    }
   }
   ck(cudaStreamSynchronize(P->stream), "dsplit");
 }
@@ -1409,18 +1405,31 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     ck(hfx::launch_cpieces(D, X, P->sp, s), "cpieces");
     if (P->t1u) {
       U.KP = P->t1u_KP;
+      U.G = P->t1u_G;
+      U.UB = P->t1u_UB;
       U.NS = P->t1u_NS;
-      U.FS = P->t1u_FS;
       U.seg = P->t1u_seg;
-      U.cu_blk = (long long)P->np * 64 * U.KP + 2LL * 4 * 64 * hfx::t1u_kp32(U.KP);
-      U.vu_blk = (long long)P->np * 4096 + 2LL * 3 * 4096;
-      ensure_buf(P, P->Yf, P->Yfcap, std::max(1LL, P->tot[0] / P->np));
-      U.Yf = P->Yf;
-      U.Df = P->Df;
+      // items divided where there are too few to balance the SMs (eight per SM);
+      // by the C pairs of the whole structure, so that neither the passes nor
+      // the plan's home atoms move the FP32 runs' ends
+      U.nsplit = std::max(1, std::min(8, (8 * hfx::sm_count() + P->nC - 1) / std::max(1, P->nC)));
+      U.cu_blk = (long long)P->np * 8 * U.G * U.KP + 2LL * 4 * 64 * hfx::t1u_kp32(U.KP);
+      U.vu_blk = (long long)P->np * 512 * U.G + 2LL * 3 * 4096;
       U.t1_idx = P->t1_idx;
-      X.Yf = P->Yf;
+      U.Dh = P->sp == hfx::kSplitHalf ? P->Dsp : P->Dh;
+      if (P->sp == hfx::kSplitHalf && P->t2u) {   // Ysp is the first product's store too
+        U.Yh = P->Ysp;
+      } else {
+        X.yh_blk = (long long)P->np * 8 * U.G * U.KP;
+        const long long hcap0 = P->Yhcap;
+        ensure_buf(P, P->Yh, P->Yhcap, std::max(1LL, P->tot[1]) * X.yh_blk);
+        if (P->Yhcap != hcap0) ck(cudaMemsetAsync(P->Yh, 0, P->Yhcap * sizeof(uint16_t), s), "memset");
+        X.Yh = P->Yh;
+        U.Yh = P->Yh;
+        U.yh_blk = X.yh_blk;
+      }
     }
-    X.yT_blk = P->t2u ? (long long)P->np * 64 * P->t1u_KP : (long long)P->np * P->MC * 128 * 16;
+    X.yT_blk = P->t2u ? (long long)P->np * 8 * P->t1u_G * P->t1u_KP : (long long)P->np * P->MC * 128 * 16;
     const long long tcap0 = P->YspTcap;
     ensure_buf(P, P->YspT, P->YspTcap, std::max(1LL, P->tot[1]) * X.yT_blk);
     if (P->t2u && P->YspTcap != tcap0) ck(cudaMemsetAsync(P->YspT, 0, P->YspTcap * sizeof(uint16_t), s), "memset");
@@ -1483,7 +1492,7 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
         ensure_buf(P, P->Vu, P->Vucap, std::max(1LL, ct[CT_T1]) * U.vu_blk);
         U.Cu = P->Cu;
         U.Vu = P->Vu;
-        ck(hfx::launch_t1u_stores(D, U, P->sp, t1items + c0, (int)ct[CT_Q], false, s), "term-1 C store");
+        ck(hfx::launch_t1u_cstore(D, U, P->sp, t1items + c0, (int)ct[CT_Q], s), "term-1 C store");
         ck(hfx::launch_vstores(D, X, U, P->sp, P->v_list + v0, (int)ct[CT_VN], s), "V stores");
         k1a.push_back(tm.mark());
         ck(hfx::launch_t1_umma(D, X, U, P->sp, t1items + c0, (int)ct[CT_Q], P->smem_t1u, P->d_work, P->d_err, s),
@@ -1804,7 +1813,7 @@ hfx_status hfx_plan_autotune(hfx_plan* P, const double* lattice, const double* p
                              hfx_tune_report* report) {
   if (!P || !lattice || !positions || reps < 1) return HFX_ERR_INVALID;
   hfx_tune_report R{};
-  R.t1_rows_per_slot = P->t1u_FS;
+  R.t1_rows_per_slot = 1;
   R.t1_slots = P->t1u_NS;
   R.t1_home_order = P->t1_order;
   R.y_tiles_per_cta = P->ybtpc;
@@ -1813,13 +1822,8 @@ hfx_status hfx_plan_autotune(hfx_plan* P, const double* lattice, const double* p
     if (report) *report = R;
     return HFX_OK;
   }
-  const int fs0 = P->t1u_FS, ns0 = P->t1u_NS;
-  const size_t smem0 = P->smem_t1u;
   const bool timing0 = P->timing;
-  auto use = [&](int fs, int ns) {
-    P->t1u_FS = fs;
-    P->t1u_NS = ns;
-    P->smem_t1u = hfx::t1u_smem(P->np, P->t1u_KP, ns, fs);
+  auto drop_graph = [&]() {
     if (P->gexec) {   // a recorded evaluation has the old launch shape
       cudaGraphExecDestroy(P->gexec);
       P->gexec = nullptr;
@@ -1842,32 +1846,16 @@ hfx_status hfx_plan_autotune(hfx_plan* P, const double* lattice, const double* p
   };
   P->timing = true;
   bool ok = time_it(R.default_ms);
-  int best_fs = fs0, best_ns = ns0;
   R.best_ms = R.default_ms;
   R.candidates = ok ? 1 : 0;
-  const int fh = (P->t1u_KP / 16 + 1) / 2;   // a run never crosses a U column chunk
-  for (int fs = 1; ok && fs <= fh; ++fs) {
-    const int ns = (int)std::min<long long>(t1u_slots(P, fs), hfx::t1u_max_slots());
-    if (ns < 2 || (fs == fs0 && ns == ns0)) continue;
-    use(fs, ns);
-    double ms = 0.0;
-    ok = time_it(ms);
-    if (!ok) break;
-    ++R.candidates;
-    if (ms < R.best_ms) {
-      R.best_ms = ms;
-      best_fs = fs;
-      best_ns = ns;
-    }
-  }
-  // the order of the items, with the best ring shape
+  // the order of the items
   const int order0 = P->t1_order;
   int best_order = order0;
   if (ok) {
-    use(best_fs, best_ns);
     for (int o = 0; o < 3 && ok; ++o) {
       if (o == order0) continue;
       P->t1_order = o;
+      drop_graph();
       double ms = 0.0;
       ok = time_it(ms);
       if (!ok) break;
@@ -1895,10 +1883,7 @@ hfx_status hfx_plan_autotune(hfx_plan* P, const double* lattice, const double* p
     for (int ai = 0; ai < 2 && ok; ++ai) {
       if (alts[ai] == 0) continue;
       knob = alts[ai];
-      if (P->gexec) {
-        cudaGraphExecDestroy(P->gexec);
-        P->gexec = nullptr;
-      }
+      drop_graph();
       double ms = 0.0;
       ok = time_it(ms);
       if (!ok) break;
@@ -1911,17 +1896,13 @@ hfx_status hfx_plan_autotune(hfx_plan* P, const double* lattice, const double* p
     knob = best;
   }
   P->timing = timing0;
+  drop_graph();
   if (!ok) {   // keep the initial choice
-    use(fs0, ns0);
-    P->smem_t1u = smem0;
     P->t1_order = order0;
     P->ybtpc = yb0;
     P->q2tpc = q20;
     return status;
   }
-  use(best_fs, best_ns);
-  R.t1_rows_per_slot = best_fs;
-  R.t1_slots = best_ns;
   R.t1_home_order = best_order;
   R.y_tiles_per_cta = P->ybtpc;
   R.q2_tiles_per_cta = P->q2tpc;

@@ -26,8 +26,10 @@ constexpr int kPieces = 2;            // pieces per operand
 // the lists cover, so that no stored element exceeds 2^15.
 struct SplitScale {
   float c = 1.f, v = 1.f, d = 1.f;   // stored piece = c * C, v * V, d * D
-  float y = 1.f, yf = 1.f;           // C.D accumulator -> stored Y; stored Y -> FP32 Y
-  float u = 1.f, uf = 1.f;           // D.Y accumulator -> stored U; FP32 U -> stored U
+  float y = 1.f, u = 1.f;            // C.D accumulator -> stored Y, D.Y accumulator -> stored U
+  // tcgen05 first product, whose Y and D operands are fp16 pieces for either
+  // piece type: stored Y -> its fp16 Y, D -> its fp16 D, their product -> stored U
+  float yh = 1.f, dh = 1.f, u1 = 1.f;
   float z = 1.f;                     // V.Y accumulator -> stored Z
   double r1 = 1.0, q1 = 1.0;         // C.U and V.U accumulators -> R, Q
   double r2 = 1.0, q2 = 1.0;         // Y.Y and Z.D accumulators -> R2, Q2
@@ -143,7 +145,10 @@ struct MixPlan {
   int* qcnt;                   // [nC] kept B per (A,F)
   long long* qoff;             // [nC] offsets into blist
   int* blist;                  // V pairs (A,B) per (A,F), in V-pair order
-  float* Yf = nullptr;         // Y^{XZ} in FP32 as [z][alpha][16], offsets y_off / 2 (tcgen05 term 1 only)
+  // tcgen05 first product: Y^{XZ} as fp16 pieces in the core-matrix layout of
+  // ycm, yh_blk per key (by y_idx); nullptr where Ysp is that store
+  uint16_t* Yh = nullptr;
+  long long yh_blk = 0;
   uint16_t* YspT = nullptr;    // Y^{XZ} transposed, bf16 pieces [piece][(alpha,x)][16 z] (z padded), yT_blk per key
   long long yT_blk = 0;        // uint16 units per key of YspT (2 pieces x 128-row tiles x 16)
   const long long* y_idx = nullptr;   // key -> its position in the needed-key list (YspT block)
@@ -154,10 +159,10 @@ struct MixPlan {
   // issues no copies, so its pipeline waits run out (HFX_ERR_TIMEOUT).
   int stall_q2 = 0;
   // tcgen05 R2 / Z kernel (k_t2_umma): with ycm the Y build writes Ysp and
-  // YspT per key as NP planes of 64 rows alpha x K columns in the tensor
-  // cores' core-matrix order (Ysp: K = (z, x), 16 n_ao(Z) columns; YspT:
-  // K = (x, z), 16 n_ao(X) columns; rows past n_abf(X) are left as they are:
-  // finite, never read into a kept result); Vz holds per second-product pair
+  // YspT per key as NP planes of rup8(n_abf(X)) rows alpha x K columns in the
+  // tensor cores' core-matrix order (Ysp: K = (z, x), 16 n_ao(Z) columns;
+  // YspT: K = (x, z), 16 n_ao(X) columns; rows past n_abf(X) are left as they
+  // are: finite, never read into a kept result); Vz holds per second-product pair
   // slot NP pieces of V [alpha 64][beta 64] in core-matrix order, then V and
   // grad V as four FP32 planes of 64 x 64 in epilogue load order.
   int ycm = 0;
@@ -182,17 +187,20 @@ __host__ __device__ inline int gc_off(int row, int f) {
 
 // Operand stores of the tcgen05 first-product kernel (hfx_t1umma.cu).
 struct T1UPlan {
-  uint16_t* Cu;                // per item (A,F): pieces of C as [alpha 64][(f,a) KP], then C, grad C FP32 [4][64][KP]
+  uint16_t* Cu;                // per item (A,F): C pieces [8-row group][piece] x (f,a) KP in core-matrix order, then C, grad C FP32 [4][64][KP32]
   long long cu_blk;            // uint16 units per item
-  uint16_t* Vu;                // per term-1 V pair: pieces of V [alpha 64][beta 64], then grad V FP32 [3][64][64]
+  uint16_t* Vu;                // per term-1 V pair: V pieces [8-row group][piece] x beta 64, then grad V FP32 [3][64][64]
   long long vu_blk;            // uint16 units per V pair
   const long long* t1_idx;     // V pair -> its position in the term-1 V list
-  float* Yf;                   // see MixPlan::Yf
-  float* Df;                   // D blocks in FP32, [16][16] each
+  const uint16_t* Yh;          // fp16 Y pieces (MixPlan::Yh or Ysp)
+  long long yh_blk;            // its block per needed key, 0: offsets y_off (Ysp)
+  const uint16_t* Dh;          // fp16 D pieces, 512 elements per block
   int KP;                      // columns (f,a) = 16 f + a: 16 * max n_ao
-  int NS;                      // Y ring slots
-  int FS;                      // rows f per Y slot (a run never crosses a U chunk)
+  int G;                       // 8-row groups of the largest n_abf
+  int UB;                      // buffers of U (1 or 2)
+  int NS;                      // Y ring slots (128-row tiles)
   int seg;                     // B per FP32 run of the Q accumulator
+  int nsplit;                  // parts an item's B are divided into
 };
 
 enum AccSlot { ACC_E = 0, ACC_W = 1, ACC_FY = 10, ACC_F1 = 11, ACC_F2 = 12, ACC_N = 16 };
@@ -234,7 +242,8 @@ cudaError_t launch_lri_fit(int batch, int n, int w, const double* A, const doubl
 
 // Split-precision kernels (hfx_mixed.cu); sp = kSplitBf16 or kSplitHalf.
 long long mixed_launch_count();
-cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, int sp, cudaStream_t s);
+// pieces of every D block, times scale, at dst + X.dsp_off
+cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, uint16_t* dst, float scale, int sp, cudaStream_t s);
 cudaError_t launch_cpieces(const DevPlan& P, const MixPlan& X, int sp, cudaStream_t s);
 cudaError_t launch_vpieces(const DevPlan& P, const MixPlan& X, int sp, const int* list, int n, cudaStream_t s);
 cudaError_t launch_ygroups(const DevPlan& P, const long long* y_idx, const long long* y_total, int* gcnt,
@@ -276,7 +285,7 @@ cudaError_t launch_t2_umma(const DevPlan& P, const MixPlan& X, int sp, const int
 
 // tcgen05 first exchange product (hfx_t1umma.cu): shapes n_abf <= 64, n_ao <= 16.
 long long t1u_launch_count();
-size_t t1u_smem(int pieces, int KP, int NS, int FS);
+size_t t1u_smem(int KP, int G, int UB, int NS);
 // Columns of one FP32 plane of C / grad C in the operand store (KP rounded up to 32).
 __host__ __device__ inline int t1u_kp32(int KP) { return (KP + 31) & ~31; }
 // Items of the first product in a chosen order: list[0..*n) (n read on the
@@ -293,8 +302,8 @@ cudaError_t t1u_set_smem(int sp);
 // set, the tcgen05 first product's V store, in one pass per pair.
 cudaError_t launch_vstores(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int sp, const int* list, int n,
                            cudaStream_t s);
-cudaError_t launch_t1u_stores(const DevPlan& P, const T1UPlan& U, int sp, const int* qlist, int nq, bool dstore,
-                              cudaStream_t s);
+cudaError_t launch_t1u_cstore(const DevPlan& P, const T1UPlan& U, int sp, const int* qlist, int nq, cudaStream_t s);
+int sm_count();
 cudaError_t launch_t1_umma(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int sp, const int* qlist, int n,
                            size_t smem, int* work, int* err, cudaStream_t s);
 

@@ -88,17 +88,17 @@ __device__ void block_sum_n(double (&v)[NV], double* red) {
 // ------------------------------------------------------------------ D split
 // D block k (n_ao(I) x n_ao(J)) -> NP planes of rup16(n_ao(I)) x rup16(n_ao(J)), zero padded.
 template <int SP>
-__global__ void k_dsplit(DevPlan P, MixPlan X) {
+__global__ void k_dsplit(DevPlan P, MixPlan X, uint16_t* dst, float scale) {
   for (long long k = blockIdx.x; k < P.n_d; k += gridDim.x) {
     const int I = P.Didx[5 * k], J = P.Didx[5 * k + 1];
     const int na = P.n_ao[P.species[I]], nb = P.n_ao[P.species[J]];
     const int pa = rup16(na), pb = rup16(nb);
-    uint16_t* out = X.Dsp + X.dsp_off[k];
+    uint16_t* out = dst + X.dsp_off[k];
     const double* src = P.Dval + P.Doff[k];
     for (int e = threadIdx.x; e < pa * pb; e += blockDim.x) {
       const int a = e / pb, b = e - a * pb;
       uint16_t pc[NP];
-      split_f<SP>((a < na && b < nb) ? (float)src[a * nb + b] * pscale<SP>(P.sc.d) : 0.f, pc);
+      split_f<SP>((a < na && b < nb) ? (float)src[a * nb + b] * pscale<SP>(scale) : 0.f, pc);
 #pragma unroll
       for (int p = 0; p < NP; ++p) out[p * pa * pb + tix(a, b)] = pc[p];
     }
@@ -1208,10 +1208,10 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
         if (ykey[i] < 0) continue;
         const int nZ = P.n_ao[P.species[zat[i]]];
         uint16_t* Yo = X.Ysp + P.y_off[ykey[i]];
-        float* Yf = X.Yf ? X.Yf + P.y_off[ykey[i]] / NP : nullptr;
-        const bool cm = X.ycm != 0;   // Ysp rows alpha (64), K = (z, x) in core-matrix order
-        const int KZc = 16 * nZ;
-        const long long plane = cm ? 64LL * KZc : (long long)mX * nZ * 16;
+        uint16_t* Yh = X.Yh ? X.Yh + X.y_idx[ykey[i]] * X.yh_blk : nullptr;
+        const bool cm = X.ycm != 0;   // Ysp rows alpha, K = (z, x) in core-matrix order
+        const int KZc = 16 * nZ, m8 = (mX + 7) & ~7;
+        const long long hplane = (long long)m8 * KZc, plane = cm ? hplane : (long long)mX * nZ * 16;
         const float* eh = ep + h * 16;
         // bf16 pieces: chunk (alpha, z, half) holds x = 8 half .. 8 half + 7
         // (core-matrix order: consecutive threads take consecutive alpha, whose
@@ -1244,31 +1244,34 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
           for (int pp = 0; pp < NP; ++pp)
             *reinterpret_cast<uint4*>(yo + pp * plane) = make_uint4(p0[pp].x, p0[pp].y, p1[pp].x, p1[pp].y);
         }
-        // FP32 copy as [z][alpha][16]; chunk c (16 bytes) of row alpha holds
-        // x = 4 (c ^ sw) .. + 3 with sw = 2 ((alpha >> 1) & 1), so that four
-        // consecutive rows read two adjacent chunks each from distinct
-        // shared-memory banks
-        if (Yf) {
-          for (int c = et; c < nal * nZ * 4; c += 128) {
-            const int cq = c & 3, za = c >> 2, zz = za / nal, al = alF + (za - zz * nal);
-            const int x0 = 4 * (cq ^ (2 * ((al >> 1) & 1)));
-            const int rl = al * nX - row0 + x0;
-            float4 o;
-            o.x = x0 < nX ? eh[rl * 33 + zz] * pscale<SP>(P.sc.yf) : 0.f;
-            o.y = x0 + 1 < nX ? eh[(rl + 1) * 33 + zz] * pscale<SP>(P.sc.yf) : 0.f;
-            o.z = x0 + 2 < nX ? eh[(rl + 2) * 33 + zz] * pscale<SP>(P.sc.yf) : 0.f;
-            o.w = x0 + 3 < nX ? eh[(rl + 3) * 33 + zz] * pscale<SP>(P.sc.yf) : 0.f;
-            *reinterpret_cast<float4*>(Yf + ((long long)zz * mX + al) * 16 + 4 * cq) = o;
+        // the first product's fp16 pieces, where Ysp is not that store
+        if (Yh) {
+          for (int c = et; c < nal * nZ * 2; c += 128) {
+            const int r2 = c / nal, al = alF + (c - r2 * nal), hf = r2 & 1, zz = r2 >> 1;
+            const int rl = al * nX - row0 + 8 * hf;
+            float f0[4], f1[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              f0[k] = 8 * hf + k < nX ? eh[(rl + k) * 33 + zz] * P.sc.yh : 0.f;
+              f1[k] = 8 * hf + 4 + k < nX ? eh[(rl + 4 + k) * 33 + zz] * P.sc.yh : 0.f;
+            }
+            uint2 p0[NP], p1[NP];
+            split4<kSplitHalf>(f0, p0);
+            split4<kSplitHalf>(f1, p1);
+            uint16_t* yo = Yh + cmx(al, zz * 16 + 8 * hf, KZc);
+#pragma unroll
+            for (int pp = 0; pp < NP; ++pp)
+              *reinterpret_cast<uint4*>(yo + pp * hplane) = make_uint4(p0[pp].x, p0[pp].y, p1[pp].x, p1[pp].y);
           }
         }
         // transposed pieces for the second product: accumulator row (alpha, x)
         // with the 16 z of key i (z >= n_ao(Z) zero); every row of the tile
         // is this CTA's own
         if (X.YspT) {
-          // row-major tiles [(alpha, x)][16 z], or (ycm) rows alpha (64), K = (x, z) in core-matrix order
+          // row-major tiles [(alpha, x)][16 z], or (ycm) rows alpha, K = (x, z) in core-matrix order
           uint16_t* ytb = X.YspT + X.y_idx[ykey[i]] * X.yT_blk;
           uint16_t* yt = ytb + (long long)row0 * 16;
-          const long long tplane = cm ? 64LL * 16 * nX : X.yT_blk / NP;
+          const long long tplane = cm ? (long long)m8 * 16 * nX : X.yT_blk / NP;
           // (core-matrix order: consecutive threads take consecutive alpha of one
           // (x, half), whose chunks are 16 bytes apart; rows outside the tile skipped)
           const int nala = alB - alA + 1;
@@ -1315,17 +1318,22 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
             uint16_t pc[NP];
             split_f<SP>(y, pc);
             const long long o = cm ? cmx(al, zz * 16, KZc) : ((long long)al * nZ + zz) * 16;   // + x (x < 16)
-            const int sw = 2 * ((al >> 1) & 1);
-            float* yr = Yf ? Yf + ((long long)zz * mX + al) * 16 : nullptr;
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp) Yo[pp * plane + o + (cm ? ((x >> 3) << 6) + (x & 7) : x)] = pc[pp];
-            if (yr) yr[(((x >> 2) ^ sw) << 2) + (x & 3)] = y * pscale<SP>(P.sc.yf);
             if (x == nX - 1)
-              for (int xp = nX; xp < 16; ++xp) {
+              for (int xp = nX; xp < 16; ++xp)
 #pragma unroll
                 for (int pp = 0; pp < NP; ++pp) Yo[pp * plane + o + (cm ? ((xp >> 3) << 6) + (xp & 7) : xp)] = 0;
-                if (yr) yr[(((xp >> 2) ^ sw) << 2) + (xp & 3)] = 0.f;
+            if (Yh) {
+              uint16_t* yo = Yh + cmx(al, zz * 16, KZc);
+              split_f<kSplitHalf>(y * P.sc.yh, pc);
+#pragma unroll
+              for (int pp = 0; pp < NP; ++pp) {
+                yo[pp * hplane + ((x >> 3) << 6) + (x & 7)] = pc[pp];
+                if (x == nX - 1)
+                  for (int xp = nX; xp < 16; ++xp) yo[pp * hplane + ((xp >> 3) << 6) + (xp & 7)] = 0;
               }
+            }
           }
         }
       }
@@ -1459,11 +1467,11 @@ int q2_umma_segments(int max_pairs_per_atom, int tpc) {
   return (max_pairs_per_atom + kmp - 1) / kmp;
 }
 
-cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, int sp, cudaStream_t s) {
+cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, uint16_t* dst, float scale, int sp, cudaStream_t s) {
   if (P.n_d == 0) return cudaSuccess;
   ++g_mix_launches;
-  if (sp == kSplitBf16) k_dsplit<kSplitBf16><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X);
-  else k_dsplit<kSplitHalf><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X);
+  if (sp == kSplitBf16) k_dsplit<kSplitBf16><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X, dst, scale);
+  else k_dsplit<kSplitHalf><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X, dst, scale);
   return cudaGetLastError();
 }
 

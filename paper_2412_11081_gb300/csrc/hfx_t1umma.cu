@@ -3,31 +3,43 @@
 //
 // For a kept C pair (A,F) (an "item") and its kept V pairs (A,B), the first
 // product of Eq. exx_expand, factorised through Y^{BF} = sum_W C_BW D_WF:
-//   U_B[beta][(f,a)] = sum_b Y^{BF}[f][beta][b] D_AB[a][b]   (CUDA cores, FP32)
+//   U_B[beta][(f,a)] = sum_b Y^{BF}[f][beta][b] D_AB[a][b]
 //   R_B = C_AF . U_B^T        (M = alpha, N = beta, K = (f,a))  -> g^V_AB = -<grad V_AB, R_B>
-//                             (two U pieces per instruction, N = 128: R is the sum of two 64-column blocks)
 //   Q  += V_AB . U_B          (M = alpha, N = (f,a), K = beta)  -> E = -<C_AF, Q>, g^C_AF = -2 <grad C_AF, Q>
 // (E through Q: <V_AB, C U^T> = <C, V_AB U>, so the per-B epilogue carries
 // only the three gradient planes of V.)
 //
-// Column order (f,a) = 16 f + a with a padded to 16: a U row of one f is two
-// whole core matrices, so the CUDA cores write U with 8-byte stores and no
-// bank conflicts.  All matrices sit in shared memory in the no-swizzle
-// core-matrix order (8 rows x 16 bytes); U serves R as a K-major B operand
-// and Q as an MN-major B operand without a second copy.
+// All three products run on the tensor cores.  U is made in tensor memory
+// from the fp16 pieces of Y (the Y build's own store, copied as it lies) and
+// D (three piece products, 22 bits), read back, split into two pieces and
+// stored to shared memory as the operand of R and Q.  Both pieces of C (and
+// of V) lie as alternating 8-row groups of one M = 128 operand and both
+// pieces of U side by side in N, so R takes one instruction per k step for
+// all four piece products and Q two; M = 64 instructions take as long as
+// M = 128 ones.
 //
-// Warp roles (16 warps, one CTA per SM, persistent over items):
-//   warp 0      Y producer: bulk copies of runs of up to FS rows Y^{BF}[f]
-//               (FP32, never crossing a U chunk) into a ring of NS slots
-//   warp 1      scheduler and producer: takes items from a global counter
-//               (dynamic load balance), hands them to the other roles through
-//               a ring two items ahead, and copies C (per item), D_AB (FP32)
-//               and V_AB pieces (per B)
-//   warp 2      tensor-memory owner; lane 0 issues the R products
-//   warp 3      lane 0 issues the Q products (a second issuing thread on
-//               another SMSP: one thread issues an MMA only every ~50 cycles)
-//   warps 4-7   epilogue: R -> g^V per B; Q -> E, g^C per run of B
-//   warps 8-15  U: one thread per (beta, 4 columns a) of each f
+// What bounds it: per kept triplet (n_ao 13, n_abf 50) about 2,500 cycles of
+// tensor-core work (18 U, 13 R, 8 Q instructions) and as much shared-memory
+// traffic, 105 KB of L2 reads.  The kernel before built U in FP32 on the CUDA
+// cores, two warps per scheduler with 64 registers of D each: 12,900 cycles
+// per triplet, most of them the latency of its shared-memory loads and FMA
+// chains.
+//
+// Column order (f,a) = 16 f + a with a padded to 16.  All matrices sit in
+// shared memory in the no-swizzle core-matrix order (8 rows x 16 bytes); U
+// serves R as a K-major B operand and Q as an MN-major one.
+//
+// Warp roles (16 warps of 128 registers, one CTA per SM, persistent over units; a unit is an
+// item or, on small cells, a part of its B):
+//   warp 0       Y producer: 128-row tiles of Y^{BF} into a ring of NS slots
+//   warp 1       scheduler and producer: takes units from a global counter
+//                (dynamic load balance), hands them to the other roles through
+//                a ring two units ahead, and copies C (per unit), D_AB and
+//                V_AB pieces (per B)
+//   warp 2       tensor-memory owner; lane 0 issues the U products
+//   warp 3       lane 0 issues the Q and R products
+//   warps 4-11   epilogue: R -> g^V per B; Q -> E, g^C per run of B
+//   warps 12-15  U tiles from tensor memory to the pieces in shared memory
 // All hand-offs are mbarriers (bounded waits; a timeout sets the error flag
 // and every role stops), no block barrier inside the pipeline.
 #include <algorithm>
@@ -45,20 +57,44 @@ using namespace dev;
 
 std::atomic<long long> g_t1u_launches{0};
 
-constexpr int kThreads = 512;
-constexpr int kWarpY = 0, kWarpV = 1, kWarpM = 2, kWarpQ = 3, kWarpE = 4, kWarpU = 8;
-constexpr int kNE = 4, kNU = 8;
+constexpr int kWarpY = 0, kWarpV = 1, kWarpU = 2, kWarpR = 3, kWarpE = 4, kNE = 8, kWarpS = 12, kNU = 4;
+constexpr int kThreads = 32 * (kWarpS + kNU);
 constexpr int kItemRing = 4;
-constexpr int kItemReaders = 3 + kNE + kNU;   // Y, R issuer, Q issuer, epilogue warps, U warps
-constexpr int kMaxNS = 16;
-constexpr int kRCol = 256;   // tensor-memory column of the first R accumulator (Q sits at column 0)
-constexpr int kRCols = 128;  // columns of one R accumulator: two 64-column blocks, R = block 0 + block 1
+constexpr int kItemReaders = 3 + kNE + kNU;   // Y, U and R / Q issuers, epilogue warps, U splitters
+constexpr int kMaxNS = 12;                    // Y ring slots
+constexpr int kYG = 32;                        // 8-row groups per Y slot: two 128-row tiles
+constexpr uint32_t kYPiece = kYG * 256;        // bytes of one piece of a slot
+constexpr uint32_t kYSlot = 2 * kYPiece;
+constexpr int kND = 4;                        // D ring slots
+constexpr int kMaxUT = 6;                     // pairs of U tiles in tensor memory
 
 __device__ __forceinline__ bool aborted(const volatile int* f) { return *f != 0; }
 
 // Every lane waits (bounded); the result is the same on all lanes.
 __device__ __forceinline__ bool wait_all(uint32_t mbar, uint32_t parity) {
   return __all_sync(0xffffffffu, mbar_wait(mbar, parity)) != 0;
+}
+
+// Position in a ring of barriers: slot and phase.  A filled slot is waited for
+// with parity ph, a free one with ph ^ 1 (true at once on the first round).
+// (Counters divided by the ring's run-time size cost the single issuing
+// threads more than the MMAs they issue.)
+struct Ring {
+  int s = 0;
+  uint32_t ph = 0, n = 0;   // n: slots passed in all
+  __device__ __forceinline__ void next(int size) {
+    ++n;
+    if (++s == size) {
+      s = 0;
+      ph ^= 1;
+    }
+  }
+};
+
+// Lets every copy issued into a ring (in order, `size` slots) land.
+__device__ __forceinline__ void drain(uint32_t full, Ring r, int size) {
+  for (uint32_t k = r.n < (uint32_t)size ? 0u : r.n - (uint32_t)size; k < r.n; ++k)
+    mbar_wait(full + 8 * (k % size), (k / size) & 1);
 }
 
 // ------------------------------------------------------------ operand stores
@@ -75,10 +111,19 @@ __device__ __forceinline__ void ep_at(int w, int& alpha, int& col) {
   col = 32 * j + 16 * (l >> 4) + 4 * t + k;
 }
 
-// Item kk (C pair q = list[kk]): NP pieces of C_AF as [alpha (64)][(f,a) (KP)]
-// in core-matrix order (8-row groups of KP/8 core matrices), then C and
-// grad C in FP32 as four planes of 64 x KP32 (KP rounded up to 32) in
-// epilogue load order (ep_at).  Zero padded.  Each plane of the C pair
+// The same for the first product, whose accumulators hold the two pieces of
+// row alpha in lanes l and l ^ 8 of quarter qd: lane l holds row
+// alpha = 16 qd + 8 (l >> 4) + (l & 7) and reads columns 32 j + 16 ((l >> 3) & 1) + 4 t .. + 3.
+__device__ __forceinline__ void ep_at1(int w, int& alpha, int& col) {
+  const int k = w & 3, l = (w >> 2) & 31, qd = (w >> 7) & 3, t = (w >> 9) & 3, j = w >> 11;
+  alpha = qd * 16 + 8 * (l >> 4) + (l & 7);
+  col = 32 * j + 16 * ((l >> 3) & 1) + 4 * t + k;
+}
+
+// Item kk (C pair q = list[kk]): the pieces of C_AF, per 8 rows alpha first
+// piece 0 and then piece 1, (f,a) (KP) columns in core-matrix order, then C
+// and grad C in FP32 as four planes of 64 x KP32 (KP rounded up to 32) in
+// epilogue load order (ep_at1).  Zero padded.  Each plane of the C pair
 // ([(alpha,a)][f]) is evaluated from the block model into shared memory as
 // FP32; the outputs are written in storage order, four elements per thread.
 constexpr int kCStoreSmem = 64 * 16 * 16 * 4;   // one plane of n_abf <= 64, n_ao <= 16
@@ -92,9 +137,9 @@ __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
     const int A = P.c_home[q], F = P.c_j[q];
     const int sA = P.species[A];
     const int nA = P.n_ao[sA], mA = P.n_abf[sA], nF = P.n_ao[P.species[F]];
-    const int ncq = mA * nA * nF;
+    const int ncq = mA * nA * nF, g8 = (mA + 7) >> 3;
     uint16_t* out = U.Cu + (long long)kk * U.cu_blk;
-    float* pl = reinterpret_cast<float*>(out + (long long)NP * 64 * KP);
+    float* pl = reinterpret_cast<float*>(out + (long long)NP * U.G * 8 * KP);
     float scf[8];   // C = G f + G' fa, grad C = G g + G' ga (block model, FP32 as k_cpieces)
 #pragma unroll
     for (int k = 0; k < 8; ++k) scf[k] = (float)P.c_sc[8 * (long long)q + k];
@@ -108,22 +153,21 @@ __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
         return (al < mA && col < KP && f < nF && a < nA) ? cs[(al * nA + a) * nF + f] : 0.f;
       };
       if (c == 0) {
-        // pieces: core-matrix element t -> (alpha, col), four consecutive columns per thread
-        for (int t4 = threadIdx.x; t4 < 16 * KP; t4 += blockDim.x) {
-          const int t = 4 * t4;
-          const int g8 = t / (KP * 8), rem = t - g8 * KP * 8;
-          const int al = g8 * 8 + ((rem >> 3) & 7), col = (rem >> 6) * 8 + (rem & 7);
-          const float x[4] = {val(al, col) * pscale<SP>(P.sc.c), val(al, col + 1) * pscale<SP>(P.sc.c), val(al, col + 2) * pscale<SP>(P.sc.c),
-                              val(al, col + 3) * pscale<SP>(P.sc.c)};
+        // pieces: element t of an 8-row group -> (alpha, col), four consecutive columns per thread
+        for (int t4 = threadIdx.x; t4 < g8 * 2 * KP; t4 += blockDim.x) {
+          const int g = t4 / (2 * KP), t = 4 * (t4 - g * 2 * KP);
+          const int al = g * 8 + ((t >> 3) & 7), col = (t >> 6) * 8 + (t & 7);
+          const float x[4] = {val(al, col) * pscale<SP>(P.sc.c), val(al, col + 1) * pscale<SP>(P.sc.c),
+                              val(al, col + 2) * pscale<SP>(P.sc.c), val(al, col + 3) * pscale<SP>(P.sc.c)};
           uint2 pc[NP];
           split4<SP>(x, pc);
 #pragma unroll
-          for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(out + (long long)pp * 64 * KP + t) = pc[pp];
+          for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(out + (long long)(g * NP + pp) * 8 * KP + t) = pc[pp];
         }
       }
       for (int w4 = threadIdx.x; w4 < PL / 4; w4 += blockDim.x) {   // FP32 plane c, storage order
         int al, col;
-        ep_at(4 * w4, al, col);
+        ep_at1(4 * w4, al, col);
         *reinterpret_cast<float4*>(pl + (long long)c * PL + 4 * w4) =
             make_float4(val(al, col), val(al, col + 1), val(al, col + 2), val(al, col + 3));
       }
@@ -137,10 +181,12 @@ __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
 //   set): NP planes [alpha][rup16(n_abf(B))] and V, grad V in FP32
 //   [4][n_abf(A) n_abf(B)];
 //   for the pairs of the first product (any bit of v_mask), the tcgen05
-//   store U.Vu at t1_idx[p]: NP pieces [alpha 64][beta 64] in core-matrix
-//   order and grad V in three planes in epilogue load order (ep_at);
+//   store U.Vu at t1_idx[p]: the pieces of V, per 8 rows alpha piece 0 then
+//   piece 1, beta 64 in core-matrix order, and grad V in three planes in
+//   epilogue load order (ep_at1);
 //   for the pairs of the second product (v_t2), with X.Vz set, the store of
-//   k_t2_umma at t2_slot[p]: the same pieces and V, grad V in four planes.
+//   k_t2_umma at t2_slot[p]: the pieces as [piece][alpha 64][beta 64] and V,
+//   grad V in four planes (ep_at).
 // Outputs are written in storage order, four elements per thread.
 constexpr int kVStoreSmem = 4 * 64 * 64 * 4;
 
@@ -202,14 +248,18 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
         uint2 pc[NP];
         split4<SP>(x, pc);
 #pragma unroll
-        for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(vu + pp * 4096 + t) = pc[pp];
+        for (int pp = 0; pp < NP; ++pp) {
+          const int o = st == 0 ? ((t >> 9) * NP + pp) * 512 + (t & 511) : pp * 4096 + t;
+          if (st == 1 || (t >> 9) < U.G) *reinterpret_cast<uint2*>(vu + o) = pc[pp];
+        }
       }
-      float* pl = reinterpret_cast<float*>(vu + NP * 4096);
+      float* pl = reinterpret_cast<float*>(vu + (st == 0 ? NP * 512 * U.G : NP * 4096));
       const int c0 = st == 0 ? 1 : 0;   // first plane: grad V (first product) or V (second)
       for (int w4 = threadIdx.x; w4 < (4 - c0) * 1024; w4 += blockDim.x) {   // epilogue load order
         const int c = c0 + (w4 >> 10);
         int al, be;
-        ep_at(4 * (w4 & 1023), al, be);
+        if (st == 0) ep_at1(4 * (w4 & 1023), al, be);
+        else ep_at(4 * (w4 & 1023), al, be);
         float4 o;
         o.x = (al < mA && be < mB) ? vsm[c * nv + al * mB + be] : 0.f;
         o.y = (al < mA && be + 1 < mB) ? vsm[c * nv + al * mB + be + 1] : 0.f;
@@ -217,21 +267,6 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
         o.w = (al < mA && be + 3 < mB) ? vsm[c * nv + al * mB + be + 3] : 0.f;
         *reinterpret_cast<float4*>(pl + 4 * w4) = o;
       }
-    }
-  }
-}
-
-// D block k as FP32 [16][16], zero padded; the four 16-byte chunks of row a
-// are permuted by (a >> 2) & 3, so that rows 4 apart read the same chunk from
-// different banks.
-__global__ void k_t1u_dstore(DevPlan P, float* Df) {
-  for (long long k = blockIdx.x; k < P.n_d; k += gridDim.x) {
-    const int na = P.n_ao[P.species[P.Didx[5 * k]]], nb = P.n_ao[P.species[P.Didx[5 * k + 1]]];
-    const double* src = P.Dval + P.Doff[k];
-    for (int e = threadIdx.x; e < 256; e += blockDim.x) {
-      const int a = e >> 4, b = e & 15;
-      Df[k * 256 + a * 16 + (((b >> 2) ^ ((a >> 2) & 3)) << 2) + (b & 3)] =
-          (a < na && b < nb) ? (float)src[a * nb + b] : 0.f;
     }
   }
 }
@@ -289,207 +324,244 @@ __global__ void k_lpt_scatter(const int* key, int asc, const int* list, const lo
 }
 
 // ------------------------------------------------------------------- kernel
+// Sizes of one launch, shared by the kernel and the host: KP columns
+// (f, a) = 16 f + a, G row groups of 8 alpha or beta (n_abf of the largest
+// species), UB buffers of U, NS slots of the Y ring.
+__host__ __device__ inline uint32_t t1_cbytes(int KP, int G) { return (uint32_t)G * 2u * 16u * KP; }   // C, or one buffer of U
+__host__ __device__ inline uint32_t t1_vbytes(int G) { return (uint32_t)G * 2048u; }
+__host__ __device__ inline uint32_t t1_base(int KP, int G, int UB) {
+  return t1_cbytes(KP, G) * (1 + UB) + 2 * t1_vbytes(G) + kND * 1024u;
+}
+// Tensor-memory columns: Q at 0, R from the next multiple of 32, then the U tiles in pairs of 32 columns.
+__host__ __device__ inline int t1_rcol(int KP) { return (KP + 31) & ~31; }
+__host__ __device__ inline int t1_utiles(int KP, int G) {
+  const int n = (512 - t1_rcol(KP) - 16 * G) / 32;
+  return n < kMaxUT ? n : kMaxUT;
+}
+
 template <int SP>
 __global__ void __launch_bounds__(kThreads, 1)
     k_t1_umma(DevPlan P, MixPlan X, T1UPlan U, const int* qlist, int n_list, int* work, int* err) {
-  const int KP = U.KP, KP32 = t1u_kp32(KP), NF = KP >> 4, FH = (NF + 1) >> 1, NS = U.NS, SEG = U.seg, FS = U.FS;
-  const int SLOT = FS * 64 * 16;                 // floats of one Y slot (FS rows f of up to 64 beta)
-  constexpr int NPROD = NP * (NP + 1) / 2;       // piece products (i, j) with i + j < NP
-  const uint32_t CPB = 64u * KP * 2u;            // bytes of one piece of C or U
+  const int KP = U.KP, KP32 = t1u_kp32(KP), G = U.G, NS = U.NS, UB = U.UB, SEG = U.seg, nsplit = U.nsplit;
+  const int NT = t1_utiles(KP, G), n_units = n_list * nsplit;
+  const uint32_t rowg = 16u * KP;                    // bytes of one 8-row group of a C or U piece
+  const uint32_t CB = t1_cbytes(KP, G), VB = t1_vbytes(G);
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  uint16_t* Cs = reinterpret_cast<uint16_t*>(smem_raw);
-  uint16_t* Us = Cs + (size_t)NP * 64 * KP;
-  uint16_t* Vs = Us + (size_t)NP * 64 * KP;
-  float* Ds = reinterpret_cast<float*>(Vs + NP * 4096);
-  float* Ys = Ds + 2 * 256;
-  __shared__ __align__(8) uint64_t b_yf[kMaxNS], b_ye[kMaxNS], b_cf, b_ce, b_vf, b_ve, b_df[2], b_de[2], b_uf[2],
-      b_ue[2], b_rf[2], b_re[2], b_qf, b_qe, b_if[kItemRing], b_ie[kItemRing];
+  __shared__ __align__(8) uint64_t b_yf[kMaxNS], b_ye[kMaxNS], b_cf, b_ce, b_vf[2], b_ve[2], b_df[kND], b_de[kND],
+      b_tf[kMaxUT], b_te[kMaxUT], b_uf[2], b_ue[2], b_rf, b_re, b_qf, b_qe, b_if[kItemRing], b_ie[kItemRing], b_done[2];
   __shared__ int s_item[kItemRing];
   __shared__ uint32_t tmem_base;
   __shared__ int s_abort;
   volatile int* abort_flag = &s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   auto sa = [](const void* p) { return (uint32_t)__cvta_generic_to_shared(p); };
-  const uint32_t yf = sa(b_yf), ye = sa(b_ye), cf = sa(&b_cf), ce = sa(&b_ce), vf = sa(&b_vf), ve = sa(&b_ve),
-                 df = sa(b_df), de = sa(b_de), uf = sa(b_uf), ue = sa(b_ue), rf = sa(b_rf), re = sa(b_re),
-                 qf = sa(&b_qf), qe = sa(&b_qe), itf = sa(b_if), ite = sa(b_ie);
+  const uint32_t Cs = sa(smem_raw), Us = Cs + CB, Vs = Us + UB * CB, Ds = Vs + 2 * VB, Ys = Ds + kND * 1024u;
+  const uint32_t yf = sa(b_yf), ye = sa(b_ye), cf = sa(&b_cf), ce = sa(&b_ce), vf = sa(b_vf), ve = sa(b_ve),
+                 df = sa(b_df), de = sa(b_de), tf = sa(b_tf), te = sa(b_te), uf = sa(b_uf), ue = sa(b_ue),
+                 rf = sa(&b_rf), re = sa(&b_re), qf = sa(&b_qf), qe = sa(&b_qe), itf = sa(b_if), ite = sa(b_ie),
+                 mdone = sa(b_done);
+  // Operand rows and columns past a block's own are read (and multiplied by
+  // zeros of the other operand, or their results dropped): everything in the
+  // buffers has to be finite from the start.
+  for (uint32_t o = tid * 16u; o < (Ys - Cs) + (uint32_t)NS * kYSlot; o += kThreads * 16u)
+    *reinterpret_cast<uint4*>(smem_raw + o) = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) {
     s_abort = 0;
     for (int s = 0; s < NS; ++s) {
       mbar_init(yf + 8 * s, 1);
-      mbar_init(ye + 8 * s, kNU);
+      mbar_init(ye + 8 * s, 1);
+    }
+    for (int s = 0; s < kND; ++s) {
+      mbar_init(df + 8 * s, 1);
+      mbar_init(de + 8 * s, 1);
+    }
+    for (int s = 0; s < NT; ++s) {
+      mbar_init(tf + 8 * s, 1);
+      mbar_init(te + 8 * s, kNU);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(vf + 8 * s, 1);
+      mbar_init(ve + 8 * s, 1);
+      mbar_init(uf + 8 * s, kNU);
+      mbar_init(ue + 8 * s, 1);
     }
     mbar_init(cf, 1);
     mbar_init(ce, 1);
-    mbar_init(vf, 1);
-    mbar_init(ve, 1);
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(df + 8 * s, 1);
-      mbar_init(de + 8 * s, kNU);
-      mbar_init(uf + 8 * s, kNU);
-      mbar_init(ue + 8 * s, 2);   // released by both issuers
-      mbar_init(rf + 8 * s, 1);
-      mbar_init(re + 8 * s, kNE);
-    }
+    mbar_init(rf, 1);
+    mbar_init(re, kNE);
     mbar_init(qf, 1);
     mbar_init(qe, kNE);
     for (int s = 0; s < kItemRing; ++s) {
       mbar_init(itf + 8 * s, 1);
       mbar_init(ite + 8 * s, kItemReaders);
     }
+    for (int s = 0; s < 2; ++s) mbar_init(mdone + 8 * s, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
   }
-  if (warp == kWarpM) {
+  if (warp == kWarpU) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sa(&tmem_base)), "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
   }
+  fence_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t T = tmem_base;
-  // Next item of the ring for a role (one reader per warp; lane 0 releases
-  // the slot).  n_list marks the end.  Every lane of the warp calls it.
-  auto next_item = [&](uint32_t& k) -> int {
+  const uint32_t T = tmem_base, TR = T + t1_rcol(KP), TU = TR + 16u * G;
+  // Next unit of the ring for a role (one reader per warp; lane 0 releases
+  // the slot).  n_units marks the end.  Every lane of the warp calls it.
+  auto next_unit = [&](uint32_t& k) -> int {
     const int s = k & (kItemRing - 1);
-    int kk = n_list;
-    if (wait_all(itf + 8 * s, (k / kItemRing) & 1)) kk = *reinterpret_cast<volatile int*>(&s_item[s]);
+    int u = n_units;
+    if (wait_all(itf + 8 * s, (k / kItemRing) & 1)) u = *reinterpret_cast<volatile int*>(&s_item[s]);
     else *abort_flag = 1;
     __syncwarp();
     if (lane == 0) mbar_arrive(ite + 8 * s);
     ++k;
-    return kk;
+    return u;
+  };
+  // Unit u: item kk = u / nsplit, its kept B [lo, hi) of the list at X.qoff.
+  struct Unit {
+    int kk, q, lo, hi;
+  };
+  auto unit = [&](int u) -> Unit {
+    Unit r;
+    r.kk = u / nsplit;
+    const int s = u - r.kk * nsplit;
+    r.q = qlist[r.kk];
+    const long long n = X.qcnt[r.q];
+    r.lo = (int)(n * s / nsplit);
+    r.hi = (int)(n * (s + 1) / nsplit);
+    return r;
   };
 
   if (warp == kWarpY) {
     // ---------------------------------------------------------- Y producer
-    uint32_t ys = 0, ik = 0;
-    for (int kk = next_item(ik); kk < n_list && !aborted(abort_flag); kk = next_item(ik)) {
-      const int q = qlist[kk];
-      const int F = P.c_j[q];
+    // Y^{BF} as [piece][(g, f)][8 beta x 16 b]: up to 32 row groups (g, f) per
+    // slot, the two pieces copied by lanes 0 and 1.
+    uint32_t ik = 0;
+    Ring y;
+    for (int u = next_unit(ik); u < n_units && !aborted(abort_flag); u = next_unit(ik)) {
+      const Unit it = unit(u);
+      const int F = P.c_j[it.q];
       const int nF = P.n_ao[P.species[F]];
-      const int* Rf = P.c_R + 3 * q;
-      const long long b0 = X.qoff[q];
-      const int nbt = X.qcnt[q];
-      for (int i0 = 0; i0 < nbt && !aborted(abort_flag); i0 += 32) {
+      const int* Rf = P.c_R + 3 * it.q;
+      const long long b0 = X.qoff[it.q];
+      for (int i0 = it.lo; i0 < it.hi && !aborted(abort_flag); i0 += 32) {
         long long yo = 0;
-        int mB = 0;
-        if (i0 + lane < nbt) {
+        int ng = 0;
+        if (i0 + lane < it.hi) {
           const int p = X.blist[b0 + i0 + lane];
           const int b = P.v_j[p];
           const int* Rb = P.v_R + 3 * p;
           const int yc = ylut_get(P, b, F, Rf[0] - Rb[0], Rf[1] - Rb[1], Rf[2] - Rb[2]);
-          yo = yc >= 0 ? P.y_off[yc] / NP : -1;
-          mB = P.n_abf[P.species[b]];
+          yo = yc < 0 ? -1 : U.yh_blk ? X.y_idx[yc] * U.yh_blk : P.y_off[yc];
+          ng = ((P.n_abf[P.species[b]] + 7) >> 3) * nF;
         }
-        const int nb = min(32, nbt - i0);
+        const int nb = min(32, it.hi - i0);
         for (int j = 0; j < nb; ++j) {
           const long long yoj = __shfl_sync(0xffffffffu, yo, j);
-          const int mBj = __shfl_sync(0xffffffffu, mB, j);
-          if (lane == 0 && !aborted(abort_flag)) {
-            if (yoj < 0) *abort_flag = 1;   // a kept triplet always has its Y block
-            // runs [fa, fb) of at most FS rows, within each U chunk, rows f < nF only
-            for (int c = 0; c < 2 && !aborted(abort_flag); ++c) {
-              const int e = min(c ? NF : FH, nF);
-              for (int fa = c ? FH : 0; fa < e && !aborted(abort_flag); fa += FS) {
-                const int fb = min(fa + FS, e);
-                const int s = (int)(ys % NS);
-                if (ys >= (uint32_t)NS && !mbar_wait(ye + 8 * s, ((ys / NS) - 1) & 1)) {
-                  *abort_flag = 1;
-                  break;
-                }
-                const uint32_t bytes = (uint32_t)((fb - fa) * mBj) * 64u;
-                mbar_expect_tx(yf + 8 * s, bytes);
-                bulk_g2s(sa(Ys + s * SLOT), U.Yf + yoj + (long long)fa * mBj * 16, bytes, yf + 8 * s);
-                ++ys;
-              }
+          const int ngj = __shfl_sync(0xffffffffu, ng, j);
+          if (yoj < 0) *abort_flag = 1;   // a kept triplet always has its Y block
+          for (int r0 = 0; r0 < ngj; r0 += kYG, y.next(NS)) {
+            const int s = y.s;
+            const uint32_t bytes = 256u * (uint32_t)min(kYG, ngj - r0);
+            bool ok = true;
+            if (lane == 0) {
+              ok = !aborted(abort_flag) && mbar_wait(ye + 8 * s, y.ph ^ 1);
+              if (ok) mbar_expect_tx(yf + 8 * s, 2 * bytes);
+              else *abort_flag = 1;
             }
+            ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+            if (!ok) break;
+            if (lane < 2)
+              bulk_g2s(Ys + s * kYSlot + lane * kYPiece, U.Yh + yoj + (long long)lane * ngj * 128 + r0 * 128, bytes,
+                       yf + 8 * s);
           }
-          __syncwarp();
+          if (__shfl_sync(0xffffffffu, (int)aborted(abort_flag), 0)) break;
         }
       }
     }
-    if (lane == 0)   // copies in flight land before the CTA leaves
-      for (int s = 0; s < NS; ++s) {
-        const uint32_t n = ys / NS + ((uint32_t)s < ys % NS ? 1u : 0u);
-        if (n) mbar_wait(yf + 8 * s, (n - 1) & 1);
-      }
+    __syncwarp();
+    if (lane == 0) drain(yf, y, NS);   // copies in flight land before the CTA leaves
   } else if (warp == kWarpV) {
     // -------------------------------------- scheduler, C, D and V producer
-    // Lane 0 publishes item indices two items ahead of this warp's own
-    // position (a slot is reused once every reader has taken its item).
+    // Lane 0 publishes units two ahead of this warp's own position (a slot
+    // is reused once every reader has taken its unit).
     uint32_t pub = 0;
     bool pub_done = false;
     auto publish = [&]() {
       const int s = pub & (kItemRing - 1);
       if (pub >= kItemRing && !mbar_wait(ite + 8 * s, ((pub / kItemRing) - 1) & 1)) {
         *abort_flag = 1;
-        s_item[s] = n_list;   // best effort: readers also stop on the flag
+        s_item[s] = n_units;   // best effort: readers also stop on the flag
         pub_done = true;
         return;
       }
-      int kk = aborted(abort_flag) ? n_list : atomicAdd(work, 1);
-      if (kk > n_list) kk = n_list;
-      s_item[s] = kk;
+      int u = n_units;
+      while (!aborted(abort_flag)) {   // units without a B (fewer B than parts) are passed over
+        u = atomicAdd(work, 1);
+        if (u >= n_units) break;
+        const Unit it = unit(u);
+        if (it.hi > it.lo) break;
+      }
+      if (u > n_units) u = n_units;
+      s_item[s] = u;
       mbar_arrive(itf + 8 * s);
       ++pub;
-      if (kk >= n_list) pub_done = true;
+      if (u >= n_units) pub_done = true;
     };
     if (lane == 0) {
       publish();
       if (!pub_done) publish();
     }
     __syncwarp();
-    uint32_t vb = 0, db = 0, it = 0, ca = 0, own = 0;
-    auto own_item = [&]() -> int {
-      int kk = n_list;
-      if (lane == 0 && own < pub) kk = *reinterpret_cast<volatile int*>(&s_item[own & (kItemRing - 1)]);
+    uint32_t it_n = 0, ca = 0, own = 0;
+    Ring v, d;
+    auto own_unit = [&]() -> int {
+      int u = n_units;
+      if (lane == 0 && own < pub) u = *reinterpret_cast<volatile int*>(&s_item[own & (kItemRing - 1)]);
       ++own;
-      return __shfl_sync(0xffffffffu, kk, 0);
+      return __shfl_sync(0xffffffffu, u, 0);
     };
-    for (int kk = own_item(); kk < n_list && !aborted(abort_flag); kk = own_item(), ++it) {
-      const int q = qlist[kk];
-      const long long b0 = X.qoff[q];
-      const int nbt = X.qcnt[q];
+    for (int u = own_unit(); u < n_units && !aborted(abort_flag); u = own_unit(), ++it_n) {
+      const Unit it = unit(u);
+      const long long b0 = X.qoff[it.q];
+      const uint32_t gA = (uint32_t)(P.n_abf[P.species[P.c_home[it.q]]] + 7) >> 3;
       if (lane == 0) {
         if (!pub_done) publish();
-        if (it >= 1 && !mbar_wait(ce, (it - 1) & 1)) *abort_flag = 1;
+        if (it_n >= 1 && !mbar_wait(ce, (it_n - 1) & 1)) *abort_flag = 1;
         if (!aborted(abort_flag)) {
-          mbar_expect_tx(cf, (uint32_t)NP * CPB);
-          const uint16_t* src = U.Cu + (long long)kk * U.cu_blk;
-#pragma unroll
-          for (int pp = 0; pp < NP; ++pp) bulk_g2s(sa(Cs) + pp * CPB, src + (long long)pp * 64 * KP, CPB, cf);
+          mbar_expect_tx(cf, gA * 2u * rowg);
+          bulk_g2s(Cs, U.Cu + (long long)it.kk * U.cu_blk, gA * 2u * rowg, cf);
           ++ca;
         }
       }
       __syncwarp();
-      for (int i0 = 0; i0 < nbt && !aborted(abort_flag); i0 += 32) {
+      for (int i0 = it.lo; i0 < it.hi && !aborted(abort_flag); i0 += 32) {
         long long vo = 0, dofs = 0;
-        if (i0 + lane < nbt) {
+        if (i0 + lane < it.hi) {
           const int p = X.blist[b0 + i0 + lane];
           vo = U.t1_idx[p] * U.vu_blk;
           const int di = P.v_didx[p];
-          dofs = di >= 0 ? (long long)di * 256 : -1;   // a kept triplet always has its D block
+          dofs = di >= 0 ? (long long)di * 512 : -1;   // a kept triplet always has its D block
         }
-        const int nb = min(32, nbt - i0);
+        const int nb = min(32, it.hi - i0);
         for (int j = 0; j < nb; ++j) {
           const long long voj = __shfl_sync(0xffffffffu, vo, j);
           const long long doj = __shfl_sync(0xffffffffu, dofs, j);
           if (lane == 0 && doj < 0) *abort_flag = 1;
           if (lane == 0 && !aborted(abort_flag)) {
-            const int s = db & 1;
-            bool ok = db < 2 || mbar_wait(de + 8 * s, ((db >> 1) - 1) & 1);
+            bool ok = mbar_wait(de + 8 * d.s, d.ph ^ 1);
             if (ok) {
-              mbar_expect_tx(df + 8 * s, 1024u);
-              bulk_g2s(sa(Ds + s * 256), U.Df + doj, 1024u, df + 8 * s);
-              ++db;
+              mbar_expect_tx(df + 8 * d.s, 1024u);
+              bulk_g2s(Ds + d.s * 1024u, U.Dh + doj, 1024u, df + 8 * d.s);
+              d.next(kND);
             }
-            ok = ok && (vb < 1 || mbar_wait(ve, (vb - 1) & 1));
+            ok = ok && mbar_wait(ve + 8 * v.s, v.ph ^ 1);
             if (ok) {
-              mbar_expect_tx(vf, (uint32_t)NP * 8192u);
-              const uint16_t* src = U.Vu + voj;
-#pragma unroll
-              for (int pp = 0; pp < NP; ++pp) bulk_g2s(sa(Vs) + pp * 8192, src + pp * 4096, 8192u, vf);
-              ++vb;
+              mbar_expect_tx(vf + 8 * v.s, gA * 2048u);
+              bulk_g2s(Vs + v.s * VB, U.Vu + voj, gA * 2048u, vf + 8 * v.s);
+              v.next(2);
             } else {
               *abort_flag = 1;
             }
@@ -500,274 +572,266 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (lane == 0) {
       if (ca) mbar_wait(cf, (ca - 1) & 1);
-      if (vb) mbar_wait(vf, (vb - 1) & 1);
-      for (int s = 0; s < 2; ++s) {
-        const uint32_t n = db / 2 + ((uint32_t)s < db % 2 ? 1u : 0u);
-        if (n) mbar_wait(df + 8 * s, (n - 1) & 1);
-      }
+      drain(vf, v, 2);
+      drain(df, d, kND);
     }
-  } else if (warp == kWarpM) {
-    // ------------------------------------------------------------ R issuer
-    // R_B = C_AF . U_B^T (M = 64 alpha, N = beta, K = (f,a), one f per k
-    // step) into one of two accumulators of kRCols columns.  A U piece
-    // plane is 64 rows, i.e. eight 8-row groups, after the previous one, so
-    // pieces 0 and 1 together are one N = 128 operand: block 0 (columns
-    // 0-63) collects the products with U_0, block 1 those with U_1, and
-    // R = block 0 + block 1: C0 [U0;U1], C1 U0.  Descriptors
-    // are formed once; a k step adds 16 (256 bytes).
-    constexpr int NR = 2;   // MMAs per k step
-    const uint32_t idR128 = idesc_split<SP>(64, 128, 0), idR64 = idesc_split<SP>(64, 64, 0);
-    const uint32_t rowg = 16u * KP;   // bytes between 8-row groups of C and U
-    const uint64_t dC = sdesc2(sa(Cs), 128, rowg), dUR = sdesc2(sa(Us), 128, rowg);
-    uint64_t pa[NR], pb[NR];
-    uint32_t pid[NR];
-    {
-      pa[0] = dC;   // C0 [U0;U1]
-      pb[0] = dUR;
-      pid[0] = idR128;
-      pa[1] = dC + ((uint64_t)CPB >> 4);   // C1 U0
-      pb[1] = dUR;
-      pid[1] = idR64;
-    }
-    uint32_t rb = 0, it = 0, ik = 0;
+  } else if (warp == kWarpU) {
+    // ------------------------------------------------------------ U issuer
+    // Tile of U: 128 rows (g, f, beta of the group) x 16 columns a,
+    // U = Y0 D1^T + Y1 D0^T + Y0 D0^T (K = 16 b), always fp16 pieces.  The
+    // products of a slot's two tiles alternate: an instruction waits for the
+    // one before on the same accumulator (72 cycles each in one chain).
+    const uint32_t idU = idesc_split<kSplitHalf>(128, 16, 0);
+    uint32_t ik = 0;
+    Ring y, t, d;
     bool ok = true;
-    for (int kk = next_item(ik); kk < n_list; kk = next_item(ik), ++it) {
-      const int q = qlist[kk];
-      const int nbt = X.qcnt[q];
-      if (lane == 0 && ok) {
-        ok = mbar_wait(cf, it & 1);
-        tc_fence_after();
-        for (int i = 0; i < nbt && ok; ++i) {
-          if (aborted(abort_flag)) {
-            ok = false;
-            break;
-          }
-          const int rbuf = rb & 1;
-          const uint32_t dR = T + kRCol + (uint32_t)kRCols * rbuf;
-          if (rb >= 2) ok = mbar_wait(re + 8 * rbuf, ((rb >> 1) - 1) & 1);
-          for (int c = 0; c < 2 && ok; ++c) {
-            ok = mbar_wait(uf + 8 * c, rb & 1);
-            if (!ok) break;
-            tc_fence_after();
-            const int f0 = c ? FH : 0, f1 = c ? NF : FH;
-            for (int f = f0; f < f1; ++f) {
-              const uint64_t o = 16u * (uint32_t)f;
-#pragma unroll
-              for (int k = 0; k < NR; ++k) umma_f16(dR, pa[k] + o, pb[k] + o, pid[k], (f > 0 || k > 0) ? 1u : 0u);
+    for (int u = next_unit(ik); u < n_units; u = next_unit(ik)) {
+      const Unit it = unit(u);
+      const int nF = P.n_ao[P.species[P.c_j[it.q]]];
+      const long long b0 = X.qoff[it.q];
+      for (int i0 = it.lo; i0 < it.hi; i0 += 32) {
+        int ng = 0;
+        if (i0 + lane < it.hi) ng = ((P.n_abf[P.species[P.v_j[X.blist[b0 + i0 + lane]]]] + 7) >> 3) * nF;
+        const int nb = min(32, it.hi - i0);
+        for (int j = 0; j < nb; ++j) {
+          const int ngj = __shfl_sync(0xffffffffu, ng, j);
+          if (lane == 0 && ok) {
+            ok = !aborted(abort_flag) && mbar_wait(df + 8 * d.s, d.ph);
+            const uint64_t dD = sdesc2(Ds + d.s * 1024u, 128, 256);
+            for (int r0 = 0; r0 < ngj && ok; r0 += kYG) {
+              ok = mbar_wait(yf + 8 * y.s, y.ph) && mbar_wait(te + 8 * t.s, t.ph ^ 1);
+              if (!ok) break;
+              tc_fence_after();
+              const uint64_t dY = sdesc2(Ys + y.s * kYSlot, 128, 256);
+              const uint32_t tu = TU + 32u * t.s;
+              const bool two = r0 + 16 < ngj;
+              umma_f16(tu, dY, dD + 32, idU, 0u);                            // Y0 D1 (a piece of D: 512 bytes)
+              if (two) umma_f16(tu + 16, dY + 256, dD + 32, idU, 0u);        // (the second tile: 4096 bytes on)
+              umma_f16(tu, dY + (kYPiece >> 4), dD, idU, 1u);                // Y1 D0
+              if (two) umma_f16(tu + 16, dY + 256 + (kYPiece >> 4), dD, idU, 1u);
+              umma_f16(tu, dY, dD, idU, 1u);                                 // Y0 D0
+              if (two) umma_f16(tu + 16, dY + 256, dD, idU, 1u);
+              umma_commit(tf + 8 * t.s);
+              umma_commit(ye + 8 * y.s);
+              y.next(NS);
+              t.next(NT);
             }
-            umma_commit(ue + 8 * c);
-            if (c == 1) umma_commit(rf + 8 * rbuf);
+            if (ok) umma_commit(de + 8 * d.s);
+            else *abort_flag = 1;
+            d.next(kND);
           }
-          ++rb;
+          __syncwarp();
         }
-        if (ok) umma_commit(ce);
-        if (!ok) *abort_flag = 1;
       }
-      __syncwarp();
     }
-  } else if (warp == kWarpQ) {
-    // ------------------------------------------------------------ Q issuer
-    // Q[:, chunk] += V_AB . U_B[:, chunk] (M = 64 alpha, N = the chunk's
-    // (f,a) columns, K = beta in four k steps; U read MN-major).
-    const int N0 = 16 * FH, N1 = 16 * (NF - FH);
-    const uint32_t idQ0 = idesc_split<SP>(64, N0, 1), idQ1 = N1 > 0 ? idesc_split<SP>(64, N1, 1) : 0u;
-    const uint32_t rowg = 16u * KP;
-    const uint64_t dV = sdesc2(sa(Vs), 128, 1024), dUQ = sdesc2(sa(Us), rowg, 128);
-    uint64_t pa[NPROD], pb[NPROD];
-    {
-      int k = 0;
-#pragma unroll
-      for (int sum = NP - 1; sum >= 0; --sum)
-#pragma unroll
-        for (int ia = 0; ia <= sum; ++ia, ++k) {
-          pa[k] = dV + ((uint64_t)(ia * 8192) >> 4);
-          pb[k] = dUQ + ((uint64_t)((sum - ia) * CPB) >> 4);
-        }
+    if (lane == 0) {
+      umma_commit(mdone);
+      mbar_wait(mdone, 0);
     }
-    const uint64_t kbA = 256 >> 4, kbB = (uint64_t)(2 * rowg) >> 4;
-    uint32_t rb = 0, seg = 0, ik = 0;
+  } else if (warp == kWarpR) {
+    // ------------------------------------------------------- Q and R issuer
+    // Q += V_AB . U_B, K = beta in steps of 16: A = both pieces of V (row
+    // groups (g, piece), M = 128), N = 16 n_ao(F) columns (f,a) of one piece
+    // of U, read MN-major.
+    // R_B = C_AF . U_B^T, K = (f,a), one f per k step: A = both pieces of C
+    // (row groups (g, piece), M = 128), B = both pieces of U (N = 16 G), so
+    // one instruction per k step makes all four piece products, and R is the
+    // sum over the two row groups of an alpha and the two columns of a beta.
+    // Q goes first: meanwhile the epilogue empties the accumulator of the R before.
+    const uint32_t idR = idesc_split<SP>(128, 16 * G, 0);
+    const uint64_t dC = sdesc2(Cs, 128, rowg);
+    const uint64_t kbB = (uint64_t)(2 * rowg) >> 4, pB = (uint64_t)(CB >> 1) >> 4;
+    uint32_t rp = 1, qp = 1, it_n = 0, ik = 0;   // phases of the free accumulators
+    Ring ub, v;
     bool ok = true;
-    for (int kk = next_item(ik); kk < n_list; kk = next_item(ik)) {
-      const int q = qlist[kk];
-      const int nbt = X.qcnt[q];
-      if (lane == 0 && ok) {
-        for (int i = 0; i < nbt && ok; ++i) {
-          if (aborted(abort_flag)) {
-            ok = false;
-            break;
-          }
-          const bool first = (i % SEG) == 0, last = (i % SEG) == SEG - 1 || i == nbt - 1;
-          for (int c = 0; c < 2 && ok; ++c) {
-            ok = mbar_wait(uf + 8 * c, rb & 1);
-            if (ok && c == 0) ok = mbar_wait(vf, rb & 1) && (!first || seg == 0 || mbar_wait(qe, (seg - 1) & 1));
-            if (!ok) break;
-            tc_fence_after();
-            const int f0 = c ? FH : 0;
-            const int Nc = c ? N1 : N0;
-            if (Nc > 0) {
-              const uint32_t idQ = c ? idQ1 : idQ0, tq = T + 16u * f0;
-              const uint64_t oB = (uint64_t)(f0 * 256) >> 4;
-              for (int kb = 0; kb < 4; ++kb)
-#pragma unroll
-                for (int k = 0; k < NPROD; ++k)
-                  umma_f16(tq, pa[k] + kbA * kb, pb[k] + oB + kbB * kb, idQ, (first && kb == 0 && k == 0) ? 0u : 1u);
+    for (int u = next_unit(ik); u < n_units; u = next_unit(ik), ++it_n) {
+      const Unit it = unit(u);
+      const int nF = P.n_ao[P.species[P.c_j[it.q]]];
+      const uint32_t idQ = idesc_split<SP>(128, 16 * nF, 1);
+      const long long b0 = X.qoff[it.q];
+      int run = 0;
+      for (int i0 = it.lo; i0 < it.hi; i0 += 32) {
+        int nk_l = 0;
+        if (i0 + lane < it.hi) nk_l = (P.n_abf[P.species[P.v_j[X.blist[b0 + i0 + lane]]]] + 15) >> 4;
+        const int nb = min(32, it.hi - i0);
+        for (int j = 0; j < nb; ++j) {
+          const int nk = __shfl_sync(0xffffffffu, nk_l, j);
+          if (lane == 0 && ok) {
+            const bool first = run == 0, last = ++run == SEG || i0 + j == it.hi - 1;
+            if (last) run = 0;
+            ok = !aborted(abort_flag) && mbar_wait(uf + 8 * ub.s, ub.ph) && mbar_wait(vf + 8 * v.s, v.ph) &&
+                 (!first || mbar_wait(qe, qp));
+            if (ok) {
+              tc_fence_after();
+              const uint64_t dV = sdesc2(Vs + v.s * VB, 128, 1024), dU = sdesc2(Us + ub.s * CB, rowg, 128);
+              for (int kb = 0; kb < nk; ++kb) {
+                umma_f16(T, dV + 16u * kb, dU + pB + kbB * kb, idQ, (first && kb == 0) ? 0u : 1u);
+                umma_f16(T, dV + 16u * kb, dU + kbB * kb, idQ, 1u);
+              }
+              umma_commit(ve + 8 * v.s);
+              v.next(2);
+              if (last) {
+                umma_commit(qf);
+                qp ^= 1;
+              }
+              ok = (i0 + j > it.lo || mbar_wait(cf, it_n & 1)) && mbar_wait(re, rp);
             }
-            umma_commit(ue + 8 * c);
+            if (ok) {
+              tc_fence_after();
+              const uint64_t dU = sdesc2(Us + ub.s * CB, 128, rowg);
+              for (int f = 0; f < nF; ++f) umma_f16(TR, dC + 16u * f, dU + 16u * f, idR, f > 0 ? 1u : 0u);
+              umma_commit(rf);
+              umma_commit(ue + 8 * ub.s);
+              ub.next(UB);
+              rp ^= 1;
+              if (i0 + j == it.hi - 1) umma_commit(ce);
+            } else {
+              *abort_flag = 1;
+            }
           }
-          if (!ok) break;
-          umma_commit(ve);
-          if (last) {
-            umma_commit(qf);
-            ++seg;
-          }
-          ++rb;
+          __syncwarp();
         }
-        if (!ok) *abort_flag = 1;
       }
-      __syncwarp();
+    }
+    if (lane == 0) {
+      umma_commit(mdone + 8);
+      mbar_wait(mdone + 8, 0);
     }
   } else if (warp >= kWarpE && warp < kWarpE + kNE) {
     // --------------------------------------------------------------- epilogue
-    const int qd = warp & 3;                 // tensor-memory lane quarter
-    const int ew = warp - kWarpE;
-    const int alpha = qd * 16 + (lane & 15); // accumulator row held by this thread
-    const int half = lane >> 4;              // columns [0,16) or [16,32) of a 32-column load
-    const uint32_t tl = T + ((uint32_t)(qd * 32) << 16);
-    uint32_t rb = 0, seg = 0, it = 0, ik = 0;
-    double fl = 0.0;
+    // Eight warps: lane quarter qd (rows alpha 16 qd .. + 15, both pieces) and
+    // half h of the columns.  Lane l holds piece (l >> 3) & 1 of row alpha; the
+    // lanes l and l ^ 8 add their rows, each keeping 16 of the 32 columns.
+    const int qd = warp & 3, h = (warp - kWarpE) >> 2, ew = warp - kWarpE;
+    const int alpha = qd * 16 + 8 * (lane >> 4) + (lane & 7), pc = (lane >> 3) & 1;
+    const uint32_t tl = (uint32_t)(qd * 32) << 16;
+    // x[t] = this lane pair's sum over columns c0 + 16 pc + t (and, with c1, over
+    // c1 + 16 pc + t): each lane sends the half that the other keeps
+    auto pair_read = [&](uint32_t c0, uint32_t c1, bool two, float (&x)[16]) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        uint32_t a0[8], a1[8], b0[8], b1[8];
+        tmem_ld8(c0 + 8u * q, a0);
+        tmem_ld8(c0 + 16u + 8u * q, a1);
+        if (two) {
+          tmem_ld8(c1 + 8u * q, b0);
+          tmem_ld8(c1 + 16u + 8u * q, b1);
+        }
+        tmem_wait_ld();
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          const float lo = two ? __uint_as_float(a0[t]) + __uint_as_float(b0[t]) : __uint_as_float(a0[t]);
+          const float hi = two ? __uint_as_float(a1[t]) + __uint_as_float(b1[t]) : __uint_as_float(a1[t]);
+          x[8 * q + t] = (pc ? hi : lo) + __shfl_xor_sync(0xffffffffu, pc ? lo : hi, 8);
+        }
+      }
+    };
+    uint32_t rb = 0, seg = 0, ik = 0;
+    unsigned long long fl = 0;
     bool ok = true;
-    for (int kk = next_item(ik); kk < n_list && ok; kk = next_item(ik), ++it) {
-      const int q = qlist[kk];
-      const int A = P.c_home[q], F = P.c_j[q];
+    for (int u = next_unit(ik); u < n_units && ok; u = next_unit(ik)) {
+      const Unit it = unit(u);
+      const int A = P.c_home[it.q], F = P.c_j[it.q];
       const int sA = P.species[A];
       const int nA = P.n_ao[sA], mA = P.n_abf[sA], nF = P.n_ao[P.species[F]];
-      const long long b0 = X.qoff[q];
-      const int nbt = X.qcnt[q];
-      const float* Cf = reinterpret_cast<const float*>(U.Cu + (long long)kk * U.cu_blk + (long long)NP * 64 * KP);
-      double e_it = 0.0, g_it[3] = {0.0, 0.0, 0.0};
-      for (int i0 = 0; i0 < nbt && ok; i0 += 32) {
+      const long long b0 = X.qoff[it.q];
+      const float* Cf = reinterpret_cast<const float*>(U.Cu + (long long)it.kk * U.cu_blk + (CB >> 1));
+      int run = 0;
+      for (int i0 = it.lo; i0 < it.hi && ok; i0 += 32) {
         int p_l = 0, mB_l = 0, nB_l = 0;
         long long vo_l = 0;
-        if (i0 + lane < nbt) {
+        if (i0 + lane < it.hi) {
           p_l = X.blist[b0 + i0 + lane];
           const int sb = P.species[P.v_j[p_l]];
           mB_l = P.n_abf[sb];
           nB_l = P.n_ao[sb];
           vo_l = U.t1_idx[p_l] * U.vu_blk;
         }
-        const int nb = min(32, nbt - i0);
+        const int nb = min(32, it.hi - i0);
         for (int j = 0; j < nb && ok; ++j) {
           ok = __all_sync(0xffffffffu, !aborted(abort_flag)) != 0;
           if (!ok) break;
-          const int i = i0 + j;
-          const int p = __shfl_sync(0xffffffffu, p_l, j);
           const int mB = __shfl_sync(0xffffffffu, mB_l, j);
-          const int nB = __shfl_sync(0xffffffffu, nB_l, j);
           const long long vo = __shfl_sync(0xffffffffu, vo_l, j);
-          const float* dV = reinterpret_cast<const float*>(U.Vu + vo + NP * 4096);
-          const bool last = (i % SEG) == SEG - 1 || i == nbt - 1;
-          const int rbuf = rb & 1;
-          // ---- R_B -> g^V_AB (the grad V rows of the first 32 columns are
-          // fetched before the wait; they do not depend on R)
-          float gv[3] = {0.f, 0.f, 0.f};
+          const bool last = ++run == SEG || i0 + j == it.hi - 1;
+          // ---- R_B -> g^V_AB (the grad V values of this lane's columns
+          // beta = cb .. cb + 15 are fetched before the wait: they do not
+          // depend on R, and their latency is the longest of the epilogue)
+          const bool any = qd * 16 < mA && 32 * h < mB;
+          const int cb = 32 * h + 16 * pc;
+          const bool act = alpha < mA && cb < mB;
           float4 w[3][4];
-          const float4* dV4 = reinterpret_cast<const float4*>(dV) + qd * 32 + lane;   // epilogue load order (ep_at)
-          {
-            const int cb = 16 * half;
-            if (alpha < mA && cb < mB)
+          if (act) {
+            const float4* dV4 = reinterpret_cast<const float4*>(U.Vu + vo + (VB >> 1)) + h * 512 + qd * 32 + lane;
 #pragma unroll
-              for (int c = 0; c < 3; ++c)
+            for (int c = 0; c < 3; ++c)
 #pragma unroll
-                for (int t4 = 0; t4 < 4; ++t4) w[c][t4] = dV4[c * 1024 + t4 * 128];
+              for (int t4 = 0; t4 < 4; ++t4) w[c][t4] = dV4[c * 1024 + t4 * 128];
           }
-          ok = wait_all(rf + 8 * rbuf, (rb >> 1) & 1);
+          ok = wait_all(rf, rb & 1);
           tc_fence_after();
-          if (ok) {
-            for (int c0 = 0; c0 < 64; c0 += 32) {
-              if (c0 >= mB) break;
-              const int cb = c0 + 16 * half;
-              const bool act = alpha < mA && cb < mB;
-              if (c0 > 0 && act)
+          float x[16];
+          if (ok && any) pair_read(TR + tl + 32u * h, TR + tl + 8u * G + 32u * h, true, x);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(re);
+          if (ok && any) {
+            float gv[3] = {0.f, 0.f, 0.f};
+            if (act) {
 #pragma unroll
-                for (int c = 0; c < 3; ++c)
+              for (int t = 0; t < 16; ++t)
+                if (cb + t >= mB) x[t] = 0.f;
 #pragma unroll
-                  for (int t4 = 0; t4 < 4; ++t4) w[c][t4] = dV4[c * 1024 + 512 + t4 * 128];
-              // R = block 0 + block 1: each block dotted in turn (the dots are linear in R)
-#pragma unroll 1
-              for (int blk = 0; blk < 2; ++blk) {
-                uint32_t v[32];
-                tmem_ld32(tl + kRCol + (uint32_t)kRCols * rbuf + 64u * blk + c0, v);
-                float x[16];
+              for (int t4 = 0; t4 < 4; ++t4)
 #pragma unroll
-                for (int t = 0; t < 16; ++t) {
-                  const float hi = __shfl_sync(0xffffffffu, __uint_as_float(v[16 + t]), lane & 15);
-                  x[t] = half ? hi : __uint_as_float(v[t]);
+                for (int c = 0; c < 3; ++c) {
+                  gv[c] = fmaf(w[c][t4].x, x[4 * t4], gv[c]);
+                  gv[c] = fmaf(w[c][t4].y, x[4 * t4 + 1], gv[c]);
+                  gv[c] = fmaf(w[c][t4].z, x[4 * t4 + 2], gv[c]);
+                  gv[c] = fmaf(w[c][t4].w, x[4 * t4 + 3], gv[c]);
                 }
-                if (act) {
+            }
 #pragma unroll
-                  for (int c = 0; c < 3; ++c) {
+            for (int c = 0; c < 3; ++c) gv[c] = warp_sum_f(gv[c]);
+            const float g = lane == 0 ? gv[0] : lane == 1 ? gv[1] : gv[2];
+            const int p = __shfl_sync(0xffffffffu, p_l, j);
+            if (lane < 3 && g != 0.f) dev::add_gV(P, 3 * p + lane, -(double)g * P.sc.r1);
+          }
+          if (ew == 0) fl += (unsigned)(mB * nF * nA) * (unsigned)(2 * __shfl_sync(0xffffffffu, nB_l, j) + 4 * mA);
+          ++rb;
+          // ---- end of a run: Q -> E, g^C (the two halves take alternate 32-column chunks)
+          if (last && ok) {
+            run = 0;
+            ok = wait_all(qf, seg & 1);
+            tc_fence_after();
+            if (ok && qd * 16 < mA) {
+              double e[4] = {0.0, 0.0, 0.0, 0.0};   // <C, Q>, <grad C, Q> of this warp's part
+              for (int jc = h; 32 * jc < 16 * nF; jc += 2) {
+                pair_read(T + tl + 32u * jc, 0u, false, x);
+                if (alpha < mA && 32 * jc + 16 * pc < 16 * nF) {
+                  const float4* src = reinterpret_cast<const float4*>(Cf) + jc * 512 + qd * 32 + lane;
+#pragma unroll
+                  for (int c = 0; c < 4; ++c) {
                     float s = 0.f;
 #pragma unroll
                     for (int t4 = 0; t4 < 4; ++t4) {
-                      s = fmaf(w[c][t4].x, x[4 * t4], s);
-                      s = fmaf(w[c][t4].y, x[4 * t4 + 1], s);
-                      s = fmaf(w[c][t4].z, x[4 * t4 + 2], s);
-                      s = fmaf(w[c][t4].w, x[4 * t4 + 3], s);
+                      const float4 y = src[(long long)c * 16 * KP32 + t4 * 128];
+                      s = fmaf(y.x, x[4 * t4], s);
+                      s = fmaf(y.y, x[4 * t4 + 1], s);
+                      s = fmaf(y.z, x[4 * t4 + 2], s);
+                      s = fmaf(y.w, x[4 * t4 + 3], s);
                     }
-                    gv[c] += s;
+                    e[c] += (double)s;
                   }
                 }
               }
-            }
-          }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(re + 8 * rbuf);
 #pragma unroll
-          for (int c = 0; c < 3; ++c) gv[c] = warp_sum_f(gv[c]);
-          if (lane == 0 && ok)
+              for (int c = 0; c < 4; ++c) e[c] = warp_sum_d(e[c]);
+              if (lane == 0) {
+                if (e[0] != 0.0) dev::add_E(P, -e[0] * P.sc.q1);
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
-              if (gv[c] != 0.f) dev::add_gV(P, 3 * p + c, -(double)gv[c] * P.sc.r1);
-          if (ew == 0 && lane == 0) fl += 2.0 * mB * nA * nB * nF + 4.0 * mA * mB * nA * nF;
-          ++rb;
-          // ---- end of a run: Q -> E, g^C
-          if (last && ok) {
-            ok = wait_all(qf, seg & 1);
-            tc_fence_after();
-            if (ok) {
-              for (int c0 = 0; c0 < KP; c0 += 32) {
-                uint32_t v[32];
-                tmem_ld32(tl + c0, v);
-                float x[16];
-#pragma unroll
-                for (int t = 0; t < 16; ++t) {
-                  const float hi = __shfl_sync(0xffffffffu, __uint_as_float(v[16 + t]), lane & 15);
-                  x[t] = half ? hi : __uint_as_float(v[t]);
-                }
-                const int cb = c0 + 16 * half;
-                if (alpha < mA && cb < KP) {
-                  float s4[4];
-#pragma unroll
-                  for (int c = 0; c < 4; ++c) {
-                    const float4* src =
-                        reinterpret_cast<const float4*>(Cf + (long long)c * 64 * KP32) + (c0 >> 5) * 512 + qd * 32 + lane;
-                    float s = 0.f;
-#pragma unroll
-                    for (int t4 = 0; t4 < 4; ++t4) {
-                      const float4 w = src[t4 * 128];
-                      s = fmaf(w.x, x[4 * t4], s);
-                      s = fmaf(w.y, x[4 * t4 + 1], s);
-                      s = fmaf(w.z, x[4 * t4 + 2], s);
-                      s = fmaf(w.w, x[4 * t4 + 3], s);
-                    }
-                    s4[c] = s;
-                  }
-                  e_it += (double)s4[0];
-                  g_it[0] += (double)s4[1];
-                  g_it[1] += (double)s4[2];
-                  g_it[2] += (double)s4[3];
-                }
+                for (int c = 0; c < 3; ++c)
+                  if (e[c + 1] != 0.0) dev::add_gC(P, 3 * it.q + c, -2.0 * e[c + 1] * P.sc.q1);
               }
             }
             tc_fence_before();
@@ -777,163 +841,70 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-      // item totals: E and g^C_AF
-      e_it = warp_sum_d(e_it);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) g_it[c] = warp_sum_d(g_it[c]);
-      if (lane == 0 && ok) {
-        if (e_it != 0.0) dev::add_E(P, -e_it * P.sc.q1);
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-          if (g_it[c] != 0.0) dev::add_gC(P, 3 * q + c, -2.0 * g_it[c] * P.sc.q1);
-      }
     }
     if (!ok) *abort_flag = 1;
-    if (ew == 0 && lane == 0 && fl != 0.0) atomicAdd(&P.acc[ACC_F1], fl);
-  } else if (warp >= kWarpU) {
-    // ---------------------------------------------------------------------- U
-    // Lane l of U warp uw: row beta = 8 uw + ((l >> 1) & 7), columns
-    // a = 4 qa .. 4 qa + 3 with qa = 2 (l >> 4) + (l & 1).  A half warp then
-    // stores one contiguous 128-byte run of U, and the four lanes of a row
-    // read the same Y row (one shared-memory wavefront per 16-byte chunk for
-    // the warp's eight rows).
-    const int uw = warp - kWarpU;
-    const int r8 = (lane >> 1) & 7, qa = 2 * (lane >> 4) + (lane & 1);
-    const int beta = 8 * uw + r8;
-    const int ysw = 2 * ((beta >> 1) & 1);          // chunk c of row beta is stored at c ^ ysw
-    uint16_t* urow = Us + (beta >> 3) * KP * 8 + (beta & 7) * 8 + (qa & 1) * 4;
-    uint32_t ub = 0, ys = 0, ik = 0;
+    if (ew == 0 && lane == 0 && fl) atomicAdd(&P.acc[ACC_F1], (double)fl);
+  } else if (warp >= kWarpS) {
+    // ------------------------------------------------------------ U splitters
+    // Lane = row (g, f, beta) of a tile, 16 values over a, split into the two
+    // pieces and stored as two core-matrix rows of 16 bytes each; two tiles
+    // at a time, so that one's conversions overlap the other's latencies.
+    const int qd = warp & 3;
+    const uint32_t tl = (uint32_t)(qd * 32) << 16;
+    const float su = P.sc.u1;
+    uint32_t ik = 0;
+    Ring ub, t;
     bool ok = true;
-    for (int kk = next_item(ik); kk < n_list && ok; kk = next_item(ik)) {
-      const int q = qlist[kk];
-      const int nF = P.n_ao[P.species[P.c_j[q]]];
-      const long long b0 = X.qoff[q];
-      const int nbt = X.qcnt[q];
-      for (int i0 = 0; i0 < nbt && ok; i0 += 32) {
-        int mB_l = 0;
-        if (i0 + lane < nbt) mB_l = P.n_abf[P.species[P.v_j[X.blist[b0 + i0 + lane]]]];
-        const int nb = min(32, nbt - i0);
+    for (int u = next_unit(ik); u < n_units && ok; u = next_unit(ik)) {
+      const Unit it = unit(u);
+      const int nF = P.n_ao[P.species[P.c_j[it.q]]];
+      const float inv = 1.0f / (float)nF;
+      const long long b0 = X.qoff[it.q];
+      for (int i0 = it.lo; i0 < it.hi && ok; i0 += 32) {
+        int ng_l = 0;
+        if (i0 + lane < it.hi) ng_l = ((P.n_abf[P.species[P.v_j[X.blist[b0 + i0 + lane]]]] + 7) >> 3) * nF;
+        const int nb = min(32, it.hi - i0);
         for (int j = 0; j < nb && ok; ++j) {
           ok = __all_sync(0xffffffffu, !aborted(abort_flag)) != 0;
           if (!ok) break;
-          const int mB = __shfl_sync(0xffffffffu, mB_l, j);
-          const int s = ub & 1;
-          ok = wait_all(df + 8 * s, (ub >> 1) & 1);
-          if (!ok) break;
-          float2 dd[2][16];   // (D_AB[4 qa + 2 j][b], D_AB[4 qa + 2 j + 1][b])
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int c4 = 0; c4 < 4; ++c4) {
-              const float4 w = *reinterpret_cast<const float4*>(Ds + s * 256 + (4 * qa + i) * 16 + 4 * (c4 ^ qa));
-              float* col = (i & 1) ? &dd[i >> 1][0].y : &dd[i >> 1][0].x;
-              col[2 * (4 * c4)] = w.x;
-              col[2 * (4 * c4 + 1)] = w.y;
-              col[2 * (4 * c4 + 2)] = w.z;
-              col[2 * (4 * c4 + 3)] = w.w;
-            }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(de + 8 * s);
-          for (int c = 0; c < 2 && ok; ++c) {
-            if (ub >= 1) ok = wait_all(ue + 8 * c, (ub - 1) & 1);
+          const int ng = __shfl_sync(0xffffffffu, ng_l, j);
+          ok = wait_all(ue + 8 * ub.s, ub.ph ^ 1);
+          unsigned char* ubase = smem_raw + CB + ub.s * CB + (lane & 7) * 16;
+          for (int r0 = 0; r0 < ng && ok; r0 += kYG) {
+            ok = wait_all(tf + 8 * t.s, t.ph);
             if (!ok) break;
-            const int f0 = c ? FH : 0, f1 = c ? NF : FH;
-            const int e = min(f1, nF);
-            // rows f < nF, one Y slot per run [fa, fb); two f per pass (eight
-            // independent FMA chains per lane)
-            for (int fa = f0; fa < e && ok; fa += FS) {
-              const int fb = min(fa + FS, e);
-              const int sl = (int)(ys % NS);
-              ok = wait_all(yf + 8 * sl, (ys / NS) & 1);
-              if (!ok) break;
-              {
-                // the run's rows rho = (f - fa) mB + beta (the slot's
-                // own order) are shared by all U warps, two per lane and pass
-                // (rho = 16 g + r8 and 16 g + 8 + r8 for row groups g = uw,
-                // uw + kNU, ...), so every warp gets the same share whatever
-                // n_abf(B) is; rows beta >= n_abf(B) are zeroed after the chunk
-                const int nrows = (fb - fa) * mB;
-                const float* ysl = Ys + sl * SLOT;
-                const float inv = 1.0f / (float)mB;
-                for (int g = uw; 16 * g < nrows; g += kNU) {
-                  int rho[2], fr[2], be[2];
-                  rho[0] = 16 * g + r8;
-                  rho[1] = rho[0] + 8;
-#pragma unroll
-                  for (int h = 0; h < 2; ++h) {   // (f - fa, beta) of row rho, exact after the correction
-                    int t = (int)((float)rho[h] * inv);
-                    if (t * mB > rho[h]) --t;
-                    else if ((t + 1) * mB <= rho[h]) ++t;
-                    fr[h] = t;
-                    be[h] = rho[h] - t * mB;
-                  }
-                  const bool v0 = rho[0] < nrows, v1 = rho[1] < nrows;
-                  // the two Y rows of this lane (16-byte chunk c stored at c ^ 2 ((beta >> 1) & 1))
-                  float y0[16], y1[16];
-  #pragma unroll
-                  for (int c4 = 0; c4 < 4; ++c4) {
-                    float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
-                    if (v0) a0 = *reinterpret_cast<const float4*>(ysl + rho[0] * 16 + 4 * (c4 ^ (2 * ((be[0] >> 1) & 1))));
-                    if (v1) a1 = *reinterpret_cast<const float4*>(ysl + rho[1] * 16 + 4 * (c4 ^ (2 * ((be[1] >> 1) & 1))));
-                    y0[4 * c4] = a0.x;
-                    y0[4 * c4 + 1] = a0.y;
-                    y0[4 * c4 + 2] = a0.z;
-                    y0[4 * c4 + 3] = a0.w;
-                    y1[4 * c4] = a1.x;
-                    y1[4 * c4 + 1] = a1.y;
-                    y1[4 * c4 + 2] = a1.z;
-                    y1[4 * c4 + 3] = a1.w;
-                  }
-                  // u[a] = sum_b y[b] D[a][b] for four a of each row
-                  float2 u0[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, u1[2] = {u0[0], u0[1]};
-  #pragma unroll
-                  for (int b = 0; b < 16; ++b)
-  #pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                      u0[j].x = fmaf(y0[b], dd[j][b].x, u0[j].x);
-                      u0[j].y = fmaf(y0[b], dd[j][b].y, u0[j].y);
-                      u1[j].x = fmaf(y1[b], dd[j][b].x, u1[j].x);
-                      u1[j].y = fmaf(y1[b], dd[j][b].y, u1[j].y);
-                    }
-                  uint2 pk[NP];
-                  if (v0) {
-                    float uf4[4] = {u0[0].x * pscale<SP>(P.sc.uf), u0[0].y * pscale<SP>(P.sc.uf), u0[1].x * pscale<SP>(P.sc.uf), u0[1].y * pscale<SP>(P.sc.uf)};
-                    split4<SP>(uf4, pk);
-                    uint16_t* ur = Us + (be[0] >> 3) * KP * 8 + (be[0] & 7) * 8 + (qa & 1) * 4 +
-                                   (2 * (fa + fr[0]) + (qa >> 1)) * 64;
-  #pragma unroll
-                    for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(ur + (size_t)pp * 64 * KP) = pk[pp];
-                  }
-                  if (v1) {
-                    float ug4[4] = {u1[0].x * pscale<SP>(P.sc.uf), u1[0].y * pscale<SP>(P.sc.uf), u1[1].x * pscale<SP>(P.sc.uf), u1[1].y * pscale<SP>(P.sc.uf)};
-                    split4<SP>(ug4, pk);
-                    uint16_t* ur = Us + (be[1] >> 3) * KP * 8 + (be[1] & 7) * 8 + (qa & 1) * 4 +
-                                   (2 * (fa + fr[1]) + (qa >> 1)) * 64;
-  #pragma unroll
-                    for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(ur + (size_t)pp * 64 * KP) = pk[pp];
-                  }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(ye + 8 * sl);   // every row of the slot has been read
-              }
-              ++ys;
-            }
-            // rows beta >= n_abf(B) (only the rows read are computed) and rows
-            // f >= nF of the chunk are zero
-            if (beta >= mB)
-              for (int f = f0; f < e; ++f)
-#pragma unroll
-                for (int pp = 0; pp < NP; ++pp)
-                  *reinterpret_cast<uint2*>(urow + (size_t)pp * 64 * KP + (2 * f + (qa >> 1)) * 64) = make_uint2(0u, 0u);
-            for (int f = max(f0, e); f < f1; ++f)
-#pragma unroll
-              for (int pp = 0; pp < NP; ++pp)
-                *reinterpret_cast<uint2*>(urow + (size_t)pp * 64 * KP + (2 * f + (qa >> 1)) * 64) = make_uint2(0u, 0u);
-            fence_async_smem();
+            tc_fence_after();
+            uint32_t v[2][16];
+            tmem_ld16(TU + tl + 32u * t.s, v[0]);
+            tmem_ld16(TU + tl + 32u * t.s + 16u, v[1]);
+            tmem_wait_ld();
+            tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(uf + 8 * c);
+            if (lane == 0) mbar_arrive(te + 8 * t.s);
+            t.next(NT);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int r = r0 + 16 * h + qd * 4 + (lane >> 3);
+              if (r >= ng) continue;
+              int g = (int)((float)r * inv);   // r / nF, exact after the correction
+              if (g * nF > r) --g;
+              else if ((g + 1) * nF <= r) ++g;
+              uint32_t w[8][NP];
+#pragma unroll
+              for (int k = 0; k < 8; ++k)
+                split2<SP>(__uint_as_float(v[h][2 * k]) * su, __uint_as_float(v[h][2 * k + 1]) * su, w[k]);
+              unsigned char* d = ubase + g * rowg + (r - g * nF) * 256;
+#pragma unroll
+              for (int pp = 0; pp < NP; ++pp) {
+                *reinterpret_cast<uint4*>(d + pp * (CB >> 1)) = make_uint4(w[0][pp], w[1][pp], w[2][pp], w[3][pp]);
+                *reinterpret_cast<uint4*>(d + pp * (CB >> 1) + 128) = make_uint4(w[4][pp], w[5][pp], w[6][pp], w[7][pp]);
+              }
+            }
           }
-          ++ub;
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(uf + 8 * ub.s);
+          ub.next(UB);
         }
       }
     }
@@ -943,7 +914,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == kWarpM) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(T), "r"(512));
+  if (warp == kWarpU) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(T), "r"(512));
   if (tid == 0 && s_abort) atomicExch(err, 1);
 }
 
@@ -970,8 +941,8 @@ __global__ void __launch_bounds__(kT2Threads, 1)
     k_t2_umma(DevPlan P, MixPlan X, const int* list, int n_list, int KKmax, long long zblk, int* err) {
   constexpr int NPROD = NP * (NP + 1) / 2;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  uint16_t* Ya = reinterpret_cast<uint16_t*>(smem_raw);   // [NP][64][KK]
-  uint16_t* Yb = Ya + (size_t)NP * 64 * KKmax;            // [NP][64][KK]
+  uint16_t* Ya = reinterpret_cast<uint16_t*>(smem_raw);   // [NP][rup8(n_abf(A))][KK]
+  uint16_t* Yb = Ya + (size_t)NP * 64 * KKmax;            // [NP][rup8(n_abf(B))][KK]
   uint16_t* Vs = Yb + (size_t)NP * 64 * KKmax;            // [NP][64][64]
   __shared__ __align__(8) uint64_t b_af, b_ae, b_bf, b_be, b_rf[2], b_re[2], b_zf, b_ze, b_done;
   __shared__ uint32_t tmem_base;
@@ -981,6 +952,11 @@ __global__ void __launch_bounds__(kT2Threads, 1)
   auto sa = [](const void* p) { return (uint32_t)__cvta_generic_to_shared(p); };
   const uint32_t mAf = sa(&b_af), mAe = sa(&b_ae), mBf = sa(&b_bf), mBe = sa(&b_be), rf = sa(b_rf), re = sa(b_re),
                  zf = sa(&b_zf), ze = sa(&b_ze), mdone = sa(&b_done);
+  // rows past n_abf are read as they lie (their results are dropped or meet
+  // zero V): the buffers start out finite
+  for (int o = tid; o < NP * (2 * 64 * KKmax + 4096) / 8; o += kT2Threads)
+    reinterpret_cast<uint4*>(smem_raw)[o] = make_uint4(0u, 0u, 0u, 0u);
+  fence_async_smem();
   if (tid == 0) {
     s_abort = 0;
     mbar_init(mAf, 1);
@@ -1020,20 +996,22 @@ __global__ void __launch_bounds__(kT2Threads, 1)
           *abort_flag = 1;
           break;
         }
-        const uint32_t ybytes = (uint32_t)NP * 64u * (uint32_t)KK * 2u;
+        // rows alpha (beta) in whole groups of 8
+        const uint32_t abytes = (uint32_t)NP * (uint32_t)((P.n_abf[P.species[A]] + 7) & ~7) * (uint32_t)KK * 2u;
+        const uint32_t bbytes = (uint32_t)NP * (uint32_t)((P.n_abf[P.species[b]] + 7) & ~7) * (uint32_t)KK * 2u;
         if (na >= 1 && !mbar_wait(mAe, (na - 1) & 1)) {
           *abort_flag = 1;
           break;
         }
-        mbar_expect_tx(mAf, ybytes);
-        bulk_g2s(sa(Ya), X.YspT + X.y_idx[y1] * X.yT_blk, ybytes, mAf);
+        mbar_expect_tx(mAf, abytes);
+        bulk_g2s(sa(Ya), X.YspT + X.y_idx[y1] * X.yT_blk, abytes, mAf);
         ++na;
         if (nb >= 1 && !mbar_wait(mBe, (nb - 1) & 1)) {
           *abort_flag = 1;
           break;
         }
-        mbar_expect_tx(mBf, ybytes + (uint32_t)NP * 8192u);
-        bulk_g2s(sa(Yb), X.Ysp + P.y_off[y2], ybytes, mBf);
+        mbar_expect_tx(mBf, bbytes + (uint32_t)NP * 8192u);
+        bulk_g2s(sa(Yb), X.Ysp + P.y_off[y2], bbytes, mBf);
         bulk_g2s(sa(Vs), X.Vz + (long long)kk * X.vz_blk, (uint32_t)NP * 8192u, mBf);
         ++nb;
       }
@@ -1052,9 +1030,11 @@ __global__ void __launch_bounds__(kT2Threads, 1)
           ok = false;
           break;
         }
-        const int nA = P.n_ao[P.species[P.v_home[list[kk]]]];
+        const int pr = list[kk], sA = P.species[P.v_home[pr]], mB = P.n_abf[P.species[P.v_j[pr]]];
+        const int nA = P.n_ao[sA];
         const int KK = 16 * nA;
-        const uint32_t PB = 64u * (uint32_t)KK * 2u;   // bytes of one piece of Y^{AB} or Y^{BA}
+        const uint32_t PA = (uint32_t)((P.n_abf[sA] + 7) & ~7) * (uint32_t)KK * 2u;   // bytes of one piece of Y^{AB}
+        const uint32_t PB = (uint32_t)((mB + 7) & ~7) * (uint32_t)KK * 2u;            // and of Y^{BA}
         const uint32_t rowg = 16u * (uint32_t)KK;      // bytes between 8-row groups
         const uint64_t dA = sdesc2(sa(Ya), 128, rowg), dBK = sdesc2(sa(Yb), 128, rowg);
         const uint64_t dV = sdesc2(sa(Vs), 128, 1024), dBM = sdesc2(sa(Yb), rowg, 128);
@@ -1072,7 +1052,7 @@ __global__ void __launch_bounds__(kT2Threads, 1)
           for (int sum = NP - 1; sum >= 0; --sum)
 #pragma unroll
             for (int ia = 0; ia <= sum; ++ia, ++k)
-              umma_f16(tR, dA + ((uint64_t)(ia * PB) >> 4) + o, dBK + ((uint64_t)((sum - ia) * PB) >> 4) + o, idR,
+              umma_f16(tR, dA + ((uint64_t)(ia * PA) >> 4) + o, dBK + ((uint64_t)((sum - ia) * PB) >> 4) + o, idR,
                         (a > 0 || k > 0) ? 1u : 0u);
         }
         umma_commit(mAe);
@@ -1080,8 +1060,8 @@ __global__ void __launch_bounds__(kT2Threads, 1)
         ok = i < 1 || mbar_wait(ze, (i - 1) & 1);
         if (!ok) break;
         tc_fence_after();
-        // Z: K = beta in four steps of 16 (V: 256 bytes; Y^{BA} MN-major: two 8-row groups)
-        for (int kb = 0; kb < 4; ++kb) {
+        // Z: K = beta in steps of 16 (V: 256 bytes; Y^{BA} MN-major: two 8-row groups)
+        for (int kb = 0; 16 * kb < mB; ++kb) {
           int k = 0;
 #pragma unroll
           for (int sum = NP - 1; sum >= 0; --sum)
@@ -1241,34 +1221,27 @@ int num_sms() {
 
 long long t1u_launch_count() { return g_t1u_launches; }
 
-size_t t1u_smem(int pieces, int KP, int NS, int FS) {
-  return (size_t)pieces * 64 * KP * 2 * 2 + (size_t)pieces * 8192 + 2 * 256 * 4 + (size_t)NS * FS * 1024 * 4;
-}
+size_t t1u_smem(int KP, int G, int UB, int NS) { return t1_base(KP, G, UB) + (size_t)NS * kYSlot; }
 
 int t1u_max_slots() { return kMaxNS; }
+
+int sm_count() { return num_sms(); }
 
 cudaError_t t1u_set_smem(int sp) {
   return allow_max_dynamic_smem(sp == kSplitBf16 ? (const void*)k_t1_umma<kSplitBf16> : (const void*)k_t1_umma<kSplitHalf>);
 }
 
-cudaError_t launch_t1u_stores(const DevPlan& P, const T1UPlan& U, int sp, const int* qlist, int nq, bool dstore,
-                              cudaStream_t s) {
-  if (nq > 0) {
-    ++g_t1u_launches;
-    static std::once_flag attr;
-    std::call_once(attr, [] {
-      cudaFuncSetAttribute(k_t1u_cstore<kSplitBf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCStoreSmem);
-      cudaFuncSetAttribute(k_t1u_cstore<kSplitHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCStoreSmem);
-    });
-    const int g = nq < 152 * 3 ? nq : 152 * 3;
-    if (sp == kSplitBf16) k_t1u_cstore<kSplitBf16><<<g, 256, kCStoreSmem, s>>>(P, U, qlist, nq);
-    else k_t1u_cstore<kSplitHalf><<<g, 256, kCStoreSmem, s>>>(P, U, qlist, nq);
-  }
-  if (dstore && P.n_d > 0) {
-    ++g_t1u_launches;
-    const long long g = P.n_d < 152 * 16 ? P.n_d : 152 * 16;
-    k_t1u_dstore<<<(unsigned)g, 256, 0, s>>>(P, U.Df);
-  }
+cudaError_t launch_t1u_cstore(const DevPlan& P, const T1UPlan& U, int sp, const int* qlist, int nq, cudaStream_t s) {
+  if (nq <= 0) return cudaSuccess;
+  ++g_t1u_launches;
+  static std::once_flag attr;
+  std::call_once(attr, [] {
+    cudaFuncSetAttribute(k_t1u_cstore<kSplitBf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCStoreSmem);
+    cudaFuncSetAttribute(k_t1u_cstore<kSplitHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCStoreSmem);
+  });
+  const int g = nq < 152 * 3 ? nq : 152 * 3;
+  if (sp == kSplitBf16) k_t1u_cstore<kSplitBf16><<<g, 256, kCStoreSmem, s>>>(P, U, qlist, nq);
+  else k_t1u_cstore<kSplitHalf><<<g, 256, kCStoreSmem, s>>>(P, U, qlist, nq);
   return cudaGetLastError();
 }
 
@@ -1321,7 +1294,7 @@ cudaError_t launch_t1_umma(const DevPlan& P, const MixPlan& X, const T1UPlan& U,
                            size_t smem, int* work, int* err, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   ++g_t1u_launches;
-  const int grid = n < num_sms() ? n : num_sms();
+  const int grid = std::min(n * U.nsplit, num_sms());
   cudaError_t e = cudaMemsetAsync(work, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   if (sp == kSplitBf16) k_t1_umma<kSplitBf16><<<grid, kThreads, smem, s>>>(P, X, U, qlist, n, work, err);
