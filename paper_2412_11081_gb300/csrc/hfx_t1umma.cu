@@ -23,7 +23,9 @@
 // traffic, 105 KB of L2 reads.  The kernel before built U in FP32 on the CUDA
 // cores, two warps per scheduler with 64 registers of D each: 12,900 cycles
 // per triplet, most of them the latency of its shared-memory loads and FMA
-// chains.
+// chains; this one takes 5,100 (64-atom Si cell 36.7 -> 13.5 ms, 8 atoms 7.0 ->
+// 1.6 ms), the hand-offs between its roles and the fetch latency of Y, one
+// triplet ahead, being what is left.
 //
 // Column order (f,a) = 16 f + a with a padded to 16.  All matrices sit in
 // shared memory in the no-swizzle core-matrix order (8 rows x 16 bytes); U
@@ -349,7 +351,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t b_yf[kMaxNS], b_ye[kMaxNS], b_cf, b_ce, b_vf[2], b_ve[2], b_df[kND], b_de[kND],
       b_tf[kMaxUT], b_te[kMaxUT], b_uf[2], b_ue[2], b_rf, b_re, b_qf, b_qe, b_if[kItemRing], b_ie[kItemRing], b_done[2];
-  __shared__ int s_item[kItemRing];
+  __shared__ int4 s_item[kItemRing];   // a unit: item kk (-1: no more), C pair q, its B [lo, hi) of the list at X.qoff
   __shared__ uint32_t tmem_base;
   __shared__ int s_abort;
   volatile int* abort_flag = &s_abort;
@@ -408,40 +410,30 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t T = tmem_base, TR = T + t1_rcol(KP), TU = TR + 16u * G;
   // Next unit of the ring for a role (one reader per warp; lane 0 releases
-  // the slot).  n_units marks the end.  Every lane of the warp calls it.
-  auto next_unit = [&](uint32_t& k) -> int {
-    const int s = k & (kItemRing - 1);
-    int u = n_units;
-    if (wait_all(itf + 8 * s, (k / kItemRing) & 1)) u = *reinterpret_cast<volatile int*>(&s_item[s]);
-    else *abort_flag = 1;
-    __syncwarp();
-    if (lane == 0) mbar_arrive(ite + 8 * s);
-    ++k;
-    return u;
-  };
-  // Unit u: item kk = u / nsplit, its kept B [lo, hi) of the list at X.qoff.
+  // the slot); kk < 0 marks the end.  Every lane of the warp calls it.
   struct Unit {
     int kk, q, lo, hi;
   };
-  auto unit = [&](int u) -> Unit {
-    Unit r;
-    r.kk = u / nsplit;
-    const int s = u - r.kk * nsplit;
-    r.q = qlist[r.kk];
-    const long long n = X.qcnt[r.q];
-    r.lo = (int)(n * s / nsplit);
-    r.hi = (int)(n * (s + 1) / nsplit);
-    return r;
+  auto next_unit = [&](Ring& r) -> Unit {
+    Unit u{-1, 0, 0, 0};
+    if (wait_all(itf + 8 * r.s, r.ph)) {
+      const volatile int* v = reinterpret_cast<const volatile int*>(&s_item[r.s]);
+      u = Unit{v[0], v[1], v[2], v[3]};
+    } else {
+      *abort_flag = 1;
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(ite + 8 * r.s);
+    r.next(kItemRing);
+    return u;
   };
 
   if (warp == kWarpY) {
     // ---------------------------------------------------------- Y producer
     // Y^{BF} as [piece][(g, f)][8 beta x 16 b]: up to 32 row groups (g, f) per
     // slot, the two pieces copied by lanes 0 and 1.
-    uint32_t ik = 0;
-    Ring y;
-    for (int u = next_unit(ik); u < n_units && !aborted(abort_flag); u = next_unit(ik)) {
-      const Unit it = unit(u);
+    Ring ik, y;
+    for (Unit it = next_unit(ik); it.kk >= 0 && !aborted(abort_flag); it = next_unit(ik)) {
       const int F = P.c_j[it.q];
       const int nF = P.n_ao[P.species[F]];
       const int* Rf = P.c_R + 3 * it.q;
@@ -487,44 +479,54 @@ __global__ void __launch_bounds__(kThreads, 1)
     // -------------------------------------- scheduler, C, D and V producer
     // Lane 0 publishes units two ahead of this warp's own position (a slot
     // is reused once every reader has taken its unit).
-    uint32_t pub = 0;
+    Ring pub;
     bool pub_done = false;
     auto publish = [&]() {
-      const int s = pub & (kItemRing - 1);
-      if (pub >= kItemRing && !mbar_wait(ite + 8 * s, ((pub / kItemRing) - 1) & 1)) {
+      volatile int* v = reinterpret_cast<volatile int*>(&s_item[pub.s]);
+      v[0] = -1;   // best effort on a timeout: readers also stop on the flag
+      if (!mbar_wait(ite + 8 * pub.s, pub.ph ^ 1)) {
         *abort_flag = 1;
-        s_item[s] = n_units;   // best effort: readers also stop on the flag
         pub_done = true;
         return;
       }
-      int u = n_units;
+      pub_done = true;
       while (!aborted(abort_flag)) {   // units without a B (fewer B than parts) are passed over
-        u = atomicAdd(work, 1);
+        const int u = atomicAdd(work, 1);
         if (u >= n_units) break;
-        const Unit it = unit(u);
-        if (it.hi > it.lo) break;
+        const int kk = u / nsplit, part = u - kk * nsplit, q = qlist[kk], n = X.qcnt[q];
+        const int lo = n * part / nsplit, hi = n * (part + 1) / nsplit;
+        if (hi <= lo) continue;
+        v[1] = q;
+        v[2] = lo;
+        v[3] = hi;
+        v[0] = kk;
+        pub_done = false;
+        break;
       }
-      if (u > n_units) u = n_units;
-      s_item[s] = u;
-      mbar_arrive(itf + 8 * s);
-      ++pub;
-      if (u >= n_units) pub_done = true;
+      mbar_arrive(itf + 8 * pub.s);
+      pub.next(kItemRing);
     };
     if (lane == 0) {
       publish();
       if (!pub_done) publish();
     }
     __syncwarp();
-    uint32_t it_n = 0, ca = 0, own = 0;
-    Ring v, d;
-    auto own_unit = [&]() -> int {
-      int u = n_units;
-      if (lane == 0 && own < pub) u = *reinterpret_cast<volatile int*>(&s_item[own & (kItemRing - 1)]);
-      ++own;
-      return __shfl_sync(0xffffffffu, u, 0);
+    uint32_t it_n = 0, ca = 0;
+    Ring own, v, d;
+    auto own_unit = [&]() -> Unit {
+      Unit u{-1, 0, 0, 0};
+      if (lane == 0 && own.n < pub.n) {
+        const volatile int* w = reinterpret_cast<const volatile int*>(&s_item[own.s]);
+        u = Unit{w[0], w[1], w[2], w[3]};
+      }
+      own.next(kItemRing);
+      u.kk = __shfl_sync(0xffffffffu, u.kk, 0);
+      u.q = __shfl_sync(0xffffffffu, u.q, 0);
+      u.lo = __shfl_sync(0xffffffffu, u.lo, 0);
+      u.hi = __shfl_sync(0xffffffffu, u.hi, 0);
+      return u;
     };
-    for (int u = own_unit(); u < n_units && !aborted(abort_flag); u = own_unit(), ++it_n) {
-      const Unit it = unit(u);
+    for (Unit it = own_unit(); it.kk >= 0 && !aborted(abort_flag); it = own_unit(), ++it_n) {
       const long long b0 = X.qoff[it.q];
       const uint32_t gA = (uint32_t)(P.n_abf[P.species[P.c_home[it.q]]] + 7) >> 3;
       if (lane == 0) {
@@ -582,11 +584,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     // products of a slot's two tiles alternate: an instruction waits for the
     // one before on the same accumulator (72 cycles each in one chain).
     const uint32_t idU = idesc_split<kSplitHalf>(128, 16, 0);
-    uint32_t ik = 0;
-    Ring y, t, d;
+    Ring ik, y, t, d;
     bool ok = true;
-    for (int u = next_unit(ik); u < n_units; u = next_unit(ik)) {
-      const Unit it = unit(u);
+    for (Unit it = next_unit(ik); it.kk >= 0; it = next_unit(ik)) {
       const int nF = P.n_ao[P.species[P.c_j[it.q]]];
       const long long b0 = X.qoff[it.q];
       for (int i0 = it.lo; i0 < it.hi; i0 += 32) {
@@ -641,11 +641,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t idR = idesc_split<SP>(128, 16 * G, 0);
     const uint64_t dC = sdesc2(Cs, 128, rowg);
     const uint64_t kbB = (uint64_t)(2 * rowg) >> 4, pB = (uint64_t)(CB >> 1) >> 4;
-    uint32_t rp = 1, qp = 1, it_n = 0, ik = 0;   // phases of the free accumulators
-    Ring ub, v;
+    uint32_t rp = 1, qp = 1, it_n = 0;   // phases of the free accumulators
+    Ring ik, ub, v;
     bool ok = true;
-    for (int u = next_unit(ik); u < n_units; u = next_unit(ik), ++it_n) {
-      const Unit it = unit(u);
+    for (Unit it = next_unit(ik); it.kk >= 0; it = next_unit(ik), ++it_n) {
       const int nF = P.n_ao[P.species[P.c_j[it.q]]];
       const uint32_t idQ = idesc_split<SP>(128, 16 * nF, 1);
       const long long b0 = X.qoff[it.q];
@@ -726,11 +725,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     };
-    uint32_t rb = 0, seg = 0, ik = 0;
+    uint32_t rb = 0, seg = 0;
+    Ring ik;
     unsigned long long fl = 0;
     bool ok = true;
-    for (int u = next_unit(ik); u < n_units && ok; u = next_unit(ik)) {
-      const Unit it = unit(u);
+    for (Unit it = next_unit(ik); it.kk >= 0 && ok; it = next_unit(ik)) {
       const int A = P.c_home[it.q], F = P.c_j[it.q];
       const int sA = P.species[A];
       const int nA = P.n_ao[sA], mA = P.n_abf[sA], nF = P.n_ao[P.species[F]];
@@ -852,11 +851,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int qd = warp & 3;
     const uint32_t tl = (uint32_t)(qd * 32) << 16;
     const float su = P.sc.u1;
-    uint32_t ik = 0;
-    Ring ub, t;
+    Ring ik, ub, t;
     bool ok = true;
-    for (int u = next_unit(ik); u < n_units && ok; u = next_unit(ik)) {
-      const Unit it = unit(u);
+    for (Unit it = next_unit(ik); it.kk >= 0 && ok; it = next_unit(ik)) {
       const int nF = P.n_ao[P.species[P.c_j[it.q]]];
       const float inv = 1.0f / (float)nF;
       const long long b0 = X.qoff[it.q];
