@@ -181,6 +181,7 @@ struct hfx_plan {
 
   // kernel shapes
   int beta_chunk = 1, alpha_chunk = 1;
+  int small = 0;               // FP64 kernels: 64-thread CTAs
   size_t smem_t1 = 0, smem_t2 = 0;
 
   // split-precision path (np = pieces per operand; 0 = FP64 path)
@@ -515,6 +516,12 @@ DevPlan make_devplan(hfx_plan* P, const double* lattice) {
   D.thD = P->opt.theta_D;
   D.thCS = P->opt.theta_CS;
   D.sc = P->scale;
+  D.small = P->small;
+  // by the V pairs of the whole structure, so that neither the passes nor the
+  // home atoms of a plan change what is summed together (about one kept pair
+  // per four of them; eight waves of 152 SMs x 3 CTAs)
+  D.parts = P->nV < 10000 ? 4 : P->nV < 40000 ? 2 : 1;
+  D.parts2 = P->small ? 1 : D.parts;   // (small blocks: the repeated sums over F cost more than the last wave)
   D.terms = P->opt.terms;
   D.h0 = P->chunks.empty() ? 0 : P->chunks.front().first;
   D.h1 = P->chunks.empty() ? P->N : P->chunks.back().second;
@@ -1000,14 +1007,26 @@ void setup_shapes(hfx_plan* P) {
     maxAO = std::max(maxAO, P->n_ao[t]);
     maxABF = std::max(maxABF, P->n_abf[t]);
   }
-  const size_t base1 = (size_t)(hfx::kMaxAO * hfx::kMaxAO + maxABF * maxABF) * sizeof(double);
+  // FP64 kernels.  U (first product): the whole block where that leaves room
+  // for three or two CTAs per SM, else as many rows as fit one.  Z (second
+  // product): 8 rows at least, for up to three CTAs per SM.
+  const size_t base1 = (size_t)(maxAO * maxAO + maxABF * maxABF) * sizeof(double);
+  const size_t base2 = (size_t)(3 * hfx::kMaxCPerAtom) * sizeof(double);
   const size_t per1 = (size_t)maxAO * maxAO * sizeof(double);
-  if (base1 + per1 > limit) fail(HFX_ERR_UNSUPPORTED, "block shapes exceed shared memory");
-  P->beta_chunk = (int)std::min<size_t>(maxABF, (limit - base1) / per1);
+  if ((size_t)(hfx::kMaxAO * hfx::kMaxAO + maxABF * maxABF) * sizeof(double) + per1 > limit)
+    fail(HFX_ERR_UNSUPPORTED, "block shapes exceed shared memory");
+  auto chunk = [&](size_t base, int least) {
+    for (int ctas = 3; ctas > 1; --ctas) {
+      const size_t room = limit / ctas - 1024;   // (each CTA's reserved kilobyte)
+      if (base + least * per1 <= room) return (int)std::min<size_t>(maxABF, (room - base) / per1);
+    }
+    return (int)std::min<size_t>(maxABF, (limit - base) / per1);
+  };
+  P->beta_chunk = chunk(base1, maxABF);
   P->smem_t1 = base1 + per1 * P->beta_chunk;
-  const size_t base2 = (size_t)(3 * hfx::kMaxCPerAtom + hfx::kMaxAO * hfx::kMaxAO) * sizeof(double);
-  P->alpha_chunk = (int)std::min<size_t>(maxABF, (limit - base2) / per1);
+  P->alpha_chunk = chunk(base2, std::min(8, maxABF));
   P->smem_t2 = base2 + per1 * P->alpha_chunk;
+  P->small = maxABF * maxAO * maxAO <= 1024 ? 1 : 0;
   ck(hfx::set_kernel_smem_limits(), "smem attributes");
   if (P->np && maxAO > 16) {
     // n_ao beyond the 16-column tiles of the tensor-memory kernels: the wide kernels

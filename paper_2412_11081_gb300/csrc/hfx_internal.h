@@ -61,6 +61,8 @@ struct DevPlan {
   double RC, omega;
   double thC, thdC, thV, thdV, thD, thCS;
   SplitScale sc;
+  int small;                   // FP64 path: blocks of at most 1024 elements of C, 64-thread CTAs
+  int parts, parts2;           // FP64 path: CTAs per Y block and pair of the first product, per pair of the second
   int terms;
   int h0, h1;                  // home atoms A whose items are screened in: [h0, h1)
 

@@ -328,9 +328,12 @@ __global__ void k_vblocks(DevPlan P, const int* list, int n_list) {
 // ---------------------------------------------------------------- K3: Y
 // One CTA per needed key (X; Z): Y[alpha,x,z] = sum_{W kept} sum_w
 // C_XW[alpha,x,w] D_WZ[w,z], D_WZ = D(w, z, R_Z - R_W) when kept.
+// A CTA takes one of P.parts ranges of the key's elements: with whole keys the
+// last wave of a small cell left most SMs idle (5-atom perovskite 17.1 ms, 13.8 now: 1.0 TFLOP/s).
 __global__ void k_ybuild(DevPlan P, const int* list, int n_list) {
   __shared__ int dsel[kMaxCPerAtom];
-  for (int k = blockIdx.x; k < n_list; k += gridDim.x) {
+  for (int u = blockIdx.x; u < n_list * P.parts; u += gridDim.x) {
+    const int k = u / P.parts, part = u - k * P.parts;
     const int y = list[k];
     const int X = P.y_home[y], z = P.y_j[y];
     const int* Rz = P.y_R + 3 * y;
@@ -353,7 +356,8 @@ __global__ void k_ybuild(DevPlan P, const int* list, int n_list) {
     const int n = rows * nZ;
     double* Y = P.Yst + P.y_off[y];
     double fl = 0.0;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    const int e1 = (int)((long long)n * (part + 1) / P.parts);
+    for (int e = (int)((long long)n * part / P.parts) + threadIdx.x; e < e1; e += blockDim.x) {
       const int row = e / nZ, col = e - row * nZ;
       double acc = 0.0;
       for (int t = 0; t < nq; ++t) {
@@ -368,37 +372,52 @@ __global__ void k_ybuild(DevPlan P, const int* list, int n_list) {
       }
       Y[e] = acc;
     }
-    if (threadIdx.x == 0) atomicAdd(&P.acc[ACC_FY], fl);
+    if (threadIdx.x == 0 && fl != 0.0) atomicAdd(&P.acc[ACC_FY], fl);
   }
 }
 
 // ---------------------------------------------------------------- K4: term 1
 // One CTA per (A,B) pair with kept F.  Shared memory: D_AB, R_AB, and a
 // beta-chunk of U (bc x n_ao(A) x n_ao(F)).
+//
+// The FP64 pipe bounds it (1.1 TFLOP/s on the whole chip).  Each warp adds its
+// own part of a gradient to the pair's sum, so the only block barriers are
+// the two around a chunk of U.  A chunk is all of U where that leaves room for
+// two or three CTAs per SM (they fill each other's barriers), else as much as
+// fits: every chunk repeats the three products with grad C.  Small blocks take
+// 64 threads per CTA, and small cells divide a pair's F over P.parts CTAs, so
+// that the last wave is short.  With block sums per F, 256 threads and whole
+// pairs: 1.31 ms on the 8-atom minimal cell (0.58 now) and 47.1 ms on the
+// 5-atom perovskite (45.6 now, 0.91 TFLOP/s).
 __global__ void k_term1(DevPlan P, const int* list, int n_list, int BC) {
   extern __shared__ double sm[];
-  __shared__ double red[kThreads / 32];
-  for (int k = blockIdx.x; k < n_list; k += gridDim.x) {
-    const int p = list[k];
+  const int lane = threadIdx.x & 31;
+  for (int u = blockIdx.x; u < n_list * P.parts; u += gridDim.x) {
+    const int part = u % P.parts, p = list[u / P.parts];
     const int A = P.v_home[p], b = P.v_j[p];
     const int* Rb = P.v_R + 3 * p;
     const int sA = P.species[A], sB = P.species[b];
     const int nA = P.n_ao[sA], nB = P.n_ao[sB], mA = P.n_abf[sA], mB = P.n_abf[sB];
     double* Dab = sm;                      // nA*nB
-    double* Rs = Dab + kMaxAO * kMaxAO;    // mA*mB
+    double* Rs = Dab + nA * nB;            // mA*mB
     double* Uc = Rs + mA * mB;             // BC*nA*nF
     const double* Dg = P.Dval + P.Doff[P.v_didx[p]];
+    const double* V = P.Vst + P.v_off[p];  // [alpha][beta]
     __syncthreads();
     for (int t = threadIdx.x; t < nA * nB; t += blockDim.x) Dab[t] = Dg[t];
     for (int t = threadIdx.x; t < mA * mB; t += blockDim.x) Rs[t] = 0.0;
     __syncthreads();
     const int q0 = P.c_ptr[A];
     double fl = 0.0;
+    int turn = 0;   // this part's F: every P.parts-th kept one
     for (int w = 0; w < kMaskWords; ++w) {
       unsigned bits = P.v_mask[(size_t)p * kMaskWords + w];
       while (bits) {
         const int s = __ffs(bits) - 1;
         bits &= bits - 1u;
+        const bool mine = turn == part;
+        if (++turn == P.parts) turn = 0;
+        if (!mine) continue;
         const int q = q0 + w * 32 + s;
         const int f = P.c_j[q];
         const int* Rf = P.c_R + 3 * q;
@@ -407,7 +426,6 @@ __global__ void k_term1(DevPlan P, const int* list, int n_list, int BC) {
         const double* Y = P.Yst + P.y_off[yc];          // [beta][b][f]
         const double* C = P.Cst + P.c_off[q];           // [alpha][a][f]
         const double* dC = P.dCst + 3 * P.c_off[q];
-        const double* V = P.Vst + P.v_off[p];           // [alpha][beta]
         const int naf = nA * nF;
         const int nc = mA * naf;
         double g0 = 0.0, g1 = 0.0, g2 = 0.0;
@@ -445,20 +463,18 @@ __global__ void k_term1(DevPlan P, const int* list, int n_list, int BC) {
           }
           __syncthreads();
         }
-        g0 = block_sum(g0, red);
-        g1 = block_sum(g1, red);
-        g2 = block_sum(g2, red);
-        if (threadIdx.x == 0) {
-          dev::add_gC(P, 3 * q + 0, -2.0 * g0);
-          dev::add_gC(P, 3 * q + 1, -2.0 * g1);
-          dev::add_gC(P, 3 * q + 2, -2.0 * g2);
-          fl += 2.0 * mB * nA * nB * nF + 4.0 * mA * mB * nA * nF;
+        g0 = warp_sum(g0);
+        g1 = warp_sum(g1);
+        g2 = warp_sum(g2);
+        if (lane == 0) {
+          if (g0 != 0.0) dev::add_gC(P, 3 * q + 0, -2.0 * g0);
+          if (g1 != 0.0) dev::add_gC(P, 3 * q + 1, -2.0 * g1);
+          if (g2 != 0.0) dev::add_gC(P, 3 * q + 2, -2.0 * g2);
         }
+        if (threadIdx.x == 0) fl += 2.0 * mB * nA * nB * nF + 4.0 * mA * mB * nA * nF;
       }
     }
-    __syncthreads();
-    // E += -<V_AB, R>,  g^V += -<grad V_AB, R>
-    const double* V = P.Vst + P.v_off[p];
+    // E += -<V_AB, R>,  g^V += -<grad V_AB, R> (the last chunk's barrier orders R)
     const int n = mA * mB;
     double e0 = 0.0, h0 = 0.0, h1 = 0.0, h2 = 0.0;
     for (int t = threadIdx.x; t < n; t += blockDim.x) {
@@ -468,32 +484,38 @@ __global__ void k_term1(DevPlan P, const int* list, int n_list, int BC) {
       h1 += V[2 * n + t] * r;
       h2 += V[3 * n + t] * r;
     }
-    e0 = block_sum(e0, red);
-    h0 = block_sum(h0, red);
-    h1 = block_sum(h1, red);
-    h2 = block_sum(h2, red);
-    if (threadIdx.x == 0) {
-      dev::add_E(P, -e0);
-      dev::add_gV(P, 3 * p + 0, -h0);
-      dev::add_gV(P, 3 * p + 1, -h1);
-      dev::add_gV(P, 3 * p + 2, -h2);
-      atomicAdd(&P.acc[ACC_F1], fl);
+    e0 = warp_sum(e0);
+    h0 = warp_sum(h0);
+    h1 = warp_sum(h1);
+    h2 = warp_sum(h2);
+    if (lane == 0) {
+      if (e0 != 0.0) dev::add_E(P, -e0);
+      if (h0 != 0.0) dev::add_gV(P, 3 * p + 0, -h0);
+      if (h1 != 0.0) dev::add_gV(P, 3 * p + 1, -h1);
+      if (h2 != 0.0) dev::add_gV(P, 3 * p + 2, -h2);
     }
+    if (threadIdx.x == 0) atomicAdd(&P.acc[ACC_F1], fl);
   }
 }
 
 // ---------------------------------------------------------------- K5: term 2
-// One CTA per (A,B) pair of the second exchange product.  Shared memory:
-// an alpha-chunk of Z (ac x n_ao(A) x n_ao(B)) and per-F gradient partials.
+// One CTA per (A,B) pair of the second exchange product and one of P.parts2
+// ranges of alpha.  Shared memory: per-F gradient partials and an alpha-chunk
+// of Z (ac x n_ao(A) x n_ao(B)).  Q2 takes one F per warp at a time (D_FB
+// straight from L1: a few KB), with no block barrier but the two around a
+// chunk of Z.  With one F per block, block sums and whole pairs: 1.99 ms on
+// the 8-atom minimal cell (0.35 now), 24.9 ms on the 5-atom perovskite (22.2
+// now).
 __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
   extern __shared__ double sm[];
-  __shared__ double red[kThreads / 32];
-  for (int k = blockIdx.x; k < n_list; k += gridDim.x) {
-    const int p = list[k];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  for (int u = blockIdx.x; u < n_list * P.parts2; u += gridDim.x) {
+    const int part = u % P.parts2, p = list[u / P.parts2];
     const int A = P.v_home[p], b = P.v_j[p];
     const int* Rb = P.v_R + 3 * p;
     const int sA = P.species[A], sB = P.species[b];
     const int nA = P.n_ao[sA], nB = P.n_ao[sB], mA = P.n_abf[sA], mB = P.n_abf[sB];
+    const int m0 = mA * part / P.parts2, m1 = mA * (part + 1) / P.parts2;   // this CTA's rows alpha
     const int y1 = ylut_get(P, A, b, Rb[0], Rb[1], Rb[2]);
     const int y2 = ylut_get(P, b, A, -Rb[0], -Rb[1], -Rb[2]);
     const double* Yab = P.Yst + P.y_off[y1];   // [alpha][a][b]
@@ -503,7 +525,7 @@ __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
     const int nab = nA * nB;
     // R2[alpha][beta] = sum_{a,b} Yab[alpha][a][b] Yba[beta][b][a], dotted at once
     double e0 = 0.0, h0 = 0.0, h1 = 0.0, h2 = 0.0;
-    for (int t = threadIdx.x; t < nvb; t += blockDim.x) {
+    for (int t = m0 * mB + threadIdx.x; t < m1 * mB; t += blockDim.x) {
       const int al = t / mB, be = t - al * mB;
       const double* Ya = Yab + (long long)al * nab;
       const double* Yb = Yba + (long long)be * nab;
@@ -515,25 +537,24 @@ __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
       h1 += V[2 * nvb + t] * s2;
       h2 += V[3 * nvb + t] * s2;
     }
-    e0 = block_sum(e0, red);
-    h0 = block_sum(h0, red);
-    h1 = block_sum(h1, red);
-    h2 = block_sum(h2, red);
-    if (threadIdx.x == 0) {
-      dev::add_E(P, -e0);
-      dev::add_gV(P, 3 * p + 0, -h0);
-      dev::add_gV(P, 3 * p + 1, -h1);
-      dev::add_gV(P, 3 * p + 2, -h2);
+    e0 = warp_sum(e0);
+    h0 = warp_sum(h0);
+    h1 = warp_sum(h1);
+    h2 = warp_sum(h2);
+    if (lane == 0) {
+      if (e0 != 0.0) dev::add_E(P, -e0);
+      if (h0 != 0.0) dev::add_gV(P, 3 * p + 0, -h0);
+      if (h1 != 0.0) dev::add_gV(P, 3 * p + 1, -h1);
+      if (h2 != 0.0) dev::add_gV(P, 3 * p + 2, -h2);
     }
     const int q0 = P.c_ptr[A], nq = P.c_ptr[A + 1] - q0;
-    double* Zc = sm;                         // AC*nA*nB
-    double* gF = Zc + (size_t)AC * nab;      // nq*3
-    double* Ds = gF + 3 * kMaxCPerAtom;      // nF*nB (one D_FB at a time)
-    __syncthreads();
-    for (int t = threadIdx.x; t < 3 * nq; t += blockDim.x) gF[t] = 0.0;
-    double fl = 4.0 * mA * mB * nA * nB;
-    for (int a0 = 0; a0 < mA; a0 += AC) {
-      const int ac = min(AC, mA - a0);
+    double* gF = sm;                        // nq*3, each F's by the warp that takes it
+    double* Zc = gF + 3 * kMaxCPerAtom;     // AC*nA*nB
+    for (int t = warp; t < nq; t += nwarp)
+      if (lane < 3) gF[3 * t + lane] = 0.0;
+    double fl = threadIdx.x == 0 ? 4.0 * (m1 - m0) * mB * nA * nB : 0.0;
+    for (int a0 = m0; a0 < m1; a0 += AC) {
+      const int ac = min(AC, m1 - a0);
       __syncthreads();
       // Z[al][a][b] = sum_beta V[a0+al][beta] Yba[beta][b][a]
       for (int e = threadIdx.x; e < ac * nab; e += blockDim.x) {
@@ -545,7 +566,7 @@ __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
         Zc[e] = s2;
       }
       __syncthreads();
-      for (int t = 0; t < nq; ++t) {
+      for (int t = warp; t < nq; t += nwarp) {
         const int q = q0 + t;
         if (!P.c_keep[q]) continue;
         const int f = P.c_j[q];
@@ -554,18 +575,16 @@ __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
         if (di < 0 || P.Dkept[di] == 0.0) continue;
         const int nF = P.n_ao[P.species[f]];
         const double* Dfb = P.Dval + P.Doff[di];   // [f][b]
-        for (int e = threadIdx.x; e < nF * nB; e += blockDim.x) Ds[e] = Dfb[e];
-        __syncthreads();
         const double* dC = P.dCst + 3 * P.c_off[q];
         const int naf = nA * nF;
         const int nc = mA * naf;
         double g0 = 0.0, g1 = 0.0, g2 = 0.0;
         // Q2[a0+al][a][f] = sum_b Z[al][a][b] D_FB[f][b]
-        for (int e = threadIdx.x; e < ac * naf; e += blockDim.x) {
+        for (int e = lane; e < ac * naf; e += 32) {
           const int al = e / naf, af = e - al * naf;
           const int a = af / nF, ff = af - a * nF;
           const double* Zr = Zc + (long long)al * nab + a * nB;
-          const double* Dr = Ds + ff * nB;
+          const double* Dr = Dfb + ff * nB;
           double s2 = 0.0;
           for (int bb = 0; bb < nB; ++bb) s2 += Zr[bb] * Dr[bb];
           const long long ci = (long long)(a0 + al) * naf + af;
@@ -573,28 +592,21 @@ __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
           g1 += dC[nc + ci] * s2;
           g2 += dC[2 * nc + ci] * s2;
         }
-        g0 = block_sum(g0, red);
-        g1 = block_sum(g1, red);
-        g2 = block_sum(g2, red);
-        if (threadIdx.x == 0) {
+        g0 = warp_sum(g0);
+        g1 = warp_sum(g1);
+        g2 = warp_sum(g2);
+        if (lane == 0) {
           gF[3 * t + 0] += g0;
           gF[3 * t + 1] += g1;
           gF[3 * t + 2] += g2;
-          if (a0 == 0) fl += 2.0 * mA * nA * nB * nF;
+          fl += 2.0 * ac * nA * nB * nF;
         }
-        __syncthreads();
       }
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nq; t += blockDim.x) {
-      if (gF[3 * t] != 0.0 || gF[3 * t + 1] != 0.0 || gF[3 * t + 2] != 0.0) {
-        const int q = q0 + t;
-        dev::add_gC(P, 3 * q + 0, -2.0 * gF[3 * t + 0]);
-        dev::add_gC(P, 3 * q + 1, -2.0 * gF[3 * t + 1]);
-        dev::add_gC(P, 3 * q + 2, -2.0 * gF[3 * t + 2]);
-      }
-    }
-    if (threadIdx.x == 0) atomicAdd(&P.acc[ACC_F2], fl);
+    for (int t = warp; t < nq; t += nwarp)
+      if (lane < 3 && gF[3 * t + lane] != 0.0) dev::add_gC(P, 3 * (q0 + t) + lane, -2.0 * gF[3 * t + lane]);
+    if (lane == 0) atomicAdd(&P.acc[ACC_F2], fl);
+    __syncthreads();   // gF and Zc are free for the next pair
   }
 }
 
@@ -869,7 +881,7 @@ cudaError_t launch_vblocks(const DevPlan& P, const int* list, int n, cudaStream_
 cudaError_t launch_ybuild(const DevPlan& P, const int* list, int n, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   ++g_launches;
-  k_ybuild<<<grid_for(n, 1, 152 * 64), kThreads, 0, s>>>(P, list, n);
+  k_ybuild<<<grid_for((long long)n * P.parts, 1, 152 * 64), P.small ? 64 : kThreads, 0, s>>>(P, list, n);
   return cudaGetLastError();
 }
 
@@ -892,14 +904,14 @@ cudaError_t set_kernel_smem_limits() {
 cudaError_t launch_term1(const DevPlan& P, const int* list, int n, int beta_chunk, size_t smem, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   ++g_launches;
-  k_term1<<<grid_for(n, 1, 152 * 64), kThreads, smem, s>>>(P, list, n, beta_chunk);
+  k_term1<<<grid_for((long long)n * P.parts, 1, 152 * 64), P.small ? 64 : kThreads, smem, s>>>(P, list, n, beta_chunk);
   return cudaGetLastError();
 }
 
 cudaError_t launch_term2(const DevPlan& P, const int* list, int n, int alpha_chunk, size_t smem, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   ++g_launches;
-  k_term2<<<grid_for(n, 1, 152 * 64), kThreads, smem, s>>>(P, list, n, alpha_chunk);
+  k_term2<<<grid_for((long long)n * P.parts2, 1, 152 * 64), P.small ? 64 : kThreads, smem, s>>>(P, list, n, alpha_chunk);
   return cudaGetLastError();
 }
 
