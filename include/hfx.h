@@ -326,8 +326,10 @@ hfx_status hfx_plan_autotune(hfx_plan* plan, const double* lattice, const double
  * dA, dB and dX must be all NULL (X only) or all non-NULL.  Pointers are
  * host memory; the call copies them to device `device`, runs one CTA per
  * pair (Cholesky factor in shared memory) on a stream of its own, copies the
- * results back and returns when they are written.  It holds no state and
- * may run beside any plan.
+ * results back and returns when they are written.  It holds no state but a
+ * stream and two buffers of 1 MiB per calling host thread (device and pinned
+ * host memory, given back when the thread ends or calls with another
+ * device), and may run beside any plan and in several threads.
  * Errors: HFX_ERR_INVALID for batch < 0, n < 1, w < 1, a NULL pointer or a
  * mixed NULL set, or a metric that is not positive definite (outputs are
  * then not written); HFX_ERR_UNSUPPORTED if n exceeds what the device's

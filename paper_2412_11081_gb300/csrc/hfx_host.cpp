@@ -4,9 +4,12 @@
 // stages of one evaluation.  Every stage of the arithmetic runs in the CUDA
 // kernels of hfx_kernels.cu.
 #include <cuda_runtime.h>
+#include <sys/mman.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <chrono>
+#include <cerrno>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -1954,6 +1957,70 @@ const char* hfx_status_string(hfx_status s) {
   return "unknown status";
 }
 
+}  // extern "C"
+
+namespace {
+
+// What hfx_lri_fit keeps per host thread between calls: a stream, and for
+// batches of at most kLriKeep bytes a device and a pinned host buffer, so that
+// a call of a few pairs is one copy each way and one launch (creating and
+// freeing the stream and the memory took most of its 97 us).  Freed when the
+// thread ends or calls with another device; larger batches allocate their own.
+constexpr size_t kLriKeep = 1 << 20;
+struct LriScratch {
+  int dev = -1;
+  cudaStream_t s = nullptr;
+  unsigned char *buf = nullptr, *pin = nullptr;
+  cudaError_t open(int device) {
+    if (dev == device) return cudaSuccess;
+    close();
+    cudaError_t e = cudaSetDevice(device);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMalloc(&buf, kLriKeep);
+    if (e == cudaSuccess) e = cudaMallocHost(&pin, kLriKeep);
+    dev = device;
+    if (e != cudaSuccess) close();
+    return e;
+  }
+  void close() {   // (errors ignored: the runtime may be gone at process exit)
+    if (dev < 0) return;
+    int now = -1;
+    cudaGetDevice(&now);
+    if (now != dev) cudaSetDevice(dev);
+    if (s) cudaStreamDestroy(s);
+    if (buf) cudaFree(buf);
+    if (pin) cudaFreeHost(pin);
+    if (now >= 0 && now != dev) cudaSetDevice(now);
+    cudaGetLastError();
+    dev = -1;
+    s = nullptr;
+    buf = pin = nullptr;
+  }
+  ~LriScratch() { close(); }
+};
+thread_local LriScratch g_lri;
+
+// Gives the pages of a result array their memory while the GPU works (their
+// contents stay): the copy into pages that were never touched takes ten times
+// as long as the copy itself (69 MB: 4.2 ms; 0.4 into present pages, and
+// 1.9 ms to make them present).  Only advice: what fails is left to the copy.
+void populate_pages(double* p, size_t n) {
+#ifdef MADV_POPULATE_WRITE
+  const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE), a = reinterpret_cast<uintptr_t>(p) & ~(page - 1);
+  const uintptr_t b = (reinterpret_cast<uintptr_t>(p + n) + page - 1) & ~(page - 1);
+  const int keep = errno;
+  madvise(reinterpret_cast<void*>(a), b - a, MADV_POPULATE_WRITE);
+  errno = keep;
+#else
+  (void)p;
+  (void)n;
+#endif
+}
+
+}  // namespace
+
+extern "C" {
+
 hfx_status hfx_lri_fit(int batch, int n, int w, const double* A, const double* B, const double* dA,
                        const double* dB, double* X, double* dX, int device) {
   g_create_error.clear();
@@ -1970,46 +2037,77 @@ hfx_status hfx_lri_fit(int batch, int n, int w, const double* A, const double* B
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   if (hfx::lri_fit_smem(n) + 2048 > (size_t)optin)
     return bad(HFX_ERR_UNSUPPORTED, "hfx_lri_fit: n too large for the Cholesky factor in shared memory");
-  const size_t nn = (size_t)batch * n * n, nw = (size_t)batch * n * w;
-  const size_t bytes = (nn + 2 * nw) * sizeof(double) * (grad ? 4 : 1) + sizeof(int);
-  cudaStream_t s = nullptr;
-  if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess)
-    return bad(HFX_ERR_CUDA, "hfx_lri_fit: stream");
-  unsigned char* buf = nullptr;
-  if (cudaMalloc(&buf, bytes) != cudaSuccess) {
+  const size_t nn = (size_t)batch * n * n, nw = (size_t)batch * n * w, k = grad ? 4 : 1;
+  const size_t in = k * (nn + nw), out = k * nw, nl = batch * hfx::lri_factor_size(n, w);
+  const size_t bytes = (in + out + 1 + nl) * sizeof(double);   // [A, dA, B, dB] [X, dX] [error flag] [factors]
+  if (g_lri.open(device) != cudaSuccess) {
     cudaGetLastError();
-    cudaStreamDestroy(s);
+    return bad(HFX_ERR_CUDA, "hfx_lri_fit: stream");
+  }
+  cudaStream_t s = g_lri.s;
+  const bool keep = bytes <= kLriKeep;
+  unsigned char* buf = g_lri.buf;
+  if (!keep && cudaMalloc(&buf, bytes) != cudaSuccess) {
+    cudaGetLastError();
     return bad(HFX_ERR_OOM, "hfx_lri_fit: device memory");
   }
-  double* A_dev = reinterpret_cast<double*>(buf);            // A, B, X [, dA, dB, dX]
-  double* B_dev = A_dev + nn;
-  double* X_dev = B_dev + nw;
-  double* gA = grad ? X_dev + nw : nullptr;
-  double* gB = grad ? gA + 3 * nn : nullptr;
-  double* gX = grad ? gB + 3 * nw : nullptr;
-  int* err = reinterpret_cast<int*>(buf + bytes - sizeof(int));
+  double* A_dev = reinterpret_cast<double*>(buf);
+  double* gA = grad ? A_dev + nn : nullptr;
+  double* B_dev = A_dev + k * nn;
+  double* gB = grad ? B_dev + nw : nullptr;
+  double* X_dev = A_dev + in;
+  double* gX = grad ? X_dev + nw : nullptr;
+  int* err = reinterpret_cast<int*>(A_dev + in + out);
+  double* Lw = nl ? A_dev + in + out + 1 : nullptr;
   int herr = 0;
-  cudaError_t e = cudaMemcpyAsync(A_dev, A, nn * sizeof(double), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(B_dev, B, nw * sizeof(double), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && grad) e = cudaMemcpyAsync(gA, dA, 3 * nn * sizeof(double), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && grad) e = cudaMemcpyAsync(gB, dB, 3 * nw * sizeof(double), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = hfx::launch_lri_fit(batch, n, w, A_dev, B_dev, gA, gB, X_dev, gX, err, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaError_t e = cudaSuccess;
+  if (keep) {   // one copy each way through the pinned buffer
+    double* h = reinterpret_cast<double*>(g_lri.pin);
+    std::memcpy(h, A, nn * sizeof(double));
+    std::memcpy(h + k * nn, B, nw * sizeof(double));
+    if (grad) {
+      std::memcpy(h + nn, dA, 3 * nn * sizeof(double));
+      std::memcpy(h + k * nn + nw, dB, 3 * nw * sizeof(double));
+    }
+    e = cudaMemcpyAsync(A_dev, h, in * sizeof(double), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
+    if (e == cudaSuccess && Lw) e = hfx::launch_lri_chol(batch, n, A_dev, Lw, err, s);
+    if (e == cudaSuccess) e = hfx::launch_lri_solve(batch, n, w, A_dev, Lw, B_dev, gA, gB, X_dev, gX, err, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, X_dev, (out + 1) * sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) std::memcpy(&herr, h + out, sizeof(int));
+  } else {
+    e = cudaMemcpyAsync(A_dev, A, nn * sizeof(double), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(B_dev, B, nw * sizeof(double), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && grad) e = cudaMemcpyAsync(gA, dA, 3 * nn * sizeof(double), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && grad) e = cudaMemcpyAsync(gB, dB, 3 * nw * sizeof(double), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), s);
+    if (e == cudaSuccess && Lw) e = hfx::launch_lri_chol(batch, n, A_dev, Lw, err, s);
+    if (e == cudaSuccess) e = hfx::launch_lri_solve(batch, n, w, A_dev, Lw, B_dev, gA, gB, X_dev, gX, err, s);
+    if (e == cudaSuccess) {
+      populate_pages(X, nw);
+      if (grad) populate_pages(dX, 3 * nw);
+      e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  }
   hfx_status st = HFX_OK;
   if (e != cudaSuccess) {
     st = bad(HFX_ERR_CUDA, cudaGetErrorString(e));
   } else if (herr) {
     st = bad(HFX_ERR_INVALID, "hfx_lri_fit: a metric block is not positive definite");
+  } else if (keep) {
+    const double* h = reinterpret_cast<const double*>(g_lri.pin);
+    std::memcpy(X, h, nw * sizeof(double));
+    if (grad) std::memcpy(dX, h + nw, 3 * nw * sizeof(double));
   } else {
     e = cudaMemcpyAsync(X, X_dev, nw * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && grad) e = cudaMemcpyAsync(dX, gX, 3 * nw * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) st = bad(HFX_ERR_CUDA, cudaGetErrorString(e));
   }
-  cudaFree(buf);
-  cudaStreamDestroy(s);
+  if (!keep) cudaFree(buf);
+  if (e != cudaSuccess) g_lri.close();   // the next call starts from a new stream and buffers
   return st;
 }
 

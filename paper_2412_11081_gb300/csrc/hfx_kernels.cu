@@ -18,6 +18,7 @@
 // CTAs meet in FP64 atomics (order-dependent only at the last bits).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -920,102 +921,192 @@ cudaError_t launch_term2(const DevPlan& P, const int* list, int n, int alpha_chu
 // a batch (one CTA per pair, grid-stride over the batch):
 //   A X = B                       X = the C^I rows, then the C^K rows
 //   A dX[c] = dB[c] - dA[c] X     c = x, y, z (gradient in K's position)
-// A (n x n, SPD) is factored as L L^T (left-looking Cholesky, L in shared
-// memory); each thread then owns RHS columns and runs the forward and back
-// substitutions on them in place in the output (row-major [n][w], so the
-// threads of a warp touch consecutive columns of one row), reading L by
-// broadcast.  A pivot <= 0 (A not positive definite) sets *err and is
-// replaced by 1 so that the CTA finishes.
+// A (n x n, SPD) is factored as L L^T (right-looking Cholesky, L in shared
+// memory as the packed lower triangle, column after column).  A CTA then
+// solves 32 RHS columns of a pair, one per lane: X in one warp, then the
+// three components of dX in three.  A lane runs the product dA[c] X and
+// both substitutions in blocks of eight rows held in registers: eight
+// independent chains, one load of the column per eight multiply-adds, and no
+// division (reciprocals of the diagonal with one correction).  Several CTAs
+// share an SM, so that one's loads and barriers hide behind another's FP64
+// work, which bounds it (n = 100, w = 169 with gradients: 512 pairs 13.9 ms =
+// 0.89 TFLOP/s; 128 pairs, 5 CTAs per SM, 4.7 + 0.2 ms.  One CTA per pair, a row
+// at a time with its column in global memory: 0.72 TFLOP/s).  A pivot <= 0 (A not positive definite)
+// sets *err and is replaced by 1 so that the CTA finishes.
 namespace {
 
-__device__ void lri_cholesky(double* L, const double* A, int n, int* err) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int e = tid; e < n * n; e += blockDim.x) L[e] = A[e];
+constexpr int kLriCols = 32;   // columns per CTA
+constexpr int kLB = 8;   // rows per block
+
+// L(i, k), i >= k, of the packed triangle
+__device__ __forceinline__ int lri_at(int i, int k, int n) { return k * n - k * (k + 1) / 2 + i; }
+
+// L and the reciprocals of its diagonal (inv).  After each column the rest of
+// the triangle is updated by all warps, a column each at a time: the work
+// spreads over the SM's four FP64 pipes.
+__device__ void lri_cholesky(double* L, double* inv, const double* A, int n, int* err) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = (blockDim.x + 31) >> 5;
+  for (int e = tid; e < n * n; e += blockDim.x) {
+    const int i = e / n, k = e - i * n;
+    if (k <= i) L[lri_at(i, k, n)] = A[e];
+  }
   __syncthreads();
   for (int j = 0; j < n; ++j) {
-    if (warp == 0) {
-      double sq = 0.0;
-      for (int k = lane; k < j; k += 32) sq += L[j * n + k] * L[j * n + k];
-      sq = warp_sum(sq);
-      if (lane == 0) {
-        double d = L[j * n + j] - sq;
-        if (!(d > 0.0)) {
-          atomicExch(err, 1);
-          d = 1.0;
-        }
-        L[j * n + j] = sqrt(d);
+    double* Lj = L + lri_at(0, j, n);   // column j, by row
+    if (tid == 0) {
+      double d = Lj[j];
+      if (!(d > 0.0)) {
+        atomicExch(err, 1);
+        d = 1.0;
       }
+      const double r = rsqrt(d);
+      Lj[j] = d * r;
+      inv[j] = r;
     }
     __syncthreads();
-    const double ljj = L[j * n + j];
+    const double ljj = Lj[j], rj = inv[j];
     for (int i = j + 1 + tid; i < n; i += blockDim.x) {
-      double a = L[i * n + j];
-      for (int k = 0; k < j; ++k) a -= L[i * n + k] * L[j * n + k];
-      L[i * n + j] = a / ljj;
+      const double t = Lj[i], y = t * rj;
+      Lj[i] = y + rj * (t - ljj * y);
+    }
+    __syncthreads();
+    for (int k = j + 1 + warp; k < n; k += nwarp) {
+      double* Lk = L + lri_at(0, k, n);
+      const double ljk = Lj[k];
+      for (int i = k + lane; i < n; i += 32) Lk[i] -= Lj[i] * ljk;
     }
     __syncthreads();
   }
 }
 
-// In-place solve L L^T x = r for the columns this thread owns of the
-// row-major n x w array R.
-__device__ void lri_substitute(const double* L, double* R, int n, int w) {
-  for (int col = threadIdx.x; col < w; col += blockDim.x) {
-    for (int i = 0; i < n; ++i) {   // L y = r
-      double a = R[(size_t)i * w + col];
-      for (int k = 0; k < i; ++k) a -= L[i * n + k] * R[(size_t)k * w + col];
-      R[(size_t)i * w + col] = a / L[i * n + i];
+// One RHS column: out = L^-T L^-1 (rhs - M x), M (n x n, row-major) and x (its
+// column, stride w) optional; rhs and out have stride w (out is written in the
+// forward pass and read back by the same thread).
+__device__ void lri_column(const double* L, const double* inv, int n, int w, const double* rhs, const double* M,
+                           const double* x, double* out) {
+  for (int i0 = 0; i0 < n; i0 += kLB) {   // L y = rhs - M x
+    const int nb = min(kLB, n - i0);
+    double a[kLB];
+#pragma unroll
+    for (int r = 0; r < kLB; ++r) a[r] = r < nb ? rhs[(size_t)(i0 + r) * w] : 0.0;
+    if (M)
+#pragma unroll 4
+      for (int j = 0; j < n; ++j) {
+        const double xj = x[(size_t)j * w];
+#pragma unroll
+        for (int r = 0; r < kLB; ++r)
+          if (r < nb) a[r] -= M[(size_t)(i0 + r) * n + j] * xj;
+      }
+#pragma unroll 4
+    for (int k = 0; k < i0; ++k) {
+      const double yk = out[(size_t)k * w];
+      const double* Lk = L + lri_at(i0, k, n);
+#pragma unroll
+      for (int r = 0; r < kLB; ++r)
+        if (r < nb) a[r] -= Lk[r] * yk;
     }
-    for (int i = n - 1; i >= 0; --i) {   // L^T x = y
-      double a = R[(size_t)i * w + col];
-      for (int k = i + 1; k < n; ++k) a -= L[k * n + i] * R[(size_t)k * w + col];
-      R[(size_t)i * w + col] = a / L[i * n + i];
+#pragma unroll
+    for (int r = 0; r < kLB; ++r)
+      if (r < nb) {
+        const double* Lr = L + lri_at(i0 + r, i0 + r, n);   // column i0 + r from the diagonal down
+        const double ri = inv[i0 + r], y0 = a[r] * ri, y = y0 + ri * (a[r] - Lr[0] * y0);
+        out[(size_t)(i0 + r) * w] = y;
+#pragma unroll
+        for (int t = r + 1; t < kLB; ++t)
+          if (t < nb) a[t] -= Lr[t - r] * y;
+      }
+  }
+  for (int i0 = (n - 1) / kLB * kLB; i0 >= 0; i0 -= kLB) {   // L^T x = y
+    const int nb = min(kLB, n - i0);
+    double a[kLB];
+#pragma unroll
+    for (int r = 0; r < kLB; ++r) a[r] = r < nb ? out[(size_t)(i0 + r) * w] : 0.0;
+#pragma unroll 4
+    for (int k = i0 + nb; k < n; ++k) {
+      const double xk = out[(size_t)k * w];
+#pragma unroll
+      for (int r = 0; r < kLB; ++r)
+        if (r < nb) a[r] -= L[lri_at(k, i0 + r, n)] * xk;
     }
+#pragma unroll
+    for (int r = kLB - 1; r >= 0; --r)
+      if (r < nb) {
+        const double ri = inv[i0 + r], y0 = a[r] * ri;
+        const double y = y0 + ri * (a[r] - L[lri_at(i0 + r, i0 + r, n)] * y0);
+        out[(size_t)(i0 + r) * w] = y;
+#pragma unroll
+        for (int t = 0; t < r; ++t) a[t] -= L[lri_at(i0 + r, i0 + t, n)] * y;
+      }
   }
 }
 
-__global__ void __launch_bounds__(kThreads) k_lri_fit(int batch, int n, int w, const double* A, const double* B,
-                                                     const double* dA, const double* dB, double* X, double* dX,
-                                                     int* err) {
-  extern __shared__ double L[];   // [n][n]
-  const size_t nn = (size_t)n * n, nw = (size_t)n * w;
+// The factor of every pair: packed triangle and reciprocals at Lw.
+__global__ void __launch_bounds__(256) k_lri_chol(int batch, int n, const double* A, double* Lw, int* err) {
+  extern __shared__ double L[];
+  const int nl = n * (n + 1) / 2;
   for (int p = blockIdx.x; p < batch; p += gridDim.x) {
-    __syncthreads();   // the previous pair's L is no longer read
-    lri_cholesky(L, A + p * nn, n, err);
-    double* Xp = X + p * nw;
-    const double* Bp = B + p * nw;
-    for (size_t e = threadIdx.x; e < nw; e += blockDim.x) Xp[e] = Bp[e];
     __syncthreads();
-    lri_substitute(L, Xp, n, w);
-    if (dX == nullptr) continue;
-    __syncthreads();   // X complete (each thread solved its own columns; rows mix below)
-    for (int c = 0; c < 3; ++c) {
-      const double* dAc = dA + (p * 3 + c) * nn;
-      const double* dBc = dB + (p * 3 + c) * nw;
-      double* R = dX + (p * 3 + c) * nw;
-      for (int col = threadIdx.x; col < w; col += blockDim.x)
-        for (int i = 0; i < n; ++i) {
-          double a = dBc[(size_t)i * w + col];
-          for (int j = 0; j < n; ++j) a -= dAc[(size_t)i * n + j] * Xp[(size_t)j * w + col];
-          R[(size_t)i * w + col] = a;
-        }
-      lri_substitute(L, R, n, w);
+    lri_cholesky(L, L + nl, A + (size_t)p * n * n, n, err);
+    for (int e = threadIdx.x; e < nl + n; e += blockDim.x) Lw[(size_t)p * (nl + n) + e] = L[e];
+  }
+}
+
+// Columns [32 part, ..) of X and dX (null: X alone) of every pair; the factor from Lw, or (Lw null) made here.
+// With gradients a CTA has four warps: one makes X, the others a component of
+// dX each; which is which turns with the unit, since a warp stays on one of the
+// SM's four FP64 pipes.
+__global__ void __launch_bounds__(4 * kLriCols) k_lri_solve(int batch, int parts, int n, int w, const double* A,
+                                                            const double* Lw, const double* B, const double* dA,
+                                                            const double* dB, double* X, double* dX, int* err) {
+  extern __shared__ double L[];   // packed triangle, then the reciprocals of the diagonal
+  const int nl = n * (n + 1) / 2, lane = threadIdx.x & 31;
+  double* inv = L + nl;
+  const size_t nn = (size_t)n * n, nw = (size_t)n * w;
+  for (long long u = blockIdx.x; u < (long long)batch * parts; u += gridDim.x) {
+    const int p = (int)(u / parts), col = kLriCols * (int)(u % parts) + lane;
+    const int c = dX ? (int)((threadIdx.x >> 5) + u) & 3 : 3;   // component of dX, or 3: X
+    __syncthreads();   // the previous unit's L is no longer read
+    if (Lw) {
+      for (int e = threadIdx.x; e < nl + n; e += blockDim.x) L[e] = Lw[(size_t)p * (nl + n) + e];
+      __syncthreads();
+    } else {
+      lri_cholesky(L, inv, A + p * nn, n, err);
     }
+    if (c == 3 && col < w) lri_column(L, inv, n, w, B + p * nw + col, nullptr, nullptr, X + p * nw + col);
+    if (dX == nullptr) continue;
+    __syncthreads();   // X of these columns complete
+    const size_t pc = (size_t)p * 3 + c;
+    if (c < 3 && col < w) lri_column(L, inv, n, w, dB + pc * nw + col, dA + pc * nn, X + p * nw + col, dX + pc * nw + col);
   }
 }
 
 }  // namespace
 
+// (the accepted n: a full n x n matrix in shared memory)
 size_t lri_fit_smem(int n) { return (size_t)n * n * sizeof(double); }
 
-cudaError_t launch_lri_fit(int batch, int n, int w, const double* A, const double* B, const double* dA,
-                           const double* dB, double* X, double* dX, int* err, cudaStream_t s) {
+size_t lri_factor_size(int n, int w) { return w <= kLriCols ? 0 : (size_t)(n * (n + 1) / 2 + n); }
+
+cudaError_t launch_lri_chol(int batch, int n, const double* A, double* Lw, int* err, cudaStream_t s) {
   if (batch <= 0) return cudaSuccess;
-  const size_t smem = lri_fit_smem(n);
-  cudaError_t e = allow_max_dynamic_smem((const void*)k_lri_fit);
+  const size_t smem = (size_t)(n * (n + 1) / 2 + n) * sizeof(double);
+  cudaError_t e = allow_max_dynamic_smem((const void*)k_lri_chol);
   if (e != cudaSuccess) return e;
   ++g_launches;
-  k_lri_fit<<<grid_for(batch, 1, 152 * 2), kThreads, smem, s>>>(batch, n, w, A, B, dA, dB, X, dX, err);
+  k_lri_chol<<<grid_for(batch, 1, 152 * 8), n <= 32 ? 64 : 256, smem, s>>>(batch, n, A, Lw, err);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_lri_solve(int batch, int n, int w, const double* A, const double* Lw, const double* B,
+                             const double* dA, const double* dB, double* X, double* dX, int* err, cudaStream_t s) {
+  if (batch <= 0) return cudaSuccess;
+  const size_t smem = (size_t)(n * (n + 1) / 2 + n) * sizeof(double);
+  cudaError_t e = allow_max_dynamic_smem((const void*)k_lri_solve);
+  if (e != cudaSuccess) return e;
+  const int parts = (w + kLriCols - 1) / kLriCols;
+  ++g_launches;
+  k_lri_solve<<<grid_for((long long)batch * parts, 1, 152 * 64), dX ? 4 * kLriCols : kLriCols, smem, s>>>(
+      batch, parts, n, w, A, Lw, B, dA, dB, X, dX, err);
   return cudaGetLastError();
 }
 
