@@ -564,15 +564,15 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
                 }
                 mma_split<SP>(acc, af[ks], bf);
               }
-              // acc[0], acc[1]: row a0 + gid, columns (beta, f) = nt * 8 + 2 tig, + 1
-              if (gid < dA) {
+              // acc[c]: row a0 + gid (+ 8 for c >= 2), column (beta, f) = nt * 8 + 2 tig + (c & 1)
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                  const int r = nt * 8 + 2 * tig + c;
-                  if (r < rowsU) {
-                    const int be = r / nF, ff = r - be * nF;
-                    put_pieces<SP>(Us, pU, be * SK + gid * nF + ff, acc[c] * pscale<SP>(P.sc.u));
-                  }
+              for (int c = 0; c < 2; ++c) {
+                const int r = nt * 8 + 2 * tig + c;
+                if (r < rowsU) {
+                  const int be = r / nF, ff = r - be * nF;
+                  if (gid < dA) put_pieces<SP>(Us, pU, be * SK + gid * nF + ff, acc[c] * pscale<SP>(P.sc.u));
+                  if (gid + 8 < dA)
+                    put_pieces<SP>(Us, pU, be * SK + (gid + 8) * nF + ff, acc[2 + c] * pscale<SP>(P.sc.u));
                 }
               }
             }
@@ -1058,7 +1058,7 @@ WideShapes wide_shapes(int maxABF, int maxAO, size_t limit) {
   WideShapes w{};
   w.MA = w.MB = (maxABF + 15) / 16 * 16;
   w.KZ = (maxAO + 15) / 16 * 16;
-  for (int da : {8, 4, 2, 1}) {
+  for (int da : {16, 8, 4, 2, 1}) {
     const int KC = (da * maxAO + 15) / 16 * 16;
     if (term1w_smem(w.MA, w.MB, KC) <= limit) {
       w.t1_da = da;
