@@ -248,13 +248,14 @@ struct hfx_plan {
   // split path for n_ao > 16 (hfx_wide.cu): FP64 C, V and D blocks, FP32 Y store
   bool wide = false;
   hfx::WideShapes ws{};
-  int wide_RB = 0;             // 64-row blocks of the largest Y block
-  int wide_maxrows = 0;        // most rows (alpha, a) of a C block
+  int KB = 1;                  // most AO sub-blocks of an atom (hfx::ao_subs)
+  int maxCv = 0;               // most column slots (C pair, sub) of an atom
+  int *vc_ptr = nullptr, *vc_list = nullptr;   // those slots per atom (KB > 1)
+  long long *y_vsize = nullptr, *y_vidx = nullptr;   // sub-blocks of each Y key's z; their place in y_vlist
+  int* y_vlist = nullptr;      // needed (key, sub), at most KB per needed key
   uint16_t* Cw = nullptr;      // C pieces of every C pair (written per call)
   float* dCf = nullptr;        // grad C of every C pair in FP32, the layout of dCst (written per call)
   long long* cw_off = nullptr;
-  uint16_t* Zw = nullptr;      // Z^{AB} of one pass's second-product pairs (bf16 pieces)
-  long long Zwcap = 0;
   uint16_t* Dw = nullptr;      // bf16 pieces of every D block (fixed for the plan)
   long long* dw_off = nullptr;
 
@@ -919,18 +920,37 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
   if (P->np) {   // key groups of the Y build
     P->gcnt = P->lalloc<int>(N);
     P->goff = P->lalloc<long long>(N);
-    P->gX = P->lalloc<int>(nY);
-    P->gS = P->lalloc<int>(nY);
-    P->gN = P->lalloc<int>(nY);
+    P->gX = P->lalloc<int>((size_t)P->KB * nY);
+    P->gS = P->lalloc<int>((size_t)P->KB * nY);
+    P->gN = P->lalloc<int>((size_t)P->KB * nY);
   }
-  if (P->np && !P->wide) {
+  P->maxCv = maxC;
+  if (P->KB > 1) {   // column slots (C pair, sub of F) and keys (key, sub of Z)
+    std::vector<int> vp(N + 1, 0), vl;
+    for (int A = 0; A < N; ++A) {
+      for (int q = c_ptr[A]; q < c_ptr[A + 1]; ++q)
+        for (int k = 0; k < hfx::ao_subs(P->n_ao[P->species[c_j[q]]]); ++k) vl.push_back(q | (k << hfx::kSubShift));
+      vp[A + 1] = (int)vl.size();
+      P->maxCv = std::max(P->maxCv, vp[A + 1] - vp[A]);
+    }
+    std::vector<long long> vs(nY);
+    for (int y = 0; y < nY; ++y) vs[y] = hfx::ao_subs(P->n_ao[P->species[y_j[y]]]);
+    P->vc_ptr = P->lalloc<int>(N + 1);
+    P->vc_list = P->lalloc<int>(vl.size());
+    P->y_vsize = P->lalloc<long long>(nY);
+    P->y_vidx = P->lalloc<long long>(nY);
+    P->y_vlist = P->lalloc<int>((size_t)P->KB * nY);
+    upload(P->vc_ptr, vp, s);
+    upload(P->vc_list, vl, s);
+    upload(P->y_vsize, vs, s);
+    ck(cudaStreamSynchronize(s), "upload lists");   // (the vectors end here)
+  }
+  if (P->np) {
     std::vector<long long> cm_off(nC + 1, 0), vm_size(nV);
     for (int p = 0; p < nC; ++p) {
       const int sA = P->species[c_home[p]], sj = P->species[c_j[p]];
       const long long rows = (long long)P->n_abf[sA] * P->n_ao[sA];
-      // bf16 tiles then FP32 grad C; each block rounded to 128 bytes (bulk copies need 16-byte alignment)
-      const long long sz = P->np * ((rows + 127) / 128) * 2048 + 2 * 3 * ((rows + 127) / 128) * 2048;
-      cm_off[p + 1] = cm_off[p] + (sz + 63) / 64 * 64;
+      cm_off[p + 1] = cm_off[p] + hfx::ao_subs(P->n_ao[sj]) * hfx::cm_size((int)rows);
     }
     for (int p = 0; p < nV; ++p) {
       const long long mA = P->n_abf[P->species[v_home[p]]], mB = P->n_abf[P->species[v_j[p]]];
@@ -1038,9 +1058,14 @@ void setup_shapes(hfx_plan* P) {
     if (!P->ws.ok) fail(HFX_ERR_UNSUPPORTED, "block shapes too large for the split-precision kernels");
     int maxrows = 0;
     for (int a = 0; a < P->S; ++a) maxrows = std::max(maxrows, P->n_abf[a] * P->n_ao[a]);
-    P->wide_RB = hfx::wide_ybuild_row_blocks(maxrows);
-    P->wide_maxrows = maxrows;
+    P->KB = hfx::ao_subs(maxAO);
+    P->MC = (maxrows + 127) / 128;
+    P->zblk = (long long)P->np * P->MC * 128 * 16;
+    P->ybtpc = 2;
+    P->q2tpc = P->sp == hfx::kSplitHalf ? 3 : 2;
+    P->q2_flush = P->sp == hfx::kSplitHalf ? 128 : 32;   // K steps per FP32 run, as for n_ao <= 16
     ck(hfx::set_wide_smem_limits(P->sp), "smem attributes");
+    ck(hfx::set_mixed_smem_limits(P->sp), "smem attributes");
     return;
   }
   if (P->np) {
@@ -1145,7 +1170,6 @@ void split_density(hfx_plan* P) {
     DevPlan D = make_devplan(P, P->lat_ref.data());
     ck(hfx::launch_dsplit_w(D, P->sp, P->Dw, P->dw_off, P->stream), "D pieces");
     ck(cudaStreamSynchronize(P->stream), "D pieces");
-    return;
   }
   std::vector<long long> off(P->n_d + 1, 0);
   for (long long k = 0; k < P->n_d; ++k) {
@@ -1157,7 +1181,7 @@ void split_density(hfx_plan* P) {
   P->Dsp = P->mem.alloc<uint16_t>(off[P->n_d] + 256);   // + one zero row (absent blocks)
   upload(P->dsp_off, off, P->stream);
   ck(cudaMemsetAsync(P->Dsp + off[P->n_d], 0, 256 * sizeof(uint16_t), P->stream), "memset");
-  {   // the split path holds n_ao <= 16: every piece is one 16 x 16 block of 512 bytes
+  {   // every piece of a sub-block is one 16 x 16 block of 512 bytes
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q{};
     ck(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q), "driver entry");
@@ -1362,9 +1386,14 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
                            P->scan_tmp, s), "scan");
     }
     if (P->np) {   // groups of up to 8 needed keys of one home atom (the Y build's CTAs)
-      ck(hfx::launch_ygroups(D, P->y_idx, T + 1, P->gcnt, nullptr, nullptr, nullptr, nullptr, 0, s), "ygroups");
+      if (P->KB > 1) {   // by (key, sub) of the keys' atoms with several sub-blocks
+        ck(hfx::scan_flags(P->y_flag, P->y_vsize, nullptr, nullptr, 1, P->nY, P->y_vidx, T + 10, P->scan_tmp, s), "scan");
+        ck(hfx::launch_yvirt(D, P->y_vidx, P->y_vlist, s), "key list");
+      }
+      const long long *yi = P->KB > 1 ? P->y_vidx : P->y_idx, *yt = P->KB > 1 ? T + 10 : T + 1;
+      ck(hfx::launch_ygroups(D, yi, yt, P->gcnt, nullptr, nullptr, nullptr, nullptr, 0, s), "ygroups");
       ck(hfx::scan_flags(P->gcnt, nullptr, nullptr, nullptr, 4, P->N, P->goff, T + 9, P->scan_tmp, s), "scan");
-      ck(hfx::launch_ygroups(D, P->y_idx, T + 1, P->gcnt, P->goff, P->gX, P->gS, P->gN, 1, s), "ygroups");
+      ck(hfx::launch_ygroups(D, yi, yt, P->gcnt, P->goff, P->gX, P->gS, P->gN, 1, s), "ygroups");
     }
     if (split) {
       // (A,F) view of the kept triplets: per C pair, its kept B in V-pair order
@@ -1398,6 +1427,12 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
   tm.mark();  // 2
   // ---- shared by every pass: the Y blocks (and the C operand pieces they read)
   hfx::T1UPlan U{};
+  X.KB = P->KB;
+  X.vc_ptr = P->vc_ptr;
+  X.vc_list = P->vc_list;
+  X.ybtpc = P->ybtpc;
+  X.q2tpc = P->q2tpc;
+  X.ytab_stride = 8 * P->maxC * P->KB;
   if (!P->np) {
     ensure_store(P, P->Yst, P->Ycap, P->tot[0]);
     D.Yst = P->Yst;
@@ -1405,8 +1440,12 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
   } else if (P->wide) {
     ensure_buf(P, P->Ysp, P->Yspcap, std::max(1LL, P->tot[0]));
     ck(hfx::launch_cpieces_w(D, P->sp, P->Cw, P->cw_off, P->dCf, s), "C pieces");
-    ck(hfx::launch_ybuild_w(D, P->sp, P->Ysp, P->Cw, P->cw_off, P->Dw, P->dw_off, P->y_list, P->gX, P->gS, P->gN,
-                            (int)P->tot[9], P->wide_RB, s),
+    ck(hfx::launch_cpieces(D, X, P->sp, s), "cpieces");
+    X.Ysp = P->Ysp;
+    ensure_buf(P, P->ytab, P->ytabcap, std::max(1LL, hfx::ytab_size((int)P->tot[9], P->maxC * P->KB)));
+    X.ytab = P->ytab;
+    ck(hfx::launch_ybuild_mma(D, X, P->sp, P->KB > 1 ? P->y_vlist : P->y_list, P->gX, P->gS, P->gN, (int)P->tot[9], P->MC,
+                              P->drows, P->d_err, s),
        "ybuild");
   } else {
     // the core-matrix Y stores' rows past n_abf are never written: zero them
@@ -1416,8 +1455,6 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     if (P->t2u && P->Yspcap != ycap0) ck(cudaMemsetAsync(P->Ysp, 0, P->Yspcap * sizeof(uint16_t), s), "memset");
     X.Ysp = P->Ysp;
     X.ycm = P->t2u ? 1 : 0;
-    X.ybtpc = P->ybtpc;
-    X.q2tpc = P->q2tpc;
     if (!reuse) {
       ensure_buf(P, P->blist, P->blist_cap, P->tot[6]);
       X.blist = P->blist;
@@ -1459,7 +1496,6 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     X.y_idx = P->y_idx;
     ensure_buf(P, P->ytab, P->ytabcap, std::max(1LL, hfx::ytab_size((int)P->tot[9], P->maxC)));
     X.ytab = P->ytab;
-    X.ytab_stride = 8 * P->maxC;
     ck(hfx::launch_ybuild_mma(D, X, P->sp, P->y_list, P->gX, P->gS, P->gN, (int)P->tot[9], P->MC, P->drows, P->d_err, s),
        "ybuild");
   }
@@ -1490,11 +1526,19 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
       m2.push_back(k1b.back());
       k2a.push_back(k1b.back());
       if (P->wide) {
-        ensure_buf(P, P->Zw, P->Zwcap,
-                   std::max(1LL, ct[CT_T2]) * P->np * hfx::wide_zplane(P->wide_maxrows, P->ws.KZ));
-        ck(hfx::launch_term2_w(D, P->sp, P->Ysp, P->Zw, P->Dw, P->dw_off, P->dCf, P->t2_list + v0, P->t2_idx, (int)ct[CT_T2],
-                               a0, a1, P->wide_maxrows, P->maxC, P->ws, s),
+        if (ct[CT_T2] * P->KB * P->zblk > P->Zcap) {
+          ensure_buf(P, P->Zst, P->Zcap, ct[CT_T2] * P->KB * P->zblk);
+          ck(cudaMemsetAsync(P->Zst, 0, (size_t)P->Zcap * sizeof(uint16_t), s), "memset");   // finite where nothing is written
+        }
+        X.Zst = P->Zst;
+        const int FC = (P->maxCv + 3) / 4;
+        ensure_buf(P, P->q2tab, P->q2tabcap, std::max(1LL, hfx::q2tab_size(ct[CT_T2] * P->KB, FC)));
+        X.q2tab = P->q2tab;
+        ck(hfx::launch_term2_w(D, P->sp, P->Ysp, P->Zst, P->zblk, P->KB, P->t2_list + v0, (int)ct[CT_T2], P->ws, s),
            "term2");
+        ck(hfx::launch_q2(D, X, P->sp, P->t2_list + v0, P->t2_idx, (int)ct[CT_T2], a0, a1, P->zblk, FC, P->MC,
+                          hfx::q2_umma_segments(P->maxV * P->KB, P->q2tpc), P->q2_flush, P->drows, P->d_err, s),
+           "Q2");
       } else
         ck(hfx::launch_term2(D, P->t2_list + v0, (int)ct[CT_T2], P->alpha_chunk, P->smem_t2, s), "term2");
     } else {

@@ -171,6 +171,15 @@ struct MixPlan {
   uint16_t* Vz = nullptr;
   long long vz_blk = 0;
   const long long* t2_slot = nullptr;   // V pair -> its slot in the pass's second-product list
+  // AO sub-blocks (ao_subs, ao_sub): the tensor-core tiles hold 16 orbitals, so
+  // an atom with more of them takes several: as K steps (C pair, sub) of the Y
+  // build and (pair, sub) of the Q2 GEMM, KB per C pair and per pair slot, and
+  // as columns: the Y build's keys carry their sub in the two top bits of the
+  // list entry, and vc_list names the (C pair, sub) of each Q2 column slot of
+  // an atom (nullptr: one slot per C pair).
+  int KB = 1;
+  const int* vc_ptr = nullptr;
+  const int* vc_list = nullptr;
   // 128-row tiles per CTA of the tcgen05 Y build and Q2 GEMM (1 or 2; the
   // autotuner's choice): two tiles share each K step's D blocks, one tile
   // runs more stages and two accumulators
@@ -204,6 +213,13 @@ struct T1UPlan {
   int seg;                     // B per FP32 run of the Q accumulator
   int nsplit;                  // parts an item's B are divided into
 };
+
+// Sub-blocks of at most 16 orbitals of an atom with n, and their size.
+constexpr int kSubShift = 30;
+__host__ __device__ inline int ao_subs(int n) { return (n + 15) >> 4; }
+__host__ __device__ inline int ao_sub(int n) { return (n + ao_subs(n) - 1) / ao_subs(n); }
+// uint16 units of one (C pair, sub) in MixPlan::Cm: the pieces, then grad C
+__host__ __device__ inline long long cm_size(int rows) { return (long long)((rows + 127) >> 7) * 2048 * (kPieces + 6); }
 
 enum AccSlot { ACC_E = 0, ACC_W = 1, ACC_FY = 10, ACC_F1 = 11, ACC_F2 = 12, ACC_N = 16 };
 enum CntSlot { CNT_C = 0, CNT_V = 1, CNT_D = 2, CNT_TRIP = 3, CNT_N = 8 };
@@ -265,7 +281,9 @@ cudaError_t launch_ybuild_mma(const DevPlan& P, const MixPlan& X, int sp, const 
                               cudaStream_t s);
 // ints of the D-block tables (MixPlan::ytab, MixPlan::q2tab)
 long long ytab_size(int ngroups, int maxC);
-long long q2tab_size(int n_slots, int FC);
+long long q2tab_size(long long n_slots, int FC);
+// (key, sub) list of the needed keys: key + (sub << kSubShift) at y_vidx[key] + sub
+cudaError_t launch_yvirt(const DevPlan& P, const long long* y_vidx, int* list, cudaStream_t s);
 cudaError_t launch_t1_lists(const DevPlan& P, const MixPlan& X, int phase, cudaStream_t s);
 size_t term1_mma_smem(int MAmax, int MBmax, int KSmax, int YRmax);
 size_t term2_mma_smem(int MAmax, int KZmax);
@@ -278,7 +296,11 @@ cudaError_t launch_term2_mma(const DevPlan& P, const MixPlan& X, int sp, const i
                              int n, int a0, int a1, int MAmax, int KZmax, long long zblk, int zrows, int FC, int MC,
                              int nseg, int flush, const DRows& drows, size_t smem, int* err, cudaStream_t s,
                              bool pairs_done = false);
-int q2_umma_segments(int max_pairs_per_atom, int tpc);
+int q2_umma_segments(int max_steps_per_atom, int tpc);
+// The Q2 GEMM alone, from a Z store of KB blocks per pair slot.
+cudaError_t launch_q2(const DevPlan& P, const MixPlan& X, int sp, const int* list, const long long* slot0, int n, int a0,
+                      int a1, long long zblk, int FC, int MC, int nseg, int flush, const DRows& drows, int* err,
+                      cudaStream_t s);
 // R2 and Z of the pass's second-product pairs on tcgen05 (hfx_t1umma.cu),
 // shapes n_abf <= 64, n_ao <= 16, with X.ycm and X.Vz set: E, g^V and the Z
 // store that k_q2_umma reads (launch_term2_mma with pairs_done then skips
@@ -318,36 +340,28 @@ cudaError_t launch_t1_umma(const DevPlan& P, const MixPlan& X, const T1UPlan& U,
 // path's layout [alpha][z][rup16(n_ao(X))]) and Z (per pass); V and grad V FP64.
 struct WideShapes {
   int MA = 0, MB = 0;          // n_abf rounded up to 16
-  int KZ = 0;                  // n_ao rounded up to 16
   int t1_da = 0, t1_KC = 0;    // first product: a per range, columns (a, f) per range (rounded to 16)
   int t2_da = 0, t2_KC = 0;    // second product: a per range, columns (a, b) per range
-  size_t smem_t1 = 0, smem_t2 = 0, smem_q2 = 0;
+  size_t smem_t1 = 0, smem_t2 = 0;
   bool ok = false;             // every shape fits the kernels' shared memory and tiles
 };
 long long wide_launch_count();
 WideShapes wide_shapes(int maxABF, int maxAO, size_t limit);
-int wide_ybuild_row_blocks(int max_rows);
 cudaError_t set_wide_smem_limits(int sp);
 // C pieces: per kept C pair, NP planes [alpha][rup8(n_ao(A) n_ao(F))] at Cw + cw_off[q]
 long long wide_cpieces_size(int n_abf, int n_ao_a, int n_ao_f);
 cudaError_t launch_cpieces_w(const DevPlan& P, int sp, uint16_t* Cw, const long long* cw_off, float* dCf,
                              cudaStream_t s);
-cudaError_t launch_ybuild_w(const DevPlan& P, int sp, uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
-                            const uint16_t* Dw, const long long* dw_off, const int* ylist, const int* gX,
-                            const int* gS, const int* gN, int ngroups, int RB, cudaStream_t s);
 cudaError_t launch_term1_w(const DevPlan& P, int sp, const uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
                            const uint16_t* Dw, const long long* dw_off, const float* dCf, const int* list, int n,
                            const WideShapes& w, cudaStream_t s);
-// elements per bf16 piece plane of one pair slot of the Z store (rows (alpha, a), row stride KZ)
-long long wide_zplane(int max_rows, int KZ);
 // bf16 pieces of every D block (fixed for the plan): NP planes of
 // rup16(n_ao(I)) x rup16(n_ao(J)) at Dw + dw_off[k] (multiples of 256)
 cudaError_t launch_dsplit_w(const DevPlan& P, int sp, uint16_t* Dw, const long long* dw_off, cudaStream_t s);
 // Second product of the home atoms [a0, a1): k_term2_w over the pass's pair
 // list (E, g^V and the Z piece store), then k_q2_w (grad C); slot0 as launch_term2_mma.
-cudaError_t launch_term2_w(const DevPlan& P, int sp, const uint16_t* Yp, uint16_t* Zw, const uint16_t* Dw,
-                           const long long* dw_off, const float* dCf, const int* list, const long long* slot0, int n,
-                           int a0, int a1, int max_rows, int max_c, const WideShapes& w, cudaStream_t s);
+cudaError_t launch_term2_w(const DevPlan& P, int sp, const uint16_t* Yp, uint16_t* Zst, long long zblk, int KB,
+                           const int* list, int n, const WideShapes& w, cudaStream_t s);
 
 // Exclusive scan helpers.  `mode` selects what is summed per element i:
 //   0: flag[i] != 0 (int32 flags)

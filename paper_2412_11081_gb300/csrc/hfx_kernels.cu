@@ -118,6 +118,10 @@ __global__ void k_cblocks(DevPlan P, int frozen) {
     const int sA = P.species[A], sj = P.species[j];
     const long long go = P.G_off[sA * P.S + sj];
     const int n = P.n_abf[sA] * P.n_ao[sA] * P.n_ao[sj];
+    if (threadIdx.x < 8) {   // the pair's scalars (c_pair_eval), for the split stores of wide plans
+      const double v[8] = {f, fa, g[0], g[1], g[2], ga[0], ga[1], ga[2]};
+      P.c_sc[8 * (long long)p + threadIdx.x] = v[threadIdx.x];
+    }
     double* C = P.Cst + P.c_off[p];
     double* dC = P.dCst + 3 * P.c_off[p];
     double sc = 0.0, sg = 0.0;

@@ -86,21 +86,23 @@ __device__ void block_sum_n(double (&v)[NV], double* red) {
 }
 
 // ------------------------------------------------------------------ D split
-// D block k (n_ao(I) x n_ao(J)) -> NP planes of rup16(n_ao(I)) x rup16(n_ao(J)), zero padded.
+// D block k (n_ao(I) x n_ao(J)) -> its sub-blocks (ao_subs), row by row, each as
+// NP planes of 16 x 16, zero padded.
 template <int SP>
 __global__ void k_dsplit(DevPlan P, MixPlan X, uint16_t* dst, float scale) {
   for (long long k = blockIdx.x; k < P.n_d; k += gridDim.x) {
     const int I = P.Didx[5 * k], J = P.Didx[5 * k + 1];
     const int na = P.n_ao[P.species[I]], nb = P.n_ao[P.species[J]];
-    const int pa = rup16(na), pb = rup16(nb);
+    const int sj = ao_subs(nb), ha = ao_sub(na), hb = ao_sub(nb), ns = ao_subs(na) * sj;
     uint16_t* out = dst + X.dsp_off[k];
     const double* src = P.Dval + P.Doff[k];
-    for (int e = threadIdx.x; e < pa * pb; e += blockDim.x) {
-      const int a = e / pb, b = e - a * pb;
+    for (int e = threadIdx.x; e < ns * 256; e += blockDim.x) {
+      const int sub = e >> 8, al = (e >> 4) & 15, bl = e & 15;
+      const int a = (sub / sj) * ha + al, b = (sub % sj) * hb + bl;
       uint16_t pc[NP];
-      split_f<SP>((a < na && b < nb) ? (float)src[a * nb + b] * pscale<SP>(scale) : 0.f, pc);
+      split_f<SP>((al < ha && a < na && bl < hb && b < nb) ? (float)src[a * nb + b] * pscale<SP>(scale) : 0.f, pc);
 #pragma unroll
-      for (int p = 0; p < NP; ++p) out[p * pa * pb + tix(a, b)] = pc[p];
+      for (int p = 0; p < NP; ++p) out[(sub * NP + p) * 256 + tix(al, bl)] = pc[p];
     }
   }
 }
@@ -108,7 +110,7 @@ __global__ void k_dsplit(DevPlan P, MixPlan X, uint16_t* dst, float scale) {
 // ------------------------------------------------------------------ pieces
 // C pair q: NP pieces of C[(alpha,a)][f] in 128-row tiles of the
 // tensor cores' core-matrix order ([tile][piece][128 x 16], f padded to 16),
-// then grad C in FP32 ([3][(alpha,a)][f]).
+// then grad C in FP32 (gc_off), per sub-block of F (cm_size apart).
 template <int SP>
 __global__ void k_cpieces(DevPlan P, MixPlan X) {
   for (int q = blockIdx.x; q < P.nC; q += gridDim.x) {
@@ -122,11 +124,14 @@ __global__ void k_cpieces(DevPlan P, MixPlan X) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) scf[k] = (float)P.c_sc[8 * (long long)q + k];
     const long long go = P.G_off[sA * P.S + sF];
-    uint16_t* out = X.Cm + X.cm_off[q];
+    const int hF = ao_sub(nF);
+    for (int sub = 0, f0 = 0; f0 < nF; ++sub, f0 += hF) {
+    const int nf = min(hF, nF - f0);
+    uint16_t* out = X.Cm + X.cm_off[q] + sub * cm_size(rows);
     for (int e = threadIdx.x; e < nt * 128 * 16; e += blockDim.x) {
       const int r = e >> 4, c = e & 15;
       uint16_t pc[NP];
-      split_f<SP>((r < rows && c < nF) ? model::c_value_f(P, scf, go, r * nF + c, 0) * pscale<SP>(P.sc.c) : 0.f, pc);
+      split_f<SP>((r < rows && c < nf) ? model::c_value_f(P, scf, go, r * nF + f0 + c, 0) * pscale<SP>(P.sc.c) : 0.f, pc);
 #pragma unroll
       for (int p = 0; p < NP; ++p) out[((r >> 7) * NP + p) * 2048 + tix(r & 127, c)] = pc[p];
     }
@@ -135,7 +140,8 @@ __global__ void k_cpieces(DevPlan P, MixPlan X) {
     for (int w = threadIdx.x; w < 3 * nt * 2048; w += blockDim.x) {
       const int c = w / (nt * 2048), wi = w - c * nt * 2048;
       const int r = ((wi >> 11) << 7) + ((wi >> 2) & 127), ff = (((wi >> 9) & 3) << 2) + (wi & 3);
-      g[w] = (r < rows && ff < nF) ? model::c_value_f(P, scf, go, r * nF + ff, c + 1) : 0.f;
+      g[w] = (r < rows && ff < nf) ? model::c_value_f(P, scf, go, r * nF + f0 + ff, c + 1) : 0.f;
+    }
     }
   }
 }
@@ -826,20 +832,23 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
   const int sA = P.species[A];
   const int nA = P.n_ao[sA], mA = P.n_abf[sA];
   const int rows = mA * nA, nt = (rows + 127) >> 7;
-  const int q0 = P.c_ptr[A], nq = P.c_ptr[A + 1] - q0;
+  const int q0 = P.c_ptr[A], nq = X.vc_ptr ? X.vc_ptr[A + 1] - X.vc_ptr[A] : P.c_ptr[A + 1] - q0;   // column slots
   if (fc * 8 >= nq || mc * 128 >= rows || P.v_ptr[A] == P.v_ptr[A + 1]) return;
   const int ntile = min(TPC, nt - mc);   // row tiles of this CTA
-  const long long s0 = slot0[P.v_ptr[A]];
-  const long long s1 = A + 1 < a1 ? slot0[P.v_ptr[A + 1]] : (long long)n_slots;
+  const long long s0 = slot0[P.v_ptr[A]] * X.KB;   // K steps (pair slot, sub)
+  const long long s1 = A + 1 < a1 ? slot0[P.v_ptr[A + 1]] * X.KB : (long long)n_slots;
   const long long p0 = s0 + (long long)seg * KMP;
   const int np = (int)max(0ll, min((long long)KMP, s1 - p0));
   if (np <= 0) return;
   const int row0 = mc * 128;
-  int qf[8];
+  int qf[8], qs[8];   // C pair (or -1) and sub of each column slot
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int j = fc * 8 + i;
-    qf[i] = (j < nq && P.c_keep[q0 + j]) ? q0 + j : -1;
+    const int code = j < nq ? (X.vc_list ? X.vc_list[X.vc_ptr[A] + j] : q0 + j) : 0;
+    const int q = code & ((1 << kSubShift) - 1);
+    qf[i] = (j < nq && P.c_keep[q]) ? q : -1;
+    qs[i] = code >> kSubShift;
   }
   // D block (units of 256 elements) of every (pair, F), or -1, from the table
   {
@@ -982,7 +991,7 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
           // grad C_AF rows in gc_off order: the warp's 32 rows of one 4-column
           // group are 512 consecutive bytes; columns f >= n_ao(F) are zero on
           // both sides
-          const float4* dC4 = reinterpret_cast<const float4*>(X.Cm + X.cm_off[qf[i]] + (long long)NP * nt * 2048) +
+          const float4* dC4 = reinterpret_cast<const float4*>(X.Cm + X.cm_off[qf[i]] + qs[i] * cm_size(rows) + (long long)NP * nt * 2048) +
                               (r >> 7) * 512 + (r & 127);
           float4 w[3][4];
 #pragma unroll
@@ -1048,8 +1057,8 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   uint16_t* stA = reinterpret_cast<uint16_t*>(smem_raw);                     // [kStages][TPC][NP][kTileElems]
   uint16_t* stB = stA + (size_t)kStages * TPC * NP * kTileElems;           // [kStages][NP][kTileElems]
-  int* m_d = reinterpret_cast<int*>(stB + (size_t)kStages * NP * kTileElems);   // [kMaxCPerAtom][8]
-  __shared__ int m_q[kMaxCPerAtom];
+  int* m_d = reinterpret_cast<int*>(stB + (size_t)kStages * NP * kTileElems);   // [K steps (C pair, sub)][8]
+  int* m_q = m_d + X.ytab_stride;                                               // the steps in use
   __shared__ int s_nsteps;
   __shared__ __align__(8) uint64_t bar_full[kStages], bar_empty[kStages], bar_accf;
   __shared__ uint32_t tmem_base;
@@ -1063,11 +1072,13 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
   const int rows = mX * nX;
   if (mc * 128 >= rows) return;
   const int ntile = min(TPC, ((rows + 127) >> 7) - mc);
-  const int q0 = P.c_ptr[Xa], nq = P.c_ptr[Xa + 1] - q0;
-  int ykey[8], zat[8];
+  const int q0 = P.c_ptr[Xa], nq = (P.c_ptr[Xa + 1] - q0) * X.KB;
+  int ykey[8], zat[8], zsub[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    ykey[i] = i < nk ? ylist[kstart + i] : -1;
+    const int code = i < nk ? ylist[kstart + i] : 0;
+    ykey[i] = i < nk ? code & ((1 << kSubShift) - 1) : -1;
+    zsub[i] = code >> kSubShift;
     zat[i] = ykey[i] >= 0 ? P.y_j[ykey[i]] : 0;
   }
   // D block of every (C pair, key), or -1, from the table
@@ -1129,7 +1140,8 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
       if (lane == 0) {
         mbar_expect_tx(mfull + 8 * s, bytes);
         bulk_g2s((uint32_t)__cvta_generic_to_shared(stA + (size_t)s * TPC * NP * kTileElems),
-                 X.Cm + X.cm_off[q0 + t] + (long long)mc * NP * kTileElems, abytes, mfull + 8 * s);
+                 X.Cm + X.cm_off[q0 + t / X.KB] + (t % X.KB) * cm_size(rows) + (long long)mc * NP * kTileElems, abytes,
+                 mfull + 8 * s);
       }
       stage_d(lane, stB + (size_t)s * NP * kTileElems, m_d + t * 8, &drows.map, drows.zero_row, mfull + 8 * s);
     }
@@ -1206,28 +1218,30 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
       for (int h = 0; h < 2; ++h) {
         const int i = (c0 >> 4) + h;
         if (ykey[i] < 0) continue;
-        const int nZ = P.n_ao[P.species[zat[i]]];
+        // columns zz < nZs of the slot are z = z0 + zz of the key's nZ; x padded to PX
+        const int nZ = P.n_ao[P.species[zat[i]]], z0 = zsub[i] * ao_sub(nZ), nZs = min(ao_sub(nZ), nZ - z0);
+        const int PX = rup16(nX), NH = PX >> 3;
         uint16_t* Yo = X.Ysp + P.y_off[ykey[i]];
         uint16_t* Yh = X.Yh ? X.Yh + X.y_idx[ykey[i]] * X.yh_blk : nullptr;
         const bool cm = X.ycm != 0;   // Ysp rows alpha, K = (z, x) in core-matrix order
         const int KZc = 16 * nZ, m8 = (mX + 7) & ~7;
-        const long long hplane = (long long)m8 * KZc, plane = cm ? hplane : (long long)mX * nZ * 16;
+        const long long hplane = (long long)m8 * KZc, plane = cm ? hplane : (long long)mX * nZ * PX;
         const float* eh = ep + h * 16;
         // bf16 pieces: chunk (alpha, z, half) holds x = 8 half .. 8 half + 7
         // (core-matrix order: consecutive threads take consecutive alpha, whose
         // chunks are 16 bytes apart)
-        for (int c = et; c < nal * nZ * 2; c += 128) {
+        for (int c = et; c < nal * nZs * NH; c += 128) {
           int hf, al, zz;
-          if (cm) {
+          if (cm) {   // (PX = 16, one sub)
             const int r2 = c / nal;
             al = alF + (c - r2 * nal);
             hf = r2 & 1;
             zz = r2 >> 1;
           } else {
-            const int az = c >> 1;
-            hf = c & 1;
-            al = alF + az / nZ;
-            zz = az - (az / nZ) * nZ;
+            const int az = c / NH;
+            hf = c - az * NH;
+            al = alF + az / nZs;
+            zz = az - (az / nZs) * nZs;
           }
           const int rl = al * nX - row0 + 8 * hf;
           float f0[4], f1[4];
@@ -1239,7 +1253,7 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
           uint2 p0[NP], p1[NP];
           split4<SP>(f0, p0);
           split4<SP>(f1, p1);
-          uint16_t* yo = Yo + (cm ? cmx(al, zz * 16 + 8 * hf, KZc) : ((long long)al * nZ + zz) * 16 + 8 * hf);
+          uint16_t* yo = Yo + (cm ? cmx(al, zz * 16 + 8 * hf, KZc) : ((long long)al * nZ + z0 + zz) * PX + 8 * hf);
 #pragma unroll
           for (int pp = 0; pp < NP; ++pp)
             *reinterpret_cast<uint4*>(yo + pp * plane) = make_uint4(p0[pp].x, p0[pp].y, p1[pp].x, p1[pp].y);
@@ -1312,16 +1326,16 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
           const int al = pa ? alB : alA;
           if (pa ? (alB <= alL || alB == alA) : (alA >= alF)) continue;
           const int r0 = max(row0, al * nX), nr = min(rend, (al + 1) * nX) - r0;
-          for (int c = et; c < nr * nZ; c += 128) {
+          for (int c = et; c < nr * nZs; c += 128) {
             const int zz = c / nr, r = r0 + (c - zz * nr), x = r - al * nX;
             const float y = eh[(r - row0) * 33 + zz];
             uint16_t pc[NP];
             split_f<SP>(y, pc);
-            const long long o = cm ? cmx(al, zz * 16, KZc) : ((long long)al * nZ + zz) * 16;   // + x (x < 16)
+            const long long o = cm ? cmx(al, zz * 16, KZc) : ((long long)al * nZ + z0 + zz) * PX;   // + x
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp) Yo[pp * plane + o + (cm ? ((x >> 3) << 6) + (x & 7) : x)] = pc[pp];
             if (x == nX - 1)
-              for (int xp = nX; xp < 16; ++xp)
+              for (int xp = nX; xp < PX; ++xp)
 #pragma unroll
                 for (int pp = 0; pp < NP; ++pp) Yo[pp * plane + o + (cm ? ((xp >> 3) << 6) + (xp & 7) : xp)] = 0;
             if (Yh) {
@@ -1380,22 +1394,26 @@ __global__ void k_ytab(DevPlan P, MixPlan X, const int* ylist, const int* gX, co
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
     const int i = (int)(e & 7);
     const long long gt = e >> 3;
-    const int g = (int)(gt / TC), t = (int)(gt - (long long)g * TC);
+    const int g = (int)(gt / TC), st = (int)(gt - (long long)g * TC);
+    const int t = st / X.KB, ws = st - t * X.KB;   // C pair slot, sub of W
     const int Xa = gX[g];
     const int q0 = P.c_ptr[Xa], nq = P.c_ptr[Xa + 1] - q0;
     if (t >= nq) continue;
-    const int key = i < gN[g] ? ylist[gS[g] + i] : -1;
+    const int code = i < gN[g] ? ylist[gS[g] + i] : 0;
+    const int key = i < gN[g] ? code & ((1 << kSubShift) - 1) : -1, zs = code >> kSubShift;
     int md = -1;
     if (key >= 0 && P.c_keep[q0 + t]) {
       const int* Rz = P.y_R + 3 * key;
       const int* Rw = P.c_R + 3 * (q0 + t);
       const int w = P.c_j[q0 + t], z = P.y_j[key];
-      const int di = dlut_get(P, w, z, Rz[0] - Rw[0], Rz[1] - Rw[1], Rz[2] - Rw[2]);
+      const int nw = P.n_ao[P.species[w]], nz = P.n_ao[P.species[z]], sw = ao_subs(nw);
+      const int di = ws < sw ? dlut_get(P, w, z, Rz[0] - Rw[0], Rz[1] - Rw[1], Rz[2] - Rw[2]) : -1;
       if (di >= 0 && P.Dkept[di] != 0.0) {
         const int mi = dlut_get(P, z, w, Rw[0] - Rz[0], Rw[1] - Rz[1], Rw[2] - Rz[2]);
-        md = (int)(X.dsp_off[mi] >> 8);
+        md = (int)(X.dsp_off[mi] >> 8) + (zs * sw + ws) * NP;
         const int sX = P.species[Xa];
-        fl += 2.0 * P.n_abf[sX] * P.n_ao[sX] * P.n_ao[P.species[z]] * P.n_ao[P.species[w]];
+        const int hz = ao_sub(nz), hw = ao_sub(nw);
+        fl += 2.0 * P.n_abf[sX] * P.n_ao[sX] * min(hz, nz - zs * hz) * min(hw, nw - ws * hw);
       }
     }
     X.ytab[e] = md;
@@ -1413,21 +1431,26 @@ __global__ void k_q2tab(DevPlan P, MixPlan X, const int* list, int n_slots, int 
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
     const int i = (int)(e & 7);
     const long long r = e >> 3;
-    const int fc = (int)(r / n_slots), slot = (int)(r - (long long)fc * n_slots);
+    const int fc = (int)(r / n_slots), st = (int)(r - (long long)fc * n_slots);
+    const int slot = st / X.KB, bs = st - slot * X.KB;   // pair slot, sub of B
     const int p = list[slot];
     const int A = P.v_home[p];
-    const int q0 = P.c_ptr[A], nq = P.c_ptr[A + 1] - q0;
+    const int q0 = P.c_ptr[A], nq = X.vc_ptr ? X.vc_ptr[A + 1] - X.vc_ptr[A] : P.c_ptr[A + 1] - q0;
     const int j = fc * 8 + i;
+    const int code = j < nq ? (X.vc_list ? X.vc_list[X.vc_ptr[A] + j] : q0 + j) : 0;
+    const int qf = code & ((1 << kSubShift) - 1), fs = code >> kSubShift;
     int db = -1;
-    if (j < nq && P.c_keep[q0 + j]) {
-      const int qf = q0 + j, b = P.v_j[p];
+    if (j < nq && P.c_keep[qf]) {
+      const int b = P.v_j[p];
       const int* Rb = P.v_R + 3 * p;
       const int* Rf = P.c_R + 3 * qf;
-      const int d = dlut_get(P, P.c_j[qf], b, Rb[0] - Rf[0], Rb[1] - Rf[1], Rb[2] - Rf[2]);
+      const int nb = P.n_ao[P.species[b]], nf = P.n_ao[P.species[P.c_j[qf]]], sb = ao_subs(nb);
+      const int d = bs < sb ? dlut_get(P, P.c_j[qf], b, Rb[0] - Rf[0], Rb[1] - Rf[1], Rb[2] - Rf[2]) : -1;
       if (d >= 0 && P.Dkept[d] != 0.0) {
-        db = (int)(X.dsp_off[d] >> 8);
+        db = (int)(X.dsp_off[d] >> 8) + (fs * sb + bs) * NP;
         const int sA = P.species[A];
-        fl += 2.0 * P.n_abf[sA] * P.n_ao[sA] * P.n_ao[P.species[b]] * P.n_ao[P.species[P.c_j[qf]]];
+        const int hb = ao_sub(nb), hf = ao_sub(nf);
+        fl += 2.0 * P.n_abf[sA] * P.n_ao[sA] * min(hb, nb - bs * hb) * min(hf, nf - fs * hf);
       }
     }
     X.q2tab[e] = db;
@@ -1436,9 +1459,9 @@ __global__ void k_q2tab(DevPlan P, MixPlan X, const int* list, int n_slots, int 
   if ((threadIdx.x & 31) == 0 && fl != 0.0) atomicAdd(&P.acc[ACC_F2], fl);
 }
 
-size_t ybuild_umma_smem(int tpc) {
+size_t ybuild_umma_smem(int tpc, int stride) {   // stride: 8 ints per K step
   return (size_t)(tpc + 1) * umma::kStages * NP * umma::kTileElems * sizeof(uint16_t) +
-         (size_t)kMaxCPerAtom * 8 * sizeof(int);
+         (size_t)(stride + stride / 8) * sizeof(int);
 }
 
 size_t q2_umma_smem(int tpc) {   // tpc 3: two tiles, the deep pipeline
@@ -1460,11 +1483,11 @@ int grid_for(long long n, int cap) {
 long long mixed_launch_count() { return g_mix_launches; }
 
 long long ytab_size(int ngroups, int maxC) { return (long long)ngroups * 8 * maxC; }
-long long q2tab_size(int n_slots, int FC) { return (long long)n_slots * ((FC * 4 + 7) / 8) * 8; }
+long long q2tab_size(long long n_slots, int FC) { return n_slots * ((FC * 4 + 7) / 8) * 8; }
 
-int q2_umma_segments(int max_pairs_per_atom, int tpc) {
+int q2_umma_segments(int max_steps_per_atom, int tpc) {
   const int kmp = tpc >= 2 ? Q2Shape<2>::kMP : Q2Shape<1>::kMP;
-  return (max_pairs_per_atom + kmp - 1) / kmp;
+  return (max_steps_per_atom + kmp - 1) / kmp;
 }
 
 cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, uint16_t* dst, float scale, int sp, cudaStream_t s) {
@@ -1507,7 +1530,7 @@ cudaError_t launch_ybuild_mma(const DevPlan& P, const MixPlan& X, int sp, const 
                                                                                           ngroups);
   const int tpc = X.ybtpc == 1 ? 1 : 2;
   const long long grid = (long long)ngroups * ((MC + tpc - 1) / tpc);
-  const size_t sm = ybuild_umma_smem(tpc);
+  const size_t sm = ybuild_umma_smem(tpc, X.ytab_stride);
   if (sp == kSplitBf16 && tpc == 2) k_ybuild_umma<kSplitBf16, 2><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
   else if (sp == kSplitBf16) k_ybuild_umma<kSplitBf16, 1><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
   else if (tpc == 2) k_ybuild_umma<kSplitHalf, 2><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
@@ -1554,34 +1577,58 @@ cudaError_t launch_term1_mma(const DevPlan& P, const MixPlan& X, int sp, const i
   return cudaGetLastError();
 }
 
-cudaError_t launch_term2_mma(const DevPlan& P, const MixPlan& X, int sp, const int* list, const long long* slot0,
-                             int n, int a0, int a1, int MAmax, int KZmax, long long zblk, int zrows, int FC, int MC,
-                             int nseg, int flush, const DRows& drows, size_t smem, int* err, cudaStream_t s,
-                             bool pairs_done) {
+__global__ void k_yvirt(DevPlan P, const long long* y_vidx, int* list) {
+  for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < P.nY; y += gridDim.x * blockDim.x)
+    if (P.y_flag[y])
+      for (int k = 0; k < ao_subs(P.n_ao[P.species[P.y_j[y]]]); ++k) list[y_vidx[y] + k] = y | (k << kSubShift);
+}
+
+cudaError_t launch_yvirt(const DevPlan& P, const long long* y_vidx, int* list, cudaStream_t s) {
+  if (P.nY == 0) return cudaSuccess;
+  ++g_mix_launches;
+  k_yvirt<<<grid_for((P.nY + 255) / 256, 152 * 16), 256, 0, s>>>(P, y_vidx, list);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_q2(const DevPlan& P, const MixPlan& X, int sp, const int* list, const long long* slot0, int n, int a0,
+                      int a1, long long zblk, int FC, int MC, int nseg, int flush, const DRows& drows, int* err,
+                      cudaStream_t s) {
   if (n == 0 || a1 <= a0) return cudaSuccess;
-  g_mix_launches += pairs_done ? 2 : 3;
-  const int FC8 = (FC * 4 + 7) / 8;     // groups of 8 C slots for the tcgen05 kernel
-  k_q2tab<<<grid_for(((long long)n * FC8 * 8 + 255) / 256, 152 * 16), 256, 0, s>>>(P, X, list, n, FC8);
+  g_mix_launches += 2;
+  const int FC8 = (FC * 4 + 7) / 8;     // groups of 8 column slots
+  const int ns = n * X.KB;              // K steps
+  k_q2tab<<<grid_for(((long long)ns * FC8 * 8 + 255) / 256, 152 * 16), 256, 0, s>>>(P, X, list, ns, FC8);
   const int tpc = X.q2tpc == 1 ? 1 : 2, deep = X.q2tpc == 3 ? 1 : 0;   // row tiles per CTA; the deep pipeline
   const size_t sq = q2_umma_smem(X.q2tpc == 1 ? 1 : (deep ? 3 : 2));
   const long long grid = (long long)(a1 - a0) * FC8 * ((MC + tpc - 1) / tpc) * nseg;
   auto q2 = [&](auto kern) {
-    kern<<<(unsigned)grid, 192, sq, s>>>(P, X, list, slot0, n, a0, a1, FC8, MC, nseg, zblk, flush, drows, err);
+    kern<<<(unsigned)grid, 192, sq, s>>>(P, X, list, slot0, ns, a0, a1, FC8, MC, nseg, zblk, flush, drows, err);
   };
   if (sp == kSplitBf16) {
-    if (!pairs_done)
-      k_term2_pairs<kSplitBf16><<<grid_for(n, 152 * 32), kWarps * 32, smem, s>>>(P, X, list, n, MAmax, KZmax, zblk, zrows);
     if (tpc == 1) q2(k_q2_umma<kSplitBf16, 1, 0>);
     else if (deep) q2(k_q2_umma<kSplitBf16, 2, 1>);
     else q2(k_q2_umma<kSplitBf16, 2, 0>);
   } else {
-    if (!pairs_done)
-      k_term2_pairs<kSplitHalf><<<grid_for(n, 152 * 32), kWarps * 32, smem, s>>>(P, X, list, n, MAmax, KZmax, zblk, zrows);
     if (tpc == 1) q2(k_q2_umma<kSplitHalf, 1, 0>);
     else if (deep) q2(k_q2_umma<kSplitHalf, 2, 1>);
     else q2(k_q2_umma<kSplitHalf, 2, 0>);
   }
   return cudaGetLastError();
+}
+
+cudaError_t launch_term2_mma(const DevPlan& P, const MixPlan& X, int sp, const int* list, const long long* slot0,
+                             int n, int a0, int a1, int MAmax, int KZmax, long long zblk, int zrows, int FC, int MC,
+                             int nseg, int flush, const DRows& drows, size_t smem, int* err, cudaStream_t s,
+                             bool pairs_done) {
+  if (n == 0 || a1 <= a0) return cudaSuccess;
+  if (!pairs_done) {
+    ++g_mix_launches;
+    if (sp == kSplitBf16)
+      k_term2_pairs<kSplitBf16><<<grid_for(n, 152 * 32), kWarps * 32, smem, s>>>(P, X, list, n, MAmax, KZmax, zblk, zrows);
+    else
+      k_term2_pairs<kSplitHalf><<<grid_for(n, 152 * 32), kWarps * 32, smem, s>>>(P, X, list, n, MAmax, KZmax, zblk, zrows);
+  }
+  return launch_q2(P, X, sp, list, slot0, n, a0, a1, zblk, FC, MC, nseg, flush, drows, err, s);
 }
 
 }  // namespace hfx

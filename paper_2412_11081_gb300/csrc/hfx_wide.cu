@@ -11,12 +11,8 @@
 //   D pieces   per D block, NP planes [rup16(n_ao(I))][rup16(n_ao(J))]   (plan)
 //   C pieces   per C pair, NP planes [alpha][rup8(n_ao(A) n_ao(F))]        (per call)
 //   Y pieces   per needed key (X; Z), NP planes [alpha][z][rup16(n_ao(X))] (Y build)
-//   Z pieces   per second-product pair, NP planes [(alpha, a)][KZ]        (per pass)
 // V and grad V stay FP64 (one pair per CTA reads them once).
 //
-//   k_ybuild_w  Y^{XZ}[alpha][x][z] = sum_W sum_w C_XW[alpha][x][w] D_WZ[w][z]
-//               per group of up to 8 keys (X; Z) of one home atom X and 64 rows
-//               (alpha, x), over the kept C pairs (X, W)
 //   k_term1_w   per kept (A,B) of the first exchange product, over its kept F
 //               and ranges of a:
 //                 U[beta][(a,f)] = sum_b D_AB[a][b] Y^{BF}[beta][b][f]
@@ -24,9 +20,10 @@
 //                 Q  = V_AB . U     (dotted with grad C_AF at once)
 //   k_term2_w   per kept (A,B) of the second product, over ranges of a:
 //                 R2 += Y^{AB} . Y^{BA}   (K = (a, b))
-//                 Z   = V_AB . Y^{BA}     (rows (alpha, a), to the Z pieces)
-//   k_q2_w      per (A, 128 rows (alpha, a), 8 C pairs (A,F)):
-//                 Q2 = sum_B Z^{AB} . D_FB^T, dotted with grad C_AF
+//                 Z   = V_AB . Y^{BA}     (rows (alpha, a), to the Z store)
+// The Y build and the Q2 GEMM are those of hfx_mixed.cu (tcgen05), which take
+// more than 16 orbitals as sub-blocks: with warp-level kernels of their own,
+// 11.5 and 12.3 ms on the 40-atom perovskite (1.2 and 1.9 ms now).
 // (Eq. exx_expand by the distributive law; Eq. Fexx1 for the gradients.)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -167,11 +164,9 @@ __global__ void k_dsplit_w(DevPlan P, uint16_t* Dw, const long long* dw_off) {
 }
 
 // ------------------------------------------------------------------ C pieces
-// Kept C pair q (evaluated this call, FP64) -> at Cw + cw_off[q]: NP bf16
-// planes of [alpha][rup8(n_ao(A) n_ao(F))] (columns (a, f) as in the FP64
-// block, zero padded; the first product's layout), then NP planes of
-// [(alpha, a)][rup16(n_ao(F))] (the Y build's A operand: every row starts on
-// a 16-byte boundary).
+// Kept C pair q (evaluated this call, FP64) -> at Cw + cw_off[q]: NP planes of
+// [alpha][rup8(n_ao(A) n_ao(F))] (columns (a, f) as in the FP64 block, zero
+// padded; the first product's layout).
 __host__ __device__ inline int cw_cols(int nA, int nF) { return (nA * nF + 7) & ~7; }
 
 // ... and grad C in FP32 (dCf, the layout of P.dCst), which the first
@@ -183,193 +178,16 @@ __global__ void k_cpieces_w(DevPlan P, uint16_t* Cw, const long long* cw_off, fl
     if (!P.c_keep[q]) continue;
     const int sA = P.species[P.c_home[q]], sF = P.species[P.c_j[q]];
     const int mA = P.n_abf[sA], nA = P.n_ao[sA], nF = P.n_ao[sF];
-    const int naf = nA * nF, CW = cw_cols(nA, nF), KW = rup16(nF);
+    const int naf = nA * nF, CW = cw_cols(nA, nF);
     const double* src = P.Cst + P.c_off[q];
     uint16_t* out = Cw + cw_off[q];
     for (int e = threadIdx.x; e < mA * CW; e += blockDim.x) {
       const int al = e / CW, c = e - al * CW;
       put_pieces<SP>(out, (long long)mA * CW, e, c < naf ? (float)src[(long long)al * naf + c] * pscale<SP>(P.sc.c) : 0.f);
     }
-    uint16_t* cy = out + (long long)NP * mA * CW;
-    for (int e = threadIdx.x; e < mA * nA * KW; e += blockDim.x) {
-      const int r = e / KW, c = e - r * KW;
-      put_pieces<SP>(cy, (long long)mA * nA * KW, e, c < nF ? (float)src[(long long)r * nF + c] * pscale<SP>(P.sc.c) : 0.f);
-    }
     const double* dsrc = P.dCst + 3 * P.c_off[q];
     float* dst = dCf + 3 * P.c_off[q];
     for (int e = threadIdx.x; e < 3 * mA * naf; e += blockDim.x) dst[e] = (float)dsrc[e];
-  }
-}
-
-// ------------------------------------------------------------------ Y build
-// CTA = (key group g, 64-row block rb).  Warp w: rows 16 (w & 3) of the block,
-// keys 4 (w >> 2) .. + 3 of the group, all z of each key (n_ao(Z) <= 32: four
-// column tiles).  K steps: 16 columns w of one kept C pair (X, W) with a D
-// block among the keys, two steps in flight (16-byte asynchronous copies):
-//   As[2][NP][64][24]          C_XW rows (alpha, x), columns w (the padded C pieces)
-//   Bs[2][NP][16][8 * 32 + 8]  D_{W Z_i} rows w, columns (i, z) (the D pieces)
-constexpr int kYRows = 64;
-constexpr int kYSA = 24;
-constexpr int kYSB = 8 * 32 + 8;
-size_t ybuild_w_smem() { return (size_t)2 * NP * (kYRows * kYSA + 16 * kYSB) * sizeof(uint16_t); }
-
-template <int SP>
-__global__ void __launch_bounds__(kWThreads) k_ybuild_w(DevPlan P, uint16_t* __restrict__ Yp,
-                                                        const uint16_t* __restrict__ Cw, const long long* cw_off,
-                                                        const uint16_t* __restrict__ Dw, const long long* dw_off,
-                                                        const int* ylist, const int* gX, const int* gS, const int* gN,
-                                                        int RB) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  constexpr long long pA = kYRows * kYSA, pB = 16 * kYSB;
-  uint16_t* As0 = reinterpret_cast<uint16_t*>(smem);   // [2][NP][64][kYSA]
-  uint16_t* Bs0 = As0 + 2 * NP * pA;                   // [2][NP][16][kYSB]
-  __shared__ int m_dw[kMaxCPerAtom][8];   // D piece block of (C pair t, key i) in 256-element units, or -1
-  __shared__ int m_step[2 * kMaxCPerAtom];
-  __shared__ int s_key[8], s_zat[8], s_nz[8];
-  __shared__ int s_nsteps;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
-  const int g = blockIdx.x / RB, rb = blockIdx.x - g * RB;
-  const int Xa = gX[g], kstart = gS[g], nk = gN[g];
-  const int sX = P.species[Xa];
-  const int mX = P.n_abf[sX], nX = P.n_ao[sX], KX = rup16(nX);
-  const int rows = mX * nX;
-  const int row0 = rb * kYRows;
-  if (row0 >= rows) return;
-  const int q0 = P.c_ptr[Xa], nq = P.c_ptr[Xa + 1] - q0;
-  if (threadIdx.x < 8) {
-    const int i = threadIdx.x;
-    const int key = i < nk ? ylist[kstart + i] : -1;
-    s_key[i] = key;
-    s_zat[i] = key >= 0 ? P.y_j[key] : 0;
-    s_nz[i] = key >= 0 ? P.n_ao[P.species[P.y_j[key]]] : 0;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < nq * 8; e += blockDim.x) {
-    const int t = e >> 3, i = e & 7;
-    const int q = q0 + t;
-    int dw = -1;
-    if (s_key[i] >= 0 && P.c_keep[q]) {
-      const int* Rw = P.c_R + 3 * q;
-      const int* Rz = P.y_R + 3 * s_key[i];
-      const int di = dlut_get(P, P.c_j[q], s_zat[i], Rz[0] - Rw[0], Rz[1] - Rw[1], Rz[2] - Rw[2]);
-      if (di >= 0 && P.Dkept[di] != 0.0) dw = (int)(dw_off[di] >> 8);
-    }
-    m_dw[t][i] = dw;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {   // K steps: (kept C pair with a D block among the keys, 16-column step)
-    int n = 0;
-    double fl = 0.0;
-    for (int t = 0; t < nq; ++t) {
-      bool any = false;
-      const int nW = P.n_ao[P.species[P.c_j[q0 + t]]];
-      for (int i = 0; i < 8; ++i)
-        if (m_dw[t][i] >= 0) {
-          any = true;
-          fl += 2.0 * rows * s_nz[i] * nW;
-        }
-      if (!any) continue;
-      for (int k0 = 0; k0 < nW; k0 += 16) m_step[n++] = (t << 8) | k0;
-    }
-    s_nsteps = n;
-    if (rb == 0) atomicAdd(&P.acc[ACC_FY], fl);
-  }
-  __syncthreads();
-  const int nsteps = s_nsteps;
-  const int mt = warp & 3, kh = warp >> 2;
-  int nz4[4];   // n_ao(Z) of this warp's four keys
-#pragma unroll
-  for (int ii = 0; ii < 4; ++ii) nz4[ii] = s_nz[4 * kh + ii];
-  float acc[4][4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[i][j][c] = 0.f;
-  // copies of step k into buffer k & 1 (rows past the block and columns past
-  // the keys' D blocks are not copied: they only meet discarded results)
-  auto issue = [&](int k) {
-    const int t = m_step[k] >> 8, k0 = m_step[k] & 255;
-    const int q = q0 + t;
-    const int nW = P.n_ao[P.species[P.c_j[q]]], pw = rup16(nW);
-    const uint16_t* Cy = Cw + cw_off[q] + (long long)NP * mX * cw_cols(nX, nW);   // [(alpha, x)][pw]
-    const long long cplane = (long long)rows * pw;
-    uint16_t* As = As0 + (k & 1) * NP * pA;
-    uint16_t* Bs = Bs0 + (k & 1) * NP * pB;
-    const int nr = min(kYRows, rows - row0);
-    for (int e = threadIdx.x; e < NP * nr * 2; e += blockDim.x) {
-      const int pp = e / (nr * 2), rr = e - pp * nr * 2, r = rr >> 1, h = rr & 1;
-      cpa16(As + pp * pA + r * kYSA + 8 * h, Cy + pp * cplane + (long long)(row0 + r) * pw + k0 + 8 * h);
-    }
-    for (int i = 0; i < 8; ++i) {
-      const int dw = m_dw[t][i];
-      if (dw < 0) continue;
-      const int pz = rup16(s_nz[i]), ch = pz >> 3;
-      const uint16_t* Dg = Dw + ((long long)dw << 8) + (long long)k0 * pz;   // rows w of D_{W Z_i} pieces [pw][pz]
-      const long long dplane = (long long)pw * pz;
-      for (int e = threadIdx.x; e < NP * 16 * ch; e += blockDim.x) {
-        const int pp = e / (16 * ch), rr = e - pp * 16 * ch, w = rr / ch, c = rr - w * ch;
-        cpa16(Bs + pp * pB + w * kYSB + i * 32 + 8 * c, Dg + pp * dplane + (long long)w * pz + 8 * c);
-      }
-    }
-  };
-  if (nsteps > 0) issue(0);
-  cpa_commit();
-  for (int k = 0; k < nsteps; ++k) {
-    if (k + 1 < nsteps) issue(k + 1);
-    cpa_commit();
-    cpa_wait<1>();
-    __syncthreads();   // step k's operands are in shared memory
-    const int t = m_step[k] >> 8;
-    const uint16_t* As = As0 + (k & 1) * NP * pA;
-    const uint16_t* Bs = Bs0 + (k & 1) * NP * pB;
-    uint32_t af[NP][4];
-#pragma unroll
-    for (int pp = 0; pp < NP; ++pp) ldm_x4(af[pp], As + pp * pA + (mt * 16 + (lane & 15)) * kYSA + ((lane >> 4) << 3));
-#pragma unroll
-    for (int ii = 0; ii < 4; ++ii) {
-      const int i = 4 * kh + ii;
-      if (m_dw[t][i] < 0) continue;
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
-        if (nt * 8 >= nz4[ii]) break;
-        uint32_t bf[NP][2];
-#pragma unroll
-        for (int pp = 0; pp < NP; ++pp) ldm_x2_trans(bf[pp], Bs + pp * pB + (lane & 15) * kYSB + i * 32 + nt * 8);
-        mma_split<SP>(acc[ii][nt], af, bf);
-      }
-    }
-    __syncthreads();   // buffer k & 1 is free for step k + 2
-  }
-  cpa_wait<0>();
-  // Y pieces [alpha][z][x] (x padded to rup16(n_ao(X)) with zeros, written
-  // with the row x = n_ao(X) - 1)
-#pragma unroll
-  for (int ii = 0; ii < 4; ++ii) {
-    const int key = s_key[4 * kh + ii];
-    if (key < 0) continue;
-    const int nZ = nz4[ii];
-    uint16_t* Y = Yp + P.y_off[key];
-    const long long plane = (long long)mX * nZ * KX;
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      if (nt * 8 >= nZ) break;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int row = row0 + mt * 16 + gid + ((c & 2) ? 8 : 0);
-        const int z = nt * 8 + 2 * tig + (c & 1);
-        if (row < rows && z < nZ) {
-          const int al = row / nX, x = row - al * nX;
-          const long long o = ((long long)al * nZ + z) * KX;
-          put_pieces<SP>(Y, plane, (int)(o + x), acc[ii][nt][c] * pscale<SP>(P.sc.y));
-          if (x == nX - 1)
-            for (int xp = nX; xp < KX; ++xp)
-#pragma unroll
-              for (int pp = 0; pp < NP; ++pp) Y[pp * plane + o + xp] = 0;
-        }
-      }
-    }
   }
 }
 
@@ -649,12 +467,13 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
 //   Vs[NP][MA][MB + 8]   V_AB
 //   Ya[NP][MA][KC + 8]   Y^{AB} columns (a, b), a in the current range
 //   Yb[NP][MB][KC + 8]   Y^{BA} as [beta][(a, b)], same columns
-// R2 gives E and g^V; Z = V_AB . Y^{BA} goes to the Z store of slot s as NP
-// bf16 planes of rows (alpha, a), columns b (row stride KZ, columns
-// n_ao(B) .. rup16(n_ao(B)) - 1 zero), for k_q2_w.
+// R2 gives E and g^V; Z = V_AB . Y^{BA} goes to the Z store of slot s: per
+// sub-block of B's orbitals (ao_sub) 128-row tiles of rows (alpha, a), 16
+// columns b, as k_q2_umma reads them (columns past the sub-block are left as
+// they are: finite, against zeros of D).
 struct T2W {
-  int MA, MB, KC, da, KZ;
-  long long zplane;    // elements per piece plane of a slot (most rows x KZ)
+  int MA, MB, KC, da, KB;
+  long long zblk;      // uint16 units per (slot, sub of B) of the Z store
 };
 
 __host__ __device__ inline size_t term2w_smem(int MA, int MB, int KC) {
@@ -663,7 +482,7 @@ __host__ __device__ inline size_t term2w_smem(int MA, int MB, int KC) {
 
 template <int SP>
 __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16_t* __restrict__ Yp,
-                                                       uint16_t* __restrict__ Zw, const int* list, int n_list, T2W S) {
+                                                       uint16_t* __restrict__ Zst, const int* list, int n_list, T2W S) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[4 * kPW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
@@ -688,16 +507,9 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
     const long long plA = (long long)mA * nB * KA, plB = (long long)mB * nA * KB;
     const double* V = P.Vst + P.v_off[p];
     const int nvb = mA * mB;
-    uint16_t* Z = Zw + (long long)kk * NP * S.zplane;   // NP planes [(alpha, a)][KZ]
+    uint16_t* Z = Zst + (long long)kk * S.KB * S.zblk;
+    const int hB = ao_sub(nB);
     __syncthreads();   // previous pair done with every buffer
-    {   // zero columns n_ao(B) .. rup16(n_ao(B)) - 1 (K padding of k_q2_w)
-      const int pad = rup16(nB) - nB;
-      for (int e = threadIdx.x; e < mA * nA * pad; e += blockDim.x) {
-        const int r = e / pad, c = nB + (e - r * pad);
-#pragma unroll
-        for (int pp = 0; pp < NP; ++pp) Z[pp * S.zplane + (long long)r * S.KZ + c] = 0;
-      }
-    }
     for (int e = threadIdx.x; e < MA * SV; e += blockDim.x) {
       const int al = e / SV, be = e - al * SV;
       put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * pscale<SP>(P.sc.v) : 0.f);
@@ -778,8 +590,10 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
               const int al = mt * 16 + gid + ((c & 2) ? 8 : 0);
               const int n = (nt0 + h) * 8 + 2 * tig + (c & 1);
               if (al < mA && n < dcols && nt0 + h < NTZ) {
-                const int bb = n / dA, a = n - bb * dA;
-                put_pieces<SP>(Z, S.zplane, (int)(((long long)al * nA + a0 + a) * S.KZ + bb), acc[h][c] * pscale<SP>(P.sc.z));
+                const int bb = n / dA, a = n - bb * dA, r = al * nA + a0 + a, sub = bb / hB;
+                put_pieces<SP>(Z + sub * S.zblk + (long long)(r >> 7) * NP * 2048, 2048,
+                               (((r & 127) >> 3) << 7) + (((bb - sub * hB) >> 3) << 6) + ((r & 7) << 3) + ((bb - sub * hB) & 7),
+                               acc[h][c] * pscale<SP>(P.sc.z));
               }
             }
         }
@@ -824,240 +638,15 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
   }
 }
 
-// k_q2_w: CTA = (home atom A of the pass, 128 rows (alpha, a), group of 8 C
-// slots F of A).  Q2^{AF}[(alpha, a)][f] = sum_B sum_b Z^{AB}[(alpha, a)][b]
-// D_FB[f][b] over the pairs (A,B) of the second product (one K step of
-// rup16(n_ao(B)) per pair), the eight F side by side in the columns (32 per
-// slot); every kQ2Run pairs the FP32 run is dotted with grad C_AF into FP64.
-// Warp w: rows 16 (w & 7) .. + 15 of the block, slots 4 (w >> 3) .. + 3.
-// Operands arrive by cp.async from the Z piece store and the D piece store,
-// two steps in flight:
-//   As[2][NP][128][KZ + 8]     Z rows, columns b
-//   Bs[2][NP][8 * 32][KZ + 8]  D_FB rows (slot, f), columns b
-constexpr int kQ2Threads = 512;
-constexpr int kQ2Rows = 128;
-constexpr int kQ2Slots = 8;
-constexpr int kQ2Seg = 256;   // pairs per segment of D-block metadata
-constexpr int kQ2Run = 64;    // pairs per FP32 run
-
-__host__ __device__ inline size_t q2w_smem(int KZ) {
-  return (size_t)2 * NP * 2 * (size_t)(kQ2Rows + kQ2Slots * 32) * (KZ + 8);
-}
-
-template <int SP>
-__global__ void __launch_bounds__(kQ2Threads, 1) k_q2_w(DevPlan P, const uint16_t* __restrict__ Zw, long long zplane,
-                                                        int KZ, const uint16_t* __restrict__ Dw,
-                                                        const long long* __restrict__ dw_off, const int* list,
-                                                        const long long* slot0, int n_slots, int a0, int a1, int RBQ,
-                                                        int SG, const float* __restrict__ dCf) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int m_dw[kQ2Seg][kQ2Slots];   // D piece block of (pair, slot) in 256-element units, or -1
-  __shared__ int m_step[kQ2Seg];
-  __shared__ int s_nsteps;
-  __shared__ int s_q[kQ2Slots], s_nf[kQ2Slots];
-  __shared__ double s_ev[kQ2Threads / 32][4][3];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
-  const int mt = warp & 7, sh = warp >> 3;
-  const int SZ = KZ + 8;
-  const long long pA = (long long)kQ2Rows * SZ, pB = (long long)kQ2Slots * 32 * SZ;
-  uint16_t* As0 = reinterpret_cast<uint16_t*>(smem);
-  uint16_t* Bs0 = As0 + 2 * NP * pA;
-  const int per_atom = RBQ * SG;
-  const int A = a0 + blockIdx.x / per_atom;
-  const int rem = blockIdx.x - (A - a0) * per_atom, rb = rem / SG, sg = rem - rb * SG;
-  if (A >= a1) return;
-  const int sA = P.species[A], mA = P.n_abf[sA], nA = P.n_ao[sA];
-  const int rows = mA * nA, row0 = rb * kQ2Rows;
-  const int q0 = P.c_ptr[A], nq = P.c_ptr[A + 1] - q0;
-  if (row0 >= rows || kQ2Slots * sg >= nq) return;
-  if (threadIdx.x < kQ2Slots) {
-    const int t = kQ2Slots * sg + threadIdx.x;
-    const int q = (t < nq && P.c_keep[q0 + t]) ? q0 + t : -1;
-    s_q[threadIdx.x] = q;
-    s_nf[threadIdx.x] = q >= 0 ? P.n_ao[P.species[P.c_j[q]]] : 0;
-  }
-  for (int e = threadIdx.x; e < (kQ2Threads / 32) * 12; e += blockDim.x) (&s_ev[0][0][0])[e] = 0.0;
-  __syncthreads();
-  bool any = false;
-#pragma unroll
-  for (int i = 0; i < kQ2Slots; ++i) any = any || s_q[i] >= 0;
-  if (!any) return;
-  int nf4[4];
-  bool live4[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    nf4[i] = s_nf[4 * sh + i];
-    live4[i] = s_q[4 * sh + i] >= 0;
-  }
-  const long long s0 = slot0[P.v_ptr[A]];
-  const long long s1 = A + 1 < a1 ? slot0[P.v_ptr[A + 1]] : (long long)n_slots;
-  float acc[4][4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[i][nt][c] = 0.f;
-  // dot of the FP32 run with grad C_AF (FP32 products, FP64 sums per warp), then the run restarts
-  auto flush = [&]() {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (!live4[i]) continue;
-      const int nF = nf4[i];
-      const float* dC = dCf + 3 * P.c_off[s_q[4 * sh + i]];   // grad C_AF in FP32 (k_cpieces_w)
-      const long long nc = (long long)rows * nF;
-      float g[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
-        if (nt * 8 >= nF) break;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int r = row0 + mt * 16 + gid + ((c & 2) ? 8 : 0);
-          const int ff = nt * 8 + 2 * tig + (c & 1);
-          if (r < rows && ff < nF) {
-            const long long ci = (long long)r * nF + ff;
-            const float v = acc[i][nt][c];
-            g[0] = fmaf((float)dC[ci], v, g[0]);
-            g[1] = fmaf((float)dC[nc + ci], v, g[1]);
-            g[2] = fmaf((float)dC[2 * nc + ci], v, g[2]);
-          }
-          acc[i][nt][c] = 0.f;
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float w = warp_sum_f(g[c]);
-        if (lane == 0) s_ev[warp][i][c] += (double)w * P.sc.q2;
-      }
-    }
-  };
-  double fl = 0.0;
-  int run = 0;
-  for (long long sb = s0; sb < s1; sb += kQ2Seg) {
-    const int nseg = (int)min((long long)kQ2Seg, s1 - sb);
-    __syncthreads();   // the previous segment is done with the metadata
-    for (int e = threadIdx.x; e < nseg * kQ2Slots; e += blockDim.x) {
-      const int j = e / kQ2Slots, i = e - j * kQ2Slots;
-      const int q = s_q[i];
-      int dw = -1;
-      if (q >= 0) {
-        const int pr = list[sb + j];
-        const int* Rb = P.v_R + 3 * pr;
-        const int* Rf = P.c_R + 3 * q;
-        const int di = dlut_get(P, P.c_j[q], P.v_j[pr], Rb[0] - Rf[0], Rb[1] - Rf[1], Rb[2] - Rf[2]);
-        if (di >= 0 && P.Dkept[di] != 0.0) dw = (int)(dw_off[di] >> 8);
-      }
-      m_dw[j][i] = dw;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int n = 0;
-      for (int j = 0; j < nseg; ++j) {
-        bool k = false;
-#pragma unroll
-        for (int i = 0; i < kQ2Slots; ++i) k = k || m_dw[j][i] >= 0;
-        if (k) m_step[n++] = j;
-      }
-      s_nsteps = n;
-    }
-    __syncthreads();
-    const int nsteps = s_nsteps;
-    // copies of step k into buffer k & 1: Z rows of the block, D_FB of every live slot
-    auto issue = [&](int k) {
-      const int j = m_step[k];
-      const long long slot = sb + j;
-      const int nB = P.n_ao[P.species[P.v_j[list[slot]]]], KB = rup16(nB), ch = KB >> 3;
-      const uint16_t* Z = Zw + slot * NP * zplane + (long long)row0 * KZ;
-      uint16_t* As = As0 + (k & 1) * NP * pA;
-      uint16_t* Bs = Bs0 + (k & 1) * NP * pB;
-      const int zr = min(kQ2Rows, rows - row0);
-      for (int e = threadIdx.x; e < NP * zr * ch; e += blockDim.x) {
-        const int pp = e / (zr * ch), rr = e - pp * zr * ch, r = rr / ch, c = rr - r * ch;
-        cpa16(As + pp * pA + r * SZ + 8 * c, Z + pp * zplane + (long long)r * KZ + 8 * c);
-      }
-      for (int i = 0; i < kQ2Slots; ++i) {
-        const int dw = m_dw[j][i];
-        if (dw < 0) continue;
-        const int pf = rup16(s_nf[i]);
-        const uint16_t* Dg = Dw + ((long long)dw << 8);
-        const long long dplane = (long long)pf * KB;
-        for (int e = threadIdx.x; e < NP * pf * ch; e += blockDim.x) {
-          const int pp = e / (pf * ch), rr = e - pp * pf * ch, f = rr / ch, c = rr - f * ch;
-          cpa16(Bs + pp * pB + (i * 32 + f) * SZ + 8 * c, Dg + pp * dplane + (long long)f * KB + 8 * c);
-        }
-      }
-    };
-    if (nsteps > 0) issue(0);
-    cpa_commit();
-    for (int k = 0; k < nsteps; ++k) {
-      if (k + 1 < nsteps) issue(k + 1);
-      cpa_commit();
-      cpa_wait<1>();
-      __syncthreads();   // step k's operands are in shared memory
-      const int j = m_step[k];
-      const int nB = P.n_ao[P.species[P.v_j[list[sb + j]]]], KB = rup16(nB);
-      const uint16_t* As = As0 + (k & 1) * NP * pA;
-      const uint16_t* Bs = Bs0 + (k & 1) * NP * pB;
-      bool on[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) on[i] = m_dw[j][4 * sh + i] >= 0;
-      for (int ks = 0; ks < KB; ks += 16) {
-        uint32_t af[NP][4];
-#pragma unroll
-        for (int pp = 0; pp < NP; ++pp)
-          ldm_x4(af[pp], As + pp * pA + (mt * 16 + (lane & 15)) * SZ + ks + ((lane >> 4) << 3));
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (!on[i]) continue;
-#pragma unroll
-          for (int nt = 0; nt < 4; ++nt) {
-            if (nt * 8 >= nf4[i]) break;
-            uint32_t bf[NP][2];
-#pragma unroll
-            for (int pp = 0; pp < NP; ++pp)
-              ldm_x2(bf[pp], Bs + pp * pB + ((4 * sh + i) * 32 + nt * 8 + (lane & 7)) * SZ + ks +
-                                 (((lane >> 3) & 1) << 3));
-            mma_split<SP>(acc[i][nt], af, bf);
-          }
-        }
-      }
-      if (rb == 0 && threadIdx.x == 0)
-        for (int i = 0; i < kQ2Slots; ++i)
-          if (m_dw[j][i] >= 0) fl += 2.0 * mA * nA * nB * s_nf[i];
-      if (++run == kQ2Run) {
-        flush();
-        run = 0;
-      }
-      __syncthreads();   // buffer k & 1 is free for step k + 2
-    }
-    cpa_wait<0>();
-  }
-  flush();
-  __syncthreads();
-  if (threadIdx.x < kQ2Slots * 3) {
-    const int i = threadIdx.x / 3, c = threadIdx.x - 3 * i;
-    const int q = s_q[i];
-    if (q >= 0) {
-      double v = 0.0;
-      for (int w = 0; w < 8; ++w) v += s_ev[(i >> 2) * 8 + w][i & 3][c];
-      dev::add_gC(P, 3 * q + c, -2.0 * v);
-    }
-  }
-  if (threadIdx.x == 0 && fl != 0.0) atomicAdd(&P.acc[ACC_F2], fl);
-}
-
 int grid_cap(long long n, int cap) { return (int)(n < cap ? (n > 0 ? n : 1) : cap); }
 
 }  // namespace
 
 long long wide_launch_count() { return g_wide_launches.load(); }
 
-int wide_ybuild_row_blocks(int max_rows) { return (max_rows + kYRows - 1) / kYRows; }
-
 WideShapes wide_shapes(int maxABF, int maxAO, size_t limit) {
   WideShapes w{};
   w.MA = w.MB = (maxABF + 15) / 16 * 16;
-  w.KZ = (maxAO + 15) / 16 * 16;
   for (int da : {16, 8, 4, 2, 1}) {
     const int KC = (da * maxAO + 15) / 16 * 16;
     if (term1w_smem(w.MA, w.MB, KC) <= limit) {
@@ -1076,9 +665,8 @@ WideShapes wide_shapes(int maxABF, int maxAO, size_t limit) {
       break;
     }
   }
-  w.smem_q2 = q2w_smem(w.KZ);
   // R tiles: (MA / 16) x (MB / 16) pairs over the warps, kPRP each
-  w.ok = w.t1_da > 0 && w.t2_da > 0 && w.smem_q2 <= limit && (w.MA / 16) * (w.MB / 16) <= kPW * kPRP &&
+  w.ok = w.t1_da > 0 && w.t2_da > 0 && (w.MA / 16) * (w.MB / 16) <= kPW * kPRP &&
          maxAO <= 32;
   return w;
 }
@@ -1090,15 +678,11 @@ cudaError_t set_wide_smem_limits(int sp) {
     if (r != cudaSuccess) e = r;
   };
   if (sp == kSplitBf16) {
-    one((const void*)k_ybuild_w<kSplitBf16>);
     one((const void*)k_term1_w<kSplitBf16>);
     one((const void*)k_term2_w<kSplitBf16>);
-    one((const void*)k_q2_w<kSplitBf16>);
   } else {
-    one((const void*)k_ybuild_w<kSplitHalf>);
     one((const void*)k_term1_w<kSplitHalf>);
     one((const void*)k_term2_w<kSplitHalf>);
-    one((const void*)k_q2_w<kSplitHalf>);
   }
   return e;
 }
@@ -1114,21 +698,7 @@ cudaError_t launch_cpieces_w(const DevPlan& P, int sp, uint16_t* Cw, const long 
 }
 
 long long wide_cpieces_size(int n_abf, int n_ao_a, int n_ao_f) {
-  return (long long)NP * n_abf * (cw_cols(n_ao_a, n_ao_f) + n_ao_a * ((n_ao_f + 15) / 16 * 16));
-}
-
-cudaError_t launch_ybuild_w(const DevPlan& P, int sp, uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
-                            const uint16_t* Dw, const long long* dw_off, const int* ylist, const int* gX,
-                            const int* gS, const int* gN, int ngroups, int RB, cudaStream_t s) {
-  if (ngroups <= 0) return cudaSuccess;
-  const long long grid = (long long)ngroups * RB;
-  const size_t smem = ybuild_w_smem();
-  if (sp == kSplitBf16)
-    k_ybuild_w<kSplitBf16><<<(unsigned)grid, kWThreads, smem, s>>>(P, Yp, Cw, cw_off, Dw, dw_off, ylist, gX, gS, gN, RB);
-  else
-    k_ybuild_w<kSplitHalf><<<(unsigned)grid, kWThreads, smem, s>>>(P, Yp, Cw, cw_off, Dw, dw_off, ylist, gX, gS, gN, RB);
-  ++g_wide_launches;
-  return cudaGetLastError();
+  return (long long)NP * n_abf * cw_cols(n_ao_a, n_ao_f);
 }
 
 cudaError_t launch_term1_w(const DevPlan& P, int sp, const uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
@@ -1143,8 +713,6 @@ cudaError_t launch_term1_w(const DevPlan& P, int sp, const uint16_t* Yp, const u
   return cudaGetLastError();
 }
 
-long long wide_zplane(int max_rows, int KZ) { return (long long)max_rows * KZ; }
-
 cudaError_t launch_dsplit_w(const DevPlan& P, int sp, uint16_t* Dw, const long long* dw_off, cudaStream_t s) {
   if (P.n_d <= 0) return cudaSuccess;
   const int grid = grid_cap(P.n_d, 1 << 16);
@@ -1154,26 +722,13 @@ cudaError_t launch_dsplit_w(const DevPlan& P, int sp, uint16_t* Dw, const long l
   return cudaGetLastError();
 }
 
-cudaError_t launch_term2_w(const DevPlan& P, int sp, const uint16_t* Yp, uint16_t* Zw, const uint16_t* Dw,
-                           const long long* dw_off, const float* dCf, const int* list, const long long* slot0, int n,
-                           int a0, int a1, int max_rows, int max_c, const WideShapes& w, cudaStream_t s) {
+cudaError_t launch_term2_w(const DevPlan& P, int sp, const uint16_t* Yp, uint16_t* Zst, long long zblk, int KB,
+                           const int* list, int n, const WideShapes& w, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const T2W S{w.MA, w.MB, w.t2_KC, w.t2_da, w.KZ, wide_zplane(max_rows, w.KZ)};
+  const T2W S{w.MA, w.MB, w.t2_KC, w.t2_da, KB, zblk};
   const int grid = grid_cap(n, 1 << 20);
-  if (sp == kSplitBf16) k_term2_w<kSplitBf16><<<grid, kPW * 32, w.smem_t2, s>>>(P, Yp, Zw, list, n, S);
-  else k_term2_w<kSplitHalf><<<grid, kPW * 32, w.smem_t2, s>>>(P, Yp, Zw, list, n, S);
-  ++g_wide_launches;
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const int RBQ = (max_rows + kQ2Rows - 1) / kQ2Rows, SG = (max_c + kQ2Slots - 1) / kQ2Slots;
-  const long long qgrid = (long long)(a1 - a0) * RBQ * SG;
-  if (qgrid <= 0) return cudaSuccess;
-  if (sp == kSplitBf16)
-    k_q2_w<kSplitBf16><<<(unsigned)qgrid, kQ2Threads, w.smem_q2, s>>>(P, Zw, S.zplane, w.KZ, Dw, dw_off, list, slot0, n, a0, a1,
-                                                             RBQ, SG, dCf);
-  else
-    k_q2_w<kSplitHalf><<<(unsigned)qgrid, kQ2Threads, w.smem_q2, s>>>(P, Zw, S.zplane, w.KZ, Dw, dw_off, list, slot0, n, a0, a1,
-                                                             RBQ, SG, dCf);
+  if (sp == kSplitBf16) k_term2_w<kSplitBf16><<<grid, kPW * 32, w.smem_t2, s>>>(P, Yp, Zst, list, n, S);
+  else k_term2_w<kSplitHalf><<<grid, kPW * 32, w.smem_t2, s>>>(P, Yp, Zst, list, n, S);
   ++g_wide_launches;
   return cudaGetLastError();
 }
