@@ -230,7 +230,9 @@ struct hfx_plan {
   size_t smem_m1 = 0, smem_m2 = 0;
   // tcgen05 first product (n_abf <= 64, n_ao <= 16): operand stores and shape
   bool t1u = false;
-  int t1u_KP = 0, t1u_G = 0, t1u_UB = 2, t1u_NS = 0, t1u_seg = 32;
+  int t1u_KP = 0, t1u_GA = 0, t1u_GB = 0, t1u_UB = 2, t1u_NS = 0, t1u_seg = 32;
+  int t1u_NAL = 1, t1u_subs = 1;   // alpha sub-blocks, items per C pair at most
+  long long* c_isize = nullptr;    // items of each C pair (wide plans)
   size_t smem_t1u = 0;
   uint16_t* Cu = nullptr;
   long long Cucap = 0;
@@ -784,6 +786,7 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
   v_ptr[N] = (int)v_j.size();
   y_ptr[N] = (int)y_j.size();
   const int nC = c_ptr[N], nV = v_ptr[N], nY = y_ptr[N];
+  if (nC >= (1 << hfx::kItemShift) || nY >= (1 << hfx::kSubShift)) fail(HFX_ERR_UNSUPPORTED, "too many pairs");
   // bound of |Y^{XZ}| = |sum_W C_XW D_WZ| at every geometry these lists cover
   // (no pair distance moves by more than the skin before they are rebuilt)
   P->ymax = 0;
@@ -864,7 +867,7 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
   P->c_off = P->lalloc<long long>(nC + 1);
   // FP64 C blocks: the FP64 path and the wide split path only (the other
   // split path evaluates C from the model where it writes its operand stores)
-  const bool fp64_c = !P->np || P->wide;
+  const bool fp64_c = !P->np || (P->wide && !P->t1u);
   P->Cst = P->lalloc<double>(fp64_c ? P->c_elems : 1);
   P->c_sc = P->lalloc<double>(8 * (size_t)nC);
   P->dCst = P->lalloc<double>(fp64_c ? 3 * P->c_elems : 1);
@@ -906,7 +909,7 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
     P->fx_words = 2 * (3 * (size_t)nC + 3 * (size_t)nV + 10 + 3 * (size_t)N);
     P->fx = P->lalloc<unsigned long long>(P->fx_words);
   }
-  if (P->wide) {   // C pieces (per call, every C pair)
+  if (P->wide && !P->t1u) {   // C pieces (per call, every C pair)
     std::vector<long long> cw_off(nC + 1, 0);
     for (int p = 0; p < nC; ++p) {
       const int sA = P->species[c_home[p]], sj = P->species[c_j[p]];
@@ -965,8 +968,18 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
     P->qcnt = P->lalloc<int>(nC);
     P->qoff = P->lalloc<long long>(nC);
     P->q_idx = P->lalloc<long long>(nC);
-    P->t1q_list = P->lalloc<int>(nC);
-    P->t1q_lpt = P->lalloc<int>(nC);
+    P->t1q_list = P->lalloc<int>((size_t)P->t1u_subs * nC);
+    P->t1q_lpt = P->lalloc<int>((size_t)P->t1u_subs * nC);
+    if (P->t1u_subs > 1) {
+      std::vector<long long> is(nC);
+      for (int q = 0; q < nC; ++q) {
+        const int sA = P->species[c_home[q]];
+        is[q] = hfx::abf_subs(P->n_abf[sA]) * hfx::ao_subs(P->n_ao[sA]) * hfx::ao_subs(P->n_ao[P->species[c_j[q]]]);
+      }
+      P->c_isize = P->lalloc<long long>(nC);
+      upload(P->c_isize, is, s);
+      ck(cudaStreamSynchronize(s), "upload lists");
+    }
     P->lpt_hist = P->lalloc<int>(hfx::kLptBuckets);
   }
   upload(P->c_ptr, c_ptr, s);
@@ -1021,6 +1034,43 @@ double list_drift(const hfx_plan* P, const double* L, const double* pos) {
   return 2.0 * disp + P->list_Rabs * dl;
 }
 
+// The tcgen05 first product for the plan's shapes: sub-blocks of at most 16
+// orbitals and 64 rows alpha; false where tensor memory (n_abf beyond ~100) or
+// shared memory do not hold them.
+bool t1u_shapes(hfx_plan* P, size_t limit) {
+  int hao = 0, habf = 0, mabf = 0, sao = 1;
+  for (int t = 0; t < P->S; ++t) {
+    hao = std::max(hao, hfx::ao_sub(P->n_ao[t]));
+    sao = std::max(sao, hfx::ao_subs(P->n_ao[t]));
+    habf = std::max(habf, hfx::abf_sub(P->n_abf[t]));
+    mabf = std::max(mabf, P->n_abf[t]);
+    P->t1u_NAL = std::max(P->t1u_NAL, hfx::abf_subs(P->n_abf[t]));
+  }
+  P->t1u_subs = P->t1u_NAL * sao * sao;
+  P->t1u_KP = 16 * hao;
+  P->t1u_GA = (habf + 7) / 8;
+  P->t1u_GB = (mabf + 7) / 8;
+  // two buffers of U where three slots of the Y ring still fit beside them
+  // (n_ao 13: n_abf up to 56), else one
+  auto slots = [&](int ub) {
+    const size_t base = hfx::t1u_smem(P->t1u_KP, P->t1u_GA, P->t1u_GB, P->KB, ub, 0);
+    return base < limit ? (int)std::min<size_t>((limit - base) / 16384, hfx::t1u_max_slots()) : 0;
+  };
+  P->t1u_UB = slots(2) >= 3 ? 2 : 1;
+  P->t1u_NS = slots(P->t1u_UB);
+  if (P->t1u_NS < 3 || hfx::t1u_utiles(P->t1u_KP, P->t1u_GB) < 2) return false;
+  P->t1u = true;
+  P->smem_t1u = hfx::t1u_smem(P->t1u_KP, P->t1u_GA, P->t1u_GB, P->KB, P->t1u_UB, P->t1u_NS);
+  // kept B per FP32 run of the Q accumulator: 32 for BF16X3, whose stress error
+  // is closest to the 1e-5 bound; 128 for BF16X6 (6.5e-6 at most on the
+  // jittered si64 geometries against 5.4e-6 with 32 when its operands were
+  // three bf16 pieces, and fewer FP64 flushes)
+  const char* sg = std::getenv("HFX_T1_SEG");
+  P->t1u_seg = sg ? std::max(1, std::atoi(sg)) : (P->sp == hfx::kSplitHalf ? 128 : 32);
+  ck(hfx::t1u_set_smem(P->sp), "smem attributes");
+  return true;
+}
+
 void setup_shapes(hfx_plan* P) {
   int dev_smem = 0;
   ck(cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, P->dev), "attr");
@@ -1059,6 +1109,9 @@ void setup_shapes(hfx_plan* P) {
     int maxrows = 0;
     for (int a = 0; a < P->S; ++a) maxrows = std::max(maxrows, P->n_abf[a] * P->n_ao[a]);
     P->KB = hfx::ao_subs(maxAO);
+    // first product: the tcgen05 kernel where the sub-blocks fit (HFX_T1_KERNEL=mma: the warp-level one)
+    const char* t1w = std::getenv("HFX_T1_KERNEL");
+    if (!(t1w && std::string(t1w) == "mma")) t1u_shapes(P, limit);
     P->MC = (maxrows + 127) / 128;
     P->zblk = (long long)P->np * P->MC * 128 * 16;
     P->ybtpc = 2;
@@ -1103,28 +1156,9 @@ void setup_shapes(hfx_plan* P) {
     const bool want_umma = !(t1k && std::string(t1k) == "mma");
     P->t1u = false;
     if (want_umma && maxABF <= 64 && maxAO <= 16) {
-      P->t1u_KP = 16 * maxAO;
-      P->t1u_G = (maxABF + 7) / 8;
-      // two buffers of U where three slots of the Y ring still fit beside them
-      // (n_ao 13: n_abf up to 56), else one
-      auto slots = [&](int ub) {
-        const size_t base = hfx::t1u_smem(P->t1u_KP, P->t1u_G, ub, 0);
-        return base < limit ? (int)std::min<size_t>((limit - base) / 16384, hfx::t1u_max_slots()) : 0;
-      };
-      P->t1u_UB = slots(2) >= 3 ? 2 : 1;
-      P->t1u_NS = slots(P->t1u_UB);
       // HFX_BF16X6 takes the shapes whose operands would fit in three pieces each
       const size_t np = P->sp == hfx::kSplitHalf ? 3 : 2;
-      if (np * (64 * P->t1u_KP * 4 + 8192) + 2048 + 8192 <= limit && P->t1u_NS >= 3) {
-        P->t1u = true;
-        P->smem_t1u = hfx::t1u_smem(P->t1u_KP, P->t1u_G, P->t1u_UB, P->t1u_NS);
-        // kept B per FP32 run of the Q accumulator: 32 for BF16X3, whose
-        // stress error is closest to the 1e-5 bound; 128 for BF16X6 (6.5e-6
-        // at most on the jittered si64 geometries against 5.4e-6 with 32,
-        // and fewer FP64 flushes)
-        const char* sg = std::getenv("HFX_T1_SEG");
-        P->t1u_seg = sg ? std::max(1, std::atoi(sg)) : (P->sp == hfx::kSplitHalf ? 128 : 32);
-        ck(hfx::t1u_set_smem(P->sp), "smem attributes");
+      if (np * (64 * 16 * maxAO * 4 + 8192) + 2048 + 8192 <= limit && t1u_shapes(P, limit)) {
         // the second product's R2 and Z on tcgen05 as well (HFX_T2_KERNEL=mma keeps the warp-level kernel)
         const char* t2k = std::getenv("HFX_T2_KERNEL");
         P->smem_t2u = hfx::t2u_smem(maxAO);
@@ -1157,7 +1191,7 @@ void setup_shapes(hfx_plan* P) {
 // bf16 pieces of every D block (fixed for the plan)
 void split_density(hfx_plan* P) {
   if (!P->np || P->n_d == 0) return;
-  if (P->wide) {   // NP planes of rup16(n_ao(I)) x rup16(n_ao(J)) per D block, row-major
+  if (P->wide && !P->t1u) {   // NP planes of rup16(n_ao(I)) x rup16(n_ao(J)) per D block, row-major
     std::vector<long long> off(P->n_d + 1, 0);
     for (long long k = 0; k < P->n_d; ++k) {
       const int* r = &P->d_index[5 * k];
@@ -1206,7 +1240,7 @@ void split_density(hfx_plan* P) {
   if (P->t1u) {
     P->d_work = P->mem.alloc<int>(1);
     if (P->sp != hfx::kSplitHalf) {
-      P->Dh = P->mem.alloc<uint16_t>((size_t)P->n_d * 512);
+      P->Dh = P->mem.alloc<uint16_t>((size_t)off[P->n_d]);
       ck(hfx::launch_dsplit(D, X, P->Dh, P->scale.dh, hfx::kSplitHalf, P->stream), "dsplit");
     }
   }
@@ -1353,7 +1387,8 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
   // the split path evaluates C from the block model where it stores the
   // operands; the FP64 path and the wide split path write the FP64 C blocks
   const bool split = P->np && !P->wide;
-  if (split)
+  const bool items = split || P->t1u;   // the (A,F) view of the kept triplets
+  if (items)
     ck(hfx::launch_cnorm(D, reuse ? 1 : 0, s), "cnorm");
   else
     ck(hfx::launch_cblocks(D, reuse ? 1 : 0, s), "cblocks");
@@ -1395,18 +1430,23 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
       ck(hfx::scan_flags(P->gcnt, nullptr, nullptr, nullptr, 4, P->N, P->goff, T + 9, P->scan_tmp, s), "scan");
       ck(hfx::launch_ygroups(D, yi, yt, P->gcnt, P->goff, P->gX, P->gS, P->gN, 1, s), "ygroups");
     }
-    if (split) {
+    if (items) {
       // (A,F) view of the kept triplets: per C pair, its kept B in V-pair order
       ck(hfx::launch_t1_lists(D, X, 0, s), "t1 count");
       ck(hfx::scan_flags(P->qcnt, nullptr, nullptr, nullptr, 4, P->nC, P->qoff, T + 6, P->scan_tmp, s), "scan");
-      for (int c = 0; c < nch; ++c) {   // per pass: its items, longest first
-        const int c0 = P->c_ptr_h[P->chunks[c].first], nc = P->c_ptr_h[P->chunks[c].second] - c0;
+      for (int c = 0; c < nch; ++c) {   // per pass: its items (a C pair's sub-blocks each), longest first
+        const int c0 = P->c_ptr_h[P->chunks[c].first], c1 = P->c_ptr_h[P->chunks[c].second], nc = c1 - c0;
+        const int sub = P->t1u_subs;
+        const size_t l0 = (size_t)sub * c0;
         long long* ct = CT + (size_t)kCT * c;
-        ck(hfx::scan_flags(P->qcnt + c0, nullptr, nullptr, nullptr, 0, nc, P->q_idx + c0, ct + CT_Q, P->scan_tmp, s),
-           "scan");
-        ck(hfx::scatter_list(P->qcnt + c0, nullptr, nullptr, 0, nc, P->q_idx + c0, P->t1q_list + c0, c0, s), "scatter");
-        ck(hfx::launch_lpt_order(P->t1_order == 2 ? P->c_j : P->qcnt, P->t1_order == 2 ? 1 : 0, P->t1q_list + c0, nc,
-                                 ct + CT_Q, P->lpt_hist, P->t1q_lpt + c0, s),
+        ck(hfx::scan_flags(P->qcnt + c0, sub > 1 ? P->c_isize + c0 : nullptr, nullptr, nullptr, sub > 1 ? 1 : 0, nc,
+                           P->q_idx + c0, ct + CT_Q, P->scan_tmp, s), "scan");
+        if (sub > 1)
+          ck(hfx::launch_t1_items(D, P->qcnt, P->q_idx, c0, c1, P->t1q_list + l0, s), "items");
+        else
+          ck(hfx::scatter_list(P->qcnt + c0, nullptr, nullptr, 0, nc, P->q_idx + c0, P->t1q_list + l0, c0, s), "scatter");
+        ck(hfx::launch_lpt_order(P->t1_order == 2 ? P->c_j : P->qcnt, P->t1_order == 2 ? 1 : 0, P->t1q_list + l0, nc * sub,
+                                 ct + CT_Q, P->lpt_hist, P->t1q_lpt + l0, s),
            "item order");
       }
     }
@@ -1433,13 +1473,57 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
   X.ybtpc = P->ybtpc;
   X.q2tpc = P->q2tpc;
   X.ytab_stride = 8 * P->maxC * P->KB;
+  auto t1u_plan = [&]() {   // the tcgen05 first product's sizes and its Y store
+    U.KP = P->t1u_KP;
+    U.GA = P->t1u_GA;
+    U.GB = P->t1u_GB;
+    U.VK = (8 * U.GB + 15) / 16 * 16;
+    U.NAL = P->t1u_NAL;
+    U.UB = P->t1u_UB;
+    U.NS = P->t1u_NS;
+    U.seg = P->t1u_seg;
+    // items divided where there are too few to balance the SMs (eight per SM);
+    // by the C pairs of the whole structure, so that neither the passes nor
+    // the plan's home atoms move the FP32 runs' ends
+    U.nsplit = std::max(1, std::min(8, (8 * hfx::sm_count() + P->nC - 1) / std::max(1, P->nC)));
+    U.cu_blk = (long long)P->np * 8 * U.GA * U.KP + 2LL * 4 * 64 * hfx::t1u_kp32(U.KP);
+    U.vu_blk = (long long)P->np * 8 * U.GA * U.VK + 2LL * 3 * 64 * ((U.VK + 31) / 32 * 32);
+    U.t1_idx = P->t1_idx;
+    U.Dh = P->sp == hfx::kSplitHalf ? P->Dsp : P->Dh;
+    if (P->sp == hfx::kSplitHalf && P->t2u) {   // Ysp is the first product's store too
+      U.Yh = P->Ysp;
+    } else {
+      X.yh_blk = 0;   // the largest key's
+      for (int a = 0; a < P->S; ++a)
+        for (int b = 0; b < P->S; ++b)
+          X.yh_blk = std::max(X.yh_blk, (long long)P->np * hfx::ao_subs(P->n_ao[a]) * ((P->n_abf[a] + 7) / 8 * 8) * 16 *
+                                            P->n_ao[b]);
+      const long long hcap0 = P->Yhcap;
+      ensure_buf(P, P->Yh, P->Yhcap, std::max(1LL, P->tot[1]) * X.yh_blk);
+      if (P->Yhcap != hcap0) ck(cudaMemsetAsync(P->Yh, 0, P->Yhcap * sizeof(uint16_t), s), "memset");
+      X.Yh = P->Yh;
+      U.Yh = P->Yh;
+      U.yh_blk = X.yh_blk;
+    }
+  };
   if (!P->np) {
     ensure_store(P, P->Yst, P->Ycap, P->tot[0]);
     D.Yst = P->Yst;
     ck(hfx::launch_ybuild(D, P->y_list, (int)P->tot[1], s), "ybuild");
   } else if (P->wide) {
     ensure_buf(P, P->Ysp, P->Yspcap, std::max(1LL, P->tot[0]));
-    ck(hfx::launch_cpieces_w(D, P->sp, P->Cw, P->cw_off, P->dCf, s), "C pieces");
+    X.y_idx = P->y_idx;
+    if (P->t1u) {
+      if (!reuse) {
+        ensure_buf(P, P->blist, P->blist_cap, P->tot[6]);
+        X.blist = P->blist;
+        ck(hfx::launch_t1_lists(D, X, 1, s), "t1 fill");
+      }
+      X.blist = P->blist;
+      t1u_plan();
+    } else {
+      ck(hfx::launch_cpieces_w(D, P->sp, P->Cw, P->cw_off, P->dCf, s), "C pieces");
+    }
     ck(hfx::launch_cpieces(D, X, P->sp, s), "cpieces");
     X.Ysp = P->Ysp;
     ensure_buf(P, P->ytab, P->ytabcap, std::max(1LL, hfx::ytab_size((int)P->tot[9], P->maxC * P->KB)));
@@ -1463,32 +1547,9 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     X.blist = P->blist;
     ck(hfx::launch_cpieces(D, X, P->sp, s), "cpieces");
     if (P->t1u) {
-      U.KP = P->t1u_KP;
-      U.G = P->t1u_G;
-      U.UB = P->t1u_UB;
-      U.NS = P->t1u_NS;
-      U.seg = P->t1u_seg;
-      // items divided where there are too few to balance the SMs (eight per SM);
-      // by the C pairs of the whole structure, so that neither the passes nor
-      // the plan's home atoms move the FP32 runs' ends
-      U.nsplit = std::max(1, std::min(8, (8 * hfx::sm_count() + P->nC - 1) / std::max(1, P->nC)));
-      U.cu_blk = (long long)P->np * 8 * U.G * U.KP + 2LL * 4 * 64 * hfx::t1u_kp32(U.KP);
-      U.vu_blk = (long long)P->np * 512 * U.G + 2LL * 3 * 4096;
-      U.t1_idx = P->t1_idx;
-      U.Dh = P->sp == hfx::kSplitHalf ? P->Dsp : P->Dh;
-      if (P->sp == hfx::kSplitHalf && P->t2u) {   // Ysp is the first product's store too
-        U.Yh = P->Ysp;
-      } else {
-        X.yh_blk = (long long)P->np * 8 * U.G * U.KP;
-        const long long hcap0 = P->Yhcap;
-        ensure_buf(P, P->Yh, P->Yhcap, std::max(1LL, P->tot[1]) * X.yh_blk);
-        if (P->Yhcap != hcap0) ck(cudaMemsetAsync(P->Yh, 0, P->Yhcap * sizeof(uint16_t), s), "memset");
-        X.Yh = P->Yh;
-        U.Yh = P->Yh;
-        U.yh_blk = X.yh_blk;
-      }
+      t1u_plan();
     }
-    X.yT_blk = P->t2u ? (long long)P->np * 8 * P->t1u_G * P->t1u_KP : (long long)P->np * P->MC * 128 * 16;
+    X.yT_blk = P->t2u ? (long long)P->np * 8 * P->t1u_GB * P->t1u_KP : (long long)P->np * P->MC * 128 * 16;
     const long long tcap0 = P->YspTcap;
     ensure_buf(P, P->YspT, P->YspTcap, std::max(1LL, P->tot[1]) * X.yT_blk);
     if (P->t2u && P->YspTcap != tcap0) ck(cudaMemsetAsync(P->YspT, 0, P->YspTcap * sizeof(uint16_t), s), "memset");
@@ -1515,12 +1576,25 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
       ensure_store(P, P->Vst, P->Vcap, ct[CT_VE]);
       D.Vst = P->Vst;
       ck(hfx::launch_vblocks(D, P->v_list + v0, (int)ct[CT_VN], s), "vblocks");
-      k1a.push_back(tm.mark());
-      if (P->wide)
+      if (P->t1u) {
+        ensure_buf(P, P->Cu, P->Cucap, std::max(1LL, ct[CT_Q]) * U.cu_blk);
+        ensure_buf(P, P->Vu, P->Vucap, std::max(1LL, ct[CT_T1]) * U.NAL * U.vu_blk);
+        U.Cu = P->Cu;
+        U.Vu = P->Vu;
+        X.Vm = nullptr;
+        const int* list = t1items + (size_t)P->t1u_subs * c0;
+        ck(hfx::launch_t1u_cstore(D, U, P->sp, list, (int)ct[CT_Q], s), "term-1 C store");
+        ck(hfx::launch_vstores(D, X, U, P->sp, P->v_list + v0, (int)ct[CT_VN], s), "V stores");
+        k1a.push_back(tm.mark());
+        ck(hfx::launch_t1_umma(D, X, U, P->sp, list, (int)ct[CT_Q], P->smem_t1u, P->d_work, P->d_err, s), "term1");
+      } else {
+        k1a.push_back(tm.mark());
+      }
+      if (P->wide && !P->t1u)
         ck(hfx::launch_term1_w(D, P->sp, P->Ysp, P->Cw, P->cw_off, P->Dw, P->dw_off, P->dCf, P->t1_list + v0,
                                (int)ct[CT_T1], P->ws, s),
            "term1");
-      else
+      else if (!P->wide)
         ck(hfx::launch_term1(D, P->t1_list + v0, (int)ct[CT_T1], P->beta_chunk, P->smem_t1, s), "term1");
       k1b.push_back(tm.mark());
       m2.push_back(k1b.back());
@@ -1543,7 +1617,7 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
         ck(hfx::launch_term2(D, P->t2_list + v0, (int)ct[CT_T2], P->alpha_chunk, P->smem_t2, s), "term2");
     } else {
       if (!P->t2u) ensure_buf(P, P->Vm, P->Vmcap, ct[CT_VM]);   // read by the warp-level kernels only
-      X.Vm = P->Vm;
+      X.Vm = P->t2u ? nullptr : P->Vm;
       // the split path evaluates V and grad V from the block model where it
       // writes the operand stores (no FP64 V blocks): one pass per needed pair
       // for both products when the tcgen05 first product runs

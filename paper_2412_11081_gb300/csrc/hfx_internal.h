@@ -147,8 +147,9 @@ struct MixPlan {
   int* qcnt;                   // [nC] kept B per (A,F)
   long long* qoff;             // [nC] offsets into blist
   int* blist;                  // V pairs (A,B) per (A,F), in V-pair order
-  // tcgen05 first product: Y^{XZ} as fp16 pieces in the core-matrix layout of
-  // ycm, yh_blk per key (by y_idx); nullptr where Ysp is that store
+  // tcgen05 first product: Y^{XZ} as fp16 pieces, yh_blk per key (by y_idx), per
+  // piece, sub of x and sub of z the row groups (g, z) of 8 alpha x 16 x in
+  // core-matrix order; nullptr where Ysp (ycm, one sub) is that store
   uint16_t* Yh = nullptr;
   long long yh_blk = 0;
   uint16_t* YspT = nullptr;    // Y^{XZ} transposed, bf16 pieces [piece][(alpha,x)][16 z] (z padded), yT_blk per key
@@ -198,16 +199,21 @@ __host__ __device__ inline int gc_off(int row, int f) {
 
 // Operand stores of the tcgen05 first-product kernel (hfx_t1umma.cu).
 struct T1UPlan {
-  uint16_t* Cu;                // per item (A,F): C pieces [8-row group][piece] x (f,a) KP in core-matrix order, then C, grad C FP32 [4][64][KP32]
+  // An item is a C pair (A,F) and sub-blocks of A's auxiliary functions
+  // (abf_sub), A's orbitals and F's orbitals (ao_sub): list entry
+  // q + (sub << kItemShift), sub = (alpha * subs(a) + a) * subs(f) + f.
+  uint16_t* Cu;                // per item: C pieces [8-row group][piece] x (f,a) KP in core-matrix order, then C, grad C FP32 [4][64][KP32]
   long long cu_blk;            // uint16 units per item
-  uint16_t* Vu;                // per term-1 V pair: V pieces [8-row group][piece] x beta 64, then grad V FP32 [3][64][64]
-  long long vu_blk;            // uint16 units per V pair
+  uint16_t* Vu;                // per term-1 V pair and alpha sub: V pieces [8-row group][piece] x beta VK, then grad V FP32 [3][64][rup32(VK)]
+  long long vu_blk;            // uint16 units per V pair and alpha sub
+  int NAL;                     // most alpha subs
   const long long* t1_idx;     // V pair -> its position in the term-1 V list
   const uint16_t* Yh;          // fp16 Y pieces (MixPlan::Yh or Ysp)
   long long yh_blk;            // its block per needed key, 0: offsets y_off (Ysp)
-  const uint16_t* Dh;          // fp16 D pieces, 512 elements per block
-  int KP;                      // columns (f,a) = 16 f + a: 16 * max n_ao
-  int G;                       // 8-row groups of the largest n_abf
+  const uint16_t* Dh;          // fp16 D pieces of the sub-blocks, offsets dsp_off
+  int KP;                      // columns (f,a) = 16 f + a of the largest sub-block of F
+  int GA, GB;                  // 8-row groups of the largest alpha sub, of the largest n_abf (beta)
+  int VK;                      // columns beta of a V row: the largest n_abf rounded up to 16
   int UB;                      // buffers of U (1 or 2)
   int NS;                      // Y ring slots (128-row tiles)
   int seg;                     // B per FP32 run of the Q accumulator
@@ -218,6 +224,10 @@ struct T1UPlan {
 constexpr int kSubShift = 30;
 __host__ __device__ inline int ao_subs(int n) { return (n + 15) >> 4; }
 __host__ __device__ inline int ao_sub(int n) { return (n + ao_subs(n) - 1) / ao_subs(n); }
+// Sub-blocks of at most 64 auxiliary functions, and their size (first product).
+__host__ __device__ inline int abf_subs(int m) { return (m + 63) >> 6; }
+__host__ __device__ inline int abf_sub(int m) { return (m + abf_subs(m) - 1) / abf_subs(m); }
+constexpr int kItemShift = 28;
 // uint16 units of one (C pair, sub) in MixPlan::Cm: the pieces, then grad C
 __host__ __device__ inline long long cm_size(int rows) { return (long long)((rows + 127) >> 7) * 2048 * (kPieces + 6); }
 
@@ -312,7 +322,11 @@ cudaError_t launch_t2_umma(const DevPlan& P, const MixPlan& X, int sp, const int
 
 // tcgen05 first exchange product (hfx_t1umma.cu): shapes n_abf <= 64, n_ao <= 16.
 long long t1u_launch_count();
-size_t t1u_smem(int KP, int G, int UB, int NS);
+size_t t1u_smem(int KP, int GA, int GB, int KB, int UB, int NS);
+int t1u_utiles(int KP, int GB);   // pairs of U tiles that fit tensor memory
+// item list entries: list[idx[q]] .. for the kept C pairs q of a slice
+cudaError_t launch_t1_items(const DevPlan& P, const int* qcnt, const long long* idx, int q0, int q1, int* list,
+                            cudaStream_t s);
 // Columns of one FP32 plane of C / grad C in the operand store (KP rounded up to 32).
 __host__ __device__ inline int t1u_kp32(int KP) { return (KP + 31) & ~31; }
 // Items of the first product in a chosen order: list[0..*n) (n read on the

@@ -1225,7 +1225,10 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
         uint16_t* Yh = X.Yh ? X.Yh + X.y_idx[ykey[i]] * X.yh_blk : nullptr;
         const bool cm = X.ycm != 0;   // Ysp rows alpha, K = (z, x) in core-matrix order
         const int KZc = 16 * nZ, m8 = (mX + 7) & ~7;
-        const long long hplane = (long long)m8 * KZc, plane = cm ? hplane : (long long)mX * nZ * PX;
+        // Yh: sub of x (hX of them) and of z first
+        const int hX = ao_sub(nX), NXS = ao_subs(nX);
+        const long long hxs = (long long)m8 * KZc, hplane = NXS * hxs, hzo = (long long)m8 * z0 * 16;
+        const long long plane = cm ? hxs : (long long)mX * nZ * PX;
         const float* eh = ep + h * 16;
         // bf16 pieces: chunk (alpha, z, half) holds x = 8 half .. 8 half + 7
         // (core-matrix order: consecutive threads take consecutive alpha, whose
@@ -1260,19 +1263,19 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
         }
         // the first product's fp16 pieces, where Ysp is not that store
         if (Yh) {
-          for (int c = et; c < nal * nZ * 2; c += 128) {
-            const int r2 = c / nal, al = alF + (c - r2 * nal), hf = r2 & 1, zz = r2 >> 1;
-            const int rl = al * nX - row0 + 8 * hf;
+          for (int c = et; c < nal * nZs * 2 * NXS; c += 128) {
+            const int r2 = c / nal, al = alF + (c - r2 * nal), hf = r2 & 1, xs = (r2 >> 1) % NXS, zz = (r2 >> 1) / NXS;
+            const int x0 = xs * hX + 8 * hf, xe = min(nX, (xs + 1) * hX), rl = al * nX - row0 + x0;
             float f0[4], f1[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              f0[k] = 8 * hf + k < nX ? eh[(rl + k) * 33 + zz] * P.sc.yh : 0.f;
-              f1[k] = 8 * hf + 4 + k < nX ? eh[(rl + 4 + k) * 33 + zz] * P.sc.yh : 0.f;
+              f0[k] = x0 + k < xe ? eh[(rl + k) * 33 + zz] * P.sc.yh : 0.f;
+              f1[k] = x0 + 4 + k < xe ? eh[(rl + 4 + k) * 33 + zz] * P.sc.yh : 0.f;
             }
             uint2 p0[NP], p1[NP];
             split4<kSplitHalf>(f0, p0);
             split4<kSplitHalf>(f1, p1);
-            uint16_t* yo = Yh + cmx(al, zz * 16 + 8 * hf, KZc);
+            uint16_t* yo = Yh + xs * hxs + hzo + cmx(al, zz * 16 + 8 * hf, 16 * nZs);
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp)
               *reinterpret_cast<uint4*>(yo + pp * hplane) = make_uint4(p0[pp].x, p0[pp].y, p1[pp].x, p1[pp].y);
@@ -1339,13 +1342,14 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
 #pragma unroll
                 for (int pp = 0; pp < NP; ++pp) Yo[pp * plane + o + (cm ? ((xp >> 3) << 6) + (xp & 7) : xp)] = 0;
             if (Yh) {
-              uint16_t* yo = Yh + cmx(al, zz * 16, KZc);
+              const int xs = x / hX, xl = x - xs * hX;
+              uint16_t* yo = Yh + xs * hxs + hzo + cmx(al, zz * 16, 16 * nZs);
               split_f<kSplitHalf>(y * P.sc.yh, pc);
 #pragma unroll
               for (int pp = 0; pp < NP; ++pp) {
-                yo[pp * hplane + ((x >> 3) << 6) + (x & 7)] = pc[pp];
-                if (x == nX - 1)
-                  for (int xp = nX; xp < 16; ++xp) yo[pp * hplane + ((xp >> 3) << 6) + (xp & 7)] = 0;
+                yo[pp * hplane + ((xl >> 3) << 6) + (xl & 7)] = pc[pp];
+                if (x == nX - 1 || xl == hX - 1)
+                  for (int xp = xl + 1; xp < 16; ++xp) yo[pp * hplane + ((xp >> 3) << 6) + (xp & 7)] = 0;
               }
             }
           }

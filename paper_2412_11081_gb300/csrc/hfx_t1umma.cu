@@ -122,33 +122,57 @@ __device__ __forceinline__ void ep_at1(int w, int& alpha, int& col) {
   col = 32 * j + 16 * ((l >> 3) & 1) + 4 * t + k;
 }
 
-// Item kk (C pair q = list[kk]): the pieces of C_AF, per 8 rows alpha first
-// piece 0 and then piece 1, (f,a) (KP) columns in core-matrix order, then C
-// and grad C in FP32 as four planes of 64 x KP32 (KP rounded up to 32) in
-// epilogue load order (ep_at1).  Zero padded.  Each plane of the C pair
-// ([(alpha,a)][f]) is evaluated from the block model into shared memory as
-// FP32; the outputs are written in storage order, four elements per thread.
-constexpr int kCStoreSmem = 64 * 16 * 16 * 4;   // one plane of n_abf <= 64, n_ao <= 16
+// An item's sub-blocks: alpha al0 .. + mA, a a0 .. + nA, f f0 .. + nF of its C pair.
+struct Sub {
+  int al0, mA, a0, nA, f0, nF, as, fs, als;
+};
+__device__ __forceinline__ Sub item_sub(int sub, int mA, int nA, int nF) {
+  const int sf = ao_subs(nF), sa = ao_subs(nA), hf = ao_sub(nF), ha = ao_sub(nA), hm = abf_sub(mA);
+  Sub r;
+  r.fs = sub % sf;
+  r.as = (sub / sf) % sa;
+  r.als = sub / sf / sa;
+  r.al0 = r.als * hm;
+  r.a0 = r.as * ha;
+  r.f0 = r.fs * hf;
+  r.mA = min(hm, mA - r.al0);
+  r.nA = min(ha, nA - r.a0);
+  r.nF = min(hf, nF - r.f0);
+  return r;
+}
+
+// Item kk: the pieces of its part of C_AF, per 8 rows alpha first piece 0 and
+// then piece 1, (f,a) (KP) columns in core-matrix order, then C and grad C in
+// FP32 as four planes of 64 x KP32 (KP rounded up to 32) in epilogue load
+// order (ep_at1).  Zero padded.  Each plane ([(alpha,a)][f]) is evaluated from
+// the block model into shared memory as FP32; the outputs are written in
+// storage order, four elements per thread.
+constexpr int kCStoreSmem = 64 * 16 * 16 * 4;   // one plane of 64 alpha, 16 a, 16 f
 
 template <int SP>
 __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
   extern __shared__ float cs[];
   const int KP = U.KP, KP32 = t1u_kp32(KP), PL = 64 * KP32;
   for (int kk = blockIdx.x; kk < n; kk += gridDim.x) {
-    const int q = list[kk];
+    const int q = list[kk] & ((1 << kItemShift) - 1);
     const int A = P.c_home[q], F = P.c_j[q];
     const int sA = P.species[A];
-    const int nA = P.n_ao[sA], mA = P.n_abf[sA], nF = P.n_ao[P.species[F]];
+    const int nAt = P.n_ao[sA], nFt = P.n_ao[P.species[F]];
+    const Sub sb = item_sub(list[kk] >> kItemShift, P.n_abf[sA], nAt, nFt);
+    const int mA = sb.mA, nA = sb.nA, nF = sb.nF;
     const int ncq = mA * nA * nF, g8 = (mA + 7) >> 3;
     uint16_t* out = U.Cu + (long long)kk * U.cu_blk;
-    float* pl = reinterpret_cast<float*>(out + (long long)NP * U.G * 8 * KP);
+    float* pl = reinterpret_cast<float*>(out + (long long)NP * U.GA * 8 * KP);
     float scf[8];   // C = G f + G' fa, grad C = G g + G' ga (block model, FP32 as k_cpieces)
 #pragma unroll
     for (int k = 0; k < 8; ++k) scf[k] = (float)P.c_sc[8 * (long long)q + k];
     const long long go = P.G_off[sA * P.S + P.species[F]];
     for (int c = 0; c < 4; ++c) {
       __syncthreads();
-      for (int e = threadIdx.x; e < ncq; e += blockDim.x) cs[e] = model::c_value_f(P, scf, go, e, c);
+      for (int e = threadIdx.x; e < ncq; e += blockDim.x) {
+        const int r = e / nF, f = e - r * nF, al = r / nA, a = r - al * nA;
+        cs[e] = model::c_value_f(P, scf, go, ((sb.al0 + al) * nAt + sb.a0 + a) * nFt + sb.f0 + f, c);
+      }
       __syncthreads();
       auto val = [&](int al, int col) -> float {
         const int f = col >> 4, a = col & 15;
@@ -190,19 +214,26 @@ __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
 //   k_t2_umma at t2_slot[p]: the pieces as [piece][alpha 64][beta 64] and V,
 //   grad V in four planes (ep_at).
 // Outputs are written in storage order, four elements per thread.
-constexpr int kVStoreSmem = 4 * 64 * 64 * 4;
+// Rows alpha are taken 64 (abf_sub) at a time; the second product's stores
+// have no more than that.
+size_t vstore_smem(int max_abf) { return (size_t)4 * 64 * max_abf * sizeof(float); }
 
 template <int SP>
 __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int n) {
-  extern __shared__ float vsm[];   // [4][mA * mB]: V, grad V
+  extern __shared__ float vsm[];   // [4][mA * mB]: V, grad V of the rows in hand
   for (int k = blockIdx.x; k < n; k += gridDim.x) {
     const int p = list[k];
     const int sA = P.species[P.v_home[p]], sB = P.species[P.v_j[p]];
-    const int mA = P.n_abf[sA], mB = P.n_abf[sB], MB = rup16(mB), nv = mA * mB;
+    const int mAt = P.n_abf[sA], mB = P.n_abf[sB], MB = rup16(mB), hm = abf_sub(mAt);
     double h, g[3];
     model::v_pair(P, p, h, g);   // V = M h, grad V = M g (block model), in FP32
     const float hf = (float)h, g0 = (float)g[0], g1 = (float)g[1], g2 = (float)g[2];
-    const float* M = P.Mf + P.M_off[sA * P.S + sB];
+    bool t1 = false;
+#pragma unroll
+    for (int w = 0; w < kMaskWords; ++w) t1 = t1 || P.v_mask[(long long)p * kMaskWords + w] != 0u;
+    for (int als = 0, al0 = 0; al0 < mAt; ++als, al0 += hm) {
+    const int mA = min(hm, mAt - al0), nv = mA * mB;
+    const float* M = P.Mf + P.M_off[sA * P.S + sB] + al0 * mB;
     __syncthreads();
     for (int e = threadIdx.x; e < nv; e += blockDim.x) {
       const float m = M[e];
@@ -212,9 +243,8 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
       vsm[3 * nv + e] = m * g2;
     }
     __syncthreads();
-    // second-product store of the warp-level R2 / Z kernel (none with the
-    // tcgen05 one, X.Vz: nothing reads it then)
-    if (!X.Vz) {
+    // second-product store of the warp-level R2 / Z kernel, where that runs
+    if (X.Vm) {
       uint16_t* out = X.Vm + X.vm_off[p];
       for (int e4 = threadIdx.x; e4 < mA * MB / 4; e4 += blockDim.x) {
         const int e = 4 * e4, al = e / MB, be = e - al * MB;
@@ -229,39 +259,35 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
       float* v32 = reinterpret_cast<float*>(out + (long long)NP * mA * MB);
       for (int e = threadIdx.x; e < 4 * nv; e += blockDim.x) v32[e] = vsm[e];
     }
-    // first-product store
-    bool t1 = false;
-#pragma unroll
-    for (int w = 0; w < kMaskWords; ++w) t1 = t1 || P.v_mask[(long long)p * kMaskWords + w] != 0u;
-    // the tcgen05 stores: the first product's (U.Vu, per first-product pair:
-    // pieces and the three grad V planes) and the second product's (X.Vz, per
-    // second-product pair: pieces and the four planes V, grad V)
+    // the tcgen05 stores: the first product's (U.Vu, per first-product pair and
+    // alpha sub: pieces and the three grad V planes) and the second product's
+    // (X.Vz, per second-product pair: pieces and the four planes V, grad V)
     for (int st = 0; st < 2; ++st) {
       uint16_t* vu = nullptr;
-      if (st == 0 && U.Vu && t1) vu = U.Vu + U.t1_idx[p] * U.vu_blk;
+      if (st == 0 && U.Vu && t1) vu = U.Vu + (U.t1_idx[p] * U.NAL + als) * U.vu_blk;
       if (st == 1 && X.Vz && P.v_t2[p]) vu = X.Vz + X.t2_slot[p] * X.vz_blk;
       if (!vu) continue;
-      for (int t4 = threadIdx.x; t4 < 1024; t4 += blockDim.x) {   // core-matrix order, 4 columns per thread
-        const int t = 4 * t4;
-        const int al = ((t >> 9) << 3) + ((t >> 3) & 7), be = (((t >> 6) & 7) << 3) + (t & 7);
+      const int VK = st == 0 ? U.VK : 64, G = st == 0 ? (mA + 7) >> 3 : 8, VC = (VK + 31) & ~31;
+      for (int t4 = threadIdx.x; t4 < G * 2 * VK; t4 += blockDim.x) {   // core-matrix order, 4 columns per thread
+        const int g8 = t4 / (2 * VK), t = 4 * (t4 - g8 * 2 * VK);
+        const int al = g8 * 8 + ((t >> 3) & 7), be = ((t >> 6) << 3) + (t & 7);
         float x[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) x[j] = (al < mA && be + j < mB) ? vsm[al * mB + be + j] * pscale<SP>(P.sc.v) : 0.f;
         uint2 pc[NP];
         split4<SP>(x, pc);
 #pragma unroll
-        for (int pp = 0; pp < NP; ++pp) {
-          const int o = st == 0 ? ((t >> 9) * NP + pp) * 512 + (t & 511) : pp * 4096 + t;
-          if (st == 1 || (t >> 9) < U.G) *reinterpret_cast<uint2*>(vu + o) = pc[pp];
-        }
+        for (int pp = 0; pp < NP; ++pp)
+          *reinterpret_cast<uint2*>(vu + (st == 0 ? (g8 * NP + pp) * 8 * VK + t : pp * 4096 + g8 * 512 + t)) = pc[pp];
       }
-      float* pl = reinterpret_cast<float*>(vu + (st == 0 ? NP * 512 * U.G : NP * 4096));
+      float* pl = reinterpret_cast<float*>(vu + (st == 0 ? NP * 8 * VK * U.GA : NP * 4096));
       const int c0 = st == 0 ? 1 : 0;   // first plane: grad V (first product) or V (second)
-      for (int w4 = threadIdx.x; w4 < (4 - c0) * 1024; w4 += blockDim.x) {   // epilogue load order
-        const int c = c0 + (w4 >> 10);
+      const int PL4 = 16 * VC;          // float4 per plane
+      for (int w4 = threadIdx.x; w4 < (4 - c0) * PL4; w4 += blockDim.x) {   // epilogue load order
+        const int c = c0 + w4 / PL4;
         int al, be;
-        if (st == 0) ep_at1(4 * (w4 & 1023), al, be);
-        else ep_at(4 * (w4 & 1023), al, be);
+        if (st == 0) ep_at1(4 * (w4 % PL4), al, be);
+        else ep_at(4 * (w4 % PL4), al, be);
         float4 o;
         o.x = (al < mA && be < mB) ? vsm[c * nv + al * mB + be] : 0.f;
         o.y = (al < mA && be + 1 < mB) ? vsm[c * nv + al * mB + be + 1] : 0.f;
@@ -269,6 +295,7 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
         o.w = (al < mA && be + 3 < mB) ? vsm[c * nv + al * mB + be + 3] : 0.f;
         *reinterpret_cast<float4*>(pl + 4 * w4) = o;
       }
+    }
     }
   }
 }
@@ -281,7 +308,7 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
 // With asc = 1 the same sort orders the items by key[q] ascending (the
 // order by F: items of one F, which share many Y^{BF} blocks, run together).
 __device__ __forceinline__ int lpt_bucket(const int* key, int q, int asc) {
-  const int k = min(key[q], kLptBuckets - 1);
+  const int k = min(key[q & ((1 << kItemShift) - 1)], kLptBuckets - 1);   // (a list entry: C pair and sub)
   return asc ? k : kLptBuckets - 1 - k;
 }
 
@@ -327,12 +354,12 @@ __global__ void k_lpt_scatter(const int* key, int asc, const int* list, const lo
 
 // ------------------------------------------------------------------- kernel
 // Sizes of one launch, shared by the kernel and the host: KP columns
-// (f, a) = 16 f + a, G row groups of 8 alpha or beta (n_abf of the largest
-// species), UB buffers of U, NS slots of the Y ring.
-__host__ __device__ inline uint32_t t1_cbytes(int KP, int G) { return (uint32_t)G * 2u * 16u * KP; }   // C, or one buffer of U
-__host__ __device__ inline uint32_t t1_vbytes(int G) { return (uint32_t)G * 2048u; }
-__host__ __device__ inline uint32_t t1_base(int KP, int G, int UB) {
-  return t1_cbytes(KP, G) * (1 + UB) + 2 * t1_vbytes(G) + kND * 1024u;
+// (f, a) = 16 f + a, GA and GB row groups of 8 alpha and 8 beta, VK columns
+// beta of V, KB sub-blocks of b, UB buffers of U, NS slots of the Y ring.
+__host__ __device__ inline uint32_t t1_ubytes(int KP, int G) { return (uint32_t)G * 2u * 16u * KP; }   // C, or one buffer of U
+__host__ __device__ inline uint32_t t1_vbytes(int GA, int VK) { return (uint32_t)GA * 2u * 16u * VK; }
+__host__ __device__ inline uint32_t t1_base(int KP, int GA, int GB, int KB, int UB) {
+  return t1_ubytes(KP, GA) + UB * t1_ubytes(KP, GB) + 2 * t1_vbytes(GA, (8 * GB + 15) & ~15) + kND * KB * 1024u;
 }
 // Tensor-memory columns: Q at 0, R from the next multiple of 32, then the U tiles in pairs of 32 columns.
 __host__ __device__ inline int t1_rcol(int KP) { return (KP + 31) & ~31; }
@@ -344,20 +371,21 @@ __host__ __device__ inline int t1_utiles(int KP, int G) {
 template <int SP>
 __global__ void __launch_bounds__(kThreads, 1)
     k_t1_umma(DevPlan P, MixPlan X, T1UPlan U, const int* qlist, int n_list, int* work, int* err) {
-  const int KP = U.KP, KP32 = t1u_kp32(KP), G = U.G, NS = U.NS, UB = U.UB, SEG = U.seg, nsplit = U.nsplit;
-  const int NT = t1_utiles(KP, G), n_units = n_list * nsplit;
+  const int KP = U.KP, KP32 = t1u_kp32(KP), GB = U.GB, VK = U.VK, NS = U.NS, UB = U.UB, SEG = U.seg, nsplit = U.nsplit;
+  const int NT = t1_utiles(KP, GB), n_units = n_list * nsplit;
   const uint32_t rowg = 16u * KP;                    // bytes of one 8-row group of a C or U piece
-  const uint32_t CB = t1_cbytes(KP, G), VB = t1_vbytes(G);
+  const uint32_t vrowg = 16u * VK;                   // and of V
+  const uint32_t CB = t1_ubytes(KP, U.GA), UBY = t1_ubytes(KP, GB), VB = t1_vbytes(U.GA, VK), DB = X.KB * 1024u;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t b_yf[kMaxNS], b_ye[kMaxNS], b_cf, b_ce, b_vf[2], b_ve[2], b_df[kND], b_de[kND],
       b_tf[kMaxUT], b_te[kMaxUT], b_uf[2], b_ue[2], b_rf, b_re, b_qf, b_qe, b_if[kItemRing], b_ie[kItemRing], b_done[2];
-  __shared__ int4 s_item[kItemRing];   // a unit: item kk (-1: no more), C pair q, its B [lo, hi) of the list at X.qoff
+  __shared__ int4 s_item[kItemRing];   // a unit: item kk (-1: no more), its list entry, its B [lo, hi) of the list at X.qoff
   __shared__ uint32_t tmem_base;
   __shared__ int s_abort;
   volatile int* abort_flag = &s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   auto sa = [](const void* p) { return (uint32_t)__cvta_generic_to_shared(p); };
-  const uint32_t Cs = sa(smem_raw), Us = Cs + CB, Vs = Us + UB * CB, Ds = Vs + 2 * VB, Ys = Ds + kND * 1024u;
+  const uint32_t Cs = sa(smem_raw), Us = Cs + CB, Vs = Us + UB * UBY, Ds = Vs + 2 * VB, Ys = Ds + kND * DB;
   const uint32_t yf = sa(b_yf), ye = sa(b_ye), cf = sa(&b_cf), ce = sa(&b_ce), vf = sa(b_vf), ve = sa(b_ve),
                  df = sa(b_df), de = sa(b_de), tf = sa(b_tf), te = sa(b_te), uf = sa(b_uf), ue = sa(b_ue),
                  rf = sa(&b_rf), re = sa(&b_re), qf = sa(&b_qf), qe = sa(&b_qe), itf = sa(b_if), ite = sa(b_ie),
@@ -408,11 +436,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t T = tmem_base, TR = T + t1_rcol(KP), TU = TR + 16u * G;
+  const uint32_t T = tmem_base, TR = T + t1_rcol(KP), TU = TR + 16u * GB;
   // Next unit of the ring for a role (one reader per warp; lane 0 releases
   // the slot); kk < 0 marks the end.  Every lane of the warp calls it.
   struct Unit {
-    int kk, q, lo, hi;
+    int kk, code, lo, hi;
+    __device__ int q() const { return code & ((1 << kItemShift) - 1); }
+    __device__ int sub() const { return code >> kItemShift; }
   };
   auto next_unit = [&](Ring& r) -> Unit {
     Unit u{-1, 0, 0, 0};
@@ -434,40 +464,48 @@ __global__ void __launch_bounds__(kThreads, 1)
     // slot, the two pieces copied by lanes 0 and 1.
     Ring ik, y;
     for (Unit it = next_unit(ik); it.kk >= 0 && !aborted(abort_flag); it = next_unit(ik)) {
-      const int F = P.c_j[it.q];
-      const int nF = P.n_ao[P.species[F]];
-      const int* Rf = P.c_R + 3 * it.q;
-      const long long b0 = X.qoff[it.q];
+      const int q = it.q(), F = P.c_j[q], sA = P.species[P.c_home[q]];
+      const int nFt = P.n_ao[P.species[F]];
+      const Sub sb = item_sub(it.sub(), P.n_abf[sA], P.n_ao[sA], nFt);
+      const int* Rf = P.c_R + 3 * q;
+      const long long b0 = X.qoff[q];
       for (int i0 = it.lo; i0 < it.hi && !aborted(abort_flag); i0 += 32) {
         long long yo = 0;
-        int ng = 0;
+        int g8 = 0, nbs = 0;   // 8-row groups of beta, subs of b
         if (i0 + lane < it.hi) {
           const int p = X.blist[b0 + i0 + lane];
           const int b = P.v_j[p];
           const int* Rb = P.v_R + 3 * p;
           const int yc = ylut_get(P, b, F, Rf[0] - Rb[0], Rf[1] - Rb[1], Rf[2] - Rb[2]);
           yo = yc < 0 ? -1 : U.yh_blk ? X.y_idx[yc] * U.yh_blk : P.y_off[yc];
-          ng = ((P.n_abf[P.species[b]] + 7) >> 3) * nF;
+          g8 = (P.n_abf[P.species[b]] + 7) >> 3;
+          nbs = ao_subs(P.n_ao[P.species[b]]);
         }
         const int nb = min(32, it.hi - i0);
         for (int j = 0; j < nb; ++j) {
           const long long yoj = __shfl_sync(0xffffffffu, yo, j);
-          const int ngj = __shfl_sync(0xffffffffu, ng, j);
+          const int g8j = __shfl_sync(0xffffffffu, g8, j), nbj = __shfl_sync(0xffffffffu, nbs, j);
+          const int ngj = g8j * sb.nF;
+          const long long xs1 = (long long)g8j * nFt * 128;   // a sub of b; the piece holds nbj of them
           if (yoj < 0) *abort_flag = 1;   // a kept triplet always has its Y block
-          for (int r0 = 0; r0 < ngj; r0 += kYG, y.next(NS)) {
-            const int s = y.s;
+          for (int r0 = 0; r0 < ngj; r0 += kYG) {
             const uint32_t bytes = 256u * (uint32_t)min(kYG, ngj - r0);
-            bool ok = true;
-            if (lane == 0) {
-              ok = !aborted(abort_flag) && mbar_wait(ye + 8 * s, y.ph ^ 1);
-              if (ok) mbar_expect_tx(yf + 8 * s, 2 * bytes);
-              else *abort_flag = 1;
+            for (int bs = 0; bs < nbj; ++bs, y.next(NS)) {
+              const int s = y.s;
+              bool ok = true;
+              if (lane == 0) {
+                ok = !aborted(abort_flag) && mbar_wait(ye + 8 * s, y.ph ^ 1);
+                if (ok) mbar_expect_tx(yf + 8 * s, 2 * bytes);
+                else *abort_flag = 1;
+              }
+              ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+              if (!ok) break;
+              if (lane < 2)
+                bulk_g2s(Ys + s * kYSlot + lane * kYPiece,
+                         U.Yh + yoj + (lane * nbj + bs) * xs1 + (long long)g8j * sb.f0 * 128 + r0 * 128, bytes,
+                         yf + 8 * s);
             }
-            ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
-            if (!ok) break;
-            if (lane < 2)
-              bulk_g2s(Ys + s * kYSlot + lane * kYPiece, U.Yh + yoj + (long long)lane * ngj * 128 + r0 * 128, bytes,
-                       yf + 8 * s);
+            if (__shfl_sync(0xffffffffu, (int)aborted(abort_flag), 0)) break;
           }
           if (__shfl_sync(0xffffffffu, (int)aborted(abort_flag), 0)) break;
         }
@@ -483,20 +521,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool pub_done = false;
     auto publish = [&]() {
       volatile int* v = reinterpret_cast<volatile int*>(&s_item[pub.s]);
-      v[0] = -1;   // best effort on a timeout: readers also stop on the flag
-      if (!mbar_wait(ite + 8 * pub.s, pub.ph ^ 1)) {
+      if (!mbar_wait(ite + 8 * pub.s, pub.ph ^ 1)) {   // every reader has taken the slot's last unit
         *abort_flag = 1;
         pub_done = true;
         return;
       }
+      v[0] = -1;
       pub_done = true;
       while (!aborted(abort_flag)) {   // units without a B (fewer B than parts) are passed over
         const int u = atomicAdd(work, 1);
         if (u >= n_units) break;
-        const int kk = u / nsplit, part = u - kk * nsplit, q = qlist[kk], n = X.qcnt[q];
+        const int kk = u / nsplit, part = u - kk * nsplit, code = qlist[kk], n = X.qcnt[code & ((1 << kItemShift) - 1)];
         const int lo = n * part / nsplit, hi = n * (part + 1) / nsplit;
         if (hi <= lo) continue;
-        v[1] = q;
+        v[1] = code;
         v[2] = lo;
         v[3] = hi;
         v[0] = kk;
@@ -521,14 +559,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       own.next(kItemRing);
       u.kk = __shfl_sync(0xffffffffu, u.kk, 0);
-      u.q = __shfl_sync(0xffffffffu, u.q, 0);
+      u.code = __shfl_sync(0xffffffffu, u.code, 0);
       u.lo = __shfl_sync(0xffffffffu, u.lo, 0);
       u.hi = __shfl_sync(0xffffffffu, u.hi, 0);
       return u;
     };
     for (Unit it = own_unit(); it.kk >= 0 && !aborted(abort_flag); it = own_unit(), ++it_n) {
-      const long long b0 = X.qoff[it.q];
-      const uint32_t gA = (uint32_t)(P.n_abf[P.species[P.c_home[it.q]]] + 7) >> 3;
+      const int q = it.q(), sA = P.species[P.c_home[q]];
+      const Sub sb = item_sub(it.sub(), P.n_abf[sA], P.n_ao[sA], P.n_ao[P.species[P.c_j[q]]]);
+      const long long b0 = X.qoff[q];
+      const uint32_t gA = (uint32_t)(sb.mA + 7) >> 3;
       if (lane == 0) {
         if (!pub_done) publish();
         if (it_n >= 1 && !mbar_wait(ce, (it_n - 1) & 1)) *abort_flag = 1;
@@ -541,28 +581,31 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       for (int i0 = it.lo; i0 < it.hi && !aborted(abort_flag); i0 += 32) {
         long long vo = 0, dofs = 0;
+        int nbs = 0;
         if (i0 + lane < it.hi) {
           const int p = X.blist[b0 + i0 + lane];
-          vo = U.t1_idx[p] * U.vu_blk;
+          vo = (U.t1_idx[p] * U.NAL + sb.als) * U.vu_blk;
           const int di = P.v_didx[p];
-          dofs = di >= 0 ? (long long)di * 512 : -1;   // a kept triplet always has its D block
+          nbs = ao_subs(P.n_ao[P.species[P.v_j[p]]]);
+          dofs = di >= 0 ? X.dsp_off[di] + sb.as * nbs * 512 : -1;   // a kept triplet always has its D block
         }
         const int nb = min(32, it.hi - i0);
         for (int j = 0; j < nb; ++j) {
           const long long voj = __shfl_sync(0xffffffffu, vo, j);
           const long long doj = __shfl_sync(0xffffffffu, dofs, j);
+          const uint32_t dbytes = 1024u * (uint32_t)__shfl_sync(0xffffffffu, nbs, j);   // the row a of sub-blocks
           if (lane == 0 && doj < 0) *abort_flag = 1;
           if (lane == 0 && !aborted(abort_flag)) {
             bool ok = mbar_wait(de + 8 * d.s, d.ph ^ 1);
             if (ok) {
-              mbar_expect_tx(df + 8 * d.s, 1024u);
-              bulk_g2s(Ds + d.s * 1024u, U.Dh + doj, 1024u, df + 8 * d.s);
+              mbar_expect_tx(df + 8 * d.s, dbytes);
+              bulk_g2s(Ds + d.s * DB, U.Dh + doj, dbytes, df + 8 * d.s);
               d.next(kND);
             }
             ok = ok && mbar_wait(ve + 8 * v.s, v.ph ^ 1);
             if (ok) {
-              mbar_expect_tx(vf + 8 * v.s, gA * 2048u);
-              bulk_g2s(Vs + v.s * VB, U.Vu + voj, gA * 2048u, vf + 8 * v.s);
+              mbar_expect_tx(vf + 8 * v.s, gA * 2u * vrowg);
+              bulk_g2s(Vs + v.s * VB, U.Vu + voj, gA * 2u * vrowg, vf + 8 * v.s);
               v.next(2);
             } else {
               *abort_flag = 1;
@@ -587,34 +630,42 @@ __global__ void __launch_bounds__(kThreads, 1)
     Ring ik, y, t, d;
     bool ok = true;
     for (Unit it = next_unit(ik); it.kk >= 0; it = next_unit(ik)) {
-      const int nF = P.n_ao[P.species[P.c_j[it.q]]];
-      const long long b0 = X.qoff[it.q];
+      const int q = it.q(), sA = P.species[P.c_home[q]];
+      const int nF = item_sub(it.sub(), P.n_abf[sA], P.n_ao[sA], P.n_ao[P.species[P.c_j[q]]]).nF;
+      const long long b0 = X.qoff[q];
       for (int i0 = it.lo; i0 < it.hi; i0 += 32) {
-        int ng = 0;
-        if (i0 + lane < it.hi) ng = ((P.n_abf[P.species[P.v_j[X.blist[b0 + i0 + lane]]]] + 7) >> 3) * nF;
+        int ng = 0, nbs = 0;
+        if (i0 + lane < it.hi) {
+          const int sB = P.species[P.v_j[X.blist[b0 + i0 + lane]]];
+          ng = ((P.n_abf[sB] + 7) >> 3) * nF;
+          nbs = ao_subs(P.n_ao[sB]);
+        }
         const int nb = min(32, it.hi - i0);
         for (int j = 0; j < nb; ++j) {
-          const int ngj = __shfl_sync(0xffffffffu, ng, j);
+          const int ngj = __shfl_sync(0xffffffffu, ng, j), nbj = __shfl_sync(0xffffffffu, nbs, j);
           if (lane == 0 && ok) {
             ok = !aborted(abort_flag) && mbar_wait(df + 8 * d.s, d.ph);
-            const uint64_t dD = sdesc2(Ds + d.s * 1024u, 128, 256);
             for (int r0 = 0; r0 < ngj && ok; r0 += kYG) {
-              ok = mbar_wait(yf + 8 * y.s, y.ph) && mbar_wait(te + 8 * t.s, t.ph ^ 1);
-              if (!ok) break;
-              tc_fence_after();
-              const uint64_t dY = sdesc2(Ys + y.s * kYSlot, 128, 256);
               const uint32_t tu = TU + 32u * t.s;
               const bool two = r0 + 16 < ngj;
-              umma_f16(tu, dY, dD + 32, idU, 0u);                            // Y0 D1 (a piece of D: 512 bytes)
-              if (two) umma_f16(tu + 16, dY + 256, dD + 32, idU, 0u);        // (the second tile: 4096 bytes on)
-              umma_f16(tu, dY + (kYPiece >> 4), dD, idU, 1u);                // Y1 D0
-              if (two) umma_f16(tu + 16, dY + 256 + (kYPiece >> 4), dD, idU, 1u);
-              umma_f16(tu, dY, dD, idU, 1u);                                 // Y0 D0
-              if (two) umma_f16(tu + 16, dY + 256, dD, idU, 1u);
-              umma_commit(tf + 8 * t.s);
-              umma_commit(ye + 8 * y.s);
-              y.next(NS);
-              t.next(NT);
+              ok = mbar_wait(te + 8 * t.s, t.ph ^ 1);
+              for (int bs = 0; bs < nbj && ok; ++bs) {
+                ok = mbar_wait(yf + 8 * y.s, y.ph);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t dD = sdesc2(Ds + d.s * DB + bs * 1024u, 128, 256);
+                const uint64_t dY = sdesc2(Ys + y.s * kYSlot, 128, 256);
+                umma_f16(tu, dY, dD + 32, idU, bs > 0);                        // Y0 D1 (a piece of D: 512 bytes)
+                if (two) umma_f16(tu + 16, dY + 256, dD + 32, idU, bs > 0);    // (the second tile: 4096 bytes on)
+                umma_f16(tu, dY + (kYPiece >> 4), dD, idU, 1u);                // Y1 D0
+                if (two) umma_f16(tu + 16, dY + 256 + (kYPiece >> 4), dD, idU, 1u);
+                umma_f16(tu, dY, dD, idU, 1u);                                 // Y0 D0
+                if (two) umma_f16(tu + 16, dY + 256, dD, idU, 1u);
+                if (bs == nbj - 1) umma_commit(tf + 8 * t.s);
+                umma_commit(ye + 8 * y.s);
+                y.next(NS);
+              }
+              if (ok) t.next(NT);
             }
             if (ok) umma_commit(de + 8 * d.s);
             else *abort_flag = 1;
@@ -638,16 +689,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     // one instruction per k step makes all four piece products, and R is the
     // sum over the two row groups of an alpha and the two columns of a beta.
     // Q goes first: meanwhile the epilogue empties the accumulator of the R before.
-    const uint32_t idR = idesc_split<SP>(128, 16 * G, 0);
+    const uint32_t idR = idesc_split<SP>(128, 16 * GB, 0);
     const uint64_t dC = sdesc2(Cs, 128, rowg);
-    const uint64_t kbB = (uint64_t)(2 * rowg) >> 4, pB = (uint64_t)(CB >> 1) >> 4;
+    const uint64_t kbB = (uint64_t)(2 * rowg) >> 4, pB = (uint64_t)(UBY >> 1) >> 4;
     uint32_t rp = 1, qp = 1, it_n = 0;   // phases of the free accumulators
     Ring ik, ub, v;
     bool ok = true;
     for (Unit it = next_unit(ik); it.kk >= 0; it = next_unit(ik), ++it_n) {
-      const int nF = P.n_ao[P.species[P.c_j[it.q]]];
+      const int q = it.q(), sA = P.species[P.c_home[q]];
+      const int nF = item_sub(it.sub(), P.n_abf[sA], P.n_ao[sA], P.n_ao[P.species[P.c_j[q]]]).nF;
       const uint32_t idQ = idesc_split<SP>(128, 16 * nF, 1);
-      const long long b0 = X.qoff[it.q];
+      const long long b0 = X.qoff[q];
       int run = 0;
       for (int i0 = it.lo; i0 < it.hi; i0 += 32) {
         int nk_l = 0;
@@ -662,7 +714,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                  (!first || mbar_wait(qe, qp));
             if (ok) {
               tc_fence_after();
-              const uint64_t dV = sdesc2(Vs + v.s * VB, 128, 1024), dU = sdesc2(Us + ub.s * CB, rowg, 128);
+              const uint64_t dV = sdesc2(Vs + v.s * VB, 128, vrowg), dU = sdesc2(Us + ub.s * UBY, rowg, 128);
               for (int kb = 0; kb < nk; ++kb) {
                 umma_f16(T, dV + 16u * kb, dU + pB + kbB * kb, idQ, (first && kb == 0) ? 0u : 1u);
                 umma_f16(T, dV + 16u * kb, dU + kbB * kb, idQ, 1u);
@@ -677,7 +729,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             if (ok) {
               tc_fence_after();
-              const uint64_t dU = sdesc2(Us + ub.s * CB, 128, rowg);
+              const uint64_t dU = sdesc2(Us + ub.s * UBY, 128, rowg);
               for (int f = 0; f < nF; ++f) umma_f16(TR, dC + 16u * f, dU + 16u * f, idR, f > 0 ? 1u : 0u);
               umma_commit(rf);
               umma_commit(ue + 8 * ub.s);
@@ -725,15 +777,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     };
+    const int VP4 = 16 * ((VK + 31) & ~31);   // float4 per plane of grad V
     uint32_t rb = 0, seg = 0;
     Ring ik;
     unsigned long long fl = 0;
     bool ok = true;
     for (Unit it = next_unit(ik); it.kk >= 0 && ok; it = next_unit(ik)) {
-      const int A = P.c_home[it.q], F = P.c_j[it.q];
-      const int sA = P.species[A];
-      const int nA = P.n_ao[sA], mA = P.n_abf[sA], nF = P.n_ao[P.species[F]];
-      const long long b0 = X.qoff[it.q];
+      const int q = it.q(), sA = P.species[P.c_home[q]];
+      const Sub sb = item_sub(it.sub(), P.n_abf[sA], P.n_ao[sA], P.n_ao[P.species[P.c_j[q]]]);
+      const int nA = sb.nA, mA = sb.mA, nF = sb.nF;
+      const long long b0 = X.qoff[q];
       const float* Cf = reinterpret_cast<const float*>(U.Cu + (long long)it.kk * U.cu_blk + (CB >> 1));
       int run = 0;
       for (int i0 = it.lo; i0 < it.hi && ok; i0 += 32) {
@@ -741,10 +794,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         long long vo_l = 0;
         if (i0 + lane < it.hi) {
           p_l = X.blist[b0 + i0 + lane];
-          const int sb = P.species[P.v_j[p_l]];
-          mB_l = P.n_abf[sb];
-          nB_l = P.n_ao[sb];
-          vo_l = U.t1_idx[p_l] * U.vu_blk;
+          const int s_b = P.species[P.v_j[p_l]];
+          mB_l = P.n_abf[s_b];
+          nB_l = P.n_ao[s_b];
+          vo_l = (U.t1_idx[p_l] * U.NAL + sb.als) * U.vu_blk;
         }
         const int nb = min(32, it.hi - i0);
         for (int j = 0; j < nb && ok; ++j) {
@@ -753,50 +806,71 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int mB = __shfl_sync(0xffffffffu, mB_l, j);
           const long long vo = __shfl_sync(0xffffffffu, vo_l, j);
           const bool last = ++run == SEG || i0 + j == it.hi - 1;
-          // ---- R_B -> g^V_AB (the grad V values of this lane's columns
-          // beta = cb .. cb + 15 are fetched before the wait: they do not
-          // depend on R, and their latency is the longest of the epilogue)
-          const bool any = qd * 16 < mA && 32 * h < mB;
-          const int cb = 32 * h + 16 * pc;
-          const bool act = alpha < mA && cb < mB;
+          // ---- R_B -> g^V_AB, 32 columns beta at a time (two halves of the
+          // warps; n_abf <= 64: one turn).  The grad V values of this lane's
+          // columns cb .. cb + 15 are fetched before the wait: they do not
+          // depend on R, and their latency is the longest of the epilogue.
+          const float4* dV4 = reinterpret_cast<const float4*>(U.Vu + vo + (VB >> 1)) + qd * 32 + lane;
           float4 w[3][4];
+          float x[16], gv[3] = {0.f, 0.f, 0.f};
+          bool act = alpha < mA && 32 * h + 16 * pc < mB;
           if (act) {
-            const float4* dV4 = reinterpret_cast<const float4*>(U.Vu + vo + (VB >> 1)) + h * 512 + qd * 32 + lane;
 #pragma unroll
             for (int c = 0; c < 3; ++c)
 #pragma unroll
-              for (int t4 = 0; t4 < 4; ++t4) w[c][t4] = dV4[c * 1024 + t4 * 128];
+              for (int t4 = 0; t4 < 4; ++t4) w[c][t4] = dV4[c * VP4 + h * 512 + t4 * 128];
           }
           ok = wait_all(rf, rb & 1);
           tc_fence_after();
-          float x[16];
-          if (ok && any) pair_read(TR + tl + 32u * h, TR + tl + 8u * G + 32u * h, true, x);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(re);
-          if (ok && any) {
-            float gv[3] = {0.f, 0.f, 0.f};
-            if (act) {
+          if (qd * 16 < mA && ok) {
+#pragma unroll 1
+            for (int jb = h; 32 * jb < mB; jb += 2) {
+              const int cb = 32 * jb + 16 * pc;
+              if (jb > h) {
+                act = alpha < mA && cb < mB;
+                if (act) {
 #pragma unroll
-              for (int t = 0; t < 16; ++t)
-                if (cb + t >= mB) x[t] = 0.f;
+                  for (int c = 0; c < 3; ++c)
 #pragma unroll
-              for (int t4 = 0; t4 < 4; ++t4)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                  gv[c] = fmaf(w[c][t4].x, x[4 * t4], gv[c]);
-                  gv[c] = fmaf(w[c][t4].y, x[4 * t4 + 1], gv[c]);
-                  gv[c] = fmaf(w[c][t4].z, x[4 * t4 + 2], gv[c]);
-                  gv[c] = fmaf(w[c][t4].w, x[4 * t4 + 3], gv[c]);
+                    for (int t4 = 0; t4 < 4; ++t4) w[c][t4] = dV4[c * VP4 + jb * 512 + t4 * 128];
                 }
+              }
+              pair_read(TR + tl + 32u * jb, TR + tl + 8u * GB + 32u * jb, true, x);
+              if (32 * (jb + 2) >= mB) {   // the last read of R
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(re);
+              }
+              if (act) {
+#pragma unroll
+                for (int t = 0; t < 16; ++t)
+                  if (cb + t >= mB) x[t] = 0.f;
+#pragma unroll
+                for (int t4 = 0; t4 < 4; ++t4)
+#pragma unroll
+                  for (int c = 0; c < 3; ++c) {
+                    gv[c] = fmaf(w[c][t4].x, x[4 * t4], gv[c]);
+                    gv[c] = fmaf(w[c][t4].y, x[4 * t4 + 1], gv[c]);
+                    gv[c] = fmaf(w[c][t4].z, x[4 * t4 + 2], gv[c]);
+                    gv[c] = fmaf(w[c][t4].w, x[4 * t4 + 3], gv[c]);
+                  }
+              }
             }
+          }
+          if (!(qd * 16 < mA && ok && 32 * h < mB)) {   // nothing to read
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(re);
+          } else {
 #pragma unroll
             for (int c = 0; c < 3; ++c) gv[c] = warp_sum_f(gv[c]);
             const float g = lane == 0 ? gv[0] : lane == 1 ? gv[1] : gv[2];
             const int p = __shfl_sync(0xffffffffu, p_l, j);
             if (lane < 3 && g != 0.f) dev::add_gV(P, 3 * p + lane, -(double)g * P.sc.r1);
           }
-          if (ew == 0) fl += (unsigned)(mB * nF * nA) * (unsigned)(2 * __shfl_sync(0xffffffffu, nB_l, j) + 4 * mA);
+          if (ew == 0)
+            fl += (unsigned)(mB * nF * nA) *
+                  (unsigned)((sb.als ? 0 : 2 * __shfl_sync(0xffffffffu, nB_l, j)) + 4 * mA);
           ++rb;
           // ---- end of a run: Q -> E, g^C (the two halves take alternate 32-column chunks)
           if (last && ok) {
@@ -830,7 +904,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (e[0] != 0.0) dev::add_E(P, -e[0] * P.sc.q1);
 #pragma unroll
                 for (int c = 0; c < 3; ++c)
-                  if (e[c + 1] != 0.0) dev::add_gC(P, 3 * it.q + c, -2.0 * e[c + 1] * P.sc.q1);
+                  if (e[c + 1] != 0.0) dev::add_gC(P, 3 * q + c, -2.0 * e[c + 1] * P.sc.q1);
               }
             }
             tc_fence_before();
@@ -854,9 +928,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     Ring ik, ub, t;
     bool ok = true;
     for (Unit it = next_unit(ik); it.kk >= 0 && ok; it = next_unit(ik)) {
-      const int nF = P.n_ao[P.species[P.c_j[it.q]]];
+      const int q = it.q(), sA = P.species[P.c_home[q]];
+      const int nF = item_sub(it.sub(), P.n_abf[sA], P.n_ao[sA], P.n_ao[P.species[P.c_j[q]]]).nF;
       const float inv = 1.0f / (float)nF;
-      const long long b0 = X.qoff[it.q];
+      const long long b0 = X.qoff[q];
       for (int i0 = it.lo; i0 < it.hi && ok; i0 += 32) {
         int ng_l = 0;
         if (i0 + lane < it.hi) ng_l = ((P.n_abf[P.species[P.v_j[X.blist[b0 + i0 + lane]]]] + 7) >> 3) * nF;
@@ -866,7 +941,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (!ok) break;
           const int ng = __shfl_sync(0xffffffffu, ng_l, j);
           ok = wait_all(ue + 8 * ub.s, ub.ph ^ 1);
-          unsigned char* ubase = smem_raw + CB + ub.s * CB + (lane & 7) * 16;
+          unsigned char* ubase = smem_raw + CB + ub.s * UBY + (lane & 7) * 16;
           for (int r0 = 0; r0 < ng && ok; r0 += kYG) {
             ok = wait_all(tf + 8 * t.s, t.ph);
             if (!ok) break;
@@ -893,8 +968,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               unsigned char* d = ubase + g * rowg + (r - g * nF) * 256;
 #pragma unroll
               for (int pp = 0; pp < NP; ++pp) {
-                *reinterpret_cast<uint4*>(d + pp * (CB >> 1)) = make_uint4(w[0][pp], w[1][pp], w[2][pp], w[3][pp]);
-                *reinterpret_cast<uint4*>(d + pp * (CB >> 1) + 128) = make_uint4(w[4][pp], w[5][pp], w[6][pp], w[7][pp]);
+                *reinterpret_cast<uint4*>(d + pp * (UBY >> 1)) = make_uint4(w[0][pp], w[1][pp], w[2][pp], w[3][pp]);
+                *reinterpret_cast<uint4*>(d + pp * (UBY >> 1) + 128) = make_uint4(w[4][pp], w[5][pp], w[6][pp], w[7][pp]);
               }
             }
           }
@@ -1218,7 +1293,11 @@ int num_sms() {
 
 long long t1u_launch_count() { return g_t1u_launches; }
 
-size_t t1u_smem(int KP, int G, int UB, int NS) { return t1_base(KP, G, UB) + (size_t)NS * kYSlot; }
+size_t t1u_smem(int KP, int GA, int GB, int KB, int UB, int NS) {
+  return t1_base(KP, GA, GB, KB, UB) + (size_t)NS * kYSlot;
+}
+
+int t1u_utiles(int KP, int GB) { return t1_utiles(KP, GB); }
 
 int t1u_max_slots() { return kMaxNS; }
 
@@ -1259,14 +1338,31 @@ cudaError_t launch_vstores(const DevPlan& P, const MixPlan& X, const T1UPlan& U,
                            cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   ++g_t1u_launches;
-  static std::once_flag attr;
-  std::call_once(attr, [] {
-    cudaFuncSetAttribute(k_vstores<kSplitBf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kVStoreSmem);
-    cudaFuncSetAttribute(k_vstores<kSplitHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, kVStoreSmem);
-  });
+  const size_t sm = vstore_smem(U.VK > 64 ? U.VK : 64);
+  cudaError_t e = allow_max_dynamic_smem(sp == kSplitBf16 ? (const void*)k_vstores<kSplitBf16>
+                                                          : (const void*)k_vstores<kSplitHalf>);
+  if (e != cudaSuccess) return e;
   const int g = n < 152 * 3 ? n : 152 * 3;
-  if (sp == kSplitBf16) k_vstores<kSplitBf16><<<g, 256, kVStoreSmem, s>>>(P, X, U, list, n);
-  else k_vstores<kSplitHalf><<<g, 256, kVStoreSmem, s>>>(P, X, U, list, n);
+  if (sp == kSplitBf16) k_vstores<kSplitBf16><<<g, 256, sm, s>>>(P, X, U, list, n);
+  else k_vstores<kSplitHalf><<<g, 256, sm, s>>>(P, X, U, list, n);
+  return cudaGetLastError();
+}
+
+// Entries (C pair, sub) of the kept C pairs q of [q0, q1) from list[idx[q]] on.
+__global__ void k_t1_items(DevPlan P, const int* qcnt, const long long* idx, int q0, int q1, int* list) {
+  for (int q = q0 + blockIdx.x * blockDim.x + threadIdx.x; q < q1; q += gridDim.x * blockDim.x) {
+    if (qcnt[q] == 0) continue;
+    const int sA = P.species[P.c_home[q]];
+    const int n = abf_subs(P.n_abf[sA]) * ao_subs(P.n_ao[sA]) * ao_subs(P.n_ao[P.species[P.c_j[q]]]);
+    for (int k = 0; k < n; ++k) list[idx[q] + k] = q | (k << kItemShift);
+  }
+}
+
+cudaError_t launch_t1_items(const DevPlan& P, const int* qcnt, const long long* idx, int q0, int q1, int* list,
+                            cudaStream_t s) {
+  if (q1 <= q0) return cudaSuccess;
+  ++g_t1u_launches;
+  k_t1_items<<<std::min((q1 - q0 + 255) / 256, 152 * 8), 256, 0, s>>>(P, qcnt, idx, q0, q1, list);
   return cudaGetLastError();
 }
 
