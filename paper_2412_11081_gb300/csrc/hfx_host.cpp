@@ -1064,9 +1064,14 @@ bool t1u_shapes(hfx_plan* P, size_t limit) {
   // kept B per FP32 run of the Q accumulator: 32 for BF16X3, whose stress error
   // is closest to the 1e-5 bound; 128 for BF16X6 (6.5e-6 at most on the
   // jittered si64 geometries against 5.4e-6 with 32 when its operands were
-  // three bf16 pieces, and fewer FP64 flushes)
+  // three bf16 pieces, and fewer FP64 flushes).  With more than 16 orbitals
+  // both products take short runs, 16 B here and 32 K steps in the Q2 GEMM:
+  // the accumulator's rounding is these cells' largest error (40-atom
+  // perovskite, relative 2-norm over three geometries, F 1.5-1.9e-6 with runs
+  // of 128, 0.9-1.0e-6 with 16, 1.1e-6 for the warp-level kernels; evaluation
+  // 15.4 and 16.0 ms).
   const char* sg = std::getenv("HFX_T1_SEG");
-  P->t1u_seg = sg ? std::max(1, std::atoi(sg)) : (P->sp == hfx::kSplitHalf ? 128 : 32);
+  P->t1u_seg = sg ? std::max(1, std::atoi(sg)) : P->wide ? 16 : (P->sp == hfx::kSplitHalf ? 128 : 32);
   ck(hfx::t1u_set_smem(P->sp), "smem attributes");
   return true;
 }
@@ -1116,7 +1121,7 @@ void setup_shapes(hfx_plan* P) {
     P->zblk = (long long)P->np * P->MC * 128 * 16;
     P->ybtpc = 2;
     P->q2tpc = P->sp == hfx::kSplitHalf ? 3 : 2;
-    P->q2_flush = P->sp == hfx::kSplitHalf ? 128 : 32;   // K steps per FP32 run, as for n_ao <= 16
+    P->q2_flush = 32;   // K steps per FP32 run (beside t1u_seg)
     ck(hfx::set_wide_smem_limits(P->sp), "smem attributes");
     ck(hfx::set_mixed_smem_limits(P->sp), "smem attributes");
     return;
