@@ -1072,7 +1072,7 @@ bool t1u_shapes(hfx_plan* P, size_t limit) {
   // 15.4 and 16.0 ms).
   const char* sg = std::getenv("HFX_T1_SEG");
   P->t1u_seg = sg ? std::max(1, std::atoi(sg)) : P->wide ? 16 : (P->sp == hfx::kSplitHalf ? 128 : 32);
-  ck(hfx::t1u_set_smem(P->sp), "smem attributes");
+  ck(hfx::t1u_set_smem(P->sp, P->t1u_subs > 1), "smem attributes");
   return true;
 }
 
@@ -1123,7 +1123,7 @@ void setup_shapes(hfx_plan* P) {
     P->q2tpc = P->sp == hfx::kSplitHalf ? 3 : 2;
     P->q2_flush = 32;   // K steps per FP32 run (beside t1u_seg)
     ck(hfx::set_wide_smem_limits(P->sp), "smem attributes");
-    ck(hfx::set_mixed_smem_limits(P->sp), "smem attributes");
+    ck(hfx::set_mixed_smem_limits(P->sp, P->KB > 1), "smem attributes");
     return;
   }
   if (P->np) {
@@ -1189,7 +1189,7 @@ void setup_shapes(hfx_plan* P) {
     P->q2tpc = qt && (std::atoi(qt) >= 1 && std::atoi(qt) <= 3) ? std::atoi(qt) : (P->sp == hfx::kSplitHalf ? 3 : 2);
     const char* qf = std::getenv("HFX_Q2_FLUSH");
     P->q2_flush = qf ? std::max(1, std::atoi(qf)) : (P->sp == hfx::kSplitHalf ? 128 : 32);   // as t1u_seg
-    ck(hfx::set_mixed_smem_limits(P->sp), "smem attributes");
+    ck(hfx::set_mixed_smem_limits(P->sp, P->KB > 1), "smem attributes");
   }
 }
 
@@ -1484,6 +1484,7 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     U.GB = P->t1u_GB;
     U.VK = (8 * U.GB + 15) / 16 * 16;
     U.NAL = P->t1u_NAL;
+    U.sub = P->t1u_subs > 1 ? 1 : 0;
     U.UB = P->t1u_UB;
     U.NS = P->t1u_NS;
     U.seg = P->t1u_seg;

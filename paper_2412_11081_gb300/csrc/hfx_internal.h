@@ -207,6 +207,7 @@ struct T1UPlan {
   uint16_t* Vu;                // per term-1 V pair and alpha sub: V pieces [8-row group][piece] x beta VK, then grad V FP32 [3][64][rup32(VK)]
   long long vu_blk;            // uint16 units per V pair and alpha sub
   int NAL;                     // most alpha subs
+  int sub;                     // 1: some block has more than one sub-block
   const long long* t1_idx;     // V pair -> its position in the term-1 V list
   const uint16_t* Yh;          // fp16 Y pieces (MixPlan::Yh or Ysp)
   long long yh_blk;            // its block per needed key, 0: offsets y_off (Ysp)
@@ -297,7 +298,7 @@ cudaError_t launch_yvirt(const DevPlan& P, const long long* y_vidx, int* list, c
 cudaError_t launch_t1_lists(const DevPlan& P, const MixPlan& X, int phase, cudaStream_t s);
 size_t term1_mma_smem(int MAmax, int MBmax, int KSmax, int YRmax);
 size_t term2_mma_smem(int MAmax, int KZmax);
-cudaError_t set_mixed_smem_limits(int sp);
+cudaError_t set_mixed_smem_limits(int sp, bool sub);
 cudaError_t launch_term1_mma(const DevPlan& P, const MixPlan& X, int sp, const int* qlist, int n, int MAmax,
                              int MBmax, int KSmax, int YRmax, size_t smem, cudaStream_t s);
 // Second product of the home atoms [a0, a1): list / slot0 / n are that pass's
@@ -338,7 +339,7 @@ constexpr int kLptBuckets = 4096;
 cudaError_t launch_lpt_order(const int* key, int asc, const int* list, int n_max, const long long* n_dev, int* hist,
                              int* out, cudaStream_t s);
 int t1u_max_slots();
-cudaError_t t1u_set_smem(int sp);
+cudaError_t t1u_set_smem(int sp, bool sub);
 // Needed V pairs: the second product's V store (MixPlan::Vm) and, with U.Vu
 // set, the tcgen05 first product's V store, in one pass per pair.
 cudaError_t launch_vstores(const DevPlan& P, const MixPlan& X, const T1UPlan& U, int sp, const int* list, int n,

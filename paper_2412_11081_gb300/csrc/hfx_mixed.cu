@@ -796,7 +796,8 @@ struct Q2Shape {
   static constexpr int kCols = kNB * TPC * 128;                        // tensor-memory columns
 };
 
-template <int SP, int TPC, int DEEP>
+// SUB: some block has more than 16 orbitals (X.KB sub-blocks at most).
+template <int SP, int TPC, int DEEP, bool SUB>
 __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int* list, const long long* slot0,
                                                  int n_slots, int a0, int a1, int FC8, int MC, int NSEG,
                                                  long long zblk, int flush, const __grid_constant__ DRows drows,
@@ -832,11 +833,11 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
   const int sA = P.species[A];
   const int nA = P.n_ao[sA], mA = P.n_abf[sA];
   const int rows = mA * nA, nt = (rows + 127) >> 7;
-  const int q0 = P.c_ptr[A], nq = X.vc_ptr ? X.vc_ptr[A + 1] - X.vc_ptr[A] : P.c_ptr[A + 1] - q0;   // column slots
+  const int q0 = P.c_ptr[A], nq = SUB ? X.vc_ptr[A + 1] - X.vc_ptr[A] : P.c_ptr[A + 1] - q0;   // column slots
   if (fc * 8 >= nq || mc * 128 >= rows || P.v_ptr[A] == P.v_ptr[A + 1]) return;
   const int ntile = min(TPC, nt - mc);   // row tiles of this CTA
-  const long long s0 = slot0[P.v_ptr[A]] * X.KB;   // K steps (pair slot, sub)
-  const long long s1 = A + 1 < a1 ? slot0[P.v_ptr[A + 1]] * X.KB : (long long)n_slots;
+  const long long s0 = slot0[P.v_ptr[A]] * (SUB ? X.KB : 1);   // K steps (pair slot, sub)
+  const long long s1 = A + 1 < a1 ? slot0[P.v_ptr[A + 1]] * (SUB ? X.KB : 1) : (long long)n_slots;
   const long long p0 = s0 + (long long)seg * KMP;
   const int np = (int)max(0ll, min((long long)KMP, s1 - p0));
   if (np <= 0) return;
@@ -845,8 +846,8 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int j = fc * 8 + i;
-    const int code = j < nq ? (X.vc_list ? X.vc_list[X.vc_ptr[A] + j] : q0 + j) : 0;
-    const int q = code & ((1 << kSubShift) - 1);
+    const int code = j < nq ? (SUB ? X.vc_list[X.vc_ptr[A] + j] : q0 + j) : 0;
+    const int q = SUB ? code & ((1 << kSubShift) - 1) : code;
     qf[i] = (j < nq && P.c_keep[q]) ? q : -1;
     qs[i] = code >> kSubShift;
   }
@@ -991,7 +992,8 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
           // grad C_AF rows in gc_off order: the warp's 32 rows of one 4-column
           // group are 512 consecutive bytes; columns f >= n_ao(F) are zero on
           // both sides
-          const float4* dC4 = reinterpret_cast<const float4*>(X.Cm + X.cm_off[qf[i]] + qs[i] * cm_size(rows) + (long long)NP * nt * 2048) +
+          const float4* dC4 = reinterpret_cast<const float4*>(X.Cm + X.cm_off[qf[i]] + (SUB ? qs[i] * cm_size(rows) : 0) +
+                                                              (long long)NP * nt * 2048) +
                               (r >> 7) * 512 + (r & 127);
           float4 w[3][4];
 #pragma unroll
@@ -1049,7 +1051,7 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
 // TPC row tiles of 128 rows per CTA share each K step's D blocks (one
 // accumulator of 128 columns per tile).
 
-template <int SP, int TPC>
+template <int SP, int TPC, bool SUB>
 __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const int* ylist, const int* gX,
                                                      const int* gS, const int* gN, int MC,
                                                      const __grid_constant__ DRows drows, int* err) {
@@ -1072,13 +1074,13 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
   const int rows = mX * nX;
   if (mc * 128 >= rows) return;
   const int ntile = min(TPC, ((rows + 127) >> 7) - mc);
-  const int q0 = P.c_ptr[Xa], nq = (P.c_ptr[Xa + 1] - q0) * X.KB;
+  const int q0 = P.c_ptr[Xa], nq = (P.c_ptr[Xa + 1] - q0) * (SUB ? X.KB : 1);
   int ykey[8], zat[8], zsub[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int code = i < nk ? ylist[kstart + i] : 0;
-    ykey[i] = i < nk ? code & ((1 << kSubShift) - 1) : -1;
-    zsub[i] = code >> kSubShift;
+    ykey[i] = i < nk ? (SUB ? code & ((1 << kSubShift) - 1) : code) : -1;
+    zsub[i] = SUB ? code >> kSubShift : 0;
     zat[i] = ykey[i] >= 0 ? P.y_j[ykey[i]] : 0;
   }
   // D block of every (C pair, key), or -1, from the table
@@ -1140,8 +1142,9 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
       if (lane == 0) {
         mbar_expect_tx(mfull + 8 * s, bytes);
         bulk_g2s((uint32_t)__cvta_generic_to_shared(stA + (size_t)s * TPC * NP * kTileElems),
-                 X.Cm + X.cm_off[q0 + t / X.KB] + (t % X.KB) * cm_size(rows) + (long long)mc * NP * kTileElems, abytes,
-                 mfull + 8 * s);
+                 X.Cm + (SUB ? X.cm_off[q0 + t / X.KB] + (t % X.KB) * cm_size(rows) : X.cm_off[q0 + t]) +
+                     (long long)mc * NP * kTileElems,
+                 abytes, mfull + 8 * s);
       }
       stage_d(lane, stB + (size_t)s * NP * kTileElems, m_d + t * 8, &drows.map, drows.zero_row, mfull + 8 * s);
     }
@@ -1219,14 +1222,15 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
         const int i = (c0 >> 4) + h;
         if (ykey[i] < 0) continue;
         // columns zz < nZs of the slot are z = z0 + zz of the key's nZ; x padded to PX
-        const int nZ = P.n_ao[P.species[zat[i]]], z0 = zsub[i] * ao_sub(nZ), nZs = min(ao_sub(nZ), nZ - z0);
-        const int PX = rup16(nX), NH = PX >> 3;
+        const int nZ = P.n_ao[P.species[zat[i]]], z0 = SUB ? zsub[i] * ao_sub(nZ) : 0;
+        const int nZs = SUB ? min(ao_sub(nZ), nZ - z0) : nZ;
+        const int PX = SUB ? rup16(nX) : 16, NH = PX >> 3;
         uint16_t* Yo = X.Ysp + P.y_off[ykey[i]];
         uint16_t* Yh = X.Yh ? X.Yh + X.y_idx[ykey[i]] * X.yh_blk : nullptr;
         const bool cm = X.ycm != 0;   // Ysp rows alpha, K = (z, x) in core-matrix order
         const int KZc = 16 * nZ, m8 = (mX + 7) & ~7;
         // Yh: sub of x (hX of them) and of z first
-        const int hX = ao_sub(nX), NXS = ao_subs(nX);
+        const int hX = SUB ? ao_sub(nX) : nX, NXS = SUB ? ao_subs(nX) : 1;
         const long long hxs = (long long)m8 * KZc, hplane = NXS * hxs, hzo = (long long)m8 * z0 * 16;
         const long long plane = cm ? hxs : (long long)mX * nZ * PX;
         const float* eh = ep + h * 16;
@@ -1477,6 +1481,27 @@ size_t q2_umma_smem(int tpc) {   // tpc 3: two tiles, the deep pipeline
          (size_t)Q2Shape<1>::kMP * 8 * sizeof(int);
 }
 
+// The Y build and Q2 GEMM of a split, tile shape (tpc as MixPlan::q2tpc) and sub-blocks or not.
+using YKern = void (*)(DevPlan, MixPlan, const int*, const int*, const int*, const int*, int, const DRows, int*);
+using Q2Kern = void (*)(DevPlan, MixPlan, const int*, const long long*, int, int, int, int, int, int, long long, int,
+                        const DRows, int*);
+template <int SP, bool SUB>
+YKern ybuild_kern(int tpc) {
+  return tpc == 1 ? k_ybuild_umma<SP, 1, SUB> : k_ybuild_umma<SP, 2, SUB>;
+}
+template <int SP, bool SUB>
+Q2Kern q2_kern(int tpc) {
+  return tpc == 1 ? k_q2_umma<SP, 1, 0, SUB> : tpc == 3 ? k_q2_umma<SP, 2, 1, SUB> : k_q2_umma<SP, 2, 0, SUB>;
+}
+YKern ybuild_kern(int sp, bool sub, int tpc) {
+  if (sp == kSplitBf16) return sub ? ybuild_kern<kSplitBf16, true>(tpc) : ybuild_kern<kSplitBf16, false>(tpc);
+  return sub ? ybuild_kern<kSplitHalf, true>(tpc) : ybuild_kern<kSplitHalf, false>(tpc);
+}
+Q2Kern q2_kern(int sp, bool sub, int tpc) {
+  if (sp == kSplitBf16) return sub ? q2_kern<kSplitBf16, true>(tpc) : q2_kern<kSplitBf16, false>(tpc);
+  return sub ? q2_kern<kSplitHalf, true>(tpc) : q2_kern<kSplitHalf, false>(tpc);
+}
+
 int grid_for(long long n, int cap) {
   long long g = n < 1 ? 1 : n;
   return (int)(g > cap ? cap : g);
@@ -1535,10 +1560,7 @@ cudaError_t launch_ybuild_mma(const DevPlan& P, const MixPlan& X, int sp, const 
   const int tpc = X.ybtpc == 1 ? 1 : 2;
   const long long grid = (long long)ngroups * ((MC + tpc - 1) / tpc);
   const size_t sm = ybuild_umma_smem(tpc, X.ytab_stride);
-  if (sp == kSplitBf16 && tpc == 2) k_ybuild_umma<kSplitBf16, 2><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
-  else if (sp == kSplitBf16) k_ybuild_umma<kSplitBf16, 1><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
-  else if (tpc == 2) k_ybuild_umma<kSplitHalf, 2><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
-  else k_ybuild_umma<kSplitHalf, 1><<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
+  ybuild_kern(sp, X.KB > 1, tpc)<<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
   return cudaGetLastError();
 }
 
@@ -1554,13 +1576,10 @@ size_t term1_mma_smem(int MAmax, int MBmax, int KSmax, int YRmax) {
 
 size_t term2_mma_smem(int MAmax, int KZmax) { return (size_t)NP * 2 * MAmax * KZmax * sizeof(uint16_t); }
 
-cudaError_t set_mixed_smem_limits(int sp) {
+cudaError_t set_mixed_smem_limits(int sp, bool sub) {
   const void* f[7] = {
-      sp == kSplitBf16 ? (const void*)k_ybuild_umma<kSplitBf16, 2> : (const void*)k_ybuild_umma<kSplitHalf, 2>,
-      sp == kSplitBf16 ? (const void*)k_ybuild_umma<kSplitBf16, 1> : (const void*)k_ybuild_umma<kSplitHalf, 1>,
-      sp == kSplitBf16 ? (const void*)k_q2_umma<kSplitBf16, 2, 0> : (const void*)k_q2_umma<kSplitHalf, 2, 0>,
-      sp == kSplitBf16 ? (const void*)k_q2_umma<kSplitBf16, 2, 1> : (const void*)k_q2_umma<kSplitHalf, 2, 1>,
-      sp == kSplitBf16 ? (const void*)k_q2_umma<kSplitBf16, 1, 0> : (const void*)k_q2_umma<kSplitHalf, 1, 0>,
+      (const void*)ybuild_kern(sp, sub, 1), (const void*)ybuild_kern(sp, sub, 2),
+      (const void*)q2_kern(sp, sub, 1), (const void*)q2_kern(sp, sub, 2), (const void*)q2_kern(sp, sub, 3),
       sp == kSplitBf16 ? (const void*)k_term1_mma<kSplitBf16> : (const void*)k_term1_mma<kSplitHalf>,
       sp == kSplitBf16 ? (const void*)k_term2_pairs<kSplitBf16> : (const void*)k_term2_pairs<kSplitHalf>};
   for (const void* k : f) {
@@ -1605,18 +1624,8 @@ cudaError_t launch_q2(const DevPlan& P, const MixPlan& X, int sp, const int* lis
   const int tpc = X.q2tpc == 1 ? 1 : 2, deep = X.q2tpc == 3 ? 1 : 0;   // row tiles per CTA; the deep pipeline
   const size_t sq = q2_umma_smem(X.q2tpc == 1 ? 1 : (deep ? 3 : 2));
   const long long grid = (long long)(a1 - a0) * FC8 * ((MC + tpc - 1) / tpc) * nseg;
-  auto q2 = [&](auto kern) {
-    kern<<<(unsigned)grid, 192, sq, s>>>(P, X, list, slot0, ns, a0, a1, FC8, MC, nseg, zblk, flush, drows, err);
-  };
-  if (sp == kSplitBf16) {
-    if (tpc == 1) q2(k_q2_umma<kSplitBf16, 1, 0>);
-    else if (deep) q2(k_q2_umma<kSplitBf16, 2, 1>);
-    else q2(k_q2_umma<kSplitBf16, 2, 0>);
-  } else {
-    if (tpc == 1) q2(k_q2_umma<kSplitHalf, 1, 0>);
-    else if (deep) q2(k_q2_umma<kSplitHalf, 2, 1>);
-    else q2(k_q2_umma<kSplitHalf, 2, 0>);
-  }
+  q2_kern(sp, X.KB > 1, tpc == 1 ? 1 : deep ? 3 : 2)<<<(unsigned)grid, 192, sq, s>>>(
+      P, X, list, slot0, ns, a0, a1, FC8, MC, nseg, zblk, flush, drows, err);
   return cudaGetLastError();
 }
 
