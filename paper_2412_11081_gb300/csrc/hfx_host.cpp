@@ -249,6 +249,8 @@ struct hfx_plan {
   long long Vzcap = 0;
   // split path for n_ao > 16 (hfx_wide.cu): FP64 C, V and D blocks, FP32 Y store
   bool wide = false;
+  bool t2w = false;            // wide: R2 and Z on tcgen05 (k_t2w_umma)
+  hfx::T2WPlan t2wp{};
   hfx::WideShapes ws{};
   int KB = 1;                  // most AO sub-blocks of an atom (hfx::ao_subs)
   int maxCv = 0;               // most column slots (C pair, sub) of an atom
@@ -1117,6 +1119,14 @@ void setup_shapes(hfx_plan* P) {
     // first product: the tcgen05 kernel where the sub-blocks fit (HFX_T1_KERNEL=mma: the warp-level one)
     const char* t1w = std::getenv("HFX_T1_KERNEL");
     if (!(t1w && std::string(t1w) == "mma")) t1u_shapes(P, limit);
+    if (P->t1u && P->sp == hfx::kSplitHalf && maxABF <= 128) {   // R2 and Z as well (HFX_T2_KERNEL=mma: warp-level)
+      const char* t2k = std::getenv("HFX_T2_KERNEL");
+      int hao = 1;
+      for (int n : P->n_ao) hao = std::max(hao, hfx::ao_sub(n));
+      P->t2wp = hfx::t2w_plan(maxABF, hao);
+      P->t2w = !(t2k && std::string(t2k) == "mma") && P->t2wp.smem <= limit;
+      if (P->t2w) ck(hfx::t2w_set_smem(), "smem attributes");
+    }
     P->MC = (maxrows + 127) / 128;
     P->zblk = (long long)P->np * P->MC * 128 * 16;
     P->ybtpc = 2;
@@ -1517,8 +1527,19 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     D.Yst = P->Yst;
     ck(hfx::launch_ybuild(D, P->y_list, (int)P->tot[1], s), "ybuild");
   } else if (P->wide) {
-    ensure_buf(P, P->Ysp, P->Yspcap, std::max(1LL, P->tot[0]));
+    if (!P->t2w) ensure_buf(P, P->Ysp, P->Yspcap, std::max(1LL, P->tot[0]));   // read by the warp-level kernels only
     X.y_idx = P->y_idx;
+    if (P->t2w) {   // (rows past n_abf are never written: finite from the start)
+      X.yT_blk = 0;   // the largest key's
+      for (int a = 0; a < P->S; ++a)
+        for (int b = 0; b < P->S; ++b)
+          X.yT_blk = std::max(X.yT_blk, (long long)P->np * hfx::ao_subs(P->n_ao[b]) * ((P->n_abf[a] + 7) / 8 * 8) * 16 *
+                                            P->n_ao[a]);
+      const long long tcap0 = P->YspTcap;
+      ensure_buf(P, P->YspT, P->YspTcap, std::max(1LL, P->tot[1]) * X.yT_blk);
+      if (P->YspTcap != tcap0) ck(cudaMemsetAsync(P->YspT, 0, P->YspTcap * sizeof(uint16_t), s), "memset");
+      X.YspT = P->YspT;
+    }
     if (P->t1u) {
       if (!reuse) {
         ensure_buf(P, P->blist, P->blist_cap, P->tot[6]);
@@ -1531,7 +1552,7 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
       ck(hfx::launch_cpieces_w(D, P->sp, P->Cw, P->cw_off, P->dCf, s), "C pieces");
     }
     ck(hfx::launch_cpieces(D, X, P->sp, s), "cpieces");
-    X.Ysp = P->Ysp;
+    X.Ysp = P->t2w ? nullptr : P->Ysp;
     ensure_buf(P, P->ytab, P->ytabcap, std::max(1LL, hfx::ytab_size((int)P->tot[9], P->maxC * P->KB)));
     X.ytab = P->ytab;
     ck(hfx::launch_ybuild_mma(D, X, P->sp, P->KB > 1 ? P->y_vlist : P->y_list, P->gX, P->gS, P->gN, (int)P->tot[9], P->MC,
@@ -1579,9 +1600,11 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     const long long* ct = P->ctot.data() + (size_t)kCT * c;
     m1.push_back(tm.mark());
     if (!split) {   // FP64 V blocks; the FP64 or the wide split kernels
-      ensure_store(P, P->Vst, P->Vcap, ct[CT_VE]);
-      D.Vst = P->Vst;
-      ck(hfx::launch_vblocks(D, P->v_list + v0, (int)ct[CT_VN], s), "vblocks");
+      if (!P->t2w) {
+        ensure_store(P, P->Vst, P->Vcap, ct[CT_VE]);
+        D.Vst = P->Vst;
+        ck(hfx::launch_vblocks(D, P->v_list + v0, (int)ct[CT_VN], s), "vblocks");
+      }
       if (P->t1u) {
         ensure_buf(P, P->Cu, P->Cucap, std::max(1LL, ct[CT_Q]) * U.cu_blk);
         ensure_buf(P, P->Vu, P->Vucap, std::max(1LL, ct[CT_T1]) * U.NAL * U.vu_blk);
@@ -1614,8 +1637,16 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
         const int FC = (P->maxCv + 3) / 4;
         ensure_buf(P, P->q2tab, P->q2tabcap, std::max(1LL, hfx::q2tab_size(ct[CT_T2] * P->KB, FC)));
         X.q2tab = P->q2tab;
-        ck(hfx::launch_term2_w(D, P->sp, P->Ysp, P->Zst, P->zblk, P->KB, P->t2_list + v0, (int)ct[CT_T2], P->ws, s),
-           "term2");
+        if (P->t2w) {
+          X.vz_blk = P->t2wp.v_blk();
+          ensure_buf(P, P->Vz, P->Vzcap, std::max(1LL, ct[CT_T2]) * X.vz_blk);
+          hfx::MixPlan X2 = X;
+          X2.Vz = P->Vz;
+          ck(hfx::launch_t2w(D, X2, P->t2wp, P->t2_list + v0, (int)ct[CT_T2], P->zblk, P->d_err, s), "term2 R2 and Z");
+        } else {
+          ck(hfx::launch_term2_w(D, P->sp, P->Ysp, P->Zst, P->zblk, P->KB, P->t2_list + v0, (int)ct[CT_T2], P->ws, s),
+             "term2");
+        }
         ck(hfx::launch_q2(D, X, P->sp, P->t2_list + v0, P->t2_idx, (int)ct[CT_T2], a0, a1, P->zblk, FC, P->MC,
                           hfx::q2_umma_segments(P->maxV * P->KB, P->q2tpc), P->q2_flush, P->drows, P->d_err, s),
            "Q2");

@@ -152,6 +152,8 @@ struct MixPlan {
   // core-matrix order; nullptr where Ysp (ycm, one sub) is that store
   uint16_t* Yh = nullptr;
   long long yh_blk = 0;
+  // (plans with sub-blocks: fp16 pieces, per piece, sub of z and sub of x the
+  // row groups (g, x) of 8 alpha x 16 z in core-matrix order)
   uint16_t* YspT = nullptr;    // Y^{XZ} transposed, bf16 pieces [piece][(alpha,x)][16 z] (z padded), yT_blk per key
   long long yT_blk = 0;        // uint16 units per key of YspT (2 pieces x 128-row tiles x 16)
   const long long* y_idx = nullptr;   // key -> its position in the needed-key list (YspT block)
@@ -320,6 +322,20 @@ size_t t2u_smem(int max_ao);
 cudaError_t t2u_set_smem(int sp);
 cudaError_t launch_t2_umma(const DevPlan& P, const MixPlan& X, int sp, const int* list, int n, long long zblk,
                            size_t smem, int* err, cudaStream_t s);
+
+// The same for plans with sub-blocks (fp16 pieces, n_abf <= 128), from X.Yh,
+// X.YspT (the Y build's sub-block stores) and V at X.Vz, which it writes.
+struct T2WPlan {
+  int M8, VK, SA;              // largest n_abf rounded up to 8, 16 (columns beta of a V row), 32 (rows of an FP32 plane)
+  uint32_t v_bytes, y_bytes;   // shared memory of V, of one Y operand
+  uint32_t smem;
+  // uint16 units per pair of X.Vz
+  long long v_blk() const { return (long long)kPieces * M8 * VK + 2LL * 4 * VK * SA; }
+};
+T2WPlan t2w_plan(int max_abf, int max_ao_sub);
+cudaError_t t2w_set_smem();
+cudaError_t launch_t2w(const DevPlan& P, const MixPlan& X, const T2WPlan& S, const int* list, int n, long long zblk,
+                       int* err, cudaStream_t s);
 
 // tcgen05 first exchange product (hfx_t1umma.cu): shapes n_abf <= 64, n_ao <= 16.
 long long t1u_launch_count();

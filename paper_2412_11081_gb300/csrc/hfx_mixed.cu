@@ -1237,7 +1237,7 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
         // bf16 pieces: chunk (alpha, z, half) holds x = 8 half .. 8 half + 7
         // (core-matrix order: consecutive threads take consecutive alpha, whose
         // chunks are 16 bytes apart)
-        for (int c = et; c < nal * nZs * NH; c += 128) {
+        for (int c = et; c < (SUB && !X.Ysp ? 0 : nal * nZs * NH); c += 128) {
           int hf, al, zz;
           if (cm) {   // (PX = 16, one sub)
             const int r2 = c / nal;
@@ -1288,7 +1288,30 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
         // transposed pieces for the second product: accumulator row (alpha, x)
         // with the 16 z of key i (z >= n_ao(Z) zero); every row of the tile
         // is this CTA's own
-        if (X.YspT) {
+        if (SUB && X.YspT) {   // sub-blocks: [sub of z][sub of x], rows alpha, K = (x, 16 z)
+          const long long tplane = (long long)m8 * 16 * nX;
+          uint16_t* yt = X.YspT + X.y_idx[ykey[i]] * X.yT_blk + zsub[i] * tplane;
+          const int nala = alB - alA + 1;
+          for (int c = et; c < nala * nX * 2; c += 128) {   // consecutive threads: consecutive alpha of one (x, half)
+            const int r2 = c / nala, al = alA + (c - r2 * nala), x = r2 >> 1, hz = r2 & 1, rl = al * nX + x - row0;
+            if (rl < 0 || row0 + rl >= rend) continue;
+            const int xs = x / hX, xl = x - xs * hX;
+            float f0[4], f1[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              f0[k] = 8 * hz + k < nZs ? eh[rl * 33 + 8 * hz + k] * P.sc.yh : 0.f;
+              f1[k] = 8 * hz + 4 + k < nZs ? eh[rl * 33 + 8 * hz + 4 + k] * P.sc.yh : 0.f;
+            }
+            uint2 p0[NP], p1[NP];
+            split4<kSplitHalf>(f0, p0);
+            split4<kSplitHalf>(f1, p1);
+            uint16_t* d = yt + (long long)m8 * 16 * xs * hX + cmx(al, xl * 16 + 8 * hz, 16 * min(hX, nX - xs * hX));
+#pragma unroll
+            for (int pp = 0; pp < NP; ++pp)
+              *reinterpret_cast<uint4*>(d + pp * ao_subs(nZ) * tplane) = make_uint4(p0[pp].x, p0[pp].y, p1[pp].x, p1[pp].y);
+          }
+        }
+        if (!SUB && X.YspT) {
           // row-major tiles [(alpha, x)][16 z], or (ycm) rows alpha, K = (x, z) in core-matrix order
           uint16_t* ytb = X.YspT + X.y_idx[ykey[i]] * X.yT_blk;
           uint16_t* yt = ytb + (long long)row0 * 16;
@@ -1340,8 +1363,9 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
             split_f<SP>(y, pc);
             const long long o = cm ? cmx(al, zz * 16, KZc) : ((long long)al * nZ + z0 + zz) * PX;   // + x
 #pragma unroll
-            for (int pp = 0; pp < NP; ++pp) Yo[pp * plane + o + (cm ? ((x >> 3) << 6) + (x & 7) : x)] = pc[pp];
-            if (x == nX - 1)
+            for (int pp = 0; pp < NP; ++pp)
+              if (!SUB || X.Ysp) Yo[pp * plane + o + (cm ? ((x >> 3) << 6) + (x & 7) : x)] = pc[pp];
+            if (x == nX - 1 && (!SUB || X.Ysp))
               for (int xp = nX; xp < PX; ++xp)
 #pragma unroll
                 for (int pp = 0; pp < NP; ++pp) Yo[pp * plane + o + (cm ? ((xp >> 3) << 6) + (xp & 7) : xp)] = 0;

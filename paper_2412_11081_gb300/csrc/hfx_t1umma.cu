@@ -1287,6 +1287,311 @@ __global__ void __launch_bounds__(kT2Threads, 1)
   if (tid == 0 && s_abort) atomicExch(err, 1);
 }
 
+// The same products for plans with sub-blocks (n_ao beyond 16, n_abf up to
+// 128, fp16 pieces): M = 128 rows alpha, and the K = (a, b) and N = (a, b)
+// columns in chunks, one sub-block of A's orbitals times one of B's, which
+// come from the Y build's sub-block stores (Y^{BA} of a chunk from X.Yh,
+// Y^{AB} from X.YspT with a and b exchanged).  R2 runs on over a pair's
+// chunks; Z of a chunk goes to the Z store of (slot, sub of b).  Roles and
+// buffers as k_t2_umma; V, grad V as four planes [beta / 4][alpha SA][4], so
+// that a warp's 32 rows are 512 consecutive bytes.
+// What bounds it: the latency of a chunk's copies (one chunk in shared memory,
+// 66 KB per operand at n_abf 75 and 13 orbitals) and of the epilogue's reads
+// of V, grad V.  The warp-level kernel (k_term2_w, still taken by HFX_BF16X3
+// and by shapes beyond shared memory) stages Y element by element and reads
+// FP64 V blocks: with the build of those 4.9 ms of a 40-atom perovskite
+// evaluation (9,896 pairs), 0.85 ms here with k_t2w_vstore.
+template <int SP>
+__global__ void __launch_bounds__(256) k_t2w_vstore(DevPlan P, MixPlan X, T2WPlan S, const int* list, int n) {
+  for (int k = blockIdx.x; k < n; k += gridDim.x) {
+    const int p = list[k], sA = P.species[P.v_home[p]], sB = P.species[P.v_j[p]];
+    const int mA = P.n_abf[sA], mB = P.n_abf[sB], m8 = (mA + 7) & ~7;
+    double h, g[3];
+    model::v_pair(P, p, h, g);
+    const float f[4] = {(float)h, (float)g[0], (float)g[1], (float)g[2]};
+    const float* M = P.Mf + P.M_off[sA * P.S + sB];
+    uint16_t* out = X.Vz + (long long)k * X.vz_blk;
+    for (int t4 = threadIdx.x; t4 < m8 * S.VK / 4; t4 += blockDim.x) {   // core-matrix order, 4 columns per thread
+      const int t = 4 * t4, g8 = t / (8 * S.VK), u = t - g8 * 8 * S.VK;
+      const int al = g8 * 8 + ((u >> 3) & 7), be = ((u >> 6) << 3) + (u & 7);
+      float x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j] = (al < mA && be + j < mB) ? M[al * mB + be + j] * f[0] * pscale<SP>(P.sc.v) : 0.f;
+      uint2 pc[NP];
+      split4<SP>(x, pc);
+#pragma unroll
+      for (int pp = 0; pp < NP; ++pp) *reinterpret_cast<uint2*>(out + pp * m8 * S.VK + t) = pc[pp];
+    }
+    float4* pl = reinterpret_cast<float4*>(out + NP * S.M8 * S.VK);
+    const int nb4 = (mB + 3) >> 2, PL = (S.VK >> 2) * S.SA;
+    for (int e = threadIdx.x; e < nb4 * mA; e += blockDim.x) {
+      const int b4 = e / mA, al = e - b4 * mA, be = 4 * b4;
+      const float* m = M + al * mB + be;
+      const float4 v = make_float4(m[0], be + 1 < mB ? m[1] : 0.f, be + 2 < mB ? m[2] : 0.f, be + 3 < mB ? m[3] : 0.f);
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        pl[c * PL + b4 * S.SA + al] = make_float4(v.x * f[c], v.y * f[c], v.z * f[c], v.w * f[c]);
+    }
+  }
+}
+
+template <int SP>
+__global__ void __launch_bounds__(kT2Threads, 1)
+    k_t2w_umma(DevPlan P, MixPlan X, T2WPlan S, const int* list, int n_list, long long zblk, int* err) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t b_af, b_ae, b_bf, b_be, b_vf, b_ve, b_rf[2], b_re[2], b_zf, b_ze, b_done;
+  __shared__ uint32_t tmem_base;
+  __shared__ int s_abort;
+  volatile int* abort_flag = &s_abort;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  auto sa = [](const void* p) { return (uint32_t)__cvta_generic_to_shared(p); };
+  const uint32_t Vs = sa(smem_raw), Ya = Vs + S.v_bytes, Yb = Ya + S.y_bytes;
+  const uint32_t mAf = sa(&b_af), mAe = sa(&b_ae), mBf = sa(&b_bf), mBe = sa(&b_be), mVf = sa(&b_vf), mVe = sa(&b_ve),
+                 rf = sa(b_rf), re = sa(b_re), zf = sa(&b_zf), ze = sa(&b_ze), mdone = sa(&b_done);
+  // rows past a block's own are read as they lie (dropped, or against zeros of V): finite from the start
+  for (uint32_t o = tid * 16u; o < S.smem; o += kT2Threads * 16u)
+    *reinterpret_cast<uint4*>(smem_raw + o) = make_uint4(0u, 0u, 0u, 0u);
+  fence_async_smem();
+  if (tid == 0) {
+    s_abort = 0;
+    for (uint32_t m : {mAf, mAe, mBf, mBe, mVf, mVe, rf, rf + 8, zf, mdone}) mbar_init(m, 1);
+    for (uint32_t m : {re, re + 8, ze}) mbar_init(m, 4);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(sa(&tmem_base)), "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t T = tmem_base;
+  // A pair's shapes and its chunks (as, bs), bs fastest.
+  struct Pair {
+    int p, A, B, nA, nB, mA, mB, a8, b8, hA, sA, sB;
+    __device__ int n() const { return sA * sB; }
+    __device__ int as(int c) const { return c / sB; }
+    __device__ int bs(int c) const { return c % sB; }
+    __device__ int na(int c) const { return min(hA, nA - as(c) * hA); }   // a of chunk c
+  };
+  auto pair_of = [&](int kk) {
+    Pair q;
+    q.p = list[kk];
+    q.A = P.v_home[q.p];
+    q.B = P.v_j[q.p];
+    const int tA = P.species[q.A], tB = P.species[q.B];
+    q.nA = P.n_ao[tA];
+    q.nB = P.n_ao[tB];
+    q.mA = P.n_abf[tA];
+    q.mB = P.n_abf[tB];
+    q.a8 = (q.mA + 7) & ~7;
+    q.b8 = (q.mB + 7) & ~7;
+    q.hA = ao_sub(q.nA);
+    q.sA = ao_subs(q.nA);
+    q.sB = ao_subs(q.nB);
+    return q;
+  };
+
+  if (warp == 0) {
+    // ------------------------------------------------------------- producer
+    if (lane == 0) {
+      uint32_t na = 0, nb = 0, nv = 0;   // copies issued into Ya, Yb, V
+      bool ok = true;
+      for (int kk = blockIdx.x; kk < n_list && ok; kk += gridDim.x) {
+        const Pair q = pair_of(kk);
+        const int* Rb = P.v_R + 3 * q.p;
+        const int y1 = ylut_get(P, q.A, q.B, Rb[0], Rb[1], Rb[2]);
+        const int y2 = ylut_get(P, q.B, q.A, -Rb[0], -Rb[1], -Rb[2]);
+        ok = y1 >= 0 && y2 >= 0;   // a kept pair always has both Y blocks
+        for (int c = 0; c < q.n() && ok; ++c) {
+          const int n = q.na(c), a0 = q.as(c) * q.hA, bs = q.bs(c);
+          const uint32_t ca = 32u * q.a8 * n, cb = 32u * q.b8 * n;   // bytes of one piece of the chunk
+          const long long ax = 16ll * q.a8 * q.nA, bx = 16ll * q.b8 * q.nA;   // elements of one sub of b
+          const uint16_t* src_a = X.YspT + X.y_idx[y1] * X.yT_blk + bs * ax + 16ll * q.a8 * a0;
+          const uint16_t* src_b = X.Yh + X.y_idx[y2] * X.yh_blk + bs * bx + 16ll * q.b8 * a0;
+          ok = !aborted(abort_flag) && (na < 1 || mbar_wait(mAe, (na - 1) & 1));
+          if (!ok) break;
+          mbar_expect_tx(mAf, NP * ca);
+          for (int pp = 0; pp < NP; ++pp) bulk_g2s(Ya + pp * ca, src_a + pp * q.sB * ax, ca, mAf);
+          ++na;
+          if (c == 0) {
+            ok = nv < 1 || mbar_wait(mVe, (nv - 1) & 1);
+            if (!ok) break;
+            const uint32_t vb = (uint32_t)NP * q.a8 * S.VK * 2u;
+            mbar_expect_tx(mVf, vb);
+            bulk_g2s(Vs, X.Vz + (long long)kk * X.vz_blk, vb, mVf);
+            ++nv;
+          }
+          ok = nb < 1 || mbar_wait(mBe, (nb - 1) & 1);
+          if (!ok) break;
+          mbar_expect_tx(mBf, NP * cb);
+          for (int pp = 0; pp < NP; ++pp) bulk_g2s(Yb + pp * cb, src_b + pp * q.sB * bx, cb, mBf);
+          ++nb;
+        }
+      }
+      if (!ok) *abort_flag = 1;
+      // copies in flight land before the CTA leaves
+      if (na) mbar_wait(mAf, (na - 1) & 1);
+      if (nv) mbar_wait(mVf, (nv - 1) & 1);
+      if (nb) mbar_wait(mBf, (nb - 1) & 1);
+    }
+  } else if (warp == 1) {
+    // ----------------------------------------------------------- MMA issuer
+    if (lane == 0) {
+      uint32_t i = 0, t = 0;   // pairs, chunks
+      bool ok = true;
+      for (int kk = blockIdx.x; kk < n_list && ok; kk += gridDim.x, ++i) {
+        const Pair q = pair_of(kk);
+        const uint32_t idR = idesc_split<SP>(128, (q.mB + 15) & ~15, 0), tR = T + kT2RCol + 128u * (i & 1);
+        const uint64_t vp = (uint64_t)(2u * q.a8 * S.VK) >> 4;   // a piece of V
+        const uint64_t dV = sdesc2(Vs, 128, 16u * S.VK);
+        ok = i < 2 || mbar_wait(re + 8 * (i & 1), ((i >> 1) - 1) & 1);
+        for (int c = 0; c < q.n() && ok; ++c, ++t) {
+          const int n = q.na(c), last = c == q.n() - 1;
+          const uint32_t rowg = 256u * n;   // bytes between 8-row groups
+          const uint64_t pa = (uint64_t)(32u * q.a8 * n) >> 4, pb = (uint64_t)(32u * q.b8 * n) >> 4;
+          const uint64_t dA = sdesc2(Ya, 128, rowg), dB = sdesc2(Yb, 128, rowg), dZ = sdesc2(Yb, rowg, 128);
+          ok = !aborted(abort_flag) && mbar_wait(mAf, t & 1) && mbar_wait(mBf, t & 1);
+          if (!ok) break;
+          tc_fence_after();
+          for (int a = 0; a < n; ++a) {   // R2: one a (16 columns, 256 bytes) per k step
+            const uint64_t o = 16u * (uint32_t)a;
+            umma_f16(tR, dA + o, dB + pb + o, idR, (c > 0 || a > 0) ? 1u : 0u);
+            umma_f16(tR, dA + pa + o, dB + o, idR, 1u);
+            umma_f16(tR, dA + o, dB + o, idR, 1u);
+          }
+          umma_commit(mAe);
+          if (last) umma_commit(rf + 8 * (i & 1));
+          ok = (c > 0 || mbar_wait(mVf, i & 1)) && (t < 1 || mbar_wait(ze, (t - 1) & 1));
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t idZ = idesc_split<SP>(128, 16 * n, 1);
+          for (int kb = 0; 16 * kb < q.mB; ++kb) {   // Z: K = beta in steps of 16 (V: 256 bytes; Y^{BA}: two 8-row groups)
+            const uint64_t o = 16u * (uint32_t)kb, oz = (uint64_t)(2 * rowg * kb) >> 4;
+            umma_f16(T, dV + o, dZ + pb + oz, idZ, kb > 0 ? 1u : 0u);
+            umma_f16(T, dV + vp + o, dZ + oz, idZ, 1u);
+            umma_f16(T, dV + o, dZ + oz, idZ, 1u);
+          }
+          umma_commit(mBe);
+          if (last) umma_commit(mVe);
+          umma_commit(zf);
+        }
+      }
+      if (!ok) *abort_flag = 1;
+      // every MMA issued has completed before tensor memory is freed
+      umma_commit(mdone);
+      mbar_wait(mdone, 0);
+    }
+  } else {
+    // ------------------------------------------------------------- epilogue
+    const int qd = warp & 3, alpha = 32 * qd + lane;   // tensor-memory lane quarter, accumulator row
+    const uint32_t tl = T + ((uint32_t)(qd * 32) << 16);
+    const int PL = (S.VK >> 2) * S.SA;   // float4 per plane
+    uint32_t i = 0, t = 0;
+    bool ok = true;
+    double fl = 0.0;
+    for (int kk = blockIdx.x; kk < n_list && ok; kk += gridDim.x, ++i) {
+      ok = __all_sync(0xffffffffu, !aborted(abort_flag)) != 0;
+      if (!ok) break;
+      const Pair q = pair_of(kk);
+      const bool rows = 32 * qd < q.mA, act = alpha < q.mA;
+      const float4* V4 = reinterpret_cast<const float4*>(X.Vz + (long long)kk * X.vz_blk + NP * S.M8 * S.VK) + alpha;
+      float4 w[4][4];
+      auto fetch = [&](int cb) {   // V, grad V of columns 16 cb .. + 15
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int t4 = 0; t4 < 4; ++t4)
+            w[c][t4] = act && 16 * cb + 4 * t4 < q.mB ? V4[c * PL + (4 * cb + t4) * S.SA] : make_float4(0.f, 0.f, 0.f, 0.f);
+      };
+      for (int c = 0; c < q.n() && ok; ++c, ++t) {
+        if (c == q.n() - 1) {   // R2 -> E, g^V
+          float ev[4] = {0.f, 0.f, 0.f, 0.f};
+          fetch(0);   // (does not depend on R2)
+          ok = wait_all(rf + 8 * (i & 1), (i >> 1) & 1);
+          tc_fence_after();
+          if (ok && rows) {
+#pragma unroll 1
+            for (int cb = 0; 16 * cb < q.mB; ++cb) {
+              if (cb) fetch(cb);
+              uint32_t v[16];
+              tmem_ld16(tl + kT2RCol + 128u * (i & 1) + 16u * cb, v);
+              tmem_wait_ld();
+              if (act) {
+                float x[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) x[k] = 16 * cb + k < q.mB ? __uint_as_float(v[k]) : 0.f;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                  float s = 0.f;
+#pragma unroll
+                  for (int t4 = 0; t4 < 4; ++t4) {
+                    s = fmaf(w[k][t4].x, x[4 * t4], s);
+                    s = fmaf(w[k][t4].y, x[4 * t4 + 1], s);
+                    s = fmaf(w[k][t4].z, x[4 * t4 + 2], s);
+                    s = fmaf(w[k][t4].w, x[4 * t4 + 3], s);
+                  }
+                  ev[k] += s;
+                }
+              }
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(re + 8 * (i & 1));
+          if (ok && rows) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) ev[k] = warp_sum_f(ev[k]);
+            if (lane == 0) {
+              if (ev[0] != 0.f) dev::add_E(P, -(double)ev[0] * P.sc.r2);
+#pragma unroll
+              for (int k = 0; k < 3; ++k)
+                if (ev[k + 1] != 0.f) dev::add_gV(P, 3 * q.p + k, -(double)ev[k + 1] * P.sc.r2);
+            }
+          }
+        }
+        // ---- Z of the chunk -> the Z store of (slot, sub of b): 128-row tiles of rows (alpha, a), 16 columns b
+        ok = ok && wait_all(zf, t & 1);
+        tc_fence_after();
+        if (ok && rows) {
+          uint16_t* Zo = X.Zst + ((long long)kk * X.KB + q.bs(c)) * zblk;
+          const int n = q.na(c), r0 = alpha * q.nA + q.as(c) * q.hA;
+#pragma unroll 1
+          for (int a = 0; a < n; ++a) {
+            uint32_t v[16];
+            tmem_ld16(tl + 16u * a, v);
+            tmem_wait_ld();
+            if (!act) continue;
+            const int r = r0 + a;
+            uint16_t* d = Zo + (long long)(r >> 7) * NP * 2048 + (((r & 127) >> 3) << 7) + ((r & 7) << 3);
+            uint32_t pc[8][NP];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+              split2<SP>(__uint_as_float(v[2 * k]) * pscale<SP>(P.sc.z), __uint_as_float(v[2 * k + 1]) * pscale<SP>(P.sc.z), pc[k]);
+#pragma unroll
+            for (int pp = 0; pp < NP; ++pp) {
+              *reinterpret_cast<uint4*>(d + pp * 2048) = make_uint4(pc[0][pp], pc[1][pp], pc[2][pp], pc[3][pp]);
+              *reinterpret_cast<uint4*>(d + pp * 2048 + 64) = make_uint4(pc[4][pp], pc[5][pp], pc[6][pp], pc[7][pp]);
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(ze);
+      }
+      if (warp == 2 && lane == 0) fl += 4.0 * q.mA * q.mB * q.nA * q.nB;
+    }
+    if (!ok) *abort_flag = 1;
+    if (warp == 2 && lane == 0 && fl != 0.0) atomicAdd(&P.acc[ACC_F2], fl);
+  }
+  // ------------------------------------------------------------------ teardown
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(T), "r"(512));
+  if (tid == 0 && s_abort) atomicExch(err, 1);
+}
+
 int num_sms() {
   static const int n = [] {
     int dev = 0, v = 0;
@@ -1394,6 +1699,34 @@ cudaError_t launch_t2_umma(const DevPlan& P, const MixPlan& X, int sp, const int
   const int KKmax = (int)(smem / NP - 8192) / (2 * 64 * 2);   // 16 x the largest n_ao
   if (sp == kSplitBf16) k_t2_umma<kSplitBf16><<<grid, kT2Threads, smem, s>>>(P, X, list, n, KKmax, zblk, err);
   else k_t2_umma<kSplitHalf><<<grid, kT2Threads, smem, s>>>(P, X, list, n, KKmax, zblk, err);
+  return cudaGetLastError();
+}
+
+T2WPlan t2w_plan(int max_abf, int max_ao_sub) {
+  T2WPlan S;
+  S.M8 = (max_abf + 7) & ~7;
+  S.VK = (max_abf + 15) & ~15;
+  S.SA = (max_abf + 31) & ~31;
+  S.v_bytes = (uint32_t)NP * S.M8 * S.VK * 2u;
+  const uint32_t col = 32u * max_ao_sub;   // bytes of a row of a chunk
+  S.y_bytes = (uint32_t)NP * S.M8 * col;
+  // the operands' reads beyond a block's rows: 128 rows of V and of Y^{AB},
+  // n_abf(B) rounded up to 16 of Y^{BA}, each from its second piece on
+  S.smem = S.v_bytes + 2 * S.y_bytes + 8 * col;
+  S.smem = std::max(S.smem, (uint32_t)(S.M8 + 128) * S.VK * 2u);
+  S.smem = std::max(S.smem, S.v_bytes + (S.M8 + 128) * col);
+  S.smem = (S.smem + 15u) & ~15u;
+  return S;
+}
+
+cudaError_t t2w_set_smem() { return allow_max_dynamic_smem((const void*)k_t2w_umma<kSplitHalf>); }
+
+cudaError_t launch_t2w(const DevPlan& P, const MixPlan& X, const T2WPlan& S, const int* list, int n, long long zblk,
+                       int* err, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  g_t1u_launches += 2;
+  k_t2w_vstore<kSplitHalf><<<std::min(n, 152 * 8), 256, 0, s>>>(P, X, S, list, n);
+  k_t2w_umma<kSplitHalf><<<std::min(n, num_sms()), kT2Threads, S.smem, s>>>(P, X, S, list, n, zblk, err);
   return cudaGetLastError();
 }
 

@@ -99,3 +99,21 @@ def test_wide_anisotropic_gradient_blocks():
     E, F, S, _ = run(w, hfx.HFX_BF16X6, aniso=(Gp, e))
     er = errs((E, F, S), (r.E, r.F, r.sigma))
     assert max(er) <= BOUND, er
+
+
+@pytest.mark.parametrize("n_ao,n_abf", [([17, 16], [64, 65]), ([18, 1], [8, 80]), ([32, 9], [33, 16]),
+                                        ([18, 13], [97, 60]), ([17, 2], [112, 3])])
+@pytest.mark.parametrize("terms", [1, 2])
+def test_sub_block_edges(n_ao, n_abf, terms):
+    """Orbitals just past one sub-block and two full ones, auxiliary sets at
+    and past the 64-row tile, up to those that fall back to the warp-level
+    kernels; each product against the FP64 GPU path, within the contract."""
+    rng = np.random.default_rng(21)
+    pos = np.array([[0.1, 0.2, 0.0], [1.6, 1.5, 1.7]]) + rng.normal(0, 0.05, (2, 3))
+    w = inputs.cut_density(inputs.tiny_model(n_ao, n_abf, [0, 1], np.eye(3) * 3.3, pos, r_c=1.4, seed=21), 4.0)
+    E0, F0, S0, st0 = run(w, hfx.HFX_FP64, terms=terms)
+    E, F, S, st = run(w, hfx.HFX_BF16X6, terms=terms)
+    er = errs((E, F, S), (E0, F0, S0))
+    assert st["triplets"] == st0["triplets"] and st["term2_pairs"] == st0["term2_pairs"]
+    assert abs(st["flops_total"] / st0["flops_total"] - 1.0) < 1e-12
+    assert max(er) <= BOUND, er
