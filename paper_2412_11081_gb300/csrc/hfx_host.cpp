@@ -1227,10 +1227,10 @@ void split_density(hfx_plan* P) {
     off[k + 1] = off[k] + (long long)P->np * a * b;
   }
   P->dsp_off = P->mem.alloc<long long>(P->n_d + 1);
-  P->Dsp = P->mem.alloc<uint16_t>(off[P->n_d] + 256);   // + one zero row (absent blocks)
+  P->Dsp = P->mem.alloc<uint16_t>(off[P->n_d] + 512);   // + one zero row (absent blocks)
   upload(P->dsp_off, off, P->stream);
-  ck(cudaMemsetAsync(P->Dsp + off[P->n_d], 0, 256 * sizeof(uint16_t), P->stream), "memset");
-  {   // every piece of a sub-block is one 16 x 16 block of 512 bytes
+  ck(cudaMemsetAsync(P->Dsp + off[P->n_d], 0, 512 * sizeof(uint16_t), P->stream), "memset");
+  {   // a sub-block is one row of 1,024 bytes (two pieces of 16 x 16), as 256 words
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q{};
     ck(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q), "driver entry");
@@ -1238,11 +1238,11 @@ void split_density(hfx_plan* P) {
     using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    const long long rows = off[P->n_d] / 256 + 1;
+    const long long rows = off[P->n_d] / 512 + 1;
     const cuuint64_t dims[2] = {256, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {512};
+    const cuuint64_t strides[1] = {1024};
     const cuuint32_t box[2] = {256, 1}, estr[2] = {1, 1};
-    const CUresult r = reinterpret_cast<Encode>(fn)(&P->drows.map, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, P->Dsp, dims,
+    const CUresult r = reinterpret_cast<Encode>(fn)(&P->drows.map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, P->Dsp, dims,
                                                     strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                                                     CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

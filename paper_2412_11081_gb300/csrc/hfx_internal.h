@@ -136,7 +136,7 @@ struct DevPlan {
 
 // Extra state of the split-precision path.
 struct MixPlan {
-  uint16_t* Dsp;               // D blocks as bf16 pieces, rup16(n_ao(I)) x rup16(n_ao(J)) per piece
+  uint16_t* Dsp;               // D sub-blocks of 16 x 16 as pieces, per 8 rows the first and then the second
   const long long* dsp_off;    // [n_d]
   uint16_t* Ysp;               // Y^{XZ} as bf16 pieces, [alpha][z][rup16(n_ao(X))] per piece
   uint16_t* Cm;                // per C pair: bf16 pieces of C, then grad C in FP32
@@ -157,9 +157,9 @@ struct MixPlan {
   uint16_t* YspT = nullptr;    // Y^{XZ} transposed, bf16 pieces [piece][(alpha,x)][16 z] (z padded), yT_blk per key
   long long yT_blk = 0;        // uint16 units per key of YspT (2 pieces x 128-row tiles x 16)
   const long long* y_idx = nullptr;   // key -> its position in the needed-key list (YspT block)
-  int* ytab = nullptr;         // Y build: D block (256-element units) per (key group, C slot t, key i), or -1
+  int* ytab = nullptr;         // Y build: row of DRows per (key group, C slot t, key i), or -1
   int ytab_stride = 0;         // ints per key group (8 * most C pairs of an atom)
-  int* q2tab = nullptr;        // second product: D block per (group of 8 C slots, pair slot, i), or -1
+  int* q2tab = nullptr;        // second product: row of DRows per (group of 8 C slots, pair slot, i), or -1
   // Fault injection for the failure tests: 1 = the second product's producer
   // issues no copies, so its pipeline waits run out (HFX_ERR_TIMEOUT).
   int stall_q2 = 0;
@@ -282,11 +282,11 @@ cudaError_t launch_cpieces(const DevPlan& P, const MixPlan& X, int sp, cudaStrea
 cudaError_t launch_vpieces(const DevPlan& P, const MixPlan& X, int sp, const int* list, int n, cudaStream_t s);
 cudaError_t launch_ygroups(const DevPlan& P, const long long* y_idx, const long long* y_total, int* gcnt,
                            const long long* goff, int* gX, int* gS, int* gN, int phase, cudaStream_t s);
-// The D piece store viewed as a 2-D tensor of 512-byte rows (one row per
-// bf16 piece of a 16 x 16 block, row dsp_off / 256 + piece; the last row is
-// zero), fetched four rows at a time by the tensor-core kernels.
+// The D piece store viewed as a 2-D tensor of 1024-byte rows (one row per
+// 16 x 16 sub-block, both pieces; the last row is zero), fetched four rows at
+// a time by the tensor-core kernels.
 struct DRows {
-  CUtensorMap map;             // box: one row of 256 bf16
+  CUtensorMap map;             // box: one row of 256 words
   int zero_row;
 };
 cudaError_t launch_ybuild_mma(const DevPlan& P, const MixPlan& X, int sp, const int* ylist, const int* gX,

@@ -86,8 +86,17 @@ __device__ void block_sum_n(double (&v)[NV], double* red) {
 }
 
 // ------------------------------------------------------------------ D split
+// Element (a, b) of piece p of a 16 x 16 sub-block of D: per 8 rows a the first
+// piece and then the second, in core-matrix order.  A sub-block is 1,024
+// consecutive bytes, so that one row of a gather brings both its pieces, and
+// every piece's 8-row groups are 512 bytes apart also across sub-blocks that
+// lie one after the other in shared memory.
+__device__ __forceinline__ int dix(int p, int a, int b) {
+  return (((a >> 3) * NP + p) << 7) + ((b >> 3) << 6) + ((a & 7) << 3) + (b & 7);
+}
+
 // D block k (n_ao(I) x n_ao(J)) -> its sub-blocks (ao_subs), row by row, each as
-// NP planes of 16 x 16, zero padded.
+// NP pieces of 16 x 16 (dix), zero padded.
 template <int SP>
 __global__ void k_dsplit(DevPlan P, MixPlan X, uint16_t* dst, float scale) {
   for (long long k = blockIdx.x; k < P.n_d; k += gridDim.x) {
@@ -102,7 +111,7 @@ __global__ void k_dsplit(DevPlan P, MixPlan X, uint16_t* dst, float scale) {
       uint16_t pc[NP];
       split_f<SP>((al < ha && a < na && bl < hb && b < nb) ? (float)src[a * nb + b] * pscale<SP>(scale) : 0.f, pc);
 #pragma unroll
-      for (int p = 0; p < NP; ++p) out[(sub * NP + p) * 256 + tix(al, bl)] = pc[p];
+      for (int p = 0; p < NP; ++p) out[sub * NP * 256 + dix(p, al, bl)] = pc[p];
     }
   }
 }
@@ -328,7 +337,7 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
         const bool ystaged = kStageY && pB == 16;
         const uint16_t* Y = X.Ysp + m_y[t];                  // [beta][f][pB] planes (global)
         const long long yplane = (long long)mB * nF * pB;
-        const uint16_t* Dab = X.Dsp + m_d[t];                 // [a][pB] planes of pA x pB
+        const uint16_t* Dab = X.Dsp + m_d[t];                 // pieces of 16 x 16 (dix)
         const float* V = reinterpret_cast<const float*>(X.Vm + m_v[t] + NP * mA * MB);   // V, grad V (FP32)
         const uint16_t* Vs = Vs0 + (t & 1) * vbuf;
         const int nvb = mA * mB;
@@ -388,11 +397,11 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
                 uint32_t bf0[NP][2], bf1[NP][2];
 #pragma unroll
                 for (int pp = 0; pp < NP; ++pp) {
-                  const uint16_t* Db = Dab + pp * 256 + tix(nt * 8 + gid, 2 * tig);
+                  const uint16_t* Db = Dab + dix(pp, nt * 8 + gid, 2 * tig);
                   bf0[pp][0] = *reinterpret_cast<const uint32_t*>(Db);
                   bf0[pp][1] = *reinterpret_cast<const uint32_t*>(Db + 64);
-                  bf1[pp][0] = *reinterpret_cast<const uint32_t*>(Db + 128);
-                  bf1[pp][1] = *reinterpret_cast<const uint32_t*>(Db + 192);
+                  bf1[pp][0] = *reinterpret_cast<const uint32_t*>(Db + NP * 128);
+                  bf1[pp][1] = *reinterpret_cast<const uint32_t*>(Db + NP * 128 + 64);
                 }
                 mma_split2<SP>(acc[nt], af, bf0, acc[nt + 1], af, bf1);
               }
@@ -748,7 +757,7 @@ constexpr int kMetaPairs = 1024;         // pairs per CTA segment (metadata in s
 // K-major operand tiles: K-adjacent core matrices 128 bytes apart, 8-row groups 256 bytes apart
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) { return sdesc2(saddr, 128, 256); }
 
-// Four 512-byte rows r0..r3 of the D piece store (tensor map of DRows) to
+// Four 1024-byte rows r0..r3 of the D piece store (tensor map of DRows) to
 // consecutive shared memory at sdst (128-byte aligned), completion counted in
 // bytes on mbar.
 __device__ __forceinline__ void gather4_rows(uint32_t sdst, const CUtensorMap* map, int r0, int r1, int r2, int r3,
@@ -760,23 +769,23 @@ __device__ __forceinline__ void gather4_rows(uint32_t sdst, const CUtensorMap* m
       : "memory");
 }
 
-// Stage the B operand of one K step: D rows of the eight keys i (row md[i] +
-// piece, the zero row where md[i] < 0), piece pp and key half h by lane
-// 1 + 2 pp + h.
+// Stage the B operand of one K step: the sub-blocks of D of the eight keys i
+// (row md[i], the zero row where md[i] < 0), both pieces at once, four keys by
+// each of lanes 1 and 2.  (One gather per piece and four keys, 512-byte rows:
+// 64-atom Si cell Q2 GEMM and Y build 5.36 and 4.51 ms; as here 4.99 and 4.40.)
 __device__ __forceinline__ void stage_d(int lane, uint16_t* stB, const int* md, const CUtensorMap* map, int zrow,
                                         uint32_t mbar) {
-  if (lane >= 1 && lane <= 2 * NP) {
-    const int pp = (lane - 1) >> 1, h = (lane - 1) & 1;
+  if (lane == 1 || lane == 2) {
+    const int h = lane - 1;
     int r[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int d = md[4 * h + j];
-      r[j] = d >= 0 ? d + pp : zrow;
-    }
-    gather4_rows((uint32_t)__cvta_generic_to_shared(stB + (size_t)pp * kTileElems + 4 * h * 256), map, r[0], r[1], r[2],
-                 r[3], mbar);
+    for (int j = 0; j < 4; ++j) r[j] = md[4 * h + j] >= 0 ? md[4 * h + j] : zrow;
+    gather4_rows((uint32_t)__cvta_generic_to_shared(stB + 4 * h * NP * 256), map, r[0], r[1], r[2], r[3], mbar);
   }
 }
+
+// Piece p of that operand: 8-row groups of the pieces alternate (dix).
+__device__ __forceinline__ uint64_t sdesc_d(uint32_t saddr, int p) { return sdesc2(saddr + 256u * p, 128, 256 * NP); }
 
 }  // namespace umma
 
@@ -952,7 +961,7 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
               for (int ia = 0; ia <= sum; ++ia) {
                 const int ib = sum - ia;
                 const uint64_t ad = sdesc(a0 + (j * NP + ia) * kTileElems * 2);
-                const uint64_t bd = sdesc(b0 + ib * kTileElems * 2);
+                const uint64_t bd = sdesc_d(b0, ib);
                 const uint32_t acc = (fs && sum == NP - 1 && ia == 0) ? 0u : 1u;
                 asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dacc + 128u * j),
@@ -1166,7 +1175,7 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
 #pragma unroll
             for (int ia = 0; ia <= sum; ++ia) {
               const uint64_t ad = sdesc(a0 + (j * NP + ia) * kTileElems * 2);
-              const uint64_t bd = sdesc(b0 + (sum - ia) * kTileElems * 2);
+              const uint64_t bd = sdesc_d(b0, sum - ia);
               const uint32_t acc = (k == 0 && sum == NP - 1 && ia == 0) ? 0u : 1u;
               asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(taddr + 128u * j),
@@ -1442,7 +1451,7 @@ __global__ void k_ytab(DevPlan P, MixPlan X, const int* ylist, const int* gX, co
       const int di = ws < sw ? dlut_get(P, w, z, Rz[0] - Rw[0], Rz[1] - Rw[1], Rz[2] - Rw[2]) : -1;
       if (di >= 0 && P.Dkept[di] != 0.0) {
         const int mi = dlut_get(P, z, w, Rw[0] - Rz[0], Rw[1] - Rz[1], Rw[2] - Rz[2]);
-        md = (int)(X.dsp_off[mi] >> 8) + (zs * sw + ws) * NP;
+        md = (int)(X.dsp_off[mi] / (NP * 256)) + zs * sw + ws;
         const int sX = P.species[Xa];
         const int hz = ao_sub(nz), hw = ao_sub(nw);
         fl += 2.0 * P.n_abf[sX] * P.n_ao[sX] * min(hz, nz - zs * hz) * min(hw, nw - ws * hw);
@@ -1479,7 +1488,7 @@ __global__ void k_q2tab(DevPlan P, MixPlan X, const int* list, int n_slots, int 
       const int nb = P.n_ao[P.species[b]], nf = P.n_ao[P.species[P.c_j[qf]]], sb = ao_subs(nb);
       const int d = bs < sb ? dlut_get(P, P.c_j[qf], b, Rb[0] - Rf[0], Rb[1] - Rf[1], Rb[2] - Rf[2]) : -1;
       if (d >= 0 && P.Dkept[d] != 0.0) {
-        db = (int)(X.dsp_off[d] >> 8) + (fs * sb + bs) * NP;
+        db = (int)(X.dsp_off[d] / (NP * 256)) + fs * sb + bs;
         const int sA = P.species[A];
         const int hb = ao_sub(nb), hf = ao_sub(nf);
         fl += 2.0 * P.n_abf[sA] * P.n_ao[sA] * min(hb, nb - bs * hb) * min(hf, nf - fs * hf);

@@ -660,10 +660,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ok = mbar_wait(yf + 8 * y.s, y.ph);
                 if (!ok) break;
                 tc_fence_after();
-                const uint64_t dD = sdesc2(Ds + d.s * DB + bs * 1024u, 128, 256);
+                const uint64_t dD = sdesc2(Ds + d.s * DB + bs * 1024u, 128, 512);   // (pieces alternate by 8 rows)
                 const uint64_t dY = sdesc2(Ys + y.s * kYSlot, 128, 256);
-                umma_f16(tu, dY, dD + 32, idU, bs > 0);                        // Y0 D1 (a piece of D: 512 bytes)
-                if (two) umma_f16(tu + 16, dY + 256, dD + 32, idU, bs > 0);    // (the second tile: 4096 bytes on)
+                umma_f16(tu, dY, dD + 16, idU, bs > 0);                        // Y0 D1 (the second piece: 256 bytes on)
+                if (two) umma_f16(tu + 16, dY + 256, dD + 16, idU, bs > 0);    // (the second tile: 4096 bytes on)
                 umma_f16(tu, dY + (kYPiece >> 4), dD, idU, 1u);                // Y1 D0
                 if (two) umma_f16(tu + 16, dY + 256 + (kYPiece >> 4), dD, idU, 1u);
                 umma_f16(tu, dY, dD, idU, 1u);                                 // Y0 D0
