@@ -1060,8 +1060,13 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
 // TPC row tiles of 128 rows per CTA share each K step's D blocks (one
 // accumulator of 128 columns per tile).
 
+// Four epilogue warps per row tile: the epilogue, which splits and writes every
+// Y block in two orders, bounds the kernel (one group of four for both tiles:
+// 64-atom Si cell Y stage 4.88 ms, 3.98 with one each).
+constexpr int yb_threads(int tpc) { return 64 + 128 * tpc; }
+
 template <int SP, int TPC, bool SUB>
-__global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const int* ylist, const int* gX,
+__global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixPlan X, const int* ylist, const int* gX,
                                                      const int* gS, const int* gN, int MC,
                                                      const __grid_constant__ DRows drows, int* err) {
   using namespace umma;
@@ -1188,7 +1193,7 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
                    : "memory");
     }
   } else {
-    // epilogue (warps 2..5): the accumulator (rows (alpha, x), columns
+    // epilogue (warps 2..5, and 6..9 for the second tile): the accumulator (rows (alpha, x), columns
     // (key, z)) passes through shared memory, two keys at a time, in the
     // stage ring (idle once the last MMA has completed), so that the Y store
     // and its FP32 copy are written as whole 16-byte chunks of complete
@@ -1196,8 +1201,8 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
     // row tiles is written element by element by both; the tile that holds
     // x = n_ao - 1 writes its padding.
     const int q = warp & 3;
-    const int et = tid - 64;
-    float* ep = reinterpret_cast<float*>(smem_raw);   // [128][33]
+    const int jt = (warp - 2) >> 2, et = (tid - 64) & 127;
+    float* ep = reinterpret_cast<float*>(smem_raw) + jt * 128 * 33;   // [128][33]
     bool have = nsteps > 0;
     if (have) {
       if (!mbar_wait<kMixTryNs>(maccf, 0u)) {
@@ -1206,7 +1211,7 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
       }
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     }
-    for (int jt = 0; jt < ntile; ++jt) {
+    if (jt < ntile) {
     const int row0 = (mc + jt) * 128;
     const int rend = min(row0 + 128, rows);
     const int alF = (row0 + nX - 1) / nX, alL = rend / nX - 1;
@@ -1225,7 +1230,7 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
 #pragma unroll
         for (int j = 0; j < 32; ++j) er[j] = __uint_as_float(v[j]) * pscale<SP>(P.sc.y);
       }
-      asm volatile("bar.sync 1, 128;\n" ::: "memory");
+      asm volatile("bar.sync %0, 128;\n" ::"r"(1 + jt) : "memory");
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         const int i = (c0 >> 4) + h;
@@ -1392,7 +1397,7 @@ __global__ void __launch_bounds__(192) k_ybuild_umma(DevPlan P, MixPlan X, const
           }
         }
       }
-      asm volatile("bar.sync 1, 128;\n" ::: "memory");
+      asm volatile("bar.sync %0, 128;\n" ::"r"(1 + jt) : "memory");
     }
     }
   }
@@ -1593,7 +1598,7 @@ cudaError_t launch_ybuild_mma(const DevPlan& P, const MixPlan& X, int sp, const 
   const int tpc = X.ybtpc == 1 ? 1 : 2;
   const long long grid = (long long)ngroups * ((MC + tpc - 1) / tpc);
   const size_t sm = ybuild_umma_smem(tpc, X.ytab_stride);
-  ybuild_kern(sp, X.KB > 1, tpc)<<<(unsigned)grid, 192, sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
+  ybuild_kern(sp, X.KB > 1, tpc)<<<(unsigned)grid, yb_threads(tpc), sm, s>>>(P, X, ylist, gX, gS, gN, MC, drows, err);
   return cudaGetLastError();
 }
 
