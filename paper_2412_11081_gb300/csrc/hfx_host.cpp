@@ -1130,7 +1130,7 @@ void setup_shapes(hfx_plan* P) {
     P->MC = (maxrows + 127) / 128;
     P->zblk = (long long)P->np * P->MC * 128 * 16;
     P->ybtpc = 2;
-    P->q2tpc = P->sp == hfx::kSplitHalf ? 3 : 2;
+    P->q2tpc = 3;
     P->q2_flush = 32;   // K steps per FP32 run (beside t1u_seg)
     ck(hfx::set_wide_smem_limits(P->sp), "smem attributes");
     ck(hfx::set_mixed_smem_limits(P->sp, P->KB > 1), "smem attributes");
@@ -1195,8 +1195,8 @@ void setup_shapes(hfx_plan* P) {
     const char* yt = std::getenv("HFX_Y_TILES");
     const char* qt = std::getenv("HFX_Q2_TILES");
     P->ybtpc = yt && std::atoi(yt) == 1 ? 1 : 2;
-    // (BF16X6 starts from the deep pipeline: si1000 second product 172.6 -> 139.6 ms)
-    P->q2tpc = qt && (std::atoi(qt) >= 1 && std::atoi(qt) <= 3) ? std::atoi(qt) : (P->sp == hfx::kSplitHalf ? 3 : 2);
+    // (the deep pipeline: 1000-atom Si cell second product 172.6 -> 139.6 ms)
+    P->q2tpc = qt && (std::atoi(qt) >= 1 && std::atoi(qt) <= 3) ? std::atoi(qt) : 3;
     const char* qf = std::getenv("HFX_Q2_FLUSH");
     P->q2_flush = qf ? std::max(1, std::atoi(qf)) : (P->sp == hfx::kSplitHalf ? 128 : 32);   // as t1u_seg
     ck(hfx::set_mixed_smem_limits(P->sp, P->KB > 1), "smem attributes");
@@ -1648,7 +1648,7 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
              "term2");
         }
         ck(hfx::launch_q2(D, X, P->sp, P->t2_list + v0, P->t2_idx, (int)ct[CT_T2], a0, a1, P->zblk, FC, P->MC,
-                          hfx::q2_umma_segments(P->maxV * P->KB, P->q2tpc), P->q2_flush, P->drows, P->d_err, s),
+                          hfx::q2_umma_segments(P->maxV * P->KB), P->q2_flush, P->drows, P->d_err, s),
            "Q2");
       } else
         ck(hfx::launch_term2(D, P->t2_list + v0, (int)ct[CT_T2], P->alpha_chunk, P->smem_t2, s), "term2");
@@ -1699,7 +1699,7 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
         ck(hfx::launch_t2_umma(D, X, P->sp, P->t2_list + v0, (int)ct[CT_T2], P->zblk, P->smem_t2u, P->d_err, s),
            "term2 R2 and Z");
       ck(hfx::launch_term2_mma(D, X, P->sp, P->t2_list + v0, P->t2_idx, (int)ct[CT_T2], a0, a1, P->MAmax, P->KZmax,
-                               P->zblk, P->ZROWS, FC, P->MC, hfx::q2_umma_segments(P->maxV, P->q2tpc), P->q2_flush,
+                               P->zblk, P->ZROWS, FC, P->MC, hfx::q2_umma_segments(P->maxV), P->q2_flush,
                                P->drows, P->smem_m2, P->d_err, s, P->t2u),
          "term2");
     }

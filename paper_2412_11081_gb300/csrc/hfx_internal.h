@@ -309,7 +309,7 @@ cudaError_t launch_term2_mma(const DevPlan& P, const MixPlan& X, int sp, const i
                              int n, int a0, int a1, int MAmax, int KZmax, long long zblk, int zrows, int FC, int MC,
                              int nseg, int flush, const DRows& drows, size_t smem, int* err, cudaStream_t s,
                              bool pairs_done = false);
-int q2_umma_segments(int max_steps_per_atom, int tpc);
+int q2_umma_segments(int max_steps_per_atom);
 // The Q2 GEMM alone, from a Z store of KB blocks per pair slot.
 cudaError_t launch_q2(const DevPlan& P, const MixPlan& X, int sp, const int* list, const long long* slot0, int n, int a0,
                       int a1, long long zblk, int FC, int MC, int nseg, int flush, const DRows& drows, int* err,

@@ -792,23 +792,26 @@ __device__ __forceinline__ uint64_t sdesc_d(uint32_t saddr, int p) { return sdes
 // TPC row tiles of 128 rows per CTA share each K step's D blocks (the B
 // operand): with TPC = 2 a step moves 3 NP tiles for two tiles' work instead
 // of 2 NP for one, in 3 stages (two CTAs fit an SM), one accumulator per tile (no double buffer; two CTAs per SM overlap
-// one's epilogue with the other's MMAs) and 512 pairs of metadata; TPC = 1
+// one's epilogue with the other's MMAs); TPC = 1
 // keeps 4 stages and two accumulators.  DEEP = 1 (with TPC = 2) runs one
 // CTA per SM instead: 6 stages to cover the copies' latency
 // and two accumulators per tile (all 512 tensor-memory columns), so the
-// epilogue of one run overlaps the next run's MMAs within the CTA.
+// epilogue of one run overlaps the next run's MMAs within the CTA, and four
+// epilogue warps for each tile, which halve what follows the last run.  With
+// parts of at most 512 steps and four epilogue warps the 64-atom Si cell's
+// second product took 6.48 ms, 6.06 as here (HFX_BF16X3 8.50 in the two-CTA
+// shape, 6.30 here).
 template <int TPC, int DEEP = 0>
 struct Q2Shape {
   static constexpr int kS = DEEP ? 6 : TPC == 2 ? 3 : umma::kStages;   // stages
-  static constexpr int kMP = TPC == 2 ? 512 : umma::kMetaPairs;        // pairs per CTA segment
   static constexpr int kNB = TPC == 2 && !DEEP ? 1 : 2;                // accumulator buffers
   static constexpr int kCols = kNB * TPC * 128;                        // tensor-memory columns
 };
 
 // SUB: some block has more than 16 orbitals (X.KB sub-blocks at most).
 template <int SP, int TPC, int DEEP, bool SUB>
-__global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int* list, const long long* slot0,
-                                                 int n_slots, int a0, int a1, int FC8, int MC, int NSEG,
+__global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevPlan P, MixPlan X, const int* list, const long long* slot0,
+                                                 int n_slots, int a0, int a1, int FC8, int MC, int NSEG, int q2parts,
                                                  long long zblk, int flush, const __grid_constant__ DRows drows,
                                                  int* err) {
   // Warp roles: warp 0 lane 0 produces (bulk async copies into a stage
@@ -816,14 +819,14 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
   // MMAs (all piece products of a pair into the TMEM accumulators, commits
   // free the stage / hand the accumulators to the epilogue); warps 2..5 read
   // the accumulators (each its 32-lane quarter of tensor memory) and dot
-  // them with grad C_AF.  No block barrier inside the pipeline.
+  // them with grad C_AF (DEEP: warps 2..9, four per tile).  No block barrier inside the pipeline.
   using namespace umma;
-  constexpr int KS = Q2Shape<TPC, DEEP>::kS, KMP = Q2Shape<TPC, DEEP>::kMP, NB = Q2Shape<TPC, DEEP>::kNB;
+  constexpr int KS = Q2Shape<TPC, DEEP>::kS, NB = Q2Shape<TPC, DEEP>::kNB;
   constexpr int TCOLS = Q2Shape<TPC, DEEP>::kCols;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   uint16_t* stA = reinterpret_cast<uint16_t*>(smem_raw);                  // [KS][TPC][NP][kTileElems]
   uint16_t* stB = stA + (size_t)KS * TPC * NP * kTileElems;               // [KS][NP][kTileElems]
-  int* m_dblk = reinterpret_cast<int*>(stB + (size_t)KS * NP * kTileElems);   // [KMP][8]
+  int* m_dblk = reinterpret_cast<int*>(stB + (size_t)KS * NP * kTileElems);   // [kMetaPairs][8]
   __shared__ __align__(8) uint64_t bar_full[KS], bar_empty[KS], bar_accf[2], bar_acce[2];
   __shared__ uint32_t tmem_base;
   __shared__ double sg[8][3];
@@ -847,8 +850,13 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
   const int ntile = min(TPC, nt - mc);   // row tiles of this CTA
   const long long s0 = slot0[P.v_ptr[A]] * (SUB ? X.KB : 1);   // K steps (pair slot, sub)
   const long long s1 = A + 1 < a1 ? slot0[P.v_ptr[A + 1]] * (SUB ? X.KB : 1) : (long long)n_slots;
-  const long long p0 = s0 + (long long)seg * KMP;
-  const int np = (int)max(0ll, min((long long)KMP, s1 - p0));
+  // A part costs a prologue and an epilogue that nothing overlaps, 0.8 ms per
+  // part and atom on the 64-atom Si cell (5 ms in all): as few as the
+  // metadata allow (q2_least: more on small cells), of equal length.
+  const int steps = (int)(s1 - s0), parts = max((steps + kMetaPairs - 1) / kMetaPairs, q2parts);
+  const int len = (steps + parts - 1) / parts;
+  const long long p0 = s0 + (long long)seg * len;
+  const int np = (int)max(0ll, min((long long)len, s1 - p0));
   if (np <= 0) return;
   const int row0 = mc * 128;
   int qf[8], qs[8];   // C pair (or -1) and sub of each column slot
@@ -878,7 +886,7 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
     }
     for (int b = 0; b < 2; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(maccf + 8 * b));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;\n" ::"r"(macce + 8 * b));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(macce + 8 * b), "r"(DEEP ? 8 : 4));
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
   }
@@ -975,7 +983,7 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
       }
     }
   } else {
-    // epilogue: warps 2..5, tensor-memory lane quarter q = warp % 4
+    // epilogue: warps 2..5 (DEEP: and 6..9, which take the second tile), tensor-memory lane quarter q = warp % 4
     const int q = warp & 3;
     double gd[8][3];
 #pragma unroll
@@ -987,7 +995,8 @@ __global__ void __launch_bounds__(192) k_q2_umma(DevPlan P, MixPlan X, const int
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      for (int j = 0; j < ntile; ++j) {
+      const int grp = (warp - 2) >> 2;
+      for (int j = grp; j < (DEEP ? min(grp + 1, ntile) : ntile); ++j) {
       const int r = row0 + 128 * j + q * 32 + lane;
       const bool rv = r < rows;
 #pragma unroll
@@ -1511,17 +1520,14 @@ size_t ybuild_umma_smem(int tpc, int stride) {   // stride: 8 ints per K step
 }
 
 size_t q2_umma_smem(int tpc) {   // tpc 3: two tiles, the deep pipeline
-  if (tpc >= 2) {
-    const int ks = tpc == 3 ? Q2Shape<2, 1>::kS : Q2Shape<2>::kS;
-    return (size_t)ks * 3 * NP * umma::kTileElems * sizeof(uint16_t) + (size_t)Q2Shape<2>::kMP * 8 * sizeof(int);
-  }
-  return (size_t)2 * Q2Shape<1>::kS * NP * umma::kTileElems * sizeof(uint16_t) +
-         (size_t)Q2Shape<1>::kMP * 8 * sizeof(int);
+  const int ks = tpc == 3 ? Q2Shape<2, 1>::kS : tpc == 2 ? Q2Shape<2>::kS : Q2Shape<1>::kS;
+  return (size_t)ks * (tpc == 1 ? 2 : 3) * NP * umma::kTileElems * sizeof(uint16_t) +
+         (size_t)umma::kMetaPairs * 8 * sizeof(int);
 }
 
 // The Y build and Q2 GEMM of a split, tile shape (tpc as MixPlan::q2tpc) and sub-blocks or not.
 using YKern = void (*)(DevPlan, MixPlan, const int*, const int*, const int*, const int*, int, const DRows, int*);
-using Q2Kern = void (*)(DevPlan, MixPlan, const int*, const long long*, int, int, int, int, int, int, long long, int,
+using Q2Kern = void (*)(DevPlan, MixPlan, const int*, const long long*, int, int, int, int, int, int, int, long long, int,
                         const DRows, int*);
 template <int SP, bool SUB>
 YKern ybuild_kern(int tpc) {
@@ -1552,9 +1558,28 @@ long long mixed_launch_count() { return g_mix_launches; }
 long long ytab_size(int ngroups, int maxC) { return (long long)ngroups * 8 * maxC; }
 long long q2tab_size(long long n_slots, int FC) { return n_slots * ((FC * 4 + 7) / 8) * 8; }
 
-int q2_umma_segments(int max_steps_per_atom, int tpc) {
-  const int kmp = tpc >= 2 ? Q2Shape<2>::kMP : Q2Shape<1>::kMP;
-  return (max_steps_per_atom + kmp - 1) / kmp;
+// Most parts of an atom's K steps, one CTA each (the kernel takes as many as
+// its own count of steps needs, and at least q2_least): by the whole
+// structure's sizes and not by the tile shape, so that neither the passes nor
+// the autotuner move the FP32 runs' ends.
+int q2_umma_segments(int max_steps_per_atom) {
+  return std::max(1, (max_steps_per_atom + umma::kMetaPairs - 1) / umma::kMetaPairs);
+}
+// Parts that finish first: waves of CTAs times the length of one, a part's
+// fixed cost being about a sixth of an atom's whole.  (8-atom Si cell, 200
+// CTAs: second product 1.00 ms in one part, 0.93 in two; large cells take one.)
+int q2_least(int n_atoms, int FC8, int MC) {
+  const int ctas = n_atoms * FC8 * ((MC + 1) / 2), sms = sm_count();
+  int best = 1;
+  double least = 0.0;
+  for (int p = 1; p <= 4; ++p) {
+    const double t = (double)(((long long)ctas * p + sms - 1) / sms) * (1.0 / p + 1.0 / 6.0);
+    if (p == 1 || t < 0.98 * least) {
+      best = p;
+      least = t;
+    }
+  }
+  return best;
 }
 
 cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, uint16_t* dst, float scale, int sp, cudaStream_t s) {
@@ -1661,9 +1686,11 @@ cudaError_t launch_q2(const DevPlan& P, const MixPlan& X, int sp, const int* lis
   k_q2tab<<<grid_for(((long long)ns * FC8 * 8 + 255) / 256, 152 * 16), 256, 0, s>>>(P, X, list, ns, FC8);
   const int tpc = X.q2tpc == 1 ? 1 : 2, deep = X.q2tpc == 3 ? 1 : 0;   // row tiles per CTA; the deep pipeline
   const size_t sq = q2_umma_smem(X.q2tpc == 1 ? 1 : (deep ? 3 : 2));
+  const int least = q2_least(P.N, FC8, MC);
+  nseg = std::max(nseg, least);
   const long long grid = (long long)(a1 - a0) * FC8 * ((MC + tpc - 1) / tpc) * nseg;
-  q2_kern(sp, X.KB > 1, tpc == 1 ? 1 : deep ? 3 : 2)<<<(unsigned)grid, 192, sq, s>>>(
-      P, X, list, slot0, ns, a0, a1, FC8, MC, nseg, zblk, flush, drows, err);
+  q2_kern(sp, X.KB > 1, tpc == 1 ? 1 : deep ? 3 : 2)<<<(unsigned)grid, deep ? 320 : 192, sq, s>>>(
+      P, X, list, slot0, ns, a0, a1, FC8, MC, nseg, least, zblk, flush, drows, err);
   return cudaGetLastError();
 }
 
