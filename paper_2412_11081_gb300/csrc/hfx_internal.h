@@ -390,7 +390,7 @@ cudaError_t launch_term1_w(const DevPlan& P, int sp, const uint16_t* Yp, const u
 // rup16(n_ao(I)) x rup16(n_ao(J)) at Dw + dw_off[k] (multiples of 256)
 cudaError_t launch_dsplit_w(const DevPlan& P, int sp, uint16_t* Dw, const long long* dw_off, cudaStream_t s);
 // Second product of the home atoms [a0, a1): k_term2_w over the pass's pair
-// list (E, g^V and the Z piece store), then k_q2_w (grad C); slot0 as launch_term2_mma.
+// list (E, g^V and the Z piece store).
 cudaError_t launch_term2_w(const DevPlan& P, int sp, const uint16_t* Yp, uint16_t* Zst, long long zblk, int KB,
                            const int* list, int n, const WideShapes& w, cudaStream_t s);
 

@@ -195,3 +195,45 @@ def test_mixed_single_atom_cell_self_images_only(prec):
     E, F, S, _ = run(w, prec)
     assert np.max(np.abs(F)) <= 1e-10 * abs(r.E)
     assert abs(E - r.E) <= BOUND * abs(r.E) and rel(S, r.sigma) <= BOUND
+
+
+def _edge_cell(n_ao, n_abf, seed=31):
+    rng = np.random.default_rng(seed)
+    pos = np.array([[0.1, 0.2, 0.0], [1.5, 1.7, 1.4]]) + rng.normal(0, 0.05, (2, 3))
+    w = inputs.tiny_model(n_ao, n_abf, [0, 1], np.eye(3) * 3.2, pos, r_c=1.3, seed=seed)
+    return inputs.cut_density(w, 3.5)
+
+
+@pytest.mark.parametrize("prec,tol", [(hfx.HFX_BF16X6, BOUND), (hfx.HFX_BF16X3, 1e-4)])
+@pytest.mark.parametrize("n_ao,n_abf", [([1, 16], [1, 64]), ([16, 15], [8, 9]), ([4, 4], [16, 17]), ([13, 2], [50, 33])])
+def test_block_shape_edges(n_ao, n_abf, prec, tol):
+    """Blocks at and beside the 16-column, 8-row and 32- and 64-row edges of
+    the tensor-memory kernels, against the FP64 GPU path.  HFX_BF16X6 within
+    its contract; HFX_BF16X3 within four operands of 2^-16 each (6e-5), taken as 1e-4."""
+    w = _edge_cell(n_ao, n_abf)
+    if prec == hfx.HFX_BF16X6 and max(n_ao) == 16 and max(n_abf) == 64:
+        # HFX_BF16X6 takes the shapes whose operands would fit in three pieces each
+        with pytest.raises(hfx.HfxError) as e:
+            run(w, prec)
+        assert e.value.status == 6
+        return
+    E0, F0, S0, st0 = run(w, hfx.HFX_FP64)
+    E, F, S, st = run(w, prec)
+    assert st["triplets"] == st0["triplets"] and st["term2_pairs"] == st0["term2_pairs"]
+    assert abs(E - E0) <= tol * abs(E0) and rel(F, F0) <= tol and rel(S, S0) <= tol
+
+
+@pytest.mark.parametrize("g,m,d", [(30, -20, 12), (-25, 18, -30), (0, 40, -8)])
+def test_operands_far_from_one(g, m, d):
+    """fp16 pieces are scaled by powers of two taken from the blocks' bounds:
+    templates and D times powers of two give the same result times their
+    product (E ~ C^2 V D^2), up to the order of the FP64 additions."""
+    import dataclasses
+    zero = dict.fromkeys(("C", "dC", "V", "dV", "D", "CS"), 0.0)
+    w = _edge_cell([5, 3], [11, 7])
+    w2 = dataclasses.replace(w, G=[x * 2.0 ** g for x in w.G], M=[x * 2.0 ** m for x in w.M], d_values=w.d_values * 2.0 ** d)
+    a, b = run(w, hfx.HFX_BF16X6, theta=zero), run(w2, hfx.HFX_BF16X6, theta=zero)
+    f = 2.0 ** (2 * g + m + 2 * d)
+    assert a[3]["triplets"] == b[3]["triplets"]
+    for x, y in zip(a[:3], b[:3]):
+        assert rel(np.asarray(y) / f, x) <= 1e-12

@@ -243,3 +243,14 @@ def test_pair_lists_on_thin_and_sheared_cells(make, seed):
     for k in ("c_pairs", "triplets", "term1_pairs", "term2_pairs", "y_blocks"):
         assert st[k] == r.counts[k], (k, st[k], r.counts[k])
     assert_parity(g, r)
+
+
+@pytest.mark.parametrize("n_ao,n_abf", [([1, 20], [1, 40]), ([5, 2], [70, 3]), ([8, 4], [16, 64])])
+def test_fp64_block_shape_edges(n_ao, n_abf):
+    """Blocks at both sides of the small-block launch shape (1,024 elements)
+    and with more than a block of rows, a small cell's pairs divided over
+    several CTAs."""
+    rng = np.random.default_rng(17)
+    pos = np.array([[0.1, 0.2, 0.0], [1.5, 1.7, 1.4]]) + rng.normal(0, 0.05, (2, 3))
+    w = inputs.cut_density(inputs.tiny_model(n_ao, n_abf, [0, 1], np.eye(3) * 3.2, pos, r_c=1.3, seed=17), 3.5)
+    assert_parity(gpu_eval(w), evaluate(w))

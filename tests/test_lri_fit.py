@@ -91,3 +91,17 @@ def test_gpu_fit_errors():
     assert ei.value.status == 6
     X = hfx.lri_fit(A, B)              # the library is still usable
     assert rel(X, oracle.fit_batch(A, B, dA, dB)[0]) <= 1e-10
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(1, 1, 1, 1, 1), (64, 64, 3, 11, 3), (17, 16, 4, 8, 33), (5, 2, 13, 13, 153)])
+def test_gpu_fit_column_and_row_blocks(shape):
+    """n and w at and beside the blocks of 8 rows and 32 columns: n 2, 128, 33
+    and 7; w 1, 33, 32 and 169."""
+    from paper_2412_11081_gb300 import hfx
+    mi, mk, ni, nk, batch = shape
+    d, A, B, dA, dB, _ = inputs.lri_pairs(batch, mi, mk, ni, nk, seed=12)
+    X, dX = hfx.lri_fit(A, B, dA, dB)
+    Xr, dXr = oracle.fit_batch(A, B, dA, dB)
+    assert rel(X, Xr) <= 1e-10 and rel(dX, dXr) <= 1e-10
+    assert rel(hfx.lri_fit(A, B), Xr) <= 1e-10
