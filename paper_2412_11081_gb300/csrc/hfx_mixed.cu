@@ -736,17 +736,19 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
 }
 
 // ------------------------------------------------------------ tcgen05 Q2 GEMM
-// Same product as k_q2_gemm on the 5th-generation tensor cores: per CTA
-// (home atom A, 8 C slots F, 128 rows (alpha,a)), D[row][(F,f)] +=
-// Z^{AB}[row][b] D_FB[f][b] over the pairs (A,B) of the second product, one
-// k16 step per pair and all bf16 piece products into one FP32 accumulator in
-// tensor memory (128 lanes x 128 columns).  Operands are staged by cp.async in
-// the K-major no-swizzle core-matrix layout (8 rows x 16 bytes per core
-// matrix; LBO = 128 B between the two K halves, SBO = 256 B between 8-row
-// groups) through a 4-stage ring; thread 0 issues the MMAs and commits each
-// stage to an mbarrier.  Every 32 pairs the accumulator is read back
-// (tcgen05.ld) and dotted with grad C_AF into FP64.  Every wait is bounded;
-// on timeout the CTA sets *err and stops.
+// Q2 = sum_B Z^{AB} D_FB^T dotted with grad C_AF: per CTA (home atom A, 8
+// column slots (F, sub), one or two tiles of 128 rows (alpha,a), a part of the
+// K steps), D[row][(F,f)] += Z^{AB}[row][b] D_FB[f][b] over the pairs (A,B)
+// of the second product, one k16 step per pair and sub of b with its three
+// piece products into one FP32 accumulator in tensor memory.  Operands lie
+// in the K-major no-swizzle core-matrix order (8 rows x 16 bytes per core
+// matrix).  Every `flush` steps the accumulator is read back and dotted with
+// grad C_AF into FP64.  Every wait is bounded; on timeout the CTA sets *err
+// and stops.
+// What bounds it: of about 800 cycles per step and two tiles 384 are tensor
+// work (six instructions of N = 128) and 24 KB come from L2 (6.7 TB/s over the
+// chip); the rest is the copies' latency, the prologue (the steps in use) and
+// the last run's epilogue of each CTA.
 namespace umma {
 
 constexpr int kStages = 4;

@@ -23,9 +23,9 @@
 // traffic, 105 KB of L2 reads.  The kernel before built U in FP32 on the CUDA
 // cores, two warps per scheduler with 64 registers of D each: 12,900 cycles
 // per triplet, most of them the latency of its shared-memory loads and FMA
-// chains; this one takes 5,100 (64-atom Si cell 36.7 -> 13.5 ms, 8 atoms 7.0 ->
-// 1.6 ms), the hand-offs between its roles and the fetch latency of Y, one
-// triplet ahead, being what is left.
+// chains; this one takes 5,200 (64-atom Si cell 36.7 -> 13.7 ms, 8 atoms 7.0 ->
+// 1.7 ms; tensor pipe active 34 %), the hand-offs between its roles being what
+// is left.  (Y and V fetched into L2 some B ahead: 14.7-20 ms.)
 //
 // Column order (f,a) = 16 f + a with a padded to 16.  All matrices sit in
 // shared memory in the no-swizzle core-matrix order (8 rows x 16 bytes); U
