@@ -846,7 +846,11 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
     const int sX = P->species[y_home[y]], sz = P->species[y_j[y]];
     if (P->t2u)  // pieces of rup8(n_abf(X)) rows alpha x (z, x) columns in core-matrix order
       y_size[y] = (long long)P->np * ((P->n_abf[sX] + 7) / 8 * 8) * 16 * P->n_ao[sz];
-    else if (P->np)  // pieces of [alpha][z][rup16(n_ao(X))]
+    else if (P->np && P->t1u) {  // the first product's store, at least as long as the second's: per sub of x (and, in
+      // the transposed store of t2w, of z) rup8(n_abf(X)) rows alpha x (z, 16 x) columns
+      const int hz = hfx::ao_subs(P->n_ao[sX]) * P->n_ao[sz], hx = P->t2w ? hfx::ao_subs(P->n_ao[sz]) * P->n_ao[sX] : 0;
+      y_size[y] = (long long)P->np * ((P->n_abf[sX] + 7) / 8 * 8) * 16 * std::max(hz, hx);
+    } else if (P->np)  // pieces of [alpha][z][rup16(n_ao(X))]
       y_size[y] = (long long)P->np * P->n_abf[sX] * P->n_ao[sz] * ((P->n_ao[sX] + 15) / 16 * 16);
     else
       y_size[y] = (long long)P->n_abf[sX] * P->n_ao[sX] * P->n_ao[sz];
@@ -1509,17 +1513,11 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     if (P->sp == hfx::kSplitHalf && P->t2u) {   // Ysp is the first product's store too
       U.Yh = P->Ysp;
     } else {
-      X.yh_blk = 0;   // the largest key's
-      for (int a = 0; a < P->S; ++a)
-        for (int b = 0; b < P->S; ++b)
-          X.yh_blk = std::max(X.yh_blk, (long long)P->np * hfx::ao_subs(P->n_ao[a]) * ((P->n_abf[a] + 7) / 8 * 8) * 16 *
-                                            P->n_ao[b]);
       const long long hcap0 = P->Yhcap;
-      ensure_buf(P, P->Yh, P->Yhcap, std::max(1LL, P->tot[1]) * X.yh_blk);
+      ensure_buf(P, P->Yh, P->Yhcap, std::max(1LL, P->tot[0]));
       if (P->Yhcap != hcap0) ck(cudaMemsetAsync(P->Yh, 0, P->Yhcap * sizeof(uint16_t), s), "memset");
       X.Yh = P->Yh;
       U.Yh = P->Yh;
-      U.yh_blk = X.yh_blk;
     }
   };
   if (!P->np) {
@@ -1530,13 +1528,8 @@ void evaluate_launches(hfx_plan* P, const double* L, hfx_stats* st, bool tail) {
     if (!P->t2w) ensure_buf(P, P->Ysp, P->Yspcap, std::max(1LL, P->tot[0]));   // read by the warp-level kernels only
     X.y_idx = P->y_idx;
     if (P->t2w) {   // (rows past n_abf are never written: finite from the start)
-      X.yT_blk = 0;   // the largest key's
-      for (int a = 0; a < P->S; ++a)
-        for (int b = 0; b < P->S; ++b)
-          X.yT_blk = std::max(X.yT_blk, (long long)P->np * hfx::ao_subs(P->n_ao[b]) * ((P->n_abf[a] + 7) / 8 * 8) * 16 *
-                                            P->n_ao[a]);
       const long long tcap0 = P->YspTcap;
-      ensure_buf(P, P->YspT, P->YspTcap, std::max(1LL, P->tot[1]) * X.yT_blk);
+      ensure_buf(P, P->YspT, P->YspTcap, std::max(1LL, P->tot[0]));
       if (P->YspTcap != tcap0) ck(cudaMemsetAsync(P->YspT, 0, P->YspTcap * sizeof(uint16_t), s), "memset");
       X.YspT = P->YspT;
     }

@@ -147,12 +147,11 @@ struct MixPlan {
   int* qcnt;                   // [nC] kept B per (A,F)
   long long* qoff;             // [nC] offsets into blist
   int* blist;                  // V pairs (A,B) per (A,F), in V-pair order
-  // tcgen05 first product: Y^{XZ} as fp16 pieces, yh_blk per key (by y_idx), per
+  // tcgen05 first product: Y^{XZ} as fp16 pieces at y_off, per
   // piece, sub of x and sub of z the row groups (g, z) of 8 alpha x 16 x in
   // core-matrix order; nullptr where Ysp (ycm, one sub) is that store
   uint16_t* Yh = nullptr;
-  long long yh_blk = 0;
-  // (plans with sub-blocks: fp16 pieces, per piece, sub of z and sub of x the
+  // (plans with sub-blocks: fp16 pieces at y_off, per piece, sub of z and sub of x the
   // row groups (g, x) of 8 alpha x 16 z in core-matrix order)
   uint16_t* YspT = nullptr;    // Y^{XZ} transposed, bf16 pieces [piece][(alpha,x)][16 z] (z padded), yT_blk per key
   long long yT_blk = 0;        // uint16 units per key of YspT (2 pieces x 128-row tiles x 16)
@@ -211,8 +210,7 @@ struct T1UPlan {
   int NAL;                     // most alpha subs
   int sub;                     // 1: some block has more than one sub-block
   const long long* t1_idx;     // V pair -> its position in the term-1 V list
-  const uint16_t* Yh;          // fp16 Y pieces (MixPlan::Yh or Ysp)
-  long long yh_blk;            // its block per needed key, 0: offsets y_off (Ysp)
+  const uint16_t* Yh;          // fp16 Y pieces (MixPlan::Yh or Ysp), at y_off
   const uint16_t* Dh;          // fp16 D pieces of the sub-blocks, offsets dsp_off
   int KP;                      // columns (f,a) = 16 f + a of the largest sub-block of F
   int GA, GB;                  // 8-row groups of the largest alpha sub, of the largest n_abf (beta)

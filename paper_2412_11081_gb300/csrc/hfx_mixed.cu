@@ -1251,7 +1251,7 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
         const int nZs = SUB ? min(ao_sub(nZ), nZ - z0) : nZ;
         const int PX = SUB ? rup16(nX) : 16, NH = PX >> 3;
         uint16_t* Yo = X.Ysp + P.y_off[ykey[i]];
-        uint16_t* Yh = X.Yh ? X.Yh + X.y_idx[ykey[i]] * X.yh_blk : nullptr;
+        uint16_t* Yh = X.Yh ? X.Yh + P.y_off[ykey[i]] : nullptr;
         const bool cm = X.ycm != 0;   // Ysp rows alpha, K = (z, x) in core-matrix order
         const int KZc = 16 * nZ, m8 = (mX + 7) & ~7;
         // Yh: sub of x (hX of them) and of z first
@@ -1315,7 +1315,7 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
         // is this CTA's own
         if (SUB && X.YspT) {   // sub-blocks: [sub of z][sub of x], rows alpha, K = (x, 16 z)
           const long long tplane = (long long)m8 * 16 * nX;
-          uint16_t* yt = X.YspT + X.y_idx[ykey[i]] * X.yT_blk + zsub[i] * tplane;
+          uint16_t* yt = X.YspT + P.y_off[ykey[i]] + zsub[i] * tplane;
           const int nala = alB - alA + 1;
           for (int c = et; c < nala * nX * 2; c += 128) {   // consecutive threads: consecutive alpha of one (x, half)
             const int r2 = c / nala, al = alA + (c - r2 * nala), x = r2 >> 1, hz = r2 & 1, rl = al * nX + x - row0;

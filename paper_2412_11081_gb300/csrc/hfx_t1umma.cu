@@ -484,7 +484,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int b = P.v_j[p];
           const int* Rb = P.v_R + 3 * p;
           const int yc = ylut_get(P, b, F, Rf[0] - Rb[0], Rf[1] - Rb[1], Rf[2] - Rb[2]);
-          yo = yc < 0 ? -1 : U.yh_blk ? X.y_idx[yc] * U.yh_blk : P.y_off[yc];
+          yo = yc < 0 ? -1 : P.y_off[yc];
           g8 = (P.n_abf[P.species[b]] + 7) >> 3;
           nbs = SUB ? ao_subs(P.n_ao[P.species[b]]) : 1;
         }
@@ -1407,8 +1407,8 @@ __global__ void __launch_bounds__(kT2Threads, 1)
           const int n = q.na(c), a0 = q.as(c) * q.hA, bs = q.bs(c);
           const uint32_t ca = 32u * q.a8 * n, cb = 32u * q.b8 * n;   // bytes of one piece of the chunk
           const long long ax = 16ll * q.a8 * q.nA, bx = 16ll * q.b8 * q.nA;   // elements of one sub of b
-          const uint16_t* src_a = X.YspT + X.y_idx[y1] * X.yT_blk + bs * ax + 16ll * q.a8 * a0;
-          const uint16_t* src_b = X.Yh + X.y_idx[y2] * X.yh_blk + bs * bx + 16ll * q.b8 * a0;
+          const uint16_t* src_a = X.YspT + P.y_off[y1] + bs * ax + 16ll * q.a8 * a0;
+          const uint16_t* src_b = X.Yh + P.y_off[y2] + bs * bx + 16ll * q.b8 * a0;
           ok = !aborted(abort_flag) && (na < 1 || mbar_wait(mAe, (na - 1) & 1));
           if (!ok) break;
           mbar_expect_tx(mAf, NP * ca);
