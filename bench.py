@@ -315,7 +315,7 @@ def perovskite_line(torch, dev, stream, local, steps=3):
         out["stages_ms"] = {k: st[k] for k in ("ms_blocks", "ms_screen", "ms_y", "ms_term1", "ms_term2", "ms_total")}
         out["gflop_per_eval"] = st["flops_total"] / 1e9
         out["achieved_tflops"] = st["flops_total"] / t / 1e12
-        out["kernels"] = "k_ybuild_w, k_term1_w, k_term2_w, k_q2_w (warp-level MMAs on bf16 pieces, n_ao up to 32)"
+        out["kernels"] = "k_ybuild_umma, k_t1_umma, k_t2w_umma, k_q2_umma by sub-blocks of at most 16 orbitals"
     return out
 
 
@@ -476,7 +476,7 @@ def run_ours(args):
                         "peak_source": "FP64 cuBLAS DGEMM 4096^3 measured in this run (FP64 pipe)"}
         else:
             pk = peaks.get("bf16_tflops_sustained") or 1717.3
-            pieces = 6 if head == "bf16x6" else 3
+            pieces = 3
             tr = t1_traffic(head)
             # DRAM bytes per launch: the capture's bytes per kept triplet times one launch's kept triplets
             traffic = tr / SI64_TRIPLETS * (flops["triplets"] / passes) if tr is not None else None
@@ -488,7 +488,7 @@ def run_ours(args):
                         "traffic_source": f"profiles/k_t1_umma_si8_{head}.md: DRAM read+write per kept triplet of "
                                           "the capture, times the kept triplets of one launch (one pass)",
                         "peak_source": "bf16 dense, sustained, of measured (MEASURED_PEAKS.json)",
-                        "note": f"achieved counts algorithmic FLOPs only; the {pieces} bf16 piece products per "
+                        "note": f"achieved counts algorithmic FLOPs only; the {pieces} 16-bit piece products per "
                                 f"multiply and the 13->16 / 50->64 tile padding are not counted",
                         "tensor_issue_tflops": achieved * pieces}
         cpu = None

@@ -249,6 +249,7 @@ struct hfx_plan {
   long long Vzcap = 0;
   // split path for n_ao > 16 (hfx_wide.cu): FP64 C, V and D blocks, FP32 Y store
   bool wide = false;
+  long long y_elems = 0;       // elements of a Y store of every candidate key
   bool t2w = false;            // wide: R2 and Z on tcgen05 (k_t2w_umma)
   hfx::T2WPlan t2wp{};
   hfx::WideShapes ws{};
@@ -856,6 +857,9 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
       y_size[y] = (long long)P->n_abf[sX] * P->n_ao[sX] * P->n_ao[sz];
   }
 
+  P->y_elems = 0;
+  for (long long n : y_size) P->y_elems += n;
+
   // (re)allocate list buffers
   P->free_lists();
   P->nC = nC;
@@ -1038,6 +1042,22 @@ double list_drift(const hfx_plan* P, const double* L, const double* pos) {
     dl = std::max(dl, std::sqrt(d2));
   }
   return 2.0 * disp + P->list_Rabs * dl;
+}
+
+// With sub-blocks the tensor-memory kernels keep two Y stores, the warp-level
+// ones one: structures whose two would take more than 35 % of the device's
+// memory (perovskites of about 2,400 atoms) stay on the warp-level kernels
+// (HFX_Y_STORE_GB: that limit in GB).
+void fit_y_stores(hfx_plan* P, const double* L, const double* pos) {
+  if (!P->wide || !P->t1u) return;
+  size_t avail = 0, total = 0;
+  ck(cudaMemGetInfo(&avail, &total), "cudaMemGetInfo");
+  const char* e = std::getenv("HFX_Y_STORE_GB");
+  const double limit = e ? 1e9 * std::atof(e) : 0.35 * (double)total;
+  if (2.0 * sizeof(uint16_t) * (double)P->y_elems <= limit) return;
+  P->t1u = P->t2w = false;
+  P->t1u_subs = P->t1u_NAL = 1;
+  build_lists(P, L, pos);
 }
 
 // The tcgen05 first product for the plan's shapes: sub-blocks of at most 16
@@ -1891,6 +1911,7 @@ hfx_status hfx_plan_create(const hfx_system* sys, const hfx_model* model, const 
     ck(cudaMemset(P->d_tot, 0, ntot * sizeof(long long)), "memset");
     setup_shapes(P);
     build_lists(P, sys->lattice, sys->positions);
+    fit_y_stores(P, sys->lattice, sys->positions);
     split_density(P);
   });
   if (st != HFX_OK) {

@@ -117,3 +117,14 @@ def test_sub_block_edges(n_ao, n_abf, terms):
     assert st["triplets"] == st0["triplets"] and st["term2_pairs"] == st0["term2_pairs"]
     assert abs(st["flops_total"] / st0["flops_total"] - 1.0) < 1e-12
     assert max(er) <= BOUND, er
+
+
+def test_warp_level_kernels_beyond_the_y_store_limit(monkeypatch):
+    """Structures whose two Y stores would not fit the device run on the
+    warp-level kernels (one store): the same kept items, within the contract."""
+    w = wide_two_species(seed=9)
+    E0, F0, S0, st0 = run(w, hfx.HFX_FP64)
+    monkeypatch.setenv("HFX_Y_STORE_GB", "0")
+    E, F, S, st = run(w, hfx.HFX_BF16X6)
+    assert st["triplets"] == st0["triplets"] and st["term2_pairs"] == st0["term2_pairs"]
+    assert max(errs((E, F, S), (E0, F0, S0))) <= BOUND
