@@ -553,7 +553,7 @@ __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
       if (h2 != 0.0) dev::add_gV(P, 3 * p + 2, -h2);
     }
     const int q0 = P.c_ptr[A], nq = P.c_ptr[A + 1] - q0;
-    double* gF = sm;                        // nq*3, each F's by the warp that takes it
+    double* gF = sm;                        // nq*3: component c of an F by lane c of the warp that takes it, and no other
     double* Zc = gF + 3 * kMaxCPerAtom;     // AC*nA*nB
     for (int t = warp; t < nq; t += nwarp)
       if (lane < 3) gF[3 * t + lane] = 0.0;
@@ -600,12 +600,8 @@ __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
         g0 = warp_sum(g0);
         g1 = warp_sum(g1);
         g2 = warp_sum(g2);
-        if (lane == 0) {
-          gF[3 * t + 0] += g0;
-          gF[3 * t + 1] += g1;
-          gF[3 * t + 2] += g2;
-          fl += 2.0 * ac * nA * nB * nF;
-        }
+        if (lane < 3) gF[3 * t + lane] += lane == 0 ? g0 : lane == 1 ? g1 : g2;
+        if (lane == 0) fl += 2.0 * ac * nA * nB * nF;
       }
     }
     for (int t = warp; t < nq; t += nwarp)

@@ -254,3 +254,19 @@ def test_fp64_block_shape_edges(n_ao, n_abf):
     pos = np.array([[0.1, 0.2, 0.0], [1.5, 1.7, 1.4]]) + rng.normal(0, 0.05, (2, 3))
     w = inputs.cut_density(inputs.tiny_model(n_ao, n_abf, [0, 1], np.eye(3) * 3.2, pos, r_c=1.3, seed=17), 3.5)
     assert_parity(gpu_eval(w), evaluate(w))
+
+
+@pytest.mark.parametrize("n_ao,n_abf", [([2, 1], [3, 5]), ([13, 4], [20, 41])])
+@pytest.mark.parametrize("deterministic", [0, 1])
+def test_second_product_gradients_of_every_f(n_ao, n_abf, deterministic):
+    """The second product alone, whose warps collect the three gradient
+    components of each of their F in shared memory: CTAs of two warps and of
+    eight."""
+    rng = np.random.default_rng(19)
+    pos = np.array([[0.1, 0.2, 0.0], [1.5, 1.7, 1.4]]) + rng.normal(0, 0.05, (2, 3))
+    w = inputs.cut_density(inputs.tiny_model(n_ao, n_abf, [0, 1], np.eye(3) * 3.2, pos, r_c=1.3, seed=19), 3.5)
+    r = evaluate(w, dataclasses.replace(Options.from_theta(w.theta), terms=2))
+    with hfx.Plan(w, terms=2, deterministic=bool(deterministic)) as p:
+        for _ in range(3):
+            E, F, S = p.evaluate(w.lattice, w.positions)
+            assert abs(E - r.E) <= TOL * abs(r.E) and rel(F, r.F) <= TOL and rel(S, r.sigma) <= TOL
