@@ -743,8 +743,10 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
 // piece products into one FP32 accumulator in tensor memory.  Operands lie
 // in the K-major no-swizzle core-matrix order (8 rows x 16 bytes per core
 // matrix).  Every `flush` steps the accumulator is read back and dotted with
-// grad C_AF into FP64.  Every wait is bounded; on timeout the CTA sets *err
-// and stops.
+// grad C_AF into FP64.  Every wait is bounded.  A warp whose wait runs out
+// sets the abort flag; nothing is committed after that, the other warps' waits
+// run out in turn, no accumulator is read that was not handed over, and the
+// CTA sets *err, waits for its copies and MMAs in flight and frees tensor memory.
 // What bounds it: of about 800 cycles per step and two tiles 384 are tensor
 // work (six instructions of N = 128) and 24 KB come from L2 (6.7 TB/s over the
 // chip); the rest is the copies' latency, the prologue (the steps in use) and
@@ -784,6 +786,24 @@ __device__ __forceinline__ void stage_d(int lane, uint16_t* stB, const int* md, 
     for (int j = 0; j < 4; ++j) r[j] = md[4 * h + j] >= 0 ? md[4 * h + j] : zrow;
     gather4_rows((uint32_t)__cvta_generic_to_shared(stB + 4 * h * NP * 256), map, r[0], r[1], r[2], r[3], mbar);
   }
+}
+
+// Every lane waits (bounded); the result is the same on all lanes, as the
+// warp-wide reads of tensor memory that follow it need.
+__device__ __forceinline__ bool wait_all(uint32_t mbar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait<kMixTryNs>(mbar, parity)) != 0;
+}
+
+// Lets the copies issued into a ring of `size` stages (`issued` in all) land.
+__device__ __forceinline__ void drain(uint32_t full, int issued, int size) {
+  for (int k = issued < size ? 0 : issued - size; k < issued; ++k)
+    mbar_wait<kMixTryNs>(full + 8 * (k % size), (uint32_t)((k / size) & 1));
+}
+
+// Lets the MMAs this thread has issued complete, by way of a barrier of their own.
+__device__ __forceinline__ void finish_mmas(uint32_t mbar) {
+  umma_commit(mbar);
+  mbar_wait<kMixTryNs>(mbar, 0u);
 }
 
 // Piece p of that operand: 8-row groups of the pieces alternate (dix).
@@ -829,12 +849,13 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
   uint16_t* stA = reinterpret_cast<uint16_t*>(smem_raw);                  // [KS][TPC][NP][kTileElems]
   uint16_t* stB = stA + (size_t)KS * TPC * NP * kTileElems;               // [KS][NP][kTileElems]
   int* m_dblk = reinterpret_cast<int*>(stB + (size_t)KS * NP * kTileElems);   // [kMetaPairs][8]
-  __shared__ __align__(8) uint64_t bar_full[KS], bar_empty[KS], bar_accf[2], bar_acce[2];
+  __shared__ __align__(8) uint64_t bar_full[KS], bar_empty[KS], bar_accf[2], bar_acce[2], bar_done;
   __shared__ uint32_t tmem_base;
   __shared__ double sg[8][3];
   __shared__ int m_q[kMetaPairs];
   __shared__ int s_nsteps;
   __shared__ int s_abort;
+  volatile int* abort_flag = &s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int rem = blockIdx.x;
   const int seg = rem % NSEG;
@@ -879,6 +900,7 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
   const uint32_t mempty = (uint32_t)__cvta_generic_to_shared(&bar_empty[0]);
   const uint32_t maccf = (uint32_t)__cvta_generic_to_shared(&bar_accf[0]);
   const uint32_t macce = (uint32_t)__cvta_generic_to_shared(&bar_acce[0]);
+  const uint32_t mdone = (uint32_t)__cvta_generic_to_shared(&bar_done);
   if (tid < 24) sg[tid / 3][tid % 3] = 0.0;
   if (tid == 0) {
     s_abort = 0;
@@ -890,6 +912,7 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(maccf + 8 * b));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(macce + 8 * b), "r"(DEEP ? 8 : 4));
     }
+    mbar_init(mdone, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
   }
   if (warp == 1) {
@@ -921,19 +944,22 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
   const int nsteps = s_nsteps;
   const int nruns = (nsteps + flush - 1) / flush;
 
-  if (warp == 0 && !X.stall_q2) {
+  if (warp == 0) {
     // producer warp: every lane waits for the stage, then lanes issue the
     // copies of one stage in parallel (lane 0 also posts the byte count)
     const uint32_t abytes = (uint32_t)ntile * NP * kTileElems * 2;
     const uint32_t bytes = abytes + (uint32_t)NP * kTileElems * 2;
-    for (int k = 0; k < nsteps; ++k) {
+    const int n = X.stall_q2 ? 0 : nsteps;
+    int k = 0;
+    for (; k < n; ++k) {
       const int s = k % KS;
       const int t = m_q[k];
-      if (k >= KS && !mbar_wait<kMixTryNs>(mempty + 8 * s, (uint32_t)((k / KS - 1) & 1))) s_abort = 1;
-      __syncwarp();
-      if (s_abort) break;
+      if (k >= KS && !wait_all(mempty + 8 * s, (uint32_t)((k / KS - 1) & 1))) {
+        *abort_flag = 1;
+        break;
+      }
       // lane 0: the NP Z piece tiles of the CTA's row tiles (contiguous, one
-      // copy); lanes 1 .. 2 NP: the eight D blocks of each piece, four per gather
+      // copy); lanes 1 and 2: the eight D sub-blocks, four per gather
       if (lane == 0) {
         mbar_expect_tx(mfull + 8 * s, bytes);
         bulk_g2s((uint32_t)__cvta_generic_to_shared(stA + (size_t)s * TPC * NP * kTileElems),
@@ -941,25 +967,23 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
       }
       stage_d(lane, stB + (size_t)s * NP * kTileElems, m_dblk + t * 8, &drows.map, drows.zero_row, mfull + 8 * s);
     }
+    if (lane == 0 && k < n) drain(mfull, k, KS);
   } else if (warp == 1) {
     if (lane == 0) {
       // MMA issuer: D f32, A/B bf16, both K-major, N = 128, M = 128
       const uint32_t idesc = idesc_split<SP>(128, 128, 0);
-      for (int r = 0; r < nruns && !s_abort; ++r) {
+      bool ok = true;
+      for (int r = 0; r < nruns && ok; ++r) {
         const int b = r % NB;
-        if (r >= NB && !mbar_wait<kMixTryNs>(macce + 8 * b, (uint32_t)((r / NB - 1) & 1))) {
-          s_abort = 1;
-          break;
-        }
+        ok = !*abort_flag && (r < NB || mbar_wait<kMixTryNs>(macce + 8 * b, (uint32_t)((r / NB - 1) & 1)));
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         const uint32_t dacc = taddr + 128u * TPC * b;
         const int k1 = min(nsteps, (r + 1) * flush);
         for (int k = r * flush; k < k1; ++k) {
           const int s = k % KS;
-          if (!mbar_wait<kMixTryNs>(mfull + 8 * s, (uint32_t)((k / KS) & 1))) {
-            s_abort = 1;
-            break;
-          }
+          ok = mbar_wait<kMixTryNs>(mfull + 8 * s, (uint32_t)((k / KS) & 1));
+          if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
           const uint32_t a0 = (uint32_t)__cvta_generic_to_shared(stA + (size_t)s * TPC * NP * kTileElems);
           const uint32_t b0 = (uint32_t)__cvta_generic_to_shared(stB + (size_t)s * NP * kTileElems);
@@ -980,9 +1004,10 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
           asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mempty + 8 * s)
                        : "memory");
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(maccf + 8 * b)
-                     : "memory");
+        if (ok) umma_commit(maccf + 8 * b);   // (an unfinished run is not handed over)
       }
+      if (!ok) *abort_flag = 1;
+      finish_mmas(mdone);   // before tensor memory is freed
     }
   } else {
     // epilogue: warps 2..5 (DEEP: and 6..9, which take the second tile), tensor-memory lane quarter q = warp % 4
@@ -990,10 +1015,12 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
     double gd[8][3];
 #pragma unroll
     for (int i = 0; i < 8; ++i) gd[i][0] = gd[i][1] = gd[i][2] = 0.0;
+    bool ok = true;
     for (int run = 0; run < nruns; ++run) {
       const int b = run % NB;
-      if (!mbar_wait<kMixTryNs>(maccf + 8 * b, (uint32_t)((run / NB) & 1))) {
-        s_abort = 1;
+      ok = wait_all(maccf + 8 * b, (uint32_t)((run / NB) & 1));
+      if (!ok) {
+        *abort_flag = 1;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -1044,7 +1071,7 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const double w = warp_sum_d(gd[i][c]);
-        if (lane == 0 && w != 0.0) {
+        if (ok && lane == 0 && w != 0.0) {
           if (P.fxC) dev::add_gC(P, 3 * qf[i] + c, -2.0 * w);   // deterministic plan: straight into the exact cell
           else atomicAdd(&sg[i][c], w);
         }
@@ -1087,9 +1114,10 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
   int* m_d = reinterpret_cast<int*>(stB + (size_t)kStages * NP * kTileElems);   // [K steps (C pair, sub)][8]
   int* m_q = m_d + X.ytab_stride;                                               // the steps in use
   __shared__ int s_nsteps;
-  __shared__ __align__(8) uint64_t bar_full[kStages], bar_empty[kStages], bar_accf;
+  __shared__ __align__(8) uint64_t bar_full[kStages], bar_empty[kStages], bar_accf, bar_done;
   __shared__ uint32_t tmem_base;
   __shared__ int s_abort;
+  volatile int* abort_flag = &s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int MCP = (MC + TPC - 1) / TPC;
   const int g = blockIdx.x / MCP, mc = (blockIdx.x - g * MCP) * TPC;   // first row tile of this CTA
@@ -1116,13 +1144,15 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
   const uint32_t mfull = (uint32_t)__cvta_generic_to_shared(&bar_full[0]);
   const uint32_t mempty = (uint32_t)__cvta_generic_to_shared(&bar_empty[0]);
   const uint32_t maccf = (uint32_t)__cvta_generic_to_shared(&bar_accf);
+  const uint32_t mdone = (uint32_t)__cvta_generic_to_shared(&bar_done);
   if (tid == 0) {
     s_abort = 0;
     for (int s = 0; s < kStages; ++s) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mfull + 8 * s));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mempty + 8 * s));
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(maccf));
+    mbar_init(maccf, 1);
+    mbar_init(mdone, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
   }
   if (warp == 1) {
@@ -1156,14 +1186,16 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
   if (warp == 0) {
     const uint32_t abytes = (uint32_t)ntile * NP * kTileElems * 2;
     const uint32_t bytes = abytes + (uint32_t)NP * kTileElems * 2;
-    for (int k = 0; k < nsteps; ++k) {
+    int k = 0;
+    for (; k < nsteps; ++k) {
       const int s = k % kStages;
-      if (k >= kStages && !mbar_wait<kMixTryNs>(mempty + 8 * s, (uint32_t)((k / kStages - 1) & 1))) s_abort = 1;
-      __syncwarp();
-      if (s_abort) break;
+      if (k >= kStages && !wait_all(mempty + 8 * s, (uint32_t)((k / kStages - 1) & 1))) {
+        *abort_flag = 1;
+        break;
+      }
       const int t = m_q[k];
       // lane 0: the NP C piece tiles of the CTA's row tiles (contiguous, one
-      // copy); lanes 1 .. 2 NP: the eight mirror D blocks of each piece, four per gather
+      // copy); lanes 1 and 2: the eight mirror D sub-blocks, four per gather
       if (lane == 0) {
         mbar_expect_tx(mfull + 8 * s, bytes);
         bulk_g2s((uint32_t)__cvta_generic_to_shared(stA + (size_t)s * TPC * NP * kTileElems),
@@ -1173,15 +1205,15 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
       }
       stage_d(lane, stB + (size_t)s * NP * kTileElems, m_d + t * 8, &drows.map, drows.zero_row, mfull + 8 * s);
     }
+    if (lane == 0 && k < nsteps) drain(mfull, k, kStages);
   } else if (warp == 1) {
     if (lane == 0 && nsteps > 0) {
       const uint32_t idesc = idesc_split<SP>(128, 128, 0);
+      bool ok = true;
       for (int k = 0; k < nsteps; ++k) {
         const int s = k % kStages;
-        if (!mbar_wait<kMixTryNs>(mfull + 8 * s, (uint32_t)((k / kStages) & 1))) {
-          s_abort = 1;
-          break;
-        }
+        ok = mbar_wait<kMixTryNs>(mfull + 8 * s, (uint32_t)((k / kStages) & 1));
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         const uint32_t a0 = (uint32_t)__cvta_generic_to_shared(stA + (size_t)s * TPC * NP * kTileElems);
         const uint32_t b0 = (uint32_t)__cvta_generic_to_shared(stB + (size_t)s * NP * kTileElems);
@@ -1200,8 +1232,9 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mempty + 8 * s)
                      : "memory");
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(maccf)
-                   : "memory");
+      if (ok) umma_commit(maccf);   // (an unfinished sum is not handed over)
+      else *abort_flag = 1;
+      finish_mmas(mdone);   // before tensor memory is freed
     }
   } else {
     // epilogue (warps 2..5, and 6..9 for the second tile): the accumulator (rows (alpha, x), columns
@@ -1214,15 +1247,20 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
     const int q = warp & 3;
     const int jt = (warp - 2) >> 2, et = (tid - 64) & 127;
     float* ep = reinterpret_cast<float*>(smem_raw) + jt * 128 * 33;   // [128][33]
-    bool have = nsteps > 0;
+    const bool have = nsteps > 0;
+    bool ok = true;
     if (have) {
-      if (!mbar_wait<kMixTryNs>(maccf, 0u)) {
-        s_abort = 1;
-        have = false;
-      }
+      ok = wait_all(maccf, 0u);
+      if (!ok) *abort_flag = 1;
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     }
-    if (jt < ntile) {
+    // the four warps of a tile go on together or not at all (they meet at a barrier below)
+    int all_ok;
+    asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %1, 0;\n bar.red.and.pred q, %2, 128, p;\n selp.b32 %0, 1, 0, q;\n}\n"
+                 : "=r"(all_ok)
+                 : "r"((int)ok), "r"(1 + jt)
+                 : "memory");
+    if (jt < ntile && all_ok) {
     const int row0 = (mc + jt) * 128;
     const int rend = min(row0 + 128, rows);
     const int alF = (row0 + nX - 1) / nX, alL = rend / nX - 1;

@@ -93,3 +93,22 @@ def test_stalled_pipeline_wait_runs_out_and_plan_recovers(prec, monkeypatch):
         monkeypatch.delenv("HFX_TEST_STALL_Q2_PRODUCER")
         E, F, S = p.evaluate(w.lattice, w.positions)
     assert abs(E - ref[0]) <= 1e-12 * abs(ref[0]) and rel(F, ref[1]) <= 1e-12 and rel(S, ref[2]) <= 1e-12
+
+
+@pytest.mark.parametrize("tiles", ["1", "2", "3"])
+def test_stalled_pipeline_in_every_q2_shape(tiles, monkeypatch):
+    """The producer warp stays out of the epilogue and nothing is read from an
+    accumulator that was not handed over, whichever way the row tiles are
+    divided over the warps; diamond8's and a 13-orbital cell's tiles (one and
+    several of 128 rows)."""
+    monkeypatch.setenv("HFX_Q2_TILES", tiles)
+    for w in (inputs.diamond8(), inputs.tiny_model([13], [50], [0], np.eye(3) * 3.4, [[0.1, 0.2, 0.0]], r_c=1.4, seed=3)):
+        with hfx.Plan(w, precision=hfx.HFX_BF16X6) as p:
+            ref = p.evaluate(w.lattice, w.positions)
+            monkeypatch.setenv("HFX_TEST_STALL_Q2_PRODUCER", "1")
+            with pytest.raises(hfx.HfxError) as ei:
+                p.evaluate(w.lattice, w.positions)
+            assert ei.value.status == 4, ei.value
+            monkeypatch.delenv("HFX_TEST_STALL_Q2_PRODUCER")
+            E, F, S = p.evaluate(w.lattice, w.positions)
+        assert abs(E - ref[0]) <= 1e-12 * abs(ref[0]) and rel(S, ref[2]) <= 1e-12
