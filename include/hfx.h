@@ -64,11 +64,17 @@ typedef enum {
  * other values select split-precision tensor-core contractions with FP32
  * accumulation and FP64 screening, force, stress and energy reduction.
  * BF16X3 writes every operand as two bf16 pieces and keeps the piece products
- * above 2^-16 of the operands' scale.  BF16X6 stands for the accuracy of six
- * products of three bf16 pieces: it writes every operand as two fp16 pieces
- * (22 significant bits) under power-of-two scales taken from bounds of the
- * blocks, and keeps the piece products above 2^-22 of the operands' scale;
- * FP32 accumulation bounds its error.  (Value 1 is not assigned.) */
+ * above 2^-16 of the operands' scale (the Y and D that make U = D Y in the
+ * first product are fp16 pieces as below where that runs on tensor memory).
+ * BF16X6 stands for the accuracy of six products of three bf16 pieces: it
+ * writes every operand as two fp16 pieces and keeps the piece products above
+ * 2^-22 of the operands' scale; FP32 accumulation bounds its error.  fp16
+ * pieces hold a value times a power of two that is fixed per atom (for D and
+ * Y: per pair of atoms) from bounds of the atom's blocks: 22 significant bits
+ * down to 2^-18 of that bound, below it an absolute error of 2^-40 of it.  An
+ * atom whose templates or D are far smaller than the others' keeps its own
+ * accuracy; what is far below the largest terms of the same atom does not.
+ * (Value 1 is not assigned.) */
 enum { HFX_FP64 = 0, HFX_BF16X3 = 2, HFX_BF16X6 = 3 };
 
 /* Exchange products of Eq. exx_expand: bit 0 = D_AB D_FG, bit 1 = D_AG D_FB. */

@@ -39,19 +39,33 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 //   kSplitBf16 (HFX_BF16X3): bf16 pieces, 16 significant bits, any FP32 range
 //   kSplitHalf (HFX_BF16X6): fp16 pieces, 22 significant bits.  fp16 has
 //     five exponent bits, so the stores hold x times a power of two
-//     (SplitScale) that keeps every element's magnitude within 2^15: the low
-//     piece is exact to 2^-25 of the stored scale, so elements down to 2^-18
-//     of that bound keep all 22 bits and the rest an absolute error of 2^-40
-//     of it.  Three products of two such pieces carry what six products of
+//     (SplitScale, per atom) that keeps every element's magnitude within 2^15:
+//     the low piece is exact to 2^-25 of the stored scale, so elements down to
+//     2^-18 of that bound keep all 22 bits and the rest an absolute error of
+//     2^-40 of it.  Three products of two such pieces carry what six products of
 //     three bf16 pieces did, at half the tensor-core work and two thirds of
 //     the operand bytes.
 constexpr int NP = kPieces;
 
-// A factor of SplitScale: 1 (and no multiplication) with bf16 pieces.
+// 2^e, e held within what the type has (terms that far from the largest of
+// their sum round to nothing).
+__device__ __forceinline__ float p2f(int e) { return __int_as_float((max(-126, min(127, e)) + 127) << 23); }
+__device__ __forceinline__ double p2d(int e) { return __hiloint2double((max(-1022, min(1023, e)) + 1023) << 20, 0); }
+
+// The factor between a value and its store, 2^e: 1 (and no multiplication) with bf16 pieces.
 template <int SP>
-__device__ __forceinline__ float pscale(float s) {
-  return SP == kSplitHalf ? s : 1.f;
+__device__ __forceinline__ float pscale(int e) {
+  return SP == kSplitHalf ? p2f(e) : 1.f;
 }
+template <int SP>
+__device__ __forceinline__ double pscale_d(int e) {
+  return SP == kSplitHalf ? p2d(e) : 1.0;
+}
+
+// Exponents of the fp16 pieces of Y^{XZ} (HFX_BF16X3), V_AB, and the product <Y^{AB}, Y^{BA}>.
+__device__ __forceinline__ int y_exp(const DevPlan& P, int X, int Z) { return max(-120, min(120, P.sc.y[X] + P.sc.d[Z])); }
+__device__ __forceinline__ int v_exp(const DevPlan& P, int A, int B) { return P.sc.q[A] - P.sc.d[B] - P.sc.y[B]; }
+__device__ __forceinline__ int r2_exp(const DevPlan& P, int A, int B) { return P.sc.y[A] + P.sc.d[B] + P.sc.y[B] + P.sc.d[A]; }
 
 template <int SP>
 __device__ __forceinline__ void split_f(float x, uint16_t (&p)[NP]) {

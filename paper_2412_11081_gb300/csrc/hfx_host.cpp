@@ -191,9 +191,11 @@ struct hfx_plan {
   int np = 0;
   int sp = 0;                  // piece type, hfx::kSplitBf16 or kSplitHalf
   std::vector<double> cmax;    // [S*S] bound of |C| / f(r)
-  double dmax = 0, vmax = 0, vrow = 0;   // bounds of |D|, |V| and sum_beta |V|
-  double ymax = 0;             // bound of |Y| over the skin of the current lists
-  hfx::SplitScale scale;
+  std::vector<double> cnorm, cpart;   // [S*S] of ||C[alpha][.][.]|| / f(r) and ||C[.][a][.]|| / f(r)
+  std::vector<double> vmax, vnorm;    // [S*S] of |V| / h(r) and ||V[alpha][.]|| / h(r)
+  std::vector<int> dexp;       // [N] d of hfx::SplitScale
+  hfx::SplitScale scale;       // exponents of the current lists
+  int* d_scale = nullptr;      // [5 N] their device arrays
   uint16_t* Dsp = nullptr;
   long long* dsp_off = nullptr;
   uint16_t* Ysp = nullptr;
@@ -330,6 +332,7 @@ void upload_model(hfx_plan* P, const hfx_system* sys, const hfx_model* m) {
     }
   std::vector<double> G(gsz), M(msz), Gp, Mnorm(S * S), Gmom(3 * S * S, 0.0);
   P->cmax.assign(S * S, 0.0);
+  for (std::vector<double>* v : {&P->cnorm, &P->cpart, &P->vmax, &P->vnorm}) v->assign(S * S, 0.0);
   double elen = 0;   // |d.e| <= |e| R_C where f(r) > 0
   for (int k = 0; k < 3; ++k) elen += m->aniso_dir[k] * m->aniso_dir[k];
   elen = m->G_aniso ? std::sqrt(elen) : 0.0;
@@ -356,14 +359,29 @@ void upload_model(hfx_plan* P, const hfx_system* sys, const hfx_model* m) {
         gm[2] += gq * gq;
         P->cmax[a * S + b] = std::max(P->cmax[a * S + b], std::fabs(gv) + elen * std::fabs(gq));
       }
-      for (int x = 0; x < P->n_abf[a]; ++x) {   // h(r) <= 1
+      const int na = P->n_ao[a], nb = P->n_ao[b];
+      auto slab = [&](const double* g, int x, int k) {   // ||g[x][.][.]|| (k = 0) or ||g[.][x][.]||
+        double t = 0;
+        for (int u = 0; u < (k ? P->n_abf[a] : na); ++u)
+          for (int f = 0; f < nb; ++f) {
+            const double v = g[((long long)(k ? u : x) * na + (k ? x : u)) * nb + f];
+            t += v * v;
+          }
+        return std::sqrt(t);
+      };
+      for (int k = 0; k < 2; ++k) {
+        double& most = (k ? P->cpart : P->cnorm)[a * S + b];
+        for (int x = 0; x < (k ? na : P->n_abf[a]); ++x)
+          most = std::max(most, slab(&G[goff[a * S + b]], x, k) + (Gp.empty() ? 0.0 : elen * slab(&Gp[goff[a * S + b]], x, k)));
+      }
+      for (int x = 0; x < P->n_abf[a]; ++x) {
         double row = 0;
         for (int y = 0; y < P->n_abf[b]; ++y) {
-          const double v = std::fabs(M[moff[a * S + b] + (long long)x * P->n_abf[b] + y]);
-          row += v;
-          P->vmax = std::max(P->vmax, v);
+          const double v = M[moff[a * S + b] + (long long)x * P->n_abf[b] + y];
+          row += v * v;
+          P->vmax[a * S + b] = std::max(P->vmax[a * S + b], std::fabs(v));
         }
-        P->vrow = std::max(P->vrow, row);
+        P->vnorm[a * S + b] = std::max(P->vnorm[a * S + b], std::sqrt(row));
       }
       Mnorm[a * S + b] = std::sqrt(s2);
       mmax = std::max(mmax, Mnorm[a * S + b]);
@@ -416,6 +434,53 @@ void upload_model(hfx_plan* P, const hfx_system* sys, const hfx_model* m) {
   ck(cudaStreamSynchronize(s), "upload model");
 }
 
+// Exponents d with 2^(d[I] + d[J]) times the 2-norm of any row or column of
+// D_IJ at most 1, and the largest of every atom's near 1: symmetric scaling by
+// the square roots of those, repeated until they settle (Ruiz's equilibration).
+void balance_density(hfx_plan* P, const std::vector<long long>& off, const double* values) {
+  const int N = P->N;
+  P->dexp.assign(N, 0);
+  if (!P->sp) return;
+  std::vector<float> lg(P->n_d);   // log2 of each block's largest norm
+  std::vector<double> row, col;
+  for (long long k = 0; k < P->n_d; ++k) {
+    const int na = P->n_ao[P->species[P->d_index[5 * k]]], nb = P->n_ao[P->species[P->d_index[5 * k + 1]]];
+    const double* d = values + off[k];
+    row.assign(na, 0.0);
+    col.assign(nb, 0.0);
+    for (int a = 0; a < na; ++a)
+      for (int b = 0; b < nb; ++b) {
+        const double t = d[a * nb + b] * d[a * nb + b];
+        row[a] += t;
+        col[b] += t;
+      }
+    const double m = std::max(*std::max_element(row.begin(), row.end()), *std::max_element(col.begin(), col.end()));
+    lg[k] = m > 0 ? (float)(0.5 * std::log2(m)) : -1e30f;
+  }
+  std::vector<float> g(N, 0.f), r(N);
+  for (int it = 0; it < 16; ++it) {
+    std::fill(r.begin(), r.end(), -1e30f);
+    for (long long k = 0; k < P->n_d; ++k) {
+      const int I = P->d_index[5 * k], J = P->d_index[5 * k + 1];
+      r[I] = std::max(r[I], lg[k] + g[I] + g[J]);
+    }
+    float worst = 0;
+    for (int I = 0; I < N; ++I)
+      if (r[I] > -1e29f) {
+        worst = std::max(worst, std::fabs(r[I]));
+        g[I] = std::max(-90.f, std::min(90.f, g[I] - 0.5f * r[I]));
+      }
+    if (worst < 1.f) break;
+  }
+  for (int I = 0; I < N; ++I) P->dexp[I] = (int)std::floor(g[I]);
+  int over = -1000;
+  for (long long k = 0; k < P->n_d; ++k)
+    if (lg[k] > -1e29f)
+      over = std::max(over, (int)std::ceil(lg[k] + 1e-3f) + P->dexp[P->d_index[5 * k]] + P->dexp[P->d_index[5 * k + 1]]);
+  if (over > 0)
+    for (int& d : P->dexp) d -= (over + 1) / 2;
+}
+
 // D blocks: validation, the dense (i, j, R) lookup table, device copies.
 void upload_density(hfx_plan* P, const hfx_model* m) {
   const int N = P->N;
@@ -439,7 +504,7 @@ void upload_density(hfx_plan* P, const hfx_model* m) {
   }
   const long long nvals = off[nd];
   if (!finite_all(m->d_values, (size_t)nvals)) fail(HFX_ERR_INVALID, "non-finite D values");
-  for (long long k = 0; k < nvals; ++k) P->dmax = std::max(P->dmax, std::fabs(m->d_values[k]));
+  balance_density(P, off, m->d_values);
   for (int c = 0; c < 3; ++c) P->HD[c] = H[c];
   const long long n0 = 2 * H[0] + 1, n1 = 2 * H[1] + 1, n2 = 2 * H[2] + 1;
   const long long lut_n = (long long)N * N * n0 * n1 * n2;
@@ -596,42 +661,74 @@ DevPlan make_devplan(hfx_plan* P, const double* lattice) {
   return D;
 }
 
-// Powers of two of the fp16 stores (hfx::SplitScale) from the bounds of the
-// blocks: |C| <= cmax f, |D| <= dmax, |V| <= vmax, |Y| <= ymax,
-// |U| <= n_ao dmax ymax, |Z| <= vrow ymax.  bf16 pieces hold the values as
-// they are.
-void set_scale(hfx_plan* P) {
-  P->scale = hfx::SplitScale{};
+// Exponents of the fp16 stores (hfx::SplitScale) from the bounds of the blocks
+// at every geometry the lists cover, no pair distance moving by more than the
+// skin before they are rebuilt: |C_AF| <= cmax f, ||row of D_IJ|| <= 2^(-d[I] -
+// d[J]), |V_AB| <= vmax h, ||Y^{XZ}[alpha][.][z]|| <= y[X] 2^-d[Z] with y[X] the
+// sum of cnorm f 2^-d[W] over W, and |Z_AB| <= vnorm h yp[B] 2^-d[A] with yp
+// that sum over cpart (||Y^{XZ}[.][x][z]||).
+void set_scale(hfx_plan* P, const double* L, const double* pos, const std::vector<int>& c_ptr,
+               const std::vector<int>& c_j, const std::vector<int>& c_R, const std::vector<int>& v_ptr,
+               const std::vector<int>& v_j, const std::vector<int>& v_R) {
   if (!P->sp) return;
-  int nao = 1;
-  for (int n : P->n_ao) nao = std::max(nao, n);
-  auto ex = [](double bound) {   // bound * 2^ex in (2^14, 2^15]
+  const int N = P->N, S = P->S;
+  auto ex = [](double bound) {   // bound * 2^ex in [2^14, 2^15)
     if (!(bound > 0)) return 0;
     int k = 0;
     std::frexp(bound, &k);
-    return std::max(-100, std::min(100, 15 - k));
+    return std::max(-200, std::min(200, 15 - k));
   };
-  const int eC = ex(*std::max_element(P->cmax.begin(), P->cmax.end())), eD = ex(P->dmax), eV = ex(P->vmax);
-  // (U with a bit to spare: rows past n_abf(B) hold other blocks' Y, bounded by 2^15 as stored)
-  const int eY = ex(P->ymax), eU = ex(2 * nao * P->dmax * P->ymax), eZ = ex(P->vrow * P->ymax);
-  auto f = [](int e) { return std::ldexp(1.f, std::max(-126, std::min(127, e))); };
-  hfx::SplitScale& s = P->scale;
-  s.dh = f(eD);
-  if (P->sp != hfx::kSplitHalf) {   // bf16 pieces hold the values as they are
-    s.yh = f(eY);
-    s.u1 = f(-eD - eY);
-    return;
+  auto dist = [&](int A, int j, const int* R) {   // the least it may become
+    double d2 = 0;
+    for (int k = 0; k < 3; ++k) {
+      const double dv = pos[3 * j + k] + R[0] * L[k] + R[1] * L[3 + k] + R[2] * L[6 + k] - pos[3 * A + k];
+      d2 += dv * dv;
+    }
+    return std::max(0.0, std::sqrt(d2) - P->opt.skin);
+  };
+  std::vector<int> sc(5 * (size_t)N);
+  int *eC = sc.data(), *eD = eC + N, *eY = eD + N, *eQ = eY + N, *eZ = eQ + N;
+  std::vector<double> ymax(N, 0.0), ypart(N, 0.0);
+  for (int A = 0; A < N; ++A) {
+    double c = 0;
+    for (int q = c_ptr[A]; q < c_ptr[A + 1]; ++q) {
+      const int st = P->species[A] * S + P->species[c_j[q]];
+      const double r = dist(A, c_j[q], &c_R[3 * q]), t = std::max(0.0, 1.0 - r * r / (P->RC * P->RC));
+      const double f = std::ldexp(t * t * t * std::exp(-0.5 * r * r), -P->dexp[c_j[q]]);
+      c = std::max(c, f * P->cmax[st]);
+      ymax[A] += f * P->cnorm[st];
+      ypart[A] += f * P->cpart[st];
+    }
+    eC[A] = ex(c);
+    eD[A] = P->dexp[A];
+    eY[A] = ymax[A] > 0 ? ex(ymax[A]) : 200;   // (no Y at all: V of such a B is stored as zero)
   }
-  s.c = f(eC);
-  s.v = f(eV);
-  s.d = f(eD);
-  s.y = f(eY - eC - eD);
-  s.u = s.u1 = f(eU - eD - eY);
-  s.z = f(eZ - eV - eY);
-  s.r1 = std::ldexp(1.0, -eC - eU);
-  s.q1 = std::ldexp(1.0, -eV - eU);
-  s.r2 = std::ldexp(1.0, -2 * eY);
-  s.q2 = std::ldexp(1.0, -eZ - eD);
+  for (int A = 0; A < N; ++A) {
+    const int s = P->species[A];
+    // the largest V y and V yp of the atom's pairs, h(r) = erfc(omega r) / (r + 1)
+    // taken where 1 / (r + 1) alone does not settle it
+    double v = 0, z = 0;
+    for (int p = v_ptr[A]; p < v_ptr[A + 1]; ++p) {
+      const int b = v_j[p], st = s * S + P->species[b];
+      const double r = dist(A, b, &v_R[3 * p]), h0 = std::ldexp(1.0, -P->dexp[b]) / (r + 1.0);
+      const double bv = P->vmax[st] * ymax[b], bz = P->vnorm[st] * ypart[b];
+      if (h0 * bv <= v && h0 * bz <= z) continue;
+      const double h = h0 * std::erfc(P->omega * r);
+      v = std::max(v, h * bv);
+      z = std::max(z, h * bz);
+    }
+    eQ[A] = ex(v) + 14;   // (the bound y[B] times 2 to its exponent is at least 2^14)
+    eZ[A] = ex(std::ldexp(z, -P->dexp[A]));
+  }
+  if (!P->d_scale) P->d_scale = P->mem.alloc<int>(5 * (size_t)N);
+  upload(P->d_scale, sc, P->stream);
+  ck(cudaStreamSynchronize(P->stream), "upload scales");
+  hfx::SplitScale& g = P->scale;
+  g.c = P->d_scale;
+  g.d = g.c + N;
+  g.y = g.d + N;
+  g.q = g.y + N;
+  g.z = g.q + N;
 }
 
 // Pair lists (K0): C pairs within R_C + skin, V pairs within the V radius
@@ -790,25 +887,7 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
   y_ptr[N] = (int)y_j.size();
   const int nC = c_ptr[N], nV = v_ptr[N], nY = y_ptr[N];
   if (nC >= (1 << hfx::kItemShift) || nY >= (1 << hfx::kSubShift)) fail(HFX_ERR_UNSUPPORTED, "too many pairs");
-  // bound of |Y^{XZ}| = |sum_W C_XW D_WZ| at every geometry these lists cover
-  // (no pair distance moves by more than the skin before they are rebuilt)
-  P->ymax = 0;
-  for (int A = 0; A < N; ++A) {
-    double y = 0;
-    for (int q = c_ptr[A]; q < c_ptr[A + 1]; ++q) {
-      double d2 = 0;
-      for (int k = 0; k < 3; ++k) {
-        const double dv = pos[3 * c_j[q] + k] + c_R[3 * q] * L[k] + c_R[3 * q + 1] * L[3 + k] +
-                          c_R[3 * q + 2] * L[6 + k] - pos[3 * A + k];
-        d2 += dv * dv;
-      }
-      const double r = std::max(0.0, std::sqrt(d2) - skin), t = std::max(0.0, 1.0 - r * r / (P->RC * P->RC));
-      y += t * t * t * std::exp(-0.5 * r * r) * P->cmax[P->species[A] * P->S + P->species[c_j[q]]] *
-           P->n_ao[P->species[c_j[q]]];
-    }
-    P->ymax = std::max(P->ymax, y * P->dmax);
-  }
-  set_scale(P);
+  set_scale(P, L, pos, c_ptr, c_j, c_R, v_ptr, v_j, v_R);
   int maxC = 0, maxV = 0;
   for (int A = 0; A < N; ++A) {
     maxC = std::max(maxC, c_ptr[A + 1] - c_ptr[A]);
@@ -1275,12 +1354,12 @@ void split_density(hfx_plan* P) {
   }
   DevPlan D = make_devplan(P, P->lat_ref.data());
   hfx::MixPlan X{P->Dsp, P->dsp_off, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  ck(hfx::launch_dsplit(D, X, P->Dsp, P->scale.d, P->sp, P->stream), "dsplit");
+  ck(hfx::launch_dsplit(D, X, P->Dsp, P->sp, P->stream), "dsplit");
   if (P->t1u) {
     P->d_work = P->mem.alloc<int>(1);
     if (P->sp != hfx::kSplitHalf) {
       P->Dh = P->mem.alloc<uint16_t>((size_t)off[P->n_d]);
-      ck(hfx::launch_dsplit(D, X, P->Dh, P->scale.dh, hfx::kSplitHalf, P->stream), "dsplit");
+      ck(hfx::launch_dsplit(D, X, P->Dh, hfx::kSplitHalf, P->stream), "dsplit");
     }
   }
   ck(cudaStreamSynchronize(P->stream), "dsplit");

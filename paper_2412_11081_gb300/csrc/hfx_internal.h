@@ -20,19 +20,27 @@ constexpr int kMaskWords = kMaxCPerAtom / 32;
 enum { kSplitBf16 = 2, kSplitHalf = 3 };
 constexpr int kPieces = 2;            // pieces per operand
 
-// Powers of two between the split path's stores and the values they stand
-// for (all 1 for bf16 pieces).  The stored C, V, D, Y, U and Z are the values
-// times 2^e with e chosen on the host from bounds that hold at every geometry
-// the lists cover, so that no stored element exceeds 2^15.
+// Exponents of the powers of two between the fp16 stores and the values they
+// stand for, per atom, so that an atom of small templates, small D or weak
+// coupling keeps its significant bits beside one of large ones.  Made on the
+// host from bounds that hold at every geometry the lists cover: no stored
+// element exceeds 2^15.  D and Y are bounded by the 2-norms of what U sums over
+// (rows of D_AB, columns of Y^{BF}), which bounds U 2^6 closer than products
+// of largest elements do: 2^-16 of the product of the two stored ones.
+//   D_IJ    15 + d[I] + d[J]   (d balances D: every row norm times 2^(d[I] + d[J]) <= 1)
+//   C_AF    c[A] - d[F]        Y^{XZ}  y[X] + d[Z]
+//   U_B     kUExp + d[A] + d[B] + y[B] + d[F]
+//   V_AB    q[A] - d[B] - y[B]
+//   Z_AB    z[A] - d[B]
+// so that the terms of every sum over atoms (W of Y, B of Q and Q2, F of R in
+// k_term1_w) have one scale.  (With one scale per kind of block and plan the
+// share of an atom whose templates were 2^24 smaller than another's was off by
+// 1e-2 and its forces by 1e-3; 5e-7 as here.)  bf16 pieces hold the values as
+// they are; of HFX_BF16X3 only the tcgen05 first product's Y and D, fp16
+// pieces in both splits, take these exponents.
+constexpr int kDExp = 15, kUExp = kDExp - 16;
 struct SplitScale {
-  float c = 1.f, v = 1.f, d = 1.f;   // stored piece = c * C, v * V, d * D
-  float y = 1.f, u = 1.f;            // C.D accumulator -> stored Y, D.Y accumulator -> stored U
-  // tcgen05 first product, whose Y and D operands are fp16 pieces for either
-  // piece type: stored Y -> its fp16 Y, D -> its fp16 D, their product -> stored U
-  float yh = 1.f, dh = 1.f, u1 = 1.f;
-  float z = 1.f;                     // V.Y accumulator -> stored Z
-  double r1 = 1.0, q1 = 1.0;         // C.U and V.U accumulators -> R, Q
-  double r2 = 1.0, q2 = 1.0;         // Y.Y and Z.D accumulators -> R2, Q2
+  const int *c = nullptr, *d = nullptr, *y = nullptr, *q = nullptr, *z = nullptr;
 };
 
 // Everything a kernel needs, passed by value.  All pointers are device
@@ -274,8 +282,8 @@ cudaError_t launch_lri_solve(int batch, int n, int w, const double* A, const dou
 
 // Split-precision kernels (hfx_mixed.cu); sp = kSplitBf16 or kSplitHalf.
 long long mixed_launch_count();
-// pieces of every D block, times scale, at dst + X.dsp_off
-cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, uint16_t* dst, float scale, int sp, cudaStream_t s);
+// pieces of every D block at dst + X.dsp_off
+cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, uint16_t* dst, int sp, cudaStream_t s);
 cudaError_t launch_cpieces(const DevPlan& P, const MixPlan& X, int sp, cudaStream_t s);
 cudaError_t launch_vpieces(const DevPlan& P, const MixPlan& X, int sp, const int* list, int n, cudaStream_t s);
 cudaError_t launch_ygroups(const DevPlan& P, const long long* y_idx, const long long* y_total, int* gcnt,

@@ -98,18 +98,19 @@ __device__ __forceinline__ int dix(int p, int a, int b) {
 // D block k (n_ao(I) x n_ao(J)) -> its sub-blocks (ao_subs), row by row, each as
 // NP pieces of 16 x 16 (dix), zero padded.
 template <int SP>
-__global__ void k_dsplit(DevPlan P, MixPlan X, uint16_t* dst, float scale) {
+__global__ void k_dsplit(DevPlan P, MixPlan X, uint16_t* dst) {
   for (long long k = blockIdx.x; k < P.n_d; k += gridDim.x) {
     const int I = P.Didx[5 * k], J = P.Didx[5 * k + 1];
     const int na = P.n_ao[P.species[I]], nb = P.n_ao[P.species[J]];
     const int sj = ao_subs(nb), ha = ao_sub(na), hb = ao_sub(nb), ns = ao_subs(na) * sj;
     uint16_t* out = dst + X.dsp_off[k];
+    const float sc = pscale<SP>(kDExp + P.sc.d[I] + P.sc.d[J]);
     const double* src = P.Dval + P.Doff[k];
     for (int e = threadIdx.x; e < ns * 256; e += blockDim.x) {
       const int sub = e >> 8, al = (e >> 4) & 15, bl = e & 15;
       const int a = (sub / sj) * ha + al, b = (sub % sj) * hb + bl;
       uint16_t pc[NP];
-      split_f<SP>((al < ha && a < na && bl < hb && b < nb) ? (float)src[a * nb + b] * pscale<SP>(scale) : 0.f, pc);
+      split_f<SP>((al < ha && a < na && bl < hb && b < nb) ? (float)src[a * nb + b] * sc : 0.f, pc);
 #pragma unroll
       for (int p = 0; p < NP; ++p) out[sub * NP * 256 + dix(p, al, bl)] = pc[p];
     }
@@ -133,6 +134,7 @@ __global__ void k_cpieces(DevPlan P, MixPlan X) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) scf[k] = (float)P.c_sc[8 * (long long)q + k];
     const long long go = P.G_off[sA * P.S + sF];
+    const float cs = pscale<SP>(P.sc.c[P.c_home[q]] - P.sc.d[P.c_j[q]]);
     const int hF = ao_sub(nF);
     for (int sub = 0, f0 = 0; f0 < nF; ++sub, f0 += hF) {
     const int nf = min(hF, nF - f0);
@@ -140,7 +142,7 @@ __global__ void k_cpieces(DevPlan P, MixPlan X) {
     for (int e = threadIdx.x; e < nt * 128 * 16; e += blockDim.x) {
       const int r = e >> 4, c = e & 15;
       uint16_t pc[NP];
-      split_f<SP>((r < rows && c < nf) ? model::c_value_f(P, scf, go, r * nF + f0 + c, 0) * pscale<SP>(P.sc.c) : 0.f, pc);
+      split_f<SP>((r < rows && c < nf) ? model::c_value_f(P, scf, go, r * nF + f0 + c, 0) * cs : 0.f, pc);
 #pragma unroll
       for (int p = 0; p < NP; ++p) out[((r >> 7) * NP + p) * 2048 + tix(r & 127, c)] = pc[p];
     }
@@ -168,11 +170,12 @@ __global__ void k_vpieces(DevPlan P, MixPlan X, const int* list, int n_list) {
     model::v_pair(P, p, h, g);
     const float hf = (float)h, g0 = (float)g[0], g1 = (float)g[1], g2 = (float)g[2];
     const float* M = P.Mf + P.M_off[sA * P.S + sB];   // FP32 products, as k_vstores
+    const float sv = pscale<SP>(v_exp(P, P.v_home[p], P.v_j[p]));
     uint16_t* out = X.Vm + X.vm_off[p];
     for (int e = threadIdx.x; e < mA * MB; e += blockDim.x) {
       const int al = e / MB, be = e - al * MB;
       uint16_t pc[NP];
-      split_f<SP>(be < mB ? M[al * mB + be] * hf * pscale<SP>(P.sc.v) : 0.f, pc);
+      split_f<SP>(be < mB ? M[al * mB + be] * hf * sv : 0.f, pc);
 #pragma unroll
       for (int pp = 0; pp < NP; ++pp) out[pp * mA * MB + e] = pc[pp];
     }
@@ -260,6 +263,8 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
     const int pA = rup16(nA);
     const int KAF = nA * nF, KP = rup16(KAF), KS = KP + 8, MA = rup16(mA);
     const int MT = MA >> 4, NTq = (KAF + 7) >> 3;
+    const float su = pscale<SP>(kUExp - kDExp);   // D.Y -> stored U
+    const double q1 = pscale_d<SP>(-(P.sc.q[A] + kUExp + P.sc.d[A] + P.sc.d[f]));
     __syncthreads();
     if (threadIdx.x == 0) {
       sacc[0] = sacc[1] = sacc[2] = sacc[3] = 0.0;
@@ -416,7 +421,7 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
                 if (r < rowsU && a < nA) {
                   const int be = r / nF, ff = r - be * nF;
                   uint16_t pc[NP];
-                  split_f<SP>(acc[nt][c] * pscale<SP>(P.sc.u), pc);
+                  split_f<SP>(acc[nt][c] * su, pc);
 #pragma unroll
                   for (int pp = 0; pp < NP; ++pp) Us[(size_t)pp * MB * KS + (size_t)be * KS + a * nF + ff] = pc[pp];
                 }
@@ -476,10 +481,12 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
         for (int c = 0; c < 4; ++c) {
           const float w = warp_sum_f(evf[c]);
           if (lane == 0) {
+            const int b = P.v_j[p];
+            const double r1 = pscale_d<SP>(-(P.sc.c[A] + kUExp + P.sc.d[A] + P.sc.d[b] + P.sc.y[b]));
             if (P.fxC)   // deterministic plan: straight into the exact cells
-              (c == 0) ? dev::add_E(P, -(double)w * P.sc.r1) : dev::add_gV(P, 3 * p + c - 1, -(double)w * P.sc.r1);
+              (c == 0) ? dev::add_E(P, -(double)w * r1) : dev::add_gV(P, 3 * p + c - 1, -(double)w * r1);
             else
-              atomicAdd(&sacc[c], (double)w * P.sc.r1);
+              atomicAdd(&sacc[c], (double)w * r1);
           }
         }
         // Q += V_AB . U (M = alpha, N = (a,f), K = beta).  Warp -> one alpha tile
@@ -535,9 +542,9 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
               qacc[i][c] = 0.f;
             }
           }
-          g[0] += (double)gf[0] * P.sc.q1;
-          g[1] += (double)gf[1] * P.sc.q1;
-          g[2] += (double)gf[2] * P.sc.q1;
+          g[0] += (double)gf[0] * q1;
+          g[1] += (double)gf[1] * q1;
+          g[2] += (double)gf[2] * q1;
         }
       }
     }
@@ -590,6 +597,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
     const uint16_t* Vp = X.Vm + X.vm_off[p];
     const float* V = reinterpret_cast<const float*>(Vp + NP * mA * MB);
     const int nvb = mA * mB;
+    const float sz = pscale<SP>(P.sc.z[A] - P.sc.q[A] - P.sc.d[A]);   // V.Y -> stored Z
+    const double r2 = pscale_d<SP>(-r2_exp(P, A, b));
     __syncthreads();
     // stage the rows [(a,b)] of Y^{BA} (by beta) and of the transposed Y^{AB}
     // (by alpha) with 16-byte copies (rows NAB long, shared-memory stride KZ;
@@ -707,8 +716,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
           if (al < mA) {
             const int a = col >> 4, bb = col & 15;
             uint16_t p0[NP], p1[NP];
-            split_f<SP>(acc[2 * h] * pscale<SP>(P.sc.z), p0);
-            split_f<SP>(acc[2 * h + 1] * pscale<SP>(P.sc.z), p1);
+            split_f<SP>(acc[2 * h] * sz, p0);
+            split_f<SP>(acc[2 * h + 1] * sz, p1);
             const int r = al * nA + a;
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp)
@@ -722,7 +731,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_term2_pairs(DevPlan P, MixPlan 
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const float w = warp_sum_f(evf[c]);
-      ev[c] = lane == 0 ? (double)w * P.sc.r2 : 0.0;
+      ev[c] = lane == 0 ? (double)w * r2 : 0.0;
     }
     block_sum_n<4>(ev, red);
     if (threadIdx.x == 0) {
@@ -1056,9 +1065,9 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
             g1 = fmaf(w[1][f4].x, x0, fmaf(w[1][f4].y, x1, fmaf(w[1][f4].z, x2, fmaf(w[1][f4].w, x3, g1))));
             g2 = fmaf(w[2][f4].x, x0, fmaf(w[2][f4].y, x1, fmaf(w[2][f4].z, x2, fmaf(w[2][f4].w, x3, g2))));
           }
-          gd[i][0] += (double)g0 * P.sc.q2;
-          gd[i][1] += (double)g1 * P.sc.q2;
-          gd[i][2] += (double)g2 * P.sc.q2;
+          gd[i][0] += (double)g0;
+          gd[i][1] += (double)g1;
+          gd[i][2] += (double)g2;
         }
       }
       }
@@ -1070,7 +1079,7 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
     for (int i = 0; i < 8; ++i)
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const double w = warp_sum_d(gd[i][c]);
+        const double w = warp_sum_d(gd[i][c]) * (qf[i] >= 0 ? pscale_d<SP>(-(P.sc.z[A] + kDExp + P.sc.d[P.c_j[qf[i]]])) : 1.0);
         if (ok && lane == 0 && w != 0.0) {
           if (P.fxC) dev::add_gC(P, 3 * qf[i] + c, -2.0 * w);   // deterministic plan: straight into the exact cell
           else atomicAdd(&sg[i][c], w);
@@ -1247,6 +1256,7 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
     const int q = warp & 3;
     const int jt = (warp - 2) >> 2, et = (tid - 64) & 127;
     float* ep = reinterpret_cast<float*>(smem_raw) + jt * 128 * 33;   // [128][33]
+    const float sy = pscale<SP>(P.sc.y[Xa] - P.sc.c[Xa] - kDExp);   // C.D -> stored Y
     const bool have = nsteps > 0;
     bool ok = true;
     if (have) {
@@ -1277,7 +1287,7 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
         }
         float* er = ep + (q * 32 + lane) * 33;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) er[j] = __uint_as_float(v[j]) * pscale<SP>(P.sc.y);
+        for (int j = 0; j < 32; ++j) er[j] = __uint_as_float(v[j]) * sy;
       }
       asm volatile("bar.sync %0, 128;\n" ::"r"(1 + jt) : "memory");
 #pragma unroll 1
@@ -1297,6 +1307,8 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
         const long long hxs = (long long)m8 * KZc, hplane = NXS * hxs, hzo = (long long)m8 * z0 * 16;
         const long long plane = cm ? hxs : (long long)mX * nZ * PX;
         const float* eh = ep + h * 16;
+        // stored Y -> its fp16 pieces (the same with fp16 pieces, 2^(y + d) with bf16 ones)
+        const float sh = SP == kSplitHalf ? 1.f : p2f(y_exp(P, Xa, zat[i]));
         // bf16 pieces: chunk (alpha, z, half) holds x = 8 half .. 8 half + 7
         // (core-matrix order: consecutive threads take consecutive alpha, whose
         // chunks are 16 bytes apart)
@@ -1336,8 +1348,8 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
             float f0[4], f1[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              f0[k] = x0 + k < xe ? eh[(rl + k) * 33 + zz] * P.sc.yh : 0.f;
-              f1[k] = x0 + 4 + k < xe ? eh[(rl + 4 + k) * 33 + zz] * P.sc.yh : 0.f;
+              f0[k] = x0 + k < xe ? eh[(rl + k) * 33 + zz] * sh : 0.f;
+              f1[k] = x0 + 4 + k < xe ? eh[(rl + 4 + k) * 33 + zz] * sh : 0.f;
             }
             uint2 p0[NP], p1[NP];
             split4<kSplitHalf>(f0, p0);
@@ -1362,8 +1374,8 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
             float f0[4], f1[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              f0[k] = 8 * hz + k < nZs ? eh[rl * 33 + 8 * hz + k] * P.sc.yh : 0.f;
-              f1[k] = 8 * hz + 4 + k < nZs ? eh[rl * 33 + 8 * hz + 4 + k] * P.sc.yh : 0.f;
+              f0[k] = 8 * hz + k < nZs ? eh[rl * 33 + 8 * hz + k] * sh : 0.f;
+              f1[k] = 8 * hz + 4 + k < nZs ? eh[rl * 33 + 8 * hz + 4 + k] * sh : 0.f;
             }
             uint2 p0[NP], p1[NP];
             split4<kSplitHalf>(f0, p0);
@@ -1435,7 +1447,7 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
             if (Yh) {
               const int xs = x / hX, xl = x - xs * hX;
               uint16_t* yo = Yh + xs * hxs + hzo + cmx(al, zz * 16, 16 * nZs);
-              split_f<kSplitHalf>(y * P.sc.yh, pc);
+              split_f<kSplitHalf>(y * sh, pc);
 #pragma unroll
               for (int pp = 0; pp < NP; ++pp) {
                 yo[pp * hplane + ((xl >> 3) << 6) + (xl & 7)] = pc[pp];
@@ -1622,11 +1634,11 @@ int q2_least(int n_atoms, int FC8, int MC) {
   return best;
 }
 
-cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, uint16_t* dst, float scale, int sp, cudaStream_t s) {
+cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, uint16_t* dst, int sp, cudaStream_t s) {
   if (P.n_d == 0) return cudaSuccess;
   ++g_mix_launches;
-  if (sp == kSplitBf16) k_dsplit<kSplitBf16><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X, dst, scale);
-  else k_dsplit<kSplitHalf><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X, dst, scale);
+  if (sp == kSplitBf16) k_dsplit<kSplitBf16><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X, dst);
+  else k_dsplit<kSplitHalf><<<grid_for(P.n_d, 152 * 64), 256, 0, s>>>(P, X, dst);
   return cudaGetLastError();
 }
 

@@ -169,6 +169,7 @@ __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) scf[k] = (float)P.c_sc[8 * (long long)q + k];
     const long long go = P.G_off[sA * P.S + P.species[F]];
+    const float sc = pscale<SP>(P.sc.c[A] - P.sc.d[F]);
     for (int c = 0; c < 4; ++c) {
       __syncthreads();
       for (int e = threadIdx.x; e < ncq; e += blockDim.x) {
@@ -185,8 +186,8 @@ __global__ void k_t1u_cstore(DevPlan P, T1UPlan U, const int* list, int n) {
         for (int t4 = threadIdx.x; t4 < g8 * 2 * KP; t4 += blockDim.x) {
           const int g = t4 / (2 * KP), t = 4 * (t4 - g * 2 * KP);
           const int al = g * 8 + ((t >> 3) & 7), col = (t >> 6) * 8 + (t & 7);
-          const float x[4] = {val(al, col) * pscale<SP>(P.sc.c), val(al, col + 1) * pscale<SP>(P.sc.c),
-                              val(al, col + 2) * pscale<SP>(P.sc.c), val(al, col + 3) * pscale<SP>(P.sc.c)};
+          const float x[4] = {val(al, col) * sc, val(al, col + 1) * sc,
+                              val(al, col + 2) * sc, val(al, col + 3) * sc};
           uint2 pc[NP];
           split4<SP>(x, pc);
 #pragma unroll
@@ -230,6 +231,7 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
     double h, g[3];
     model::v_pair(P, p, h, g);   // V = M h, grad V = M g (block model), in FP32
     const float hf = (float)h, g0 = (float)g[0], g1 = (float)g[1], g2 = (float)g[2];
+    const float sv = pscale<SP>(v_exp(P, P.v_home[p], P.v_j[p]));
     bool t1 = false;
 #pragma unroll
     for (int w = 0; w < kMaskWords; ++w) t1 = t1 || P.v_mask[(long long)p * kMaskWords + w] != 0u;
@@ -252,7 +254,7 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
         const int e = 4 * e4, al = e / MB, be = e - al * MB;
         float x[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] = be + j < mB ? vsm[al * mB + be + j] * pscale<SP>(P.sc.v) : 0.f;
+        for (int j = 0; j < 4; ++j) x[j] = be + j < mB ? vsm[al * mB + be + j] * sv : 0.f;
         uint2 pc[NP];
         split4<SP>(x, pc);
 #pragma unroll
@@ -277,7 +279,7 @@ __global__ void k_vstores(DevPlan P, MixPlan X, T1UPlan U, const int* list, int 
         const int al = g8 * 8 + ((t >> 3) & 7), be = ((t >> 6) << 3) + (t & 7);
         float x[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] = (al < mA && be + j < mB) ? vsm[al * mB + be + j] * pscale<SP>(P.sc.v) : 0.f;
+        for (int j = 0; j < 4; ++j) x[j] = (al < mA && be + j < mB) ? vsm[al * mB + be + j] * sv : 0.f;
         uint2 pc[NP];
         split4<SP>(x, pc);
 #pragma unroll
@@ -793,15 +795,18 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int q = it.q(), sA = P.species[P.c_home[q]];
       const Sub sb = item_sub<SUB>(it.sub(), P.n_abf[sA], P.n_ao[sA], P.n_ao[P.species[P.c_j[q]]]);
       const int nA = sb.nA, mA = sb.mA, nF = sb.nF;
+      const int hA = P.c_home[q], eR = P.sc.c[hA] + kUExp + P.sc.d[hA];   // (R: and d[B] + y[B])
+      const double q1 = pscale_d<SP>(-(P.sc.q[hA] + kUExp + P.sc.d[hA] + P.sc.d[P.c_j[q]]));
       const long long b0 = X.qoff[q];
       const float* Cf = reinterpret_cast<const float*>(U.Cu + (long long)it.kk * U.cu_blk + (CB >> 1));
       int run = 0;
       for (int i0 = it.lo; i0 < it.hi && ok; i0 += 32) {
-        int p_l = 0, mB_l = 0, nB_l = 0;
+        int p_l = 0, mB_l = 0, nB_l = 0, yB_l = 0;
         long long vo_l = 0;
         if (i0 + lane < it.hi) {
           p_l = X.blist[b0 + i0 + lane];
-          const int s_b = P.species[P.v_j[p_l]];
+          const int b = P.v_j[p_l], s_b = P.species[b];
+          if (SP == kSplitHalf) yB_l = P.sc.d[b] + P.sc.y[b];
           mB_l = P.n_abf[s_b];
           nB_l = P.n_ao[s_b];
           vo_l = (SUB ? U.t1_idx[p_l] * U.NAL + sb.als : U.t1_idx[p_l]) * U.vu_blk;
@@ -874,7 +879,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int c = 0; c < 3; ++c) gv[c] = warp_sum_f(gv[c]);
             const float g = lane == 0 ? gv[0] : lane == 1 ? gv[1] : gv[2];
             const int p = __shfl_sync(0xffffffffu, p_l, j);
-            if (lane < 3 && g != 0.f) dev::add_gV(P, 3 * p + lane, -(double)g * P.sc.r1);
+            const int yB = SP == kSplitHalf ? __shfl_sync(0xffffffffu, yB_l, j) : 0;
+            if (lane < 3 && g != 0.f) dev::add_gV(P, 3 * p + lane, -(double)g * pscale_d<SP>(-(eR + yB)));
           }
           if (ew == 0)
             fl += (unsigned)(mB * nF * nA) *
@@ -909,10 +915,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
               for (int c = 0; c < 4; ++c) e[c] = warp_sum_d(e[c]);
               if (lane == 0) {
-                if (e[0] != 0.0) dev::add_E(P, -e[0] * P.sc.q1);
+                if (e[0] != 0.0) dev::add_E(P, -e[0] * q1);
 #pragma unroll
                 for (int c = 0; c < 3; ++c)
-                  if (e[c + 1] != 0.0) dev::add_gC(P, 3 * q + c, -2.0 * e[c + 1] * P.sc.q1);
+                  if (e[c + 1] != 0.0) dev::add_gC(P, 3 * q + c, -2.0 * e[c + 1] * q1);
               }
             }
             tc_fence_before();
@@ -932,7 +938,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // at a time, so that one's conversions overlap the other's latencies.
     const int qd = warp & 3;
     const uint32_t tl = (uint32_t)(qd * 32) << 16;
-    const float su = P.sc.u1;
+    float su = p2f(kUExp - kDExp);   // D.Y -> stored U (bf16 pieces: per B)
     Ring ik, ub, t;
     bool ok = true;
     for (Unit it = next_unit(ik); it.kk >= 0 && ok; it = next_unit(ik)) {
@@ -941,13 +947,18 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float inv = 1.0f / (float)nF;
       const long long b0 = X.qoff[q];
       for (int i0 = it.lo; i0 < it.hi && ok; i0 += 32) {
-        int ng_l = 0;
-        if (i0 + lane < it.hi) ng_l = ((P.n_abf[P.species[P.v_j[X.blist[b0 + i0 + lane]]]] + 7) >> 3) * nF;
+        int ng_l = 0, eU_l = 0;
+        if (i0 + lane < it.hi) {
+          const int b = P.v_j[X.blist[b0 + i0 + lane]];
+          ng_l = ((P.n_abf[P.species[b]] + 7) >> 3) * nF;
+          if (SP == kSplitBf16) eU_l = kDExp + P.sc.d[P.c_home[q]] + P.sc.d[b] + y_exp(P, b, P.c_j[q]);
+        }
         const int nb = min(32, it.hi - i0);
         for (int j = 0; j < nb && ok; ++j) {
           ok = __all_sync(0xffffffffu, !aborted(abort_flag)) != 0;
           if (!ok) break;
           const int ng = __shfl_sync(0xffffffffu, ng_l, j);
+          if (SP == kSplitBf16) su = p2f(-__shfl_sync(0xffffffffu, eU_l, j));
           ok = wait_all(ue + 8 * ub.s, ub.ph ^ 1);
           unsigned char* ubase = smem_raw + CB + ub.s * UBY + (lane & 7) * 16;
           for (int r0 = 0; r0 < ng && ok; r0 += kYG) {
@@ -1177,6 +1188,9 @@ __global__ void __launch_bounds__(kT2Threads, 1)
       const int nA = P.n_ao[sA], nB = P.n_ao[sB], mA = P.n_abf[sA], mB = P.n_abf[sB];
       const int KK = 16 * nA;
       const int rbuf = i & 1;
+      const int hA = P.v_home[p], hB = P.v_j[p];
+      const float sz = pscale<SP>(P.sc.z[hA] - P.sc.q[hA] - P.sc.d[hA]);   // V.Y -> stored Z
+      const double r2 = pscale_d<SP>(-r2_exp(P, hA, hB));
       // ---- R2 -> E, g^V (the V, grad V rows of the first 32 columns are
       // fetched before the wait; they do not depend on R2)
       const float4* V4 = reinterpret_cast<const float4*>(X.Vz + (long long)kk * X.vz_blk + NP * 4096) + qd * 32 + lane;
@@ -1228,10 +1242,10 @@ __global__ void __launch_bounds__(kT2Threads, 1)
 #pragma unroll
       for (int c = 0; c < 4; ++c) ev[c] = warp_sum_f(ev[c]);
       if (lane == 0 && ok) {
-        if (ev[0] != 0.f) dev::add_E(P, -(double)ev[0] * P.sc.r2);
+        if (ev[0] != 0.f) dev::add_E(P, -(double)ev[0] * r2);
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-          if (ev[c + 1] != 0.f) dev::add_gV(P, 3 * p + c, -(double)ev[c + 1] * P.sc.r2);
+          if (ev[c + 1] != 0.f) dev::add_gV(P, 3 * p + c, -(double)ev[c + 1] * r2);
       }
       // ---- Z -> the Z store: NP planes of 128-row tiles of rows (alpha, a),
       // 16 columns b each, in the core-matrix order of tix; a thread writes
@@ -1258,8 +1272,8 @@ __global__ void __launch_bounds__(kT2Threads, 1)
               float x0[4], x1[4];
 #pragma unroll
               for (int k = 0; k < 4; ++k) {
-                x0[k] = x[8 * hb + k] * pscale<SP>(P.sc.z);
-                x1[k] = x[8 * hb + 4 + k] * pscale<SP>(P.sc.z);
+                x0[k] = x[8 * hb + k] * sz;
+                x1[k] = x[8 * hb + 4 + k] * sz;
               }
               uint2 p0[NP], p1[NP];
               split4<SP>(x0, p0);
@@ -1310,13 +1324,14 @@ __global__ void __launch_bounds__(256) k_t2w_vstore(DevPlan P, MixPlan X, T2WPla
     model::v_pair(P, p, h, g);
     const float f[4] = {(float)h, (float)g[0], (float)g[1], (float)g[2]};
     const float* M = P.Mf + P.M_off[sA * P.S + sB];
+    const float sv = pscale<SP>(v_exp(P, P.v_home[p], P.v_j[p]));
     uint16_t* out = X.Vz + (long long)k * X.vz_blk;
     for (int t4 = threadIdx.x; t4 < m8 * S.VK / 4; t4 += blockDim.x) {   // core-matrix order, 4 columns per thread
       const int t = 4 * t4, g8 = t / (8 * S.VK), u = t - g8 * 8 * S.VK;
       const int al = g8 * 8 + ((u >> 3) & 7), be = ((u >> 6) << 3) + (u & 7);
       float x[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) x[j] = (al < mA && be + j < mB) ? M[al * mB + be + j] * f[0] * pscale<SP>(P.sc.v) : 0.f;
+      for (int j = 0; j < 4; ++j) x[j] = (al < mA && be + j < mB) ? M[al * mB + be + j] * f[0] * sv : 0.f;
       uint2 pc[NP];
       split4<SP>(x, pc);
 #pragma unroll
@@ -1495,6 +1510,8 @@ __global__ void __launch_bounds__(kT2Threads, 1)
       if (!ok) break;
       const Pair q = pair_of(kk);
       const bool rows = 32 * qd < q.mA, act = alpha < q.mA;
+      const float sz = pscale<SP>(P.sc.z[q.A] - P.sc.q[q.A] - P.sc.d[q.A]);   // V.Y -> stored Z
+      const double r2 = pscale_d<SP>(-r2_exp(P, q.A, q.B));
       const float4* V4 = reinterpret_cast<const float4*>(X.Vz + (long long)kk * X.vz_blk + NP * S.M8 * S.VK) + alpha;
       float4 w[4][4];
       auto fetch = [&](int cb) {   // V, grad V of columns 16 cb .. + 15
@@ -1543,10 +1560,10 @@ __global__ void __launch_bounds__(kT2Threads, 1)
 #pragma unroll
             for (int k = 0; k < 4; ++k) ev[k] = warp_sum_f(ev[k]);
             if (lane == 0) {
-              if (ev[0] != 0.f) dev::add_E(P, -(double)ev[0] * P.sc.r2);
+              if (ev[0] != 0.f) dev::add_E(P, -(double)ev[0] * r2);
 #pragma unroll
               for (int k = 0; k < 3; ++k)
-                if (ev[k + 1] != 0.f) dev::add_gV(P, 3 * q.p + k, -(double)ev[k + 1] * P.sc.r2);
+                if (ev[k + 1] != 0.f) dev::add_gV(P, 3 * q.p + k, -(double)ev[k + 1] * r2);
             }
           }
         }
@@ -1567,7 +1584,7 @@ __global__ void __launch_bounds__(kT2Threads, 1)
             uint32_t pc[8][NP];
 #pragma unroll
             for (int k = 0; k < 8; ++k)
-              split2<SP>(__uint_as_float(v[2 * k]) * pscale<SP>(P.sc.z), __uint_as_float(v[2 * k + 1]) * pscale<SP>(P.sc.z), pc[k]);
+              split2<SP>(__uint_as_float(v[2 * k]) * sz, __uint_as_float(v[2 * k + 1]) * sz, pc[k]);
 #pragma unroll
             for (int pp = 0; pp < NP; ++pp) {
               *reinterpret_cast<uint4*>(d + pp * 2048) = make_uint4(pc[0][pp], pc[1][pp], pc[2][pp], pc[3][pp]);

@@ -158,7 +158,7 @@ __global__ void k_dsplit_w(DevPlan P, uint16_t* Dw, const long long* dw_off) {
     uint16_t* out = Dw + dw_off[k];
     for (int e = threadIdx.x; e < pa * pb; e += blockDim.x) {
       const int a = e / pb, b = e - a * pb;
-      put_pieces<SP>(out, (long long)pa * pb, e, (a < na && b < nb) ? (float)src[a * nb + b] * pscale<SP>(P.sc.d) : 0.f);
+      put_pieces<SP>(out, (long long)pa * pb, e, (a < na && b < nb) ? (float)src[a * nb + b] * pscale<SP>(kDExp + P.sc.d[I] + P.sc.d[J]) : 0.f);
     }
   }
 }
@@ -181,9 +181,10 @@ __global__ void k_cpieces_w(DevPlan P, uint16_t* Cw, const long long* cw_off, fl
     const int naf = nA * nF, CW = cw_cols(nA, nF);
     const double* src = P.Cst + P.c_off[q];
     uint16_t* out = Cw + cw_off[q];
+    const float sc = pscale<SP>(P.sc.c[P.c_home[q]] - P.sc.d[P.c_j[q]]);
     for (int e = threadIdx.x; e < mA * CW; e += blockDim.x) {
       const int al = e / CW, c = e - al * CW;
-      put_pieces<SP>(out, (long long)mA * CW, e, c < naf ? (float)src[(long long)al * naf + c] * pscale<SP>(P.sc.c) : 0.f);
+      put_pieces<SP>(out, (long long)mA * CW, e, c < naf ? (float)src[(long long)al * naf + c] * sc : 0.f);
     }
     const double* dsrc = P.dCst + 3 * P.c_off[q];
     float* dst = dCf + 3 * P.c_off[q];
@@ -235,6 +236,9 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
     const int nvb = mA * mB;
     const int pa = rup16(nA);
     const uint16_t* Dg = Dw + dw_off[P.v_didx[p]];   // D_AB pieces [pa][KB]
+    const float sv = pscale<SP>(v_exp(P, A, b));
+    const float su = pscale<SP>(kUExp - kDExp);   // D.Y -> stored U
+    const double r1 = pscale_d<SP>(-(P.sc.c[A] + kUExp + P.sc.d[A] + P.sc.d[b] + P.sc.y[b]));
     __syncthreads();   // previous pair done with every buffer
     if (threadIdx.x == 0) {
       s_g[0] = s_g[1] = s_g[2] = 0.0;
@@ -242,7 +246,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
     }
     for (int e = threadIdx.x; e < MA * SV; e += blockDim.x) {
       const int al = e / SV, be = e - al * SV;
-      put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * pscale<SP>(P.sc.v) : 0.f);
+      put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * sv : 0.f);
     }
     for (int e = threadIdx.x; e < 48 * SD; e += blockDim.x) {
       const int a = e / SD, bb = e - a * SD;
@@ -289,7 +293,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
           }
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c) ev[c] += (double)evf[c] * P.sc.r1;
+      for (int c = 0; c < 4; ++c) ev[c] += (double)evf[c] * r1;
     };
     const int q0 = P.c_ptr[A];
     double fl = 0.0;
@@ -388,9 +392,9 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
                 const int r = nt * 8 + 2 * tig + c;
                 if (r < rowsU) {
                   const int be = r / nF, ff = r - be * nF;
-                  if (gid < dA) put_pieces<SP>(Us, pU, be * SK + gid * nF + ff, acc[c] * pscale<SP>(P.sc.u));
+                  if (gid < dA) put_pieces<SP>(Us, pU, be * SK + gid * nF + ff, acc[c] * su);
                   if (gid + 8 < dA)
-                    put_pieces<SP>(Us, pU, be * SK + (gid + 8) * nF + ff, acc[2 + c] * pscale<SP>(P.sc.u));
+                    put_pieces<SP>(Us, pU, be * SK + (gid + 8) * nF + ff, acc[2 + c] * su);
                 }
               }
             }
@@ -435,7 +439,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
         for (int c = 0; c < 3; ++c) {
           const float w = warp_sum_f(gq[c]);
           if (lane == 0) {
-            const double wd = (double)w * P.sc.q1;
+            const double wd = (double)w * pscale_d<SP>(-(P.sc.q[A] + kUExp + P.sc.d[A] + P.sc.d[f]));
             if (P.fxC) dev::add_gC(P, 3 * q + c, -2.0 * wd);   // deterministic plan: straight into the exact cell
             else atomicAdd(&s_g[c], wd);
           }
@@ -509,10 +513,12 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
     const int nvb = mA * mB;
     uint16_t* Z = Zst + (long long)kk * S.KB * S.zblk;
     const int hB = ao_sub(nB);
+    const float sv = pscale<SP>(v_exp(P, A, b)), sz = pscale<SP>(P.sc.z[A] - P.sc.q[A] - P.sc.d[A]);
+    const double r2 = pscale_d<SP>(-r2_exp(P, A, b));
     __syncthreads();   // previous pair done with every buffer
     for (int e = threadIdx.x; e < MA * SV; e += blockDim.x) {
       const int al = e / SV, be = e - al * SV;
-      put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * pscale<SP>(P.sc.v) : 0.f);
+      put_pieces<SP>(Vs, pV, e, (al < mA && be < mB) ? (float)V[al * mB + be] * sv : 0.f);
     }
     // Y^{BA} rows beyond n_abf(B) stay zero (K of Z)
     for (int e = threadIdx.x; e < (MB - mB) * SK; e += blockDim.x)
@@ -593,7 +599,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
                 const int bb = n / dA, a = n - bb * dA, r = al * nA + a0 + a, sub = bb / hB;
                 put_pieces<SP>(Z + sub * S.zblk + (long long)(r >> 7) * NP * 2048, 2048,
                                (((r & 127) >> 3) << 7) + (((bb - sub * hB) >> 3) << 6) + ((r & 7) << 3) + ((bb - sub * hB) & 7),
-                               acc[h][c] * pscale<SP>(P.sc.z));
+                               acc[h][c] * sz);
               }
             }
         }
@@ -625,7 +631,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term2_w(DevPlan P, const uint16
           }
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c) ev[c] = (double)evf[c] * P.sc.r2;
+      for (int c = 0; c < 4; ++c) ev[c] = (double)evf[c] * r2;
     }
     block_sum_w<4, kPW>(ev, red);
     if (threadIdx.x == 0) {

@@ -237,3 +237,45 @@ def test_operands_far_from_one(g, m, d):
     assert a[3]["triplets"] == b[3]["triplets"]
     for x, y in zip(a[:3], b[:3]):
         assert rel(np.asarray(y) / f, x) <= 1e-12
+
+
+def _uneven(n_ao, n_abf, what, k):
+    """A two-species cell whose second species has templates C, templates V or
+    density blocks 2^k times smaller (D_11 and M_11 by 2^2k)."""
+    import dataclasses
+    w = _edge_cell(n_ao, n_abf)
+    G, M, d = [x.copy() for x in w.G], [x.copy() for x in w.M], w.d_values.copy()
+    if what == "C":
+        G[2] *= 2.0 ** -k
+        G[3] *= 2.0 ** -k
+    elif what == "V":
+        M[1] *= 2.0 ** -k
+        M[2] *= 2.0 ** -k
+        M[3] *= 2.0 ** (-2 * k)
+    else:
+        for b, (i, j) in enumerate(w.d_index[:, :2]):
+            d[w.d_offset[b]:w.d_offset[b + 1]] *= 2.0 ** (-k * (int(i == 1) + int(j == 1)))
+    return dataclasses.replace(w, G=G, M=M, d_values=d)
+
+
+UNEVEN_ENV = {"tensor memory": {}, "warp-level": {"HFX_T1_KERNEL": "mma", "HFX_T2_KERNEL": "mma"},
+              "one Y store": {"HFX_Y_STORE_GB": "0"}}
+
+
+@pytest.mark.parametrize("what,k", [("C", 12), ("C", 24), ("C", 36), ("V", 24), ("D", 12), ("D", 24)])
+@pytest.mark.parametrize("n_ao,n_abf,route", [([5, 3], [11, 7], "tensor memory"), ([5, 3], [11, 7], "warp-level"),
+                                              ([9, 5], [70, 30], "tensor memory"), ([18, 5], [23, 11], "tensor memory"),
+                                              ([18, 5], [23, 11], "one Y store")])
+@pytest.mark.parametrize("prec,tol", [(hfx.HFX_BF16X6, BOUND), (hfx.HFX_BF16X3, 1e-4)])
+def test_small_species_beside_a_large_one(n_ao, n_abf, route, what, k, prec, tol, monkeypatch):
+    """The share of each atom keeps its relative accuracy however much smaller
+    than the other's its blocks are: HFX_BF16X6 within its contract, HFX_BF16X3
+    as in test_block_shape_edges."""
+    for name, value in UNEVEN_ENV[route].items():
+        monkeypatch.setenv(name, value)
+    w = _uneven(n_ao, n_abf, what, k)
+    zero = dict.fromkeys(("C", "dC", "V", "dV", "D", "CS"), 0.0)
+    for home in ((0, 1), (1, 2)):
+        E0, F0, S0, _ = run(w, hfx.HFX_FP64, theta=zero, home=home)
+        E, F, S, _ = run(w, prec, theta=zero, home=home)
+        assert abs(E - E0) <= tol * abs(E0) and rel(F, F0) <= tol and rel(S, S0) <= tol, (home, abs(E - E0) / abs(E0), rel(F, F0), rel(S, S0))
