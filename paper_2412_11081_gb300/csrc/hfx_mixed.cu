@@ -1024,6 +1024,23 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
     double gd[8][3];
 #pragma unroll
     for (int i = 0; i < 8; ++i) gd[i][0] = gd[i][1] = gd[i][2] = 0.0;
+    // This warp's sums so far, into the CTA's or, for a deterministic plan,
+    // straight into the exact cells.  Those take each run of each tile by
+    // itself, so that what is rounded together does not depend on how the
+    // tiles are divided over warps and CTAs.
+    auto give = [&]() {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const double w = warp_sum_d(gd[i][c]) * (qf[i] >= 0 ? pscale_d<SP>(-(P.sc.z[A] + kDExp + P.sc.d[P.c_j[qf[i]]])) : 1.0);
+          gd[i][c] = 0.0;
+          if (lane == 0 && w != 0.0) {
+            if (P.fxC) dev::add_gC(P, 3 * qf[i] + c, -2.0 * w);
+            else atomicAdd(&sg[i][c], w);
+          }
+        }
+    };
     bool ok = true;
     for (int run = 0; run < nruns; ++run) {
       const int b = run % NB;
@@ -1070,21 +1087,13 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
           gd[i][2] += (double)g2;
         }
       }
+      if (P.fxC) give();
       }
       asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(macce + 8 * b) : "memory");
     }
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const double w = warp_sum_d(gd[i][c]) * (qf[i] >= 0 ? pscale_d<SP>(-(P.sc.z[A] + kDExp + P.sc.d[P.c_j[qf[i]]])) : 1.0);
-        if (ok && lane == 0 && w != 0.0) {
-          if (P.fxC) dev::add_gC(P, 3 * qf[i] + c, -2.0 * w);   // deterministic plan: straight into the exact cell
-          else atomicAdd(&sg[i][c], w);
-        }
-      }
+    if (ok && !P.fxC) give();
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();

@@ -74,3 +74,23 @@ def test_graph_replay_same_bits():
         assert p.stats.graph_replayed == 1
     for d, r in zip(direct, replayed):
         assert same_bits(d, r)
+
+
+@pytest.mark.parametrize("prec", [hfx.HFX_BF16X6, hfx.HFX_BF16X3])
+def test_same_bits_for_every_tile_shape(prec, monkeypatch):
+    """Each choice of row tiles per CTA by itself, on a cell whose sums over
+    pairs span many orders of magnitude (D down to 1e-10 of its largest
+    block), so that FP64 additions in another order do round differently."""
+    monkeypatch.setenv("HFX_Q2_FLUSH", "4")
+    w = inputs.diamond8()
+    w2 = inputs.make_workload("diamond", 1, 5.43, [13], [50], 3.7, seed=11)
+    for w in (w, w2):
+        ref = None
+        for y in ("1", "2"):
+            for q2 in ("1", "2", "3"):
+                monkeypatch.setenv("HFX_Y_TILES", y)
+                monkeypatch.setenv("HFX_Q2_TILES", q2)
+                with hfx.Plan(w, precision=prec, deterministic=True) as p:
+                    r = p.evaluate(w.lattice, w.positions)
+                ref = ref or r
+                assert same_bits(ref, r), (y, q2)
