@@ -282,6 +282,9 @@ cudaError_t launch_lri_solve(int batch, int n, int w, const double* A, const dou
 
 // Split-precision kernels (hfx_mixed.cu); sp = kSplitBf16 or kSplitHalf.
 long long mixed_launch_count();
+// log2 of the largest row norm of every D block (-1e30 for a zero block)
+cudaError_t launch_drow(long long n_d, const double* Dval, const long long* Doff, const int* Didx, const int* species,
+                        const int* n_ao, float* lg, cudaStream_t s);
 // pieces of every D block at dst + X.dsp_off
 cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, uint16_t* dst, int sp, cudaStream_t s);
 cudaError_t launch_cpieces(const DevPlan& P, const MixPlan& X, int sp, cudaStream_t s);

@@ -95,6 +95,23 @@ __device__ __forceinline__ int dix(int p, int a, int b) {
   return (((a >> 3) * NP + p) << 7) + ((b >> 3) << 6) + ((a & 7) << 3) + (b & 7);
 }
 
+// One warp per D block, a row per lane (n_ao <= 32): 0.5 log2 of the largest sum of squares.
+__global__ void k_drow(long long n_d, const double* Dval, const long long* Doff, const int* Didx, const int* species,
+                       const int* n_ao, float* lg) {
+  const int lane = threadIdx.x & 31;
+  const long long step = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long k = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < n_d; k += step) {
+    const int na = n_ao[species[Didx[5 * k]]], nb = n_ao[species[Didx[5 * k + 1]]];
+    const double* d = Dval + Doff[k] + (long long)lane * nb;
+    double t = 0.0;
+    if (lane < na)
+      for (int b = 0; b < nb; ++b) t += d[b] * d[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t = fmax(t, __shfl_xor_sync(0xffffffffu, t, o));
+    if (lane == 0) lg[k] = t > 0.0 ? (float)(0.5 * log2(t)) : -1e30f;
+  }
+}
+
 // D block k (n_ao(I) x n_ao(J)) -> its sub-blocks (ao_subs), row by row, each as
 // NP pieces of 16 x 16 (dix), zero padded.
 template <int SP>
@@ -1641,6 +1658,14 @@ int q2_least(int n_atoms, int FC8, int MC) {
     }
   }
   return best;
+}
+
+cudaError_t launch_drow(long long n_d, const double* Dval, const long long* Doff, const int* Didx, const int* species,
+                        const int* n_ao, float* lg, cudaStream_t s) {
+  if (n_d == 0) return cudaSuccess;
+  ++g_mix_launches;
+  k_drow<<<grid_for((n_d + 7) / 8, 152 * 64), 256, 0, s>>>(n_d, Dval, Doff, Didx, species, n_ao, lg);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_dsplit(const DevPlan& P, const MixPlan& X, uint16_t* dst, int sp, cudaStream_t s) {

@@ -128,3 +128,17 @@ def test_warp_level_kernels_beyond_the_y_store_limit(monkeypatch):
     E, F, S, st = run(w, hfx.HFX_BF16X6)
     assert st["triplets"] == st0["triplets"] and st["term2_pairs"] == st0["term2_pairs"]
     assert max(errs((E, F, S), (E0, F0, S0))) <= BOUND
+
+
+def test_errors_of_the_135_atom_perovskite():
+    """The FP32 sums over many pairs are this cell's largest error: relative
+    2-norms no larger than the warp-level kernels' with three bf16 pieces per
+    operand (E 2.3e-6, F 1.2e-6, and 1.5e-6 of the first product's stress, the
+    whole one being a difference of the two products')."""
+    w = inputs.perovskite_supercell(3)
+    E0, F0, S0, _ = run(w, hfx.HFX_FP64)
+    S1 = run(w, hfx.HFX_FP64, terms=1)[2]
+    E, F, S, _ = run(w, hfx.HFX_BF16X6)
+    norm = np.linalg.norm
+    assert abs(E - E0) <= 2.3e-6 * abs(E0) and norm(F - F0) <= 1.2e-6 * norm(F0)
+    assert norm(S - S0) <= 1.5e-6 * norm(S1), norm(S - S0) / norm(S1)
