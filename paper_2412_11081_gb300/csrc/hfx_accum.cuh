@@ -70,7 +70,8 @@ __device__ __forceinline__ double fx_get(const unsigned long long* cell) {
 }
 
 // ------------------------------------------------------ the plan's sums
-// FP64 atomic adds, or the fixed-point cells of a deterministic plan
+// FP64 atomic adds (E in kESlots sums by CTA, since each addition rounds at the
+// size the sum has reached), or the fixed-point cells of a deterministic plan
 // (P.fxC != nullptr).  Indices are those of the FP64 arrays.
 __device__ __forceinline__ void add_gC(const DevPlan& P, long long i, double v) {
   if (P.fxC) fx_add(P.fxC + 2 * i, v);
@@ -82,7 +83,7 @@ __device__ __forceinline__ void add_gV(const DevPlan& P, long long i, double v) 
 }
 __device__ __forceinline__ void add_E(const DevPlan& P, double v) {
   if (P.fxC) fx_add(P.fxA, v);
-  else atomicAdd(P.acc + ACC_E, v);
+  else atomicAdd(P.acc + ACC_E + (blockIdx.x & (kESlots - 1)), v);
 }
 __device__ __forceinline__ void add_W(const DevPlan& P, int c, double v) {   // virial component c
   if (P.fxC) fx_add(P.fxA + 2 * (1 + c), v);
@@ -90,7 +91,12 @@ __device__ __forceinline__ void add_W(const DevPlan& P, int c, double v) {   // 
 }
 __device__ __forceinline__ double get_gC(const DevPlan& P, long long i) { return P.fxC ? fx_get(P.fxC + 2 * i) : P.gC[i]; }
 __device__ __forceinline__ double get_gV(const DevPlan& P, long long i) { return P.fxC ? fx_get(P.fxV + 2 * i) : P.gV[i]; }
-__device__ __forceinline__ double get_E(const DevPlan& P) { return P.fxC ? fx_get(P.fxA) : P.acc[ACC_E]; }
+__device__ __forceinline__ double get_E(const DevPlan& P) {
+  if (P.fxC) return fx_get(P.fxA);
+  double e = 0.0;
+  for (int k = 0; k < kESlots; ++k) e += P.acc[ACC_E + k];
+  return e;
+}
 __device__ __forceinline__ double get_W(const DevPlan& P, int c) {
   return P.fxC ? fx_get(P.fxA + 2 * (1 + c)) : P.acc[ACC_W + c];
 }

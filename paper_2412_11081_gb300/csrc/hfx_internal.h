@@ -131,7 +131,7 @@ struct DevPlan {
   // accumulators
   double* gC;                  // [nC*3] dE/dd for C pairs
   double* gV;                  // [nV*3]
-  double* acc;                 // [0] E, [1..9] virial sum g (x) d, [10] flops y, [11] t1, [12] t2
+  double* acc;                 // AccSlot: virial sum g (x) d, flops, partial sums of E
   unsigned long long* cnt;     // [0] c kept, [1] v kept, [2] d kept, [3] triplets
   // deterministic plans: exact fixed-point cells (hfx_accum.cuh) of gC, gV,
   // E and the virial (fxA: E, then the nine virial components) and F, in
@@ -240,7 +240,8 @@ constexpr int kItemShift = 28;
 // uint16 units of one (C pair, sub) in MixPlan::Cm: the pieces, then grad C
 __host__ __device__ inline long long cm_size(int rows) { return (long long)((rows + 127) >> 7) * 2048 * (kPieces + 6); }
 
-enum AccSlot { ACC_E = 0, ACC_W = 1, ACC_FY = 10, ACC_F1 = 11, ACC_F2 = 12, ACC_N = 16 };
+constexpr int kESlots = 32;           // partial sums of E
+enum AccSlot { ACC_W = 1, ACC_FY = 10, ACC_F1 = 11, ACC_F2 = 12, ACC_E = 16, ACC_N = ACC_E + kESlots };
 enum CntSlot { CNT_C = 0, CNT_V = 1, CNT_D = 2, CNT_TRIP = 3, CNT_N = 8 };
 
 // Kernels launched by this library since load (every launcher adds its

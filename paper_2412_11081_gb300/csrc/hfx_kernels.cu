@@ -381,13 +381,26 @@ __global__ void k_ybuild(DevPlan P, const int* list, int n_list) {
   }
 }
 
+// The warps' parts of <V_AB, R> and <grad V_AB, R>, added up by four threads
+// into E and g^V of pair p (behind a barrier).
+__device__ __forceinline__ void add_pair(const DevPlan& P, int p, const double (*ew)[4], int nwarp) {
+  if (threadIdx.x >= 4) return;
+  double s = 0.0;
+  for (int k = 0; k < nwarp; ++k) s += ew[k][threadIdx.x];
+  if (s == 0.0) return;
+  if (threadIdx.x == 0) dev::add_E(P, -s);
+  else dev::add_gV(P, 3 * p + (int)threadIdx.x - 1, -s);
+}
+
 // ---------------------------------------------------------------- K4: term 1
 // One CTA per (A,B) pair with kept F.  Shared memory: D_AB, R_AB, and a
 // beta-chunk of U (bc x n_ao(A) x n_ao(F)).
 //
-// The FP64 pipe bounds it (1.1 TFLOP/s on the whole chip).  Each warp adds its
-// own part of a gradient to the pair's sum, so the only block barriers are
-// the two around a chunk of U.  A chunk is all of U where that leaves room for
+// The FP64 pipe bounds it (1.1 TFLOP/s on the whole chip).  The warps leave
+// their parts of a gradient in shared memory, where three threads add them up
+// behind the next F's barrier, so the only block barriers are the two around a
+// chunk of U.  (Eight atomic additions, one per warp, cost the same time and
+// left E and F 2 to 5 times further off.)  A chunk is all of U where that leaves room for
 // two or three CTAs per SM (they fill each other's barriers), else as much as
 // fits: every chunk repeats the three products with grad C.  Small blocks take
 // 64 threads per CTA, and small cells divide a pair's F over P.parts CTAs, so
@@ -396,7 +409,8 @@ __global__ void k_ybuild(DevPlan P, const int* list, int n_list) {
 // 5-atom perovskite (45.6 now, 0.91 TFLOP/s).
 __global__ void k_term1(DevPlan P, const int* list, int n_list, int BC) {
   extern __shared__ double sm[];
-  const int lane = threadIdx.x & 31;
+  __shared__ double gw[2][kThreads / 32][3], ew[kThreads / 32][4];   // the warps' parts, of this and the last F
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   for (int u = blockIdx.x; u < n_list * P.parts; u += gridDim.x) {
     const int part = u % P.parts, p = list[u / P.parts];
     const int A = P.v_home[p], b = P.v_j[p];
@@ -415,6 +429,13 @@ __global__ void k_term1(DevPlan P, const int* list, int n_list, int BC) {
     const int q0 = P.c_ptr[A];
     double fl = 0.0;
     int turn = 0;   // this part's F: every P.parts-th kept one
+    int last = -1, buf = 0;   // C pair whose parts are in gw[buf ^ 1]
+    auto add_last = [&]() {   // (behind a barrier)
+      if (last < 0 || threadIdx.x >= 3) return;
+      double g = 0.0;
+      for (int k = 0; k < nwarp; ++k) g += gw[buf ^ 1][k][threadIdx.x];
+      if (g != 0.0) dev::add_gC(P, 3 * last + threadIdx.x, -2.0 * g);
+    };
     for (int w = 0; w < kMaskWords; ++w) {
       unsigned bits = P.v_mask[(size_t)p * kMaskWords + w];
       while (bits) {
@@ -447,6 +468,7 @@ __global__ void k_term1(DevPlan P, const int* list, int n_list, int BC) {
             Uc[e] = s2;
           }
           __syncthreads();
+          if (b0 == 0) add_last();
           // R[alpha][b0+bl] += sum_{a,f} C[alpha][a][f] U_c[bl][a][f]
           for (int e = threadIdx.x; e < mA * bc; e += blockDim.x) {
             const int al = e / bc, bl = e - al * bc;
@@ -471,11 +493,9 @@ __global__ void k_term1(DevPlan P, const int* list, int n_list, int BC) {
         g0 = warp_sum(g0);
         g1 = warp_sum(g1);
         g2 = warp_sum(g2);
-        if (lane == 0) {
-          if (g0 != 0.0) dev::add_gC(P, 3 * q + 0, -2.0 * g0);
-          if (g1 != 0.0) dev::add_gC(P, 3 * q + 1, -2.0 * g1);
-          if (g2 != 0.0) dev::add_gC(P, 3 * q + 2, -2.0 * g2);
-        }
+        if (lane < 3) gw[buf][warp][lane] = lane == 0 ? g0 : lane == 1 ? g1 : g2;
+        last = q;
+        buf ^= 1;
         if (threadIdx.x == 0) fl += 2.0 * mB * nA * nB * nF + 4.0 * mA * mB * nA * nF;
       }
     }
@@ -493,12 +513,10 @@ __global__ void k_term1(DevPlan P, const int* list, int n_list, int BC) {
     h0 = warp_sum(h0);
     h1 = warp_sum(h1);
     h2 = warp_sum(h2);
-    if (lane == 0) {
-      if (e0 != 0.0) dev::add_E(P, -e0);
-      if (h0 != 0.0) dev::add_gV(P, 3 * p + 0, -h0);
-      if (h1 != 0.0) dev::add_gV(P, 3 * p + 1, -h1);
-      if (h2 != 0.0) dev::add_gV(P, 3 * p + 2, -h2);
-    }
+    if (lane < 4) ew[warp][lane] = lane == 0 ? e0 : lane == 1 ? h0 : lane == 2 ? h1 : h2;
+    __syncthreads();
+    add_last();
+    add_pair(P, p, ew, nwarp);
     if (threadIdx.x == 0) atomicAdd(&P.acc[ACC_F1], fl);
   }
 }
@@ -513,6 +531,7 @@ __global__ void k_term1(DevPlan P, const int* list, int n_list, int BC) {
 // now).
 __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
   extern __shared__ double sm[];
+  __shared__ double ew[kThreads / 32][4];   // the warps' parts of E and g^V
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   for (int u = blockIdx.x; u < n_list * P.parts2; u += gridDim.x) {
     const int part = u % P.parts2, p = list[u / P.parts2];
@@ -546,12 +565,7 @@ __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
     h0 = warp_sum(h0);
     h1 = warp_sum(h1);
     h2 = warp_sum(h2);
-    if (lane == 0) {
-      if (e0 != 0.0) dev::add_E(P, -e0);
-      if (h0 != 0.0) dev::add_gV(P, 3 * p + 0, -h0);
-      if (h1 != 0.0) dev::add_gV(P, 3 * p + 1, -h1);
-      if (h2 != 0.0) dev::add_gV(P, 3 * p + 2, -h2);
-    }
+    if (lane < 4) ew[warp][lane] = lane == 0 ? e0 : lane == 1 ? h0 : lane == 2 ? h1 : h2;
     const int q0 = P.c_ptr[A], nq = P.c_ptr[A + 1] - q0;
     double* gF = sm;                        // nq*3: component c of an F by lane c of the warp that takes it, and no other
     double* Zc = gF + 3 * kMaxCPerAtom;     // AC*nA*nB
@@ -561,6 +575,7 @@ __global__ void k_term2(DevPlan P, const int* list, int n_list, int AC) {
     for (int a0 = m0; a0 < m1; a0 += AC) {
       const int ac = min(AC, m1 - a0);
       __syncthreads();
+      if (a0 == m0) add_pair(P, p, ew, nwarp);
       // Z[al][a][b] = sum_beta V[a0+al][beta] Yba[beta][b][a]
       for (int e = threadIdx.x; e < ac * nab; e += blockDim.x) {
         const int al = e / nab, ab = e - al * nab;

@@ -94,3 +94,17 @@ def test_same_bits_for_every_tile_shape(prec, monkeypatch):
                     r = p.evaluate(w.lattice, w.positions)
                 ref = ref or r
                 assert same_bits(ref, r), (y, q2)
+
+
+def test_fp64_atomic_sums_round_little():
+    """The default FP64 sums against the exact ones: E within 6e-15 (one atomic
+    addition per pair into one sum left up to 5.4e-15 on such cells), F and
+    sigma within 1e-14."""
+    for n_ao, n_abf, r_c, seed in ((12, 44, 2.8, 5), (9, 31, 2.6, 6), (4, 9, 2.6, 7)):
+        w = inputs.make_workload("diamond", 1, 5.43, [n_ao], [n_abf], r_c, seed=seed)
+        with hfx.Plan(w, deterministic=True) as p:
+            E0, F0, S0 = p.evaluate(w.lattice, w.positions)
+        with hfx.Plan(w) as p:
+            for _ in range(3):
+                E, F, S = p.evaluate(w.lattice, w.positions)
+                assert abs(E - E0) <= 6e-15 * abs(E0) and rel(F, F0) <= 1e-14 and rel(S, S0) <= 1e-14
