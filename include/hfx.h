@@ -330,12 +330,15 @@ hfx_status hfx_plan_autotune(hfx_plan* plan, const double* lattice, const double
  *   X   [batch][n][w]     X = A^-1 B: the C^I rows, then the C^K rows;
  *   dX  [batch][3][n][w]  dX[c] = A^-1 (dB[c] - dA[c] X).
  * dA, dB and dX must be all NULL (X only) or all non-NULL.  Pointers are
- * host memory; the call copies them to device `device`, runs one CTA per
- * pair (Cholesky factor in shared memory) on a stream of its own, copies the
- * results back and returns when they are written.  It holds no state but a
- * stream and two buffers of 1 MiB per calling host thread (device and pinned
- * host memory, given back when the thread ends or calls with another
- * device), and may run beside any plan and in several threads.
+ * host memory; the call copies them to device `device`, factors every pair
+ * and solves its columns 32 to a CTA (Cholesky factor in shared memory) on a
+ * stream of its own, copies the results back and returns when they are
+ * written.  Per calling host thread it keeps a stream and, once a batch of at
+ * most 1 MiB has been solved, two buffers of 1 MiB (device and pinned host
+ * memory) until the thread ends or calls with another device; while they
+ * cannot be had, such a batch takes memory of its own like a larger one.  It
+ * may run beside any plan and in several threads.  As the thread keeps a
+ * stream, do not reset the device (cudaDeviceReset) and call it again.
  * Errors: HFX_ERR_INVALID for batch < 0, n < 1, w < 1, a NULL pointer or a
  * mixed NULL set, or a metric that is not positive definite (outputs are
  * then not written); HFX_ERR_UNSUPPORTED if n exceeds what the device's

@@ -2228,8 +2228,15 @@ namespace {
 // batches of at most kLriKeep bytes a device and a pinned host buffer, so that
 // a call of a few pairs is one copy each way and one launch (creating and
 // freeing the stream and the memory took most of its 97 us).  Freed when the
-// thread ends or calls with another device; larger batches allocate their own.
+// thread ends or calls with another device; larger batches allocate their own,
+// and so does a small one while the two buffers cannot be had.
 constexpr size_t kLriKeep = 1 << 20;
+// Test-only fault injection: HFX_TEST_LRI_OOM=scratch refuses the kept buffers,
+// =all the call's own memory too.
+bool lri_oom(const char* what) {
+  const char* t = std::getenv("HFX_TEST_LRI_OOM");
+  return t && (!std::strcmp(t, "all") || !std::strcmp(t, what));
+}
 struct LriScratch {
   int dev = -1;
   cudaStream_t s = nullptr;
@@ -2239,11 +2246,23 @@ struct LriScratch {
     close();
     cudaError_t e = cudaSetDevice(device);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaMalloc(&buf, kLriKeep);
-    if (e == cudaSuccess) e = cudaMallocHost(&pin, kLriKeep);
     dev = device;
     if (e != cudaSuccess) close();
     return e;
+  }
+  bool buffers() {   // the kept buffers, if they can be had
+    if (buf && !lri_oom("scratch")) return true;
+    if (lri_oom("scratch") || cudaMalloc(&buf, kLriKeep) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (cudaMallocHost(&pin, kLriKeep) != cudaSuccess) {
+      cudaGetLastError();
+      cudaFree(buf);
+      buf = pin = nullptr;
+      return false;
+    }
+    return true;
   }
   void close() {   // (errors ignored: the runtime may be gone at process exit)
     if (dev < 0) return;
@@ -2301,18 +2320,29 @@ hfx_status hfx_lri_fit(int batch, int n, int w, const double* A, const double* B
   if (hfx::lri_fit_smem(n) + 2048 > (size_t)optin)
     return bad(HFX_ERR_UNSUPPORTED, "hfx_lri_fit: n too large for the Cholesky factor in shared memory");
   const size_t nn = (size_t)batch * n * n, nw = (size_t)batch * n * w, k = grad ? 4 : 1;
-  const size_t in = k * (nn + nw), out = k * nw, nl = batch * hfx::lri_factor_size(n, w);
-  const size_t bytes = (in + out + 1 + nl) * sizeof(double);   // [A, dA, B, dB] [X, dX] [error flag] [factors]
-  if (g_lri.open(device) != cudaSuccess) {
+  const size_t in = k * (nn + nw), out = k * nw;
+  size_t nl = batch * hfx::lri_factor_size(n, w);
+  const size_t bytes = (in + out + 1) * sizeof(double);   // [A, dA, B, dB] [X, dX] [error flag], then [factors]
+  const cudaError_t opened = g_lri.open(device);
+  if (opened != cudaSuccess) {
     cudaGetLastError();
-    return bad(HFX_ERR_CUDA, "hfx_lri_fit: stream");
+    return bad(opened == cudaErrorMemoryAllocation ? HFX_ERR_OOM : HFX_ERR_CUDA, "hfx_lri_fit: stream");
   }
   cudaStream_t s = g_lri.s;
-  const bool keep = bytes <= kLriKeep;
+  const bool keep = bytes + nl * sizeof(double) <= kLriKeep && g_lri.buffers();
   unsigned char* buf = g_lri.buf;
-  if (!keep && cudaMalloc(&buf, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return bad(HFX_ERR_OOM, "hfx_lri_fit: device memory");
+  if (!keep) {
+    auto get = [&](size_t n_bytes) {
+      if (!lri_oom("call") && cudaMalloc(&buf, n_bytes) == cudaSuccess) return true;
+      cudaGetLastError();
+      return false;
+    };
+    bool got = get(bytes + nl * sizeof(double));
+    if (!got && nl) {   // without room for the factors the solving CTAs make their own
+      nl = 0;
+      got = get(bytes);
+    }
+    if (!got) return bad(HFX_ERR_OOM, "hfx_lri_fit: device memory");
   }
   double* A_dev = reinterpret_cast<double*>(buf);
   double* gA = grad ? A_dev + nn : nullptr;

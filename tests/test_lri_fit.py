@@ -134,3 +134,22 @@ def test_gpu_fit_rounding():
             r = _solve_extended(np.tril(a) + np.tril(a, -1).T, b)
             err.append(float(np.linalg.norm((x - r).astype(float)) / np.linalg.norm(r.astype(float))))
     assert np.exp(np.mean(np.log(err))) <= 4.6e-16, err
+
+
+@pytest.mark.gpu
+def test_gpu_fit_without_memory(monkeypatch):
+    """A small batch needs no more memory than its own arrays take: without
+    the kept buffers it is solved all the same, and without any memory the
+    call says so (status 2) and works again afterwards."""
+    from paper_2412_11081_gb300 import hfx
+    d, A, B, dA, dB, _ = inputs.lri_pairs(3, 20, 15, 4, 9, seed=4)
+    ref = hfx.lri_fit(A, B, dA, dB)
+    monkeypatch.setenv("HFX_TEST_LRI_OOM", "scratch")
+    for got, want in zip(hfx.lri_fit(A, B, dA, dB), ref):
+        assert np.array_equal(got, want)
+    monkeypatch.setenv("HFX_TEST_LRI_OOM", "all")
+    with pytest.raises(hfx.HfxError) as e:
+        hfx.lri_fit(A, B, dA, dB)
+    assert e.value.status == 2
+    monkeypatch.delenv("HFX_TEST_LRI_OOM")
+    assert np.array_equal(hfx.lri_fit(A, B, dA, dB)[0], ref[0])
