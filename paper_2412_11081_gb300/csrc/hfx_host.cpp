@@ -954,7 +954,9 @@ void build_lists(hfx_plan* P, const double* L, const double* pos) {
   P->y_elems = 0;
   for (long long n : y_size) P->y_elems += n;
 
-  // (re)allocate list buffers
+  // (re)allocate list buffers (a plan whose memory runs out here has no lists
+  // until the next call makes them)
+  P->lists_ready = false;
   P->free_lists();
   P->nC = nC;
   P->nV = nV;
@@ -1919,6 +1921,10 @@ thread_local std::string g_create_error;
 
 void prepare_call(hfx_plan* P, const double* lattice, const double* positions_host) {
   validate_geometry(P->N, lattice, positions_host);
+  if (!P->lists_ready) {
+    build_lists(P, lattice, positions_host);
+    return;
+  }
   const double drift = list_drift(P, lattice, positions_host);
   if (2.0 * drift >= P->opt.skin) {
     if (P->opt.freeze_lists) fail(HFX_ERR_PAIRLIST_STALE, "atoms moved beyond skin/2 on a frozen plan");
@@ -2456,7 +2462,7 @@ extern "C" hfx_status hfx_energy_force_stress_noalloc(hfx_plan* P, const double*
     ck(cudaSetDevice(P->dev), "cudaSetDevice");
     double* base = noalloc_scratch(P->dev);
     validate_geometry(P->N, lattice, positions);
-    if (2.0 * list_drift(P, lattice, positions) >= P->opt.skin)
+    if (!P->lists_ready || 2.0 * list_drift(P, lattice, positions) >= P->opt.skin)
       fail(HFX_ERR_PAIRLIST_STALE,
            "atoms moved beyond skin/2; rebuilding the pair lists allocates (call hfx_energy_force_stress once)");
     // scratch layout: scan temporaries | Y blocks | V blocks

@@ -112,3 +112,24 @@ def test_stalled_pipeline_in_every_q2_shape(tiles, monkeypatch):
             monkeypatch.delenv("HFX_TEST_STALL_Q2_PRODUCER")
             E, F, S = p.evaluate(w.lattice, w.positions)
         assert abs(E - ref[0]) <= 1e-12 * abs(ref[0]) and rel(S, ref[2]) <= 1e-12
+
+
+@pytest.mark.parametrize("prec", [hfx.HFX_FP64, hfx.HFX_BF16X6])
+def test_list_rebuild_out_of_memory_leaves_the_plan_usable(prec):
+    """Memory that runs out while stale pair lists are made again: the old ones
+    are gone by then, so the next call makes them, at whatever geometry."""
+    pytest.importorskip("torch")
+    w = inputs.diamond8()
+    far = w.positions + np.random.default_rng(2).normal(0, 0.3, w.positions.shape)
+    a = CountingAllocator()
+    with hfx.Plan(w, precision=prec, allocator=a.hooks()) as p:
+        ref = p.evaluate(w.lattice, w.positions)
+        for more in (0, 7, 20):
+            a.budget = a.allocs + more
+            with pytest.raises(hfx.HfxError) as ei:
+                p.evaluate(w.lattice, far)
+            assert ei.value.status == 2
+            a.budget = 10 ** 9
+            E, F, S = p.evaluate(w.lattice, w.positions)
+            assert abs(E - ref[0]) <= 1e-12 * abs(ref[0]) and rel(F, ref[1]) <= 1e-12
+    assert not a.live
