@@ -1140,22 +1140,6 @@ double list_drift(const hfx_plan* P, const double* L, const double* pos) {
   return 2.0 * disp + P->list_Rabs * dl;
 }
 
-// With sub-blocks the tensor-memory kernels keep two Y stores, the warp-level
-// ones one: structures whose two would take more than 35 % of the device's
-// memory (perovskites of about 2,400 atoms) stay on the warp-level kernels
-// (HFX_Y_STORE_GB: that limit in GB).
-void fit_y_stores(hfx_plan* P, const double* L, const double* pos) {
-  if (!P->wide || !P->t1u) return;
-  size_t avail = 0, total = 0;
-  ck(cudaMemGetInfo(&avail, &total), "cudaMemGetInfo");
-  const char* e = std::getenv("HFX_Y_STORE_GB");
-  const double limit = e ? 1e9 * std::atof(e) : 0.35 * (double)total;
-  if (2.0 * sizeof(uint16_t) * (double)P->y_elems <= limit) return;
-  P->t1u = P->t2w = false;
-  P->t1u_subs = P->t1u_NAL = 1;
-  build_lists(P, L, pos);
-}
-
 // The tcgen05 first product for the plan's shapes: sub-blocks of at most 16
 // orbitals and 64 rows alpha; false where tensor memory (n_abf beyond ~100) or
 // shared memory do not hold them.
@@ -1323,23 +1307,50 @@ void setup_shapes(hfx_plan* P) {
   }
 }
 
+// D for the warp-level wide kernels: NP planes of rup16(n_ao(I)) x rup16(n_ao(J)) per block, row-major
+void split_density_w(hfx_plan* P) {
+  if (P->n_d == 0 || P->Dw) return;
+  std::vector<long long> off(P->n_d + 1, 0);
+  for (long long k = 0; k < P->n_d; ++k) {
+    const int* r = &P->d_index[5 * k];
+    const long long a = (P->n_ao[P->species[r[0]]] + 15) / 16 * 16, b = (P->n_ao[P->species[r[1]]] + 15) / 16 * 16;
+    off[k + 1] = off[k] + (long long)P->np * a * b;
+  }
+  if (!P->dw_off) P->dw_off = P->mem.alloc<long long>(P->n_d + 1);
+  P->Dw = P->mem.alloc<uint16_t>(off[P->n_d]);
+  upload(P->dw_off, off, P->stream);
+  DevPlan D = make_devplan(P, P->lat_ref.data());
+  ck(hfx::launch_dsplit_w(D, P->sp, P->Dw, P->dw_off, P->stream), "D pieces");
+  ck(cudaStreamSynchronize(P->stream), "D pieces");
+}
+
+// With sub-blocks the tensor-memory kernels keep two Y stores, the warp-level
+// ones one.  A plan whose memory runs out goes over to the latter: its per-call
+// stores are given back and the lists, whose buffers differ, made again.
+void use_one_y_store(hfx_plan* P) {
+  ck(cudaStreamSynchronize(P->stream), "stores");
+  auto drop = [&](uint16_t*& b, long long& cap) {
+    if (b) P->mem.release(b);
+    b = nullptr;
+    cap = 0;
+  };
+  drop(P->Cu, P->Cucap);
+  drop(P->Vu, P->Vucap);
+  drop(P->Yh, P->Yhcap);
+  drop(P->YspT, P->YspTcap);
+  drop(P->Vz, P->Vzcap);
+  drop(P->Zst, P->Zcap);
+  P->t1u = P->t2w = false;
+  P->t1u_subs = P->t1u_NAL = 1;
+  const std::vector<double> L = P->lat_ref, pos = P->pos_ref;
+  build_lists(P, L.data(), pos.data());
+  split_density_w(P);
+}
+
 // bf16 pieces of every D block (fixed for the plan)
 void split_density(hfx_plan* P) {
   if (!P->np || P->n_d == 0) return;
-  if (P->wide && !P->t1u) {   // NP planes of rup16(n_ao(I)) x rup16(n_ao(J)) per D block, row-major
-    std::vector<long long> off(P->n_d + 1, 0);
-    for (long long k = 0; k < P->n_d; ++k) {
-      const int* r = &P->d_index[5 * k];
-      const long long a = (P->n_ao[P->species[r[0]]] + 15) / 16 * 16, b = (P->n_ao[P->species[r[1]]] + 15) / 16 * 16;
-      off[k + 1] = off[k] + (long long)P->np * a * b;
-    }
-    P->dw_off = P->mem.alloc<long long>(P->n_d + 1);
-    P->Dw = P->mem.alloc<uint16_t>(off[P->n_d]);
-    upload(P->dw_off, off, P->stream);
-    DevPlan D = make_devplan(P, P->lat_ref.data());
-    ck(hfx::launch_dsplit_w(D, P->sp, P->Dw, P->dw_off, P->stream), "D pieces");
-    ck(cudaStreamSynchronize(P->stream), "D pieces");
-  }
+  if (P->wide && !P->t1u) split_density_w(P);
   std::vector<long long> off(P->n_d + 1, 0);
   for (long long k = 0; k < P->n_d; ++k) {
     const int* r = &P->d_index[5 * k];
@@ -1459,10 +1470,18 @@ void finish_evaluation(hfx_plan* P, hfx_stats* st, hfx_stats S, long long launch
 void evaluate(hfx_plan* P, const double* L, hfx_stats* st) {
   cudaStream_t s = P->stream;
   ck(cudaMemcpyAsync(P->d_lat, L, 9 * sizeof(double), cudaMemcpyHostToDevice, s), "H2D lattice");
+  if (P->wide && !P->t1u) split_density_w(P);   // (nothing, once made)
   const bool reuse = P->opt.freeze_lists && P->frozen_ready;
   const bool graph = P->opt.graph && reuse && !P->timing && !P->noalloc_call;
   if (!graph) {
-    evaluate_launches(P, L, st);
+    try {
+      evaluate_launches(P, L, st);
+    } catch (const Failure& f) {
+      // (a frozen plan's decisions sit in the lists: not after its first call)
+      if (f.status != HFX_ERR_OOM || !P->wide || !P->t1u || reuse) throw;
+      use_one_y_store(P);
+      evaluate_launches(P, L, st);
+    }
     if (st) st->graph_replayed = 0;
     return;
   }
@@ -2011,7 +2030,9 @@ hfx_status hfx_plan_create(const hfx_system* sys, const hfx_model* model, const 
     ck(cudaMemset(P->d_tot, 0, ntot * sizeof(long long)), "memset");
     setup_shapes(P);
     build_lists(P, sys->lattice, sys->positions);
-    fit_y_stores(P, sys->lattice, sys->positions);
+    // HFX_Y_STORE_GB: the most two Y stores may take (without it, until memory runs out)
+    const char* ys = std::getenv("HFX_Y_STORE_GB");
+    if (ys && P->wide && P->t1u && 2.0 * sizeof(uint16_t) * (double)P->y_elems > 1e9 * std::atof(ys)) use_one_y_store(P);
     split_density(P);
   });
   if (st != HFX_OK) {

@@ -114,6 +114,55 @@ def test_stalled_pipeline_in_every_q2_shape(tiles, monkeypatch):
         assert abs(E - ref[0]) <= 1e-12 * abs(ref[0]) and rel(S, ref[2]) <= 1e-12
 
 
+def test_wide_plan_without_room_for_two_y_stores():
+    """n_ao > 16: the tensor-memory kernels keep two Y stores, the warp-level
+    ones one.  Whichever store of the first evaluation cannot be had, the plan
+    goes on with one Y store and gives the same result; one that gets no more
+    memory at all says so and works again afterwards."""
+    pytest.importorskip("torch")
+    rng = np.random.default_rng(5)
+    pos = np.array([[0.1, 0.2, 0.0], [1.6, 1.5, 1.7]]) + rng.normal(0, 0.05, (2, 3))
+    w = inputs.cut_density(inputs.tiny_model([18, 7], [23, 11], [0, 1], np.eye(3) * 3.3, pos, r_c=1.4, seed=5), 4.0)
+
+    class Refusing(CountingAllocator):
+        refuse = ()
+
+        def alloc(self, n):
+            self.allocs += 1
+            if self.allocs in self.refuse:
+                self.refused = getattr(self, "refused", 0) + 1
+                return 0
+            p = self.torch.cuda.caching_allocator_alloc(n, 0, self.torch.cuda.current_stream())
+            self.live[int(p)] = n
+            return int(p)
+
+    a = Refusing()
+    with hfx.Plan(w, precision=hfx.HFX_BF16X6, allocator=a.hooks()) as p:
+        made = a.allocs
+        two = p.evaluate(w.lattice, w.positions, stats=True)
+        launches, stores = p.stats.kernel_launches, a.allocs - made
+    assert not a.live and stores >= 6
+    for k in range(1, stores + 1):
+        a = Refusing()
+        with hfx.Plan(w, precision=hfx.HFX_BF16X6, allocator=a.hooks()) as p:
+            a.refuse = (a.allocs + k,)
+            E, F, S = p.evaluate(w.lattice, w.positions, stats=True)
+            assert a.refused == 1 and p.stats.kernel_launches != launches, k   # (the other kernels ran)
+            assert abs(E - two[0]) <= 1e-5 * abs(two[0]) and rel(F, two[1]) <= 1e-5 and rel(S, two[2]) <= 1e-5
+            assert rel(p.evaluate(w.lattice, w.positions)[1], F) <= 1e-12
+        assert not a.live
+    a = Refusing()
+    with hfx.Plan(w, precision=hfx.HFX_BF16X6, allocator=a.hooks()) as p:
+        a.refuse = range(a.allocs + 2, 10 ** 9)
+        with pytest.raises(hfx.HfxError) as ei:
+            p.evaluate(w.lattice, w.positions)
+        assert ei.value.status == 2
+        a.refuse = ()
+        E, F, S = p.evaluate(w.lattice, w.positions)
+        assert rel(F, two[1]) <= 1e-5
+    assert not a.live
+
+
 @pytest.mark.parametrize("prec", [hfx.HFX_FP64, hfx.HFX_BF16X6])
 def test_list_rebuild_out_of_memory_leaves_the_plan_usable(prec):
     """Memory that runs out while stale pair lists are made again: the old ones
