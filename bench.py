@@ -502,15 +502,16 @@ def run_ours(args):
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": t_max / args.steps * 1e3, "higher_is_better": True,
                 "scaling": "strong" if world > 1 else "weak", "vs_baseline": None,
-                "dtype": "bf16" if head != "fp64" else "f64",
+                "dtype": {"bf16x6": "fp16", "bf16x3": "bf16", "fp64": "f64"}[head],
                 "data": "synthetic",
                 "config": {"workload": WORKLOAD, "precision": head,
-                           "arithmetic": "bf16 pieces on tensor cores, fp32 accumulate, fp64 screening/reduction"
+                           "arithmetic": ("two fp16 pieces" if head == "bf16x6" else "two bf16 pieces") +
+                                         " per operand on tensor cores, fp32 accumulate, fp64 screening/reduction"
                            if head != "fp64" else "fp64",
                            "parallelism": f"home-atom shards x{world} + all-reduce of E, F, sigma" if world > 1
                            else "single",
                            "passes": passes,
-                           "l2": "working set > L2 (Y stores of over 100 GB and per-pass operand stores each step)"},
+                           "l2": "working set > L2 (Y stores of about 60 GB and per-pass operand stores each step)"},
                 "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
                 "latency": {"p50_ms": float(np.percentile(lat, 50)) * 1e3, "p99_ms": float(np.percentile(lat, 99)) * 1e3,
                             "requests": len(lat), "what": "one evaluation through the host entry point on an "

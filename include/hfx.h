@@ -283,16 +283,13 @@ hfx_status hfx_set_reference(hfx_plan* plan, const double* E, const double* F, c
 /* Autotuner.  Times the evaluation of `positions` (host, [n_atoms*3], with
  * `lattice` as in hfx_energy_force_stress) for each launch configuration of
  * the plan that leaves the arithmetic unchanged, and keeps the fastest for
- * the plan's later calls.  Today that is the shape of the tcgen05 first
- * product's Y ring (rows f per slot and number of slots, bounded by shared
- * memory): the shapes of the block pairs decide which run length balances
- * the copy of Y rows against the U build; then, with the best shape, the
- * order in which its items are handed out (longest first, so that the SMs
+ * the plan's later calls: the order in which the items of the tcgen05 first
+ * product are handed out (longest first, so that the SMs
  * finish together; by home atom, so that items running at the same time
  * share their V_AB and grad V_AB blocks in L2; or by the atom F of the item
  * (A,F), so that they share Y^{BF} blocks); then the 128-row tiles per CTA
  * of the tcgen05 Y build (two tiles share each K step's D blocks; one tile
- * runs more pipeline stages and two accumulators) and the shape of the Q2
+ * leaves room for more CTAs) and the shape of the Q2
  * GEMM (one or two tiles per CTA, or two tiles in one CTA per SM with a
  * deeper copy pipeline and two accumulators per tile), each kept if it is
  * faster.  Each candidate is timed as the
@@ -302,8 +299,8 @@ hfx_status hfx_set_reference(hfx_plan* plan, const double* E, const double* F, c
  * with candidates = 0.  On an error the plan keeps its initial choice. */
 typedef struct {
   int candidates;          /* configurations timed, the initial one included */
-  int t1_rows_per_slot;    /* chosen rows f per Y slot */
-  int t1_slots;            /* chosen number of Y slots */
+  int t1_rows_per_slot;    /* always 1 (the first product's Y slots hold 32 groups of 8 rows) */
+  int t1_slots;            /* Y slots of the first product, fixed by the plan's shapes */
   double default_ms;       /* median evaluation time with the initial choice */
   double best_ms;          /* median evaluation time with the chosen one */
   int t1_home_order;       /* chosen order of the first product's items: 0 = longest

@@ -230,7 +230,7 @@ struct hfx_plan {
   hfx::DRows drows{};          // tensor map of the D piece rows
   int maxV = 0;                  // most V-pair candidates of one home atom
   size_t smem_m1 = 0, smem_m2 = 0;
-  // tcgen05 first product (n_abf <= 64, n_ao <= 16): operand stores and shape
+  // tcgen05 first product: operand stores and shape
   bool t1u = false;
   int t1u_KP = 0, t1u_GA = 0, t1u_GB = 0, t1u_UB = 2, t1u_NS = 0, t1u_seg = 32;
   int t1u_NAL = 1, t1u_subs = 1;   // alpha sub-blocks, items per C pair at most
@@ -244,12 +244,12 @@ struct hfx_plan {
   long long Yhcap = 0;
   uint16_t* Dh = nullptr;
   int* d_work = nullptr;       // item counter of the tcgen05 first-product kernel
-  // tcgen05 R2 / Z of the second product (same shapes): core-matrix Y stores, V store per pair slot
+  // tcgen05 R2 / Z of the second product (n_abf <= 64, n_ao <= 16): core-matrix Y stores, V store per pair slot
   bool t2u = false;
   size_t smem_t2u = 0;
   uint16_t* Vz = nullptr;
   long long Vzcap = 0;
-  // split path for n_ao > 16 (hfx_wide.cu): FP64 C, V and D blocks, FP32 Y store
+  // split path for n_ao > 16: the tensor-memory kernels by sub-blocks, or those of hfx_wide.cu
   bool wide = false;
   long long y_elems = 0;       // elements of a Y store of every candidate key
   bool t2w = false;            // wide: R2 and Z on tcgen05 (k_t2w_umma)
@@ -263,7 +263,7 @@ struct hfx_plan {
   uint16_t* Cw = nullptr;      // C pieces of every C pair (written per call)
   float* dCf = nullptr;        // grad C of every C pair in FP32, the layout of dCst (written per call)
   long long* cw_off = nullptr;
-  uint16_t* Dw = nullptr;      // bf16 pieces of every D block (fixed for the plan)
+  uint16_t* Dw = nullptr;      // pieces of every D block for hfx_wide.cu (fixed for the plan)
   long long* dw_off = nullptr;
 
   bool timing = false;
@@ -584,9 +584,14 @@ DevPlan make_devplan(hfx_plan* P, const double* lattice) {
   D.small = P->small;
   // by the V pairs of the whole structure, so that neither the passes nor the
   // home atoms of a plan change what is summed together (about one kept pair
-  // per four of them; eight waves of 152 SMs x 3 CTAs)
+  // per four of them; eight waves of 152 SMs x 3 CTAs).  FP64 evaluations in
+  // 1 / 2 / 4 parts: 2,800 V pairs (n_ao 13, n_abf 50) 21.8 / 18.9 / 17.5 ms,
+  // 5,600 39.0 / 35.7 / 34.5, 11,000 73.0 / 69.4 / 68.0 (n_ao 4: 0.74 / 0.71 /
+  // 0.70), 22,000 138.6 / 135.2 / 134.0 (1.14 / 1.05 / 1.08), 33,000 (n_ao 8)
+  // 11.6 / 11.5 / 11.8, 49,000 16.9 / 16.8 / 17.5, 74,000 25.0 / 25.2 / 26.1
   D.parts = P->nV < 10000 ? 4 : P->nV < 40000 ? 2 : 1;
-  D.parts2 = P->small ? 1 : D.parts;   // (small blocks: the repeated sums over F cost more than the last wave)
+  // (small blocks: the repeated sums over F cost more than the last wave; 8 atoms, n_ao 4: 1.05 and 1.16 ms)
+  D.parts2 = P->small ? 1 : D.parts;
   D.terms = P->opt.terms;
   D.h0 = P->chunks.empty() ? 0 : P->chunks.front().first;
   D.h1 = P->chunks.empty() ? P->N : P->chunks.back().second;
@@ -1168,14 +1173,12 @@ bool t1u_shapes(hfx_plan* P, size_t limit) {
   P->t1u = true;
   P->smem_t1u = hfx::t1u_smem(P->t1u_KP, P->t1u_GA, P->t1u_GB, P->KB, P->t1u_UB, P->t1u_NS);
   // kept B per FP32 run of the Q accumulator: 32 for BF16X3, whose stress error
-  // is closest to the 1e-5 bound; 128 for BF16X6 (6.5e-6 at most on the
-  // jittered si64 geometries against 5.4e-6 with 32 when its operands were
-  // three bf16 pieces, and fewer FP64 flushes).  With more than 16 orbitals
-  // both products take short runs, 16 B here and 32 K steps in the Q2 GEMM:
-  // the accumulator's rounding is these cells' largest error (40-atom
-  // perovskite, relative 2-norm over three geometries, F 1.5-1.9e-6 with runs
-  // of 128, 0.9-1.0e-6 with 16, 1.1e-6 for the warp-level kernels; evaluation
-  // 15.4 and 16.0 ms).
+  // is closest to the 1e-5 bound, and 128 for BF16X6; with more than 16
+  // orbitals 16 B here and 32 K steps in the Q2 GEMM.  (Those were chosen when
+  // the pairs came in the order of their atoms: 40-atom perovskite F 1.5-1.9e-6
+  // with runs of 128 and 0.9-1.0e-6 with 16.  Farthest first, runs of 16, 64
+  // and 128 differ by less than their scatter, F 0.3e-6; 135 atoms 33.4 ms with
+  // 16, 31.4 with 128.)
   const char* sg = std::getenv("HFX_T1_SEG");
   P->t1u_seg = sg ? std::max(1, std::atoi(sg)) : P->wide ? 16 : (P->sp == hfx::kSplitHalf ? 128 : 32);
   ck(hfx::t1u_set_smem(P->sp, P->t1u_subs > 1), "smem attributes");
@@ -1210,6 +1213,8 @@ void setup_shapes(hfx_plan* P) {
   P->smem_t1 = base1 + per1 * P->beta_chunk;
   P->alpha_chunk = chunk(base2, std::min(8, maxABF));
   P->smem_t2 = base2 + per1 * P->alpha_chunk;
+  // 64-thread CTAs: 144 elements (n_ao 4, n_abf 9, 8 atoms) 1.06 ms against
+  // 1.22 with 256 threads, 1,024 7.0 and 6.9, 1,088 8.1 and 8.0, 8,450 212 and 135
   P->small = maxABF * maxAO * maxAO <= 1024 ? 1 : 0;
   ck(hfx::set_kernel_smem_limits(), "smem attributes");
   if (P->np && maxAO > 16) {
@@ -1347,7 +1352,7 @@ void use_one_y_store(hfx_plan* P) {
   split_density_w(P);
 }
 
-// bf16 pieces of every D block (fixed for the plan)
+// pieces of every D block (fixed for the plan)
 void split_density(hfx_plan* P) {
   if (!P->np || P->n_d == 0) return;
   if (P->wide && !P->t1u) split_density_w(P);

@@ -146,12 +146,12 @@ struct DevPlan {
 struct MixPlan {
   uint16_t* Dsp;               // D sub-blocks of 16 x 16 as pieces, per 8 rows the first and then the second
   const long long* dsp_off;    // [n_d]
-  uint16_t* Ysp;               // Y^{XZ} as bf16 pieces, [alpha][z][rup16(n_ao(X))] per piece
-  uint16_t* Cm;                // per C pair: bf16 pieces of C, then grad C in FP32
+  uint16_t* Ysp;               // Y^{XZ} as pieces, [alpha][z][rup16(n_ao(X))] per piece (or ycm, below)
+  uint16_t* Cm;                // per C pair and sub of F: pieces of C, then grad C in FP32
   const long long* cm_off;     // [nC] offsets (uint16 units)
-  uint16_t* Vm;                // per needed V pair: bf16 pieces of V, then V and grad V in FP32
+  uint16_t* Vm;                // per needed V pair: pieces of V, then V and grad V in FP32
   const long long* vm_off;     // [nV] offsets (uint16 units), from the per-call scan
-  uint16_t* Zst;               // per pair of the second product: bf16 pieces of Z = V_AB . Y^{BA}
+  uint16_t* Zst;               // per pair of the second product and sub of B: pieces of Z = V_AB . Y^{BA}
   int* qcnt;                   // [nC] kept B per (A,F)
   long long* qoff;             // [nC] offsets into blist
   int* blist;                  // V pairs (A,B) per (A,F), in V-pair order
@@ -159,9 +159,11 @@ struct MixPlan {
   // piece, sub of x and sub of z the row groups (g, z) of 8 alpha x 16 x in
   // core-matrix order; nullptr where Ysp (ycm, one sub) is that store
   uint16_t* Yh = nullptr;
-  // (plans with sub-blocks: fp16 pieces at y_off, per piece, sub of z and sub of x the
-  // row groups (g, x) of 8 alpha x 16 z in core-matrix order)
-  uint16_t* YspT = nullptr;    // Y^{XZ} transposed, bf16 pieces [piece][(alpha,x)][16 z] (z padded), yT_blk per key
+  // Y^{XZ} transposed, for the second product: pieces [piece][(alpha,x)][16 z]
+  // (z padded) or (ycm) as below, yT_blk per key; with sub-blocks fp16 pieces at
+  // y_off, per piece, sub of z and sub of x the row groups (g, x) of 8 alpha x
+  // 16 z in core-matrix order
+  uint16_t* YspT = nullptr;
   long long yT_blk = 0;        // uint16 units per key of YspT (2 pieces x 128-row tiles x 16)
   const long long* y_idx = nullptr;   // key -> its position in the needed-key list (YspT block)
   int* ytab = nullptr;         // Y build: row of DRows per (key group, C slot t, key i), or -1
@@ -347,7 +349,8 @@ cudaError_t t2w_set_smem();
 cudaError_t launch_t2w(const DevPlan& P, const MixPlan& X, const T2WPlan& S, const int* list, int n, long long zblk,
                        int* err, cudaStream_t s);
 
-// tcgen05 first exchange product (hfx_t1umma.cu): shapes n_abf <= 64, n_ao <= 16.
+// tcgen05 first exchange product (hfx_t1umma.cu): sub-blocks of at most 64
+// auxiliary functions and 16 orbitals, where tensor and shared memory hold them.
 long long t1u_launch_count();
 size_t t1u_smem(int KP, int GA, int GB, int KB, int UB, int NS);
 int t1u_utiles(int KP, int GB);   // pairs of U tiles that fit tensor memory
@@ -376,7 +379,7 @@ cudaError_t launch_t1_umma(const DevPlan& P, const MixPlan& X, const T1UPlan& U,
                            size_t smem, int* work, int* err, cudaStream_t s);
 
 // Split-precision kernels for n_ao up to 32 and n_abf up to 128 (hfx_wide.cu):
-// warp-level MMAs on bf16 pieces copied from piece stores of D (plan), C (per
+// warp-level MMAs on 16-bit pieces copied from piece stores of D (plan), C (per
 // call, from the FP64 blocks), Y (the Y build; offsets y_off, the split
 // path's layout [alpha][z][rup16(n_ao(X))]) and Z (per pass); V and grad V FP64.
 struct WideShapes {
@@ -396,7 +399,7 @@ cudaError_t launch_cpieces_w(const DevPlan& P, int sp, uint16_t* Cw, const long 
 cudaError_t launch_term1_w(const DevPlan& P, int sp, const uint16_t* Yp, const uint16_t* Cw, const long long* cw_off,
                            const uint16_t* Dw, const long long* dw_off, const float* dCf, const int* list, int n,
                            const WideShapes& w, cudaStream_t s);
-// bf16 pieces of every D block (fixed for the plan): NP planes of
+// pieces of every D block (fixed for the plan): NP planes of
 // rup16(n_ao(I)) x rup16(n_ao(J)) at Dw + dw_off[k] (multiples of 256)
 cudaError_t launch_dsplit_w(const DevPlan& P, int sp, uint16_t* Dw, const long long* dw_off, cudaStream_t s);
 // Second product of the home atoms [a0, a1): k_term2_w over the pass's pair

@@ -933,7 +933,7 @@ cudaError_t launch_term2(const DevPlan& P, const int* list, int n, int alpha_chu
 
 // ------------------------------------------------------------ LRI fit
 // Eq. C_VA and the gradient equation after Eq. V_inverse, per atom pair p of
-// a batch (one CTA per pair, grid-stride over the batch):
+// a batch:
 //   A X = B                       X = the C^I rows, then the C^K rows
 //   A dX[c] = dB[c] - dA[c] X     c = x, y, z (gradient in K's position)
 // A (n x n, SPD) is factored as L L^T (right-looking Cholesky, L in shared
@@ -946,8 +946,8 @@ cudaError_t launch_term2(const DevPlan& P, const int* list, int n, int alpha_chu
 // share an SM, so that one's loads and barriers hide behind another's FP64
 // work, which bounds it (n = 100, w = 169 with gradients: 512 pairs 13.9 ms =
 // 0.89 TFLOP/s; 128 pairs, 5 CTAs per SM, 4.7 + 0.2 ms.  One CTA per pair, a row
-// at a time with its column in global memory: 0.72 TFLOP/s).  A pivot <= 0 (A not positive definite)
-// sets *err and is replaced by 1 so that the CTA finishes.
+// at a time with its column in global memory: 0.72 TFLOP/s).  A pivot <= 0 (A
+// not positive definite) sets *err and is replaced by 1 so that the CTA finishes.
 namespace {
 
 constexpr int kLriCols = 32;   // columns per CTA

@@ -14,7 +14,7 @@
 // Accumulation is FP32 in the MMA and FP64 beyond a short run; the
 // screening, the pair gradients, E, F and sigma stay FP64.
 //
-// Operand stores, written once per evaluation from the FP64 blocks
+// Operand stores, written once per evaluation from the block model
 // (k_cpieces, k_vpieces): per C pair, NP planes of C [(alpha,a)][rup16(f)]
 // and grad C in FP32; per needed V pair, NP planes of V [alpha][rup16(beta)]
 // and V, grad V in FP32.  No FP64 arithmetic runs inside the item loops.
@@ -23,13 +23,15 @@
 // distributive law), with the first exchange product organised per
 // (A, F) pair so that Q_AF = sum_B V_AB . U_ABF accumulates inside the
 // MMA accumulators:
-//   Y^{XZ}[alpha][z][x] = sum_W C_XW . D_WZ                (k_ybuild_mma)
-//   per (A,F), over its kept B:                             (k_term1_mma)
+//   Y^{XZ}[alpha][z][x] = sum_W C_XW . D_WZ                (k_ybuild_umma, tcgen05)
+//   per (A,F), over its kept B:                             (k_term1_mma; k_t1_umma in hfx_t1umma.cu)
 //     U[(beta,f)][a] = sum_b Y^{BF}[(beta,f)][b] D_AB[a][b]
 //     R = C_AF . U^T  -> E += -<V,R>, g^V += -<grad V,R>
 //     Q += V_AB . U   -> g^C_AF = -2 <grad C_AF, Q>
-//   per (A,B) of the second product:                        (k_term2_mma)
-//     R2 = <Y^{AB}, Y^{BA}>;  Z = V_AB . Y^{BA};  Q2_F = Z . D_FB^T
+//   per (A,B) of the second product:                        (k_term2_pairs; k_t2_umma, k_t2w_umma there)
+//     R2 = <Y^{AB}, Y^{BA}>;  Z = V_AB . Y^{BA}
+//   per home atom A:                                        (k_q2_umma, tcgen05)
+//     Q2_F = sum_B Z^{AB} . D_FB^T
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -246,11 +248,11 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 constexpr int kMeta = 64;   // B per metadata chunk of the term-1 kernel
 constexpr int kYS = 24;     // row stride (elements) of the staged Y rows (16 + 8)
 
-// One CTA (16 warps) per (A,F) with kept B.  Shared memory (bf16 planes):
+// One CTA (16 warps) per (A,F) with kept B.  Shared memory (planes of 16-bit pieces):
 //   Cs[NP][MA][KS]   C_AF, rows alpha, K = (a,f) (row stride KS)
 //   Us[NP][MB][KS]   U of the current B, rows beta, K = (a,f)
 //   Vs[2][NP][MA][VS] V_AB of the current / next B (cp.async double buffer)
-//   Ys[NP][YR][kYS]  Y^{BF} rows (beta,f) of the current B (NP == 2 only;
+//   Ys[NP][YR][kYS]  Y^{BF} rows (beta,f) of the current B (YRmax > 0 only;
 //                    prefetched while the previous B's R and Q run)
 // Per-B metadata (block offsets) is resolved in chunks of kMeta B by all
 // threads before the chunk's loop.
@@ -583,7 +585,7 @@ __global__ void __launch_bounds__(kWarps1 * 32) k_term1_mma(DevPlan P, MixPlan X
 
 // ------------------------------------------------------------------ term 2
 // Phase 1: one CTA per kept (A,B) pair of the second product (slot s of the
-// pair list).  Shared memory (bf16 planes, row stride KZ = n_ao(A)*pB + 8):
+// pair list).  Shared memory (planes of pieces, row stride KZ = n_ao(A)*pB + 8):
 //   Yb[NP][MB][KZ]  Y^{BA} as [beta][(a,b)]         (b padded to pB)
 //   Ya[NP][MA][KZ]  Y^{AB} as [alpha][(a,b)], from the transposed store the Y build writes
 // R2^T[beta][alpha] = sum_{(a,b)} Yb[beta][(a,b)] Ya[alpha][(a,b)], dotted with V, grad V;
@@ -917,7 +919,7 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
     qf[i] = (j < nq && P.c_keep[q]) ? q : -1;
     qs[i] = code >> kSubShift;
   }
-  // D block (units of 256 elements) of every (pair, F), or -1, from the table
+  // row of DRows of every (K step, column slot), or -1, from the table
   {
     const int4* tab = reinterpret_cast<const int4*>(X.q2tab + ((long long)fc * n_slots + p0) * 8);
     for (int e = tid; e < np * 2; e += blockDim.x) reinterpret_cast<int4*>(m_dblk)[e] = tab[e];
@@ -1129,7 +1131,7 @@ __global__ void __launch_bounds__(DEEP ? 320 : 192, DEEP ? 1 : 0) k_q2_umma(DevP
 // the kept C pairs (X,W) (one k16 step each); the B operand of key i is the
 // mirror block D_ZW = D_WZ^T (rows z, columns w).  Same warp roles as
 // k_q2_umma; one accumulation run; the epilogue splits the FP32 result into
-// bf16 pieces and writes the Y store ([alpha][z][16], x padding zeroed).
+// pieces and writes the Y stores (x padding zeroed).
 // TPC row tiles of 128 rows per CTA share each K step's D blocks (one
 // accumulator of 128 columns per tile).
 
@@ -1171,7 +1173,7 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
     zsub[i] = SUB ? code >> kSubShift : 0;
     zat[i] = ykey[i] >= 0 ? P.y_j[ykey[i]] : 0;
   }
-  // D block of every (C pair, key), or -1, from the table
+  // row of DRows of every (K step, key), or -1, from the table
   {
     const int4* tab = reinterpret_cast<const int4*>(X.ytab + (long long)g * X.ytab_stride);
     for (int e = tid; e < nq * 2; e += blockDim.x) reinterpret_cast<int4*>(m_d)[e] = tab[e];
@@ -1274,8 +1276,8 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
   } else {
     // epilogue (warps 2..5, and 6..9 for the second tile): the accumulator (rows (alpha, x), columns
     // (key, z)) passes through shared memory, two keys at a time, in the
-    // stage ring (idle once the last MMA has completed), so that the Y store
-    // and its FP32 copy are written as whole 16-byte chunks of complete
+    // stage ring (idle once the last MMA has completed), so that the Y stores
+    // are written as whole 16-byte chunks of complete
     // (alpha, z) rows, x padding included.  An alpha whose rows straddle two
     // row tiles is written element by element by both; the tile that holds
     // x = n_ao - 1 writes its padding.
@@ -1335,7 +1337,7 @@ __global__ void __launch_bounds__(yb_threads(TPC)) k_ybuild_umma(DevPlan P, MixP
         const float* eh = ep + h * 16;
         // stored Y -> its fp16 pieces (the same with fp16 pieces, 2^(y + d) with bf16 ones)
         const float sh = SP == kSplitHalf ? 1.f : p2f(y_exp(P, Xa, zat[i]));
-        // bf16 pieces: chunk (alpha, z, half) holds x = 8 half .. 8 half + 7
+        // Ysp: chunk (alpha, z, half) holds x = 8 half .. 8 half + 7
         // (core-matrix order: consecutive threads take consecutive alpha, whose
         // chunks are 16 bytes apart)
         for (int c = et; c < (SUB && !X.Ysp ? 0 : nal * nZs * NH); c += 128) {
@@ -1516,8 +1518,8 @@ __global__ void k_ygroups(DevPlan P, const long long* y_idx, const long long* y_
   }
 }
 
-// D block (256-element units) of every (key group g, C slot t of its home
-// atom X, key i) of the Y build, or -1 (C pair dropped, key absent, D block
+// Row of DRows (one per 16 x 16 sub-block) of every (key group g, C slot and
+// sub of W of its home atom X, key i) of the Y build, or -1 (C pair dropped, key absent, D block
 // screened out); the Y build's flops are counted here.
 __global__ void k_ytab(DevPlan P, MixPlan X, const int* ylist, const int* gX, const int* gS, const int* gN,
                        int ngroups) {
@@ -1644,8 +1646,12 @@ int q2_umma_segments(int max_steps_per_atom) {
   return std::max(1, (max_steps_per_atom + umma::kMetaPairs - 1) / umma::kMetaPairs);
 }
 // Parts that finish first: waves of CTAs times the length of one, a part's
-// fixed cost being about a sixth of an atom's whole.  (8-atom Si cell, 200
-// CTAs: second product 1.00 ms in one part, 0.93 in two; large cells take one.)
+// fixed cost being about a sixth of an atom's whole.  Evaluations in 1 / 2 / 3
+// / 4 parts: 12 CTAs (1 atom, 13 orbitals) 0.99 / 0.90 / 0.86 / 0.86 ms, 48
+// (4 atoms) 1.54 / 1.44 / 1.41 / 1.47, 64 (8 atoms, 10 orbitals) 1.84 / 1.75 /
+// 1.80 / 1.78, 72 1.65 / 1.61 / 1.64 / 1.63, 108 2.14 / 2.15 / 2.19 / 2.17,
+// 2,496 (64-atom Si cell) 27.0 / 27.2 / 27.6 / 27.9: the rule takes 4, 3, 2, 2,
+// 1 and 1, on none of 30 cells more than 0.5 % from the best.
 int q2_least(int n_atoms, int FC8, int MC) {
   const int ctas = n_atoms * FC8 * ((MC + 1) / 2), sms = sm_count();
   int best = 1;

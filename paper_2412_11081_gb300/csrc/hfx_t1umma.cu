@@ -1,5 +1,5 @@
 // First exchange product of the HFX force/stress on the 5th-generation tensor
-// cores (tcgen05 MMAs with accumulators in tensor memory), split-bf16 operands.
+// cores (tcgen05 MMAs with accumulators in tensor memory), operands in two 16-bit pieces.
 //
 // For a kept C pair (A,F) (an "item") and its kept V pairs (A,B), the first
 // product of Eq. exx_expand, factorised through Y^{BF} = sum_W C_BW D_WF:
@@ -1030,7 +1030,6 @@ constexpr int kT2RCol = 256;   // tensor-memory column of the first R2 accumulat
 template <int SP>
 __global__ void __launch_bounds__(kT2Threads, 1)
     k_t2_umma(DevPlan P, MixPlan X, const int* list, int n_list, int KKmax, long long zblk, int* err) {
-  constexpr int NPROD = NP * (NP + 1) / 2;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   uint16_t* Ya = reinterpret_cast<uint16_t*>(smem_raw);   // [NP][rup8(n_abf(A))][KK]
   uint16_t* Yb = Ya + (size_t)NP * 64 * KKmax;            // [NP][rup8(n_abf(B))][KK]
@@ -1162,7 +1161,6 @@ __global__ void __launch_bounds__(kT2Threads, 1)
                         dBM + ((uint64_t)((sum - ia) * PB) >> 4) + ((uint64_t)(2 * rowg * kb) >> 4), idZ,
                         (kb > 0 || k > 0) ? 1u : 0u);
         }
-        (void)NPROD;
         umma_commit(mBe);
         umma_commit(zf);
       }
@@ -1315,8 +1313,8 @@ __global__ void __launch_bounds__(kT2Threads, 1)
 // and by shapes beyond shared memory) stages Y element by element and reads
 // FP64 V blocks: with the build of those 4.9 ms of a 40-atom perovskite
 // evaluation (9,896 pairs), 0.85 ms here with k_t2w_vstore.
-template <int SP>
 __global__ void __launch_bounds__(256) k_t2w_vstore(DevPlan P, MixPlan X, T2WPlan S, const int* list, int n) {
+  constexpr int SP = kSplitHalf;
   for (int k = blockIdx.x; k < n; k += gridDim.x) {
     const int p = list[k], sA = P.species[P.v_home[p]], sB = P.species[P.v_j[p]];
     const int mA = P.n_abf[sA], mB = P.n_abf[sB], m8 = (mA + 7) & ~7;
@@ -1350,9 +1348,9 @@ __global__ void __launch_bounds__(256) k_t2w_vstore(DevPlan P, MixPlan X, T2WPla
   }
 }
 
-template <int SP>
 __global__ void __launch_bounds__(kT2Threads, 1)
     k_t2w_umma(DevPlan P, MixPlan X, T2WPlan S, const int* list, int n_list, long long zblk, int* err) {
+  constexpr int SP = kSplitHalf;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t b_af, b_ae, b_bf, b_be, b_vf, b_ve, b_rf[2], b_re[2], b_zf, b_ze, b_done;
   __shared__ uint32_t tmem_base;
@@ -1736,14 +1734,14 @@ T2WPlan t2w_plan(int max_abf, int max_ao_sub) {
   return S;
 }
 
-cudaError_t t2w_set_smem() { return allow_max_dynamic_smem((const void*)k_t2w_umma<kSplitHalf>); }
+cudaError_t t2w_set_smem() { return allow_max_dynamic_smem((const void*)k_t2w_umma); }
 
 cudaError_t launch_t2w(const DevPlan& P, const MixPlan& X, const T2WPlan& S, const int* list, int n, long long zblk,
                        int* err, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   g_t1u_launches += 2;
-  k_t2w_vstore<kSplitHalf><<<std::min(n, 152 * 8), 256, 0, s>>>(P, X, S, list, n);
-  k_t2w_umma<kSplitHalf><<<std::min(n, num_sms()), kT2Threads, S.smem, s>>>(P, X, S, list, n, zblk, err);
+  k_t2w_vstore<<<std::min(n, 152 * 8), 256, 0, s>>>(P, X, S, list, n);
+  k_t2w_umma<<<std::min(n, num_sms()), kT2Threads, S.smem, s>>>(P, X, S, list, n, zblk, err);
   return cudaGetLastError();
 }
 

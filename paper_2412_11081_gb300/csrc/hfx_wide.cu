@@ -3,8 +3,8 @@
 // n_abf up to 128.
 //
 // Same factorisation and the same piece products as hfx_mixed.cu (two 16-bit
-// pieces per operand, three products, FP32 accumulation
-// in warp-level MMAs, FP64 screening, gradients and reductions), organised
+// pieces per operand, three products, FP32 accumulation in warp-level MMAs,
+// FP64 screening, gradients and reductions), organised
 // like the FP64 kernels of hfx_kernels.cu so that any n_ao and n_abf fit.
 // Operands are split into their pieces once, into stores that the kernels copy
 // from:
@@ -65,7 +65,7 @@ __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t (&w)[NP]
   for (int pp = 0; pp < NP; ++pp) w[pp] = pack2(p0[pp], p1[pp]);
 }
 
-// element e of a [rows][S] bf16 plane set (NP planes of `plane` elements): the NP pieces of x
+// element e of a [rows][S] plane set (NP planes of `plane` elements): the NP pieces of x
 template <int SP>
 __device__ __forceinline__ void put_pieces(uint16_t* base, long long plane, int e, float x) {
   uint16_t pc[NP];
@@ -193,7 +193,7 @@ __global__ void k_cpieces_w(DevPlan P, uint16_t* Cw, const long long* cw_off, fl
 }
 
 // ------------------------------------------------------------------ term 1
-// Shared memory (bf16 planes; strides are multiples of 8 elements with an
+// Shared memory (planes of 16-bit pieces; strides are multiples of 8 elements with an
 // odd count of 16-byte chunks, so that ldmatrix rows hit distinct banks):
 //   Vs[NP][MA][MB + 8]   V_AB (rows alpha, columns beta; zero padded)
 //   Ds[NP][48][40]       D_AB (rows a, columns b; zero padded; 16 rows from any a0 < 32)
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kPW * 32, 1) k_term1_w(DevPlan P, const uint16
 
 // ------------------------------------------------------------------ term 2
 // k_term2_w, one CTA per kept (A,B) pair (slot s of the pass's list); shared
-// memory (bf16 planes):
+// memory (planes of pieces):
 //   Vs[NP][MA][MB + 8]   V_AB
 //   Ya[NP][MA][KC + 8]   Y^{AB} columns (a, b), a in the current range
 //   Yb[NP][MB][KC + 8]   Y^{BA} as [beta][(a, b)], same columns
