@@ -70,8 +70,9 @@ __device__ __forceinline__ double fx_get(const unsigned long long* cell) {
 }
 
 // ------------------------------------------------------ the plan's sums
-// FP64 atomic adds (E in kESlots sums by CTA, since each addition rounds at the
-// size the sum has reached), or the fixed-point cells of a deterministic plan
+// FP64 atomic adds (the FP64 kernels add E to kESlots sums by CTA, since each
+// addition rounds at the size the sum has reached; the split kernels, whose E
+// is good to 1e-6, to one), or the fixed-point cells of a deterministic plan
 // (P.fxC != nullptr).  Indices are those of the FP64 arrays.
 __device__ __forceinline__ void add_gC(const DevPlan& P, long long i, double v) {
   if (P.fxC) fx_add(P.fxC + 2 * i, v);
@@ -81,9 +82,9 @@ __device__ __forceinline__ void add_gV(const DevPlan& P, long long i, double v) 
   if (P.fxC) fx_add(P.fxV + 2 * i, v);
   else atomicAdd(P.gV + i, v);
 }
-__device__ __forceinline__ void add_E(const DevPlan& P, double v) {
+__device__ __forceinline__ void add_E(const DevPlan& P, double v, int slot = 0) {
   if (P.fxC) fx_add(P.fxA, v);
-  else atomicAdd(P.acc + ACC_E + (blockIdx.x & (kESlots - 1)), v);
+  else atomicAdd(P.acc + ACC_E + slot, v);
 }
 __device__ __forceinline__ void add_W(const DevPlan& P, int c, double v) {   // virial component c
   if (P.fxC) fx_add(P.fxA + 2 * (1 + c), v);

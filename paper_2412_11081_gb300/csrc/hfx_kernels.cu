@@ -388,7 +388,7 @@ __device__ __forceinline__ void add_pair(const DevPlan& P, int p, const double (
   double s = 0.0;
   for (int k = 0; k < nwarp; ++k) s += ew[k][threadIdx.x];
   if (s == 0.0) return;
-  if (threadIdx.x == 0) dev::add_E(P, -s);
+  if (threadIdx.x == 0) dev::add_E(P, -s, blockIdx.x & (kESlots - 1));
   else dev::add_gV(P, 3 * p + (int)threadIdx.x - 1, -s);
 }
 

@@ -796,7 +796,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       const Sub sb = item_sub<SUB>(it.sub(), P.n_abf[sA], P.n_ao[sA], P.n_ao[P.species[P.c_j[q]]]);
       const int nA = sb.nA, mA = sb.mA, nF = sb.nF;
       const int hA = P.c_home[q], eR = P.sc.c[hA] + kUExp + P.sc.d[hA];   // (R: and d[B] + y[B])
-      const double q1 = pscale_d<SP>(-(P.sc.q[hA] + kUExp + P.sc.d[hA] + P.sc.d[P.c_j[q]]));
       const long long b0 = X.qoff[q];
       const float* Cf = reinterpret_cast<const float*>(U.Cu + (long long)it.kk * U.cu_blk + (CB >> 1));
       int run = 0;
@@ -915,6 +914,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
               for (int c = 0; c < 4; ++c) e[c] = warp_sum_d(e[c]);
               if (lane == 0) {
+                const double q1 = pscale_d<SP>(-(P.sc.q[hA] + kUExp + P.sc.d[hA] + P.sc.d[P.c_j[q]]));
                 if (e[0] != 0.0) dev::add_E(P, -e[0] * q1);
 #pragma unroll
                 for (int c = 0; c < 3; ++c)
