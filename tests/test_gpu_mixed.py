@@ -279,3 +279,17 @@ def test_small_species_beside_a_large_one(n_ao, n_abf, route, what, k, prec, tol
         E0, F0, S0, _ = run(w, hfx.HFX_FP64, theta=zero, home=home)
         E, F, S, _ = run(w, prec, theta=zero, home=home)
         assert abs(E - E0) <= tol * abs(E0) and rel(F, F0) <= tol and rel(S, S0) <= tol, (home, abs(E - E0) / abs(E0), rel(F, F0), rel(S, S0))
+
+
+@pytest.mark.parametrize("prec,tol", [(hfx.HFX_BF16X6, BOUND), (hfx.HFX_BF16X3, 1e-4)])
+@pytest.mark.parametrize("n_ao,n_abf", [([5, 3], [11, 7]), ([9, 5], [70, 30]), ([18, 5], [23, 11])])
+@pytest.mark.parametrize("what", ["C", "V", "D"])
+def test_species_without_blocks(n_ao, n_abf, what, prec, tol):
+    """A species whose C templates, V templates or density blocks are all zero
+    has no bound to scale by: the other's results stay as they are."""
+    w = _uneven(n_ao, n_abf, what, 2000)   # (2^-2000 is zero)
+    E0, F0, S0, _ = run(w, hfx.HFX_FP64)
+    E, F, S, _ = run(w, prec)
+    assert np.isfinite(E) and np.isfinite(F).all() and np.isfinite(S).all()
+    assert abs(E - E0) <= tol * abs(E0) and rel(S, S0) <= tol
+    assert np.max(np.abs(F - F0)) <= tol * max(np.max(np.abs(F0)), abs(E0))

@@ -142,3 +142,32 @@ def test_errors_of_the_135_atom_perovskite():
     norm = np.linalg.norm
     assert abs(E - E0) <= 2.3e-6 * abs(E0) and norm(F - F0) <= 1.2e-6 * norm(F0)
     assert norm(S - S0) <= 1.5e-6 * norm(S1), norm(S - S0) / norm(S1)
+
+
+@pytest.mark.parametrize("n_ao,n_abf", [([17, 16], [64, 65]), ([18, 13], [97, 60]), ([32, 9], [33, 16]), ([17, 2], [112, 3])])
+def test_sub_block_edges_bf16x3(n_ao, n_abf):
+    """HFX_BF16X3 with n_ao > 16: the tensor-memory first product over one and
+    two sub-blocks of auxiliary functions (and shapes beyond it), the
+    warp-level second product.  Four operands of 2^-16 each (6e-5), taken as
+    1e-4, of the FP64 path's values; the energy of either product (the first
+    one's nearly vanishes in one of these cells) in parts of the whole."""
+    rng = np.random.default_rng(21)
+    pos = np.array([[0.1, 0.2, 0.0], [1.6, 1.5, 1.7]]) + rng.normal(0, 0.05, (2, 3))
+    w = inputs.cut_density(inputs.tiny_model(n_ao, n_abf, [0, 1], np.eye(3) * 3.3, pos, r_c=1.4, seed=21), 4.0)
+    whole = abs(run(w, hfx.HFX_FP64)[0])
+    for terms in (1, 2):
+        E0, F0, S0, st0 = run(w, hfx.HFX_FP64, terms=terms)
+        E, F, S, st = run(w, hfx.HFX_BF16X3, terms=terms)
+        assert st["triplets"] == st0["triplets"] and st["term2_pairs"] == st0["term2_pairs"]
+        assert abs(E - E0) <= 1e-4 * whole and rel(F, F0) <= 1e-4 and rel(S, S0) <= 1e-4
+
+
+def test_the_y_store_limit_changes_the_kernels(monkeypatch):
+    """HFX_Y_STORE_GB=0 runs the warp-level kernels (other launches), and they
+    agree with the tensor-memory ones within the contract."""
+    w = wide_two_species(seed=9)
+    E0, F0, S0, st0 = run(w, hfx.HFX_BF16X6)
+    monkeypatch.setenv("HFX_Y_STORE_GB", "0")
+    E, F, S, st = run(w, hfx.HFX_BF16X6)
+    assert st["kernel_launches"] != st0["kernel_launches"]
+    assert max(errs((E, F, S), (E0, F0, S0))) <= BOUND
